@@ -1,0 +1,196 @@
+// gf_coop.cuh -- one ray per warp: the warp traverses the ray's tree together
+// and shares out its chords.
+#pragma once
+#include "gf_device.cuh"
+#include "gf_trace.cuh"
+
+namespace gf {
+
+// Traversal of one ray by a whole warp: a shared stack of four-wide nodes, up to
+// 32 popped per step (one per lane) and their hit children pushed; the leaves
+// reached are queued, and every 32 queued leaves (and the last ones) make a
+// round, in which round(j) is called by every lane, j the sorted primitive of the
+// lane's leaf or -1.
+//
+// The ray lives in registers (the same in every lane), so a step has no lane-
+// dependent ray data and no branch that parts the lanes.  A step pushes at most
+// 128 nodes; above kCoopStack - kCoopMargin entries the warp goes depth first
+// (one node per step, at most 3 more entries per tree level, 32 levels), so the
+// stack holds a full step plus a whole descent.
+constexpr int kCoopStack = 512;
+constexpr int kCoopMargin = 200;
+constexpr int kCoopLeafQ = 160;  // <= 31 left + 128 new
+static_assert(kCoopStack - kCoopMargin + 96 + 3 * 32 <= kCoopStack, "a full step, then a descent");
+struct CoopTrav {
+  int stk[kCoopStack];
+  int lq[kCoopLeafQ];
+};
+
+template <class Round>
+__device__ __forceinline__ void coop_traverse(const DevField& F, CoopTrav& Q,
+                                              unsigned long long mask, float3 o, float3 inv,
+                                              float t0, float t1, uint32_t lane, Counters& cnt,
+                                              Round&& round) {
+  const unsigned lt = (1u << lane) - 1u;
+  // a one-primitive field has no internal node: its leaf is queued at once
+  int sp = F.root >= 0 ? 1 : 0, lq_n = F.root >= 0 ? 0 : 1;
+  if (lane == 0) {
+    if (F.root >= 0) Q.stk[0] = 0;
+    else Q.lq[0] = 0;
+  }
+  __syncwarp();
+  // every node enters the stack at most once
+  const long long max_it = F.n_nodes4 + 64;
+  for (long long it = 0;; ++it) {
+    if (it > max_it) {
+      if (lane == 0) set_err(F, ERR_GUARD);
+      break;
+    }
+    int take = sp < 32 ? sp : 32;
+    if (sp > kCoopStack - kCoopMargin) take = 1;  // near capacity: depth first
+    const int node = (int)lane < take ? Q.stk[sp - take + (int)lane] : -1;
+    __syncwarp();
+    sp -= take;
+    int ch[4] = {0, 0, 0, 0};
+    unsigned hit = 0u;
+    if (node >= 0 && (int64_t)node >= F.n_nodes4) {
+      set_err(F, ERR_INDEX);  // a node beyond the tree: skipped
+    } else if (node >= 0) {
+      ++cnt.nodes;
+      hit = node4_hits(F.nodes4 + node, o, inv, mask, t0, t1, ch);
+    }
+    // push internal children, queue leaves (ballots keep the entries contiguous)
+    int np = 0, nl = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const bool h = (hit >> k & 1u) != 0u;
+      const unsigned bp = __ballot_sync(kFull, h && ch[k] >= 0);
+      const unsigned bl = __ballot_sync(kFull, h && ch[k] < 0);
+      if (h && ch[k] >= 0) {
+        const int pos = sp + np + __popc(bp & lt);
+        if (pos < kCoopStack) Q.stk[pos] = ch[k];
+      }
+      if (h && ch[k] < 0) Q.lq[lq_n + nl + __popc(bl & lt)] = ~ch[k];
+      np += __popc(bp);
+      nl += __popc(bl);
+    }
+    if (sp + np > kCoopStack) {
+      if (lane == 0) set_err(F, ERR_STACK);
+      np = kCoopStack - sp;
+    }
+    sp += np;
+    lq_n += nl;
+    __syncwarp();
+    const bool more = sp > 0;
+    while (lq_n >= 32 || (!more && lq_n > 0)) {
+      const int tk = lq_n < 32 ? lq_n : 32;
+      int j = (int)lane < tk ? Q.lq[lq_n - tk + (int)lane] : -1;
+      __syncwarp();
+      lq_n -= tk;
+      if (j >= 0) ++cnt.leaves;
+      if ((int64_t)j >= F.n) {  // a leaf beyond the records
+        set_err(F, ERR_INDEX);
+        j = -1;
+      }
+      round(j);
+      __syncwarp();
+    }
+    if (!more && lq_n == 0) break;
+  }
+}
+
+// inclusive prefix sum over the warp's lanes
+__device__ __forceinline__ int warp_incl_sum(int x, uint32_t lane) {
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int y = __shfl_up_sync(kFull, x, d);
+    if ((int)lane >= d) x += y;
+  }
+  return x;
+}
+
+// the lanes' compensated sums combined in a fixed butterfly order: every lane
+// receives the total as a pair
+__device__ __forceinline__ void warp_sum_pair(float& s, float& c) {
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const float so = __shfl_xor_sync(kFull, s, off), co = __shfl_xor_sync(kFull, c, off);
+    float t, e;
+    two_sum(s, so, t, e);
+    s = t;
+    c = __fadd_rn(__fadd_rn(c, co), e);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Optical depth of one ray (Eq. 2-3).  A round sets up the chords of 32 leaves,
+// one per lane.  Gauss-Legendre mode: the nodes of those chords are shared out
+// evenly among the lanes (the rule per chord as in det_tau): every chord writes
+// its lane number over its stretch of the round's node list, so that node f of the
+// round finds its chord with one byte load.  Closed form: each lane integrates its
+// own chord.  Every term goes into its lane's compensated sum.
+// ---------------------------------------------------------------------------
+struct CoopChord {
+  float mid, hl, y2, y1, y0, scale, B, delta;
+  int off;  // first node of the chord's rule in the tables, less its start in the round
+};
+struct CoopQ {
+  CoopTrav t;
+  CoopChord ch[32];  // the round's chords, one per lane
+  unsigned char own[32 * gl_n(kNumRules - 1)];  // node of the round -> lane of its chord
+};
+
+template <int MODE>  // GF_TR_DETERMINISTIC or GF_TR_CLOSED_FORM
+__device__ __forceinline__ void coop_tau(const DevField& F, CoopQ& Q, const Mask& M, float3 o,
+                                         float3 v, float tmin, float tmax, const float* glx,
+                                         const float* glw, uint32_t lane, float& s_acc,
+                                         float& c_acc, Counters& cnt) {
+  const float3 inv = safe_inv(v);
+  float t0, t1;
+  if (M.bits == 0ull || !scene_span(F, o, inv, tmin, tmax, t0, t1)) return;
+  if (lane == 0) cnt.windows += 1;
+  coop_traverse(F, Q.t, M.bits, o, inv, t0, t1, lane, cnt, [&](int j) {
+    int n = 0, off = 0;
+    Chord ch;
+    float w;
+    const bool ok = j >= 0 && prim_chord(F, j, o, v, tmin, tmax,
+                                         [&](uint32_t cl) { return mask_weight(M, cl); }, w, ch);
+    if (ok) ++cnt.chords;
+    if (MODE == GF_TR_CLOSED_FORM) {
+      if (ok) neumaier_add(s_acc, c_acc, w * chord_closed(F.wd, ch));
+      return;
+    }
+    const float len = ch.dtout - ch.dtin;
+    if (ok) gl_pick(gl_rule(sqrtf(ch.a) * len + 0.5f * fabsf(ch.B) * len), n, off);
+    const int incl = warp_incl_sum(n, lane);
+    const int total = __shfl_sync(kFull, incl, 31);
+    if (ok) {
+      const int start = incl - n;
+      CoopChord C;
+      C.mid = 0.5f * (ch.dtin + ch.dtout);
+      C.hl = 0.5f * len;
+      C.y2 = -0.5f * kLog2e * ch.a;
+      C.y1 = -kLog2e * ch.b;
+      C.y0 = -0.5f * kLog2e * ch.g;
+      C.scale = w * ch.absA * C.hl;
+      C.B = ch.B;
+      C.delta = ch.delta;
+      C.off = off - start;
+      Q.ch[lane] = C;
+      // rules hold a multiple of 4 nodes, so a stretch is whole 32-bit words
+      uint32_t* own4 = reinterpret_cast<uint32_t*>(Q.own) + (start >> 2);
+      for (int k = 0; k < (n >> 2); ++k) own4[k] = lane * 0x01010101u;
+    }
+    __syncwarp();
+    for (int f = (int)lane; f < total; f += 32) {
+      const CoopChord& C = Q.ch[Q.own[f]];
+      const int k = C.off + f;
+      const float dt = fmaf(C.hl, glx[k], C.mid);
+      const float y = fmaf(fmaf(C.y2, dt, C.y1), dt, C.y0);
+      neumaier_add(s_acc, c_acc, C.scale * glw[k] * ex2f(y) * cosf(fmaf(C.B, dt, C.delta)));
+      ++cnt.evals;
+    }
+  });
+}
+
+}  // namespace gf

@@ -523,36 +523,14 @@ __device__ __forceinline__ void slab_interval(float3 o, float3 inv, float lx, fl
   tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fmaxf(tz0, tz1));
 }
 
-// the subtree that lane `sub` of a group of `group` lanes (a power of two)
-// walks: log2(group) levels down from the root along the bits of sub, most
-// significant first, so the group's lanes cover the tree without overlap.  A
-// leaf met on the way belongs to the lane whose remaining bits are all zero.
-// Returns an internal node (>= 0), a leaf ~j (< 0), or kNoStart.
-constexpr int kNoStart = -2147483647 - 1;
-__device__ __forceinline__ int group_start(const DevField& F, int sub, int group) {
-  int node = F.root < 0 ? ~0 : F.root;
-  for (int l = 31 - __clz(group) - 1; l >= 0; --l) {
-    if (node < 0) return (sub & ((2 << l) - 1)) == 0 ? node : kNoStart;
-    const int4 d = __ldg(&F.nodes[node].d);
-    node = (sub >> l & 1) ? d.y : d.x;
-  }
-  return node;
-}
-
-// traversal of the subtree `start` (group_start's result)
 template <class TestFn, class LeafFn>
-__device__ __forceinline__ void traverse_from(const DevField& F, int start, float3 o, float3 inv,
-                                              unsigned long long mask, TestFn& test, LeafFn& leaf,
-                                              unsigned long long& nvis,
-                                              unsigned long long& nleaves) {
-  if (start == kNoStart) return;
-  if (start < 0) {
-    if ((int64_t)~start >= F.n) {
-      set_err(F, ERR_INDEX);
-      return;
-    }
+__device__ __forceinline__ void traverse_ray(const DevField& F, float3 o, float3 inv,
+                                             unsigned long long mask, TestFn& test, LeafFn& leaf,
+                                             unsigned long long& nvis,
+                                             unsigned long long& nleaves) {
+  if (F.root < 0) {  // a one-primitive field has no internal node
     ++nleaves;
-    leaf(~start);
+    leaf(0);
     return;
   }
   // lanes that entered together stay together: they reconverge after every
@@ -561,7 +539,7 @@ __device__ __forceinline__ void traverse_from(const DevField& F, int start, floa
   int st_node[kStack];
   float st_tn[kStack];
   int sp = 0;
-  int node = start;            // next internal node, -1 once the tree is exhausted
+  int node = F.root;           // next internal node, -1 once the tree is exhausted
   int pend0 = -1, pend1 = -1;  // queued leaves
   // each internal node is fetched at most once per traversal
   const long long max_steps = F.n + 64;
@@ -646,13 +624,48 @@ __device__ __forceinline__ void traverse_from(const DevField& F, int start, floa
   }
 }
 
-// traversal of the whole tree
-template <class TestFn, class LeafFn>
-__device__ __forceinline__ void traverse_ray(const DevField& F, float3 o, float3 inv,
-                                             unsigned long long mask, TestFn& test, LeafFn& leaf,
-                                             unsigned long long& nvis,
-                                             unsigned long long& nleaves) {
-  traverse_from(F, F.root < 0 ? ~0 : F.root, o, inv, mask, test, leaf, nvis, nleaves);
+// byte k of x as a float, exactly: 0x4B0000xx is 2^23 + xx
+__device__ __forceinline__ float byte_float(uint32_t x, int k) {
+  return __int_as_float((int)__byte_perm(x, 0x4Bu, (uint32_t)k | 0x4550u)) - 8388608.0f;
+}
+
+// The children of a four-wide node that overlap [ta, te] of the ray and hold one
+// of the ray's cells (bit k: child k); ch receives the children.
+__device__ __forceinline__ unsigned node4_hits(const Node4* N, float3 o, float3 inv,
+                                               unsigned long long mask, float ta, float te,
+                                               int ch[4]) {
+  const float4 v0 = __ldg(&N->v0), v1 = __ldg(&N->v1);
+  const uint4 q = __ldg(&N->q);
+  const int4 c4 = __ldg(&N->child);
+  const uint4 m01 = __ldg(&N->m01), m23 = __ldg(&N->m23);
+  const uint32_t qlx = __float_as_uint(v1.z), qly = __float_as_uint(v1.w);
+  // slab distances straight from the codes: t = (lo + c s - o) inv = c (s inv) + (lo - o) inv
+  const float ax = v0.w * inv.x, ay = v1.x * inv.y, az = v1.y * inv.z;
+  const float bx = (v0.x - o.x) * inv.x, by = (v0.y - o.y) * inv.y, bz = (v0.z - o.z) * inv.z;
+  const unsigned long long mk[4] = {
+      (unsigned long long)m01.x | ((unsigned long long)m01.y << 32),
+      (unsigned long long)m01.z | ((unsigned long long)m01.w << 32),
+      (unsigned long long)m23.x | ((unsigned long long)m23.y << 32),
+      (unsigned long long)m23.z | ((unsigned long long)m23.w << 32)};
+  ch[0] = c4.x;
+  ch[1] = c4.y;
+  ch[2] = c4.z;
+  ch[3] = c4.w;
+  // near and far planes by the ray's direction signs, chosen once per node
+  const uint32_t nx = inv.x >= 0.f ? qlx : q.y, fx = inv.x >= 0.f ? q.y : qlx;
+  const uint32_t ny = inv.y >= 0.f ? qly : q.z, fy = inv.y >= 0.f ? q.z : qly;
+  const uint32_t nz = inv.z >= 0.f ? q.x : q.w, fz = inv.z >= 0.f ? q.w : q.x;
+  unsigned hit = 0u;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float txn = fmaf(byte_float(nx, k), ax, bx), txf = fmaf(byte_float(fx, k), ax, bx);
+    const float tyn = fmaf(byte_float(ny, k), ay, by), tyf = fmaf(byte_float(fy, k), ay, by);
+    const float tzn = fmaf(byte_float(nz, k), az, bz), tzf = fmaf(byte_float(fz, k), az, bz);
+    const float tn = fmaxf(fmaxf(txn, tyn), fmaxf(tzn, ta));
+    const float tf = fminf(fminf(txf, tyf), fminf(tzf, te));
+    if ((mk[k] & mask) && tn <= tf) hit |= 1u << k;
+  }
+  return hit;
 }
 
 }  // namespace gf

@@ -373,9 +373,6 @@ struct DetLeaf {
   const float* glw;
   float s = 0.f, c = 0.f;
   unsigned long long nch = 0, nev = 0;
-  // lane `sub` of `group` lanes takes the Gauss-Legendre nodes sub, sub + group, ...
-  // (the transmittance kernel splits a ray's tree instead and passes 0 and 1)
-  int sub = 0, group = 1;
   __device__ __forceinline__ void operator()(int j) {
     const Mask& Mk = *M;
     Chord ch;
@@ -391,25 +388,22 @@ struct DetLeaf {
     const float scale = w * ch.absA * hl;
     // every node's term goes into the ray's compensated sum (the node sums of
     // a chord can cancel as much as the chords of a ray)
-    for (int k = sub; k < n; k += group) {
+    for (int k = 0; k < n; ++k) {
       const float dt = fmaf(hl, glx[off + k], mid);
       const float y = fmaf(fmaf(y2, dt, y1), dt, y0);
       neumaier_add(s, c, scale * glw[off + k] * ex2f(y) * cosf(fmaf(ch.B, dt, ch.delta)));
     }
-    nev += (unsigned long long)((n - sub + group - 1) / group);
+    nev += (unsigned long long)n;
   }
 };
 
 __device__ __forceinline__ float det_tau(const DevField& F, const Mask& M, float3 o, float3 v,
                                          float tmin, float tmax, const float* glx,
-                                         const float* glw, Counters& cnt, int sub = 0,
-                                         int group = 1) {
+                                         const float* glw, Counters& cnt) {
   const float3 inv = safe_inv(v);
   float t0, t1;
   if (M.bits == 0ull || !scene_span(F, o, inv, tmin, tmax, t0, t1)) return 0.f;
   DetLeaf leaf;
-  leaf.sub = 0;
-  leaf.group = 1;
   leaf.F = &F;
   leaf.M = &M;
   leaf.o = o;
@@ -419,12 +413,8 @@ __device__ __forceinline__ float det_tau(const DevField& F, const Mask& M, float
   leaf.glx = glx;
   leaf.glw = glw;
   SpanTest test{t0, t1};
-  // the lanes of a group walk disjoint subtrees of the same ray
-  unsigned long long nodes = 0, leaves = 0;
-  traverse_from(F, group_start(F, sub, group), o, inv, M.bits, test, leaf, nodes, leaves);
-  cnt.nodes += nodes;
-  cnt.leaves += leaves;
-  if (sub == 0) cnt.windows += 1;
+  traverse_ray(F, o, inv, M.bits, test, leaf, cnt.nodes, cnt.leaves);
+  cnt.windows += 1;
   cnt.chords += leaf.nch;
   cnt.evals += leaf.nev;
   return __fadd_rn(leaf.s, leaf.c);
@@ -497,8 +487,8 @@ struct ClosedLeaf {
 };
 
 __device__ __forceinline__ float closed_tau(const DevField& F, const Mask& M, float3 o, float3 v,
-                                            float tmin, float tmax, Counters& cnt, int sub = 0,
-                                            int group = 1, float* tend = nullptr) {
+                                            float tmin, float tmax, Counters& cnt,
+                                            float* tend = nullptr) {
   const float3 inv = safe_inv(v);
   float t0, t1;
   if (tend) *tend = -INFINITY;
@@ -511,12 +501,8 @@ __device__ __forceinline__ float closed_tau(const DevField& F, const Mask& M, fl
   leaf.tmin = tmin;
   leaf.tmax = tmax;
   SpanTest test{t0, t1};
-  // the lanes of a group walk disjoint subtrees of the same ray
-  unsigned long long nodes = 0, leaves = 0;
-  traverse_from(F, group_start(F, sub, group), o, inv, M.bits, test, leaf, nodes, leaves);
-  cnt.nodes += nodes;
-  cnt.leaves += leaves;
-  if (sub == 0) cnt.windows += 1;
+  traverse_ray(F, o, inv, M.bits, test, leaf, cnt.nodes, cnt.leaves);
+  cnt.windows += 1;
   cnt.chords += leaf.nch;
   if (tend) *tend = leaf.tend;
   return __fadd_rn(leaf.s, leaf.c);
@@ -535,7 +521,7 @@ __device__ __forceinline__ bool cdf_flight(const DevField& F, const Mask& M, flo
   const uint4 y = rng4(seed, 0, kNoPrim, ray, word);
   const float target = -log1pf(-u01(y.x));
   float tend;
-  const float total = closed_tau(F, M, o, v, 0.f, INFINITY, cnt, 0, 1, &tend);
+  const float total = closed_tau(F, M, o, v, 0.f, INFINITY, cnt, &tend);
   if (!(tend > 0.f) || total < target) return false;
   float lo = 0.f, hi = tend;
   for (int it = 0; it < 32; ++it) {
@@ -595,7 +581,7 @@ __device__ __forceinline__ bool segment_flight(const DevField& F, const Mask& M,
   const uint4 y = rng4(seed, 0, kNoPrim, ray, word);
   const float target = -log1pf(-u01(y.x));
   float tend;
-  const float total = closed_tau(F, M, o, v, 0.f, INFINITY, cnt, 0, 1, &tend);
+  const float total = closed_tau(F, M, o, v, 0.f, INFINITY, cnt, &tend);
   if (!(tend > 0.f) || total < target) return false;
   const float3 inv = safe_inv(v);
   float t0, t1;

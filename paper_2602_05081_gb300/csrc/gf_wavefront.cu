@@ -101,11 +101,6 @@ __device__ __forceinline__ float ray_weight(const LaneRay& R, uint32_t cell) {
   return R.bw[b] * cone_factor(R.cx, cell, b);
 }
 
-// byte k of x as a float, exactly: 0x4B0000xx is 2^23 + xx
-__device__ __forceinline__ float byte_float(uint32_t x, int k) {
-  return __int_as_float((int)__byte_perm(x, 0x4Bu, (uint32_t)k | 0x4550u)) - 8388608.0f;
-}
-
 __device__ __forceinline__ uint64_t slot_seed(const LaneRay& R) {
   return (uint64_t)R.seed_lo | ((uint64_t)R.seed_hi << 32);
 }
@@ -220,39 +215,8 @@ __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, c
       const LaneRay& R = Q.r[slot];
       const float3 o = make_float3(R.o[0], R.o[1], R.o[2]);
       const float3 inv = make_float3(R.inv[0], R.inv[1], R.inv[2]);
-      const unsigned long long mask = slot_mask(R);
-      const Node4* N = Wk.field(R.asset).nodes4 + node;
-      const float4 v0 = __ldg(&N->v0), v1 = __ldg(&N->v1);
-      const uint4 q = __ldg(&N->q);
-      const int4 c4 = __ldg(&N->child);
-      const uint4 m01 = __ldg(&N->m01), m23 = __ldg(&N->m23);
       ++cnt.nodes;
-      const uint32_t qlx = __float_as_uint(v1.z), qly = __float_as_uint(v1.w);
-      // slab distances straight from the codes: t = (lo + c s - o) inv = c (s inv) + (lo - o) inv
-      const float ax = v0.w * inv.x, ay = v1.x * inv.y, az = v1.y * inv.z;
-      const float bx = (v0.x - o.x) * inv.x, by = (v0.y - o.y) * inv.y, bz = (v0.z - o.z) * inv.z;
-      const unsigned long long mk[4] = {
-          (unsigned long long)m01.x | ((unsigned long long)m01.y << 32),
-          (unsigned long long)m01.z | ((unsigned long long)m01.w << 32),
-          (unsigned long long)m23.x | ((unsigned long long)m23.y << 32),
-          (unsigned long long)m23.z | ((unsigned long long)m23.w << 32)};
-      ch[0] = c4.x;
-      ch[1] = c4.y;
-      ch[2] = c4.z;
-      ch[3] = c4.w;
-      // near and far planes by the ray's direction signs, chosen once per node
-      const uint32_t nx = inv.x >= 0.f ? qlx : q.y, fx = inv.x >= 0.f ? q.y : qlx;
-      const uint32_t ny = inv.y >= 0.f ? qly : q.z, fy = inv.y >= 0.f ? q.z : qly;
-      const uint32_t nz = inv.z >= 0.f ? q.x : q.w, fz = inv.z >= 0.f ? q.w : q.x;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float txn = fmaf(byte_float(nx, k), ax, bx), txf = fmaf(byte_float(fx, k), ax, bx);
-        const float tyn = fmaf(byte_float(ny, k), ay, by), tyf = fmaf(byte_float(fy, k), ay, by);
-        const float tzn = fmaf(byte_float(nz, k), az, bz), tzf = fmaf(byte_float(fz, k), az, bz);
-        const float tn = fmaxf(fmaxf(txn, tyn), fmaxf(tzn, R.ta));
-        const float tf = fminf(fminf(txf, tyf), fminf(tzf, R.te));
-        if ((mk[k] & mask) && tn <= tf) hit |= 1u << k;
-      }
+      hit = node4_hits(Wk.field(R.asset).nodes4 + node, o, inv, slot_mask(R), R.ta, R.te, ch);
     }
     // ---------------- push internal children, queue leaves: per child slot k a
     // ballot places the lanes' entries contiguously (no bank conflicts)
