@@ -954,31 +954,17 @@ __device__ __forceinline__ unsigned long long fov_cells(const DevField& F, const
   return m;
 }
 
-// One sample of pixel (px, py): tomography exp(-tau) or scattering radiance.
-// Called by all lanes of a warp together (inactive lanes with active = false):
-// every phase (camera tracking, NEE, scattering) runs with the lanes that need
-// it converged, and the lanes regroup after each phase.
-// FF selects the free flight at compile time (GF_FLIGHT_DELTA, GF_FLIGHT_CDF or
-// GF_FLIGHT_SEGMENT), so that each kernel carries only the stack of the path it runs.
+// One sample of pixel (px, py): scattering radiance with the free flight FF
+// (GF_FLIGHT_CDF or GF_FLIGHT_SEGMENT).  Called by all lanes of a warp together
+// (inactive lanes with active = false): every phase (flight, NEE, scattering) runs
+// with the lanes that need it converged, and the lanes regroup after each phase.
 template <int FF>
 static __device__ float path_sample(const DevField& F, const PathParams& P, bool active, int px,
-                                    int py, int s, const float* glx, const float* glw,
-                                    const float* env, Counters& cnt) {
+                                    int py, int s, Counters& cnt) {
   float3 o = make_float3(0.f, 0.f, 0.f), v = make_float3(0.f, 0.f, 1.f);
   if (active) camera_ray(P.cam, P.seed, px, py, s, o, v);
   const uint32_t pix = (uint32_t)py * (uint32_t)P.cam.W + (uint32_t)px;
   const unsigned long long allow = fov_cells(F, P, v, pix, (uint32_t)s);
-  if (P.integrator == 0) {
-    float T = 0.f;
-    if (active) {
-      Mask m = sample_mask(F, P.lod, v, P.seed, pix, (uint32_t)s, 0, TAG_MASK);
-      m.bits &= allow;
-      cnt.rays += 1;
-      T = expf(-det_tau(F, m, o, v, 0.f, INFINITY, glx, glw, cnt));
-    }
-    __syncwarp();
-    return T;
-  }
   float thr = 1.f, Lsum = 0.f;
   bool alive = active;
   GF_TIC(ct);
@@ -993,10 +979,8 @@ static __device__ float path_sample(const DevField& F, const PathParams& P, bool
       const uint32_t tw = stream_word((uint32_t)s, (uint32_t)b, TAG_TRACK);
       if constexpr (FF == GF_FLIGHT_CDF)
         hit = cdf_flight(F, m, o, v, P.seed, pix, tw, th, cnt) ? 1.f : 0.f;
-      else if constexpr (FF == GF_FLIGHT_SEGMENT)
-        hit = segment_flight(F, m, o, v, P.seed, pix, tw, th, cnt) ? 1.f : 0.f;
       else
-        hit = track<true>(F, m, o, v, 0.f, INFINITY, true, P.seed, pix, tw, env, cnt, &th);
+        hit = segment_flight(F, m, o, v, P.seed, pix, tw, th, cnt) ? 1.f : 0.f;
     }
     __syncwarp();
     alive = alive && hit != 0.f;
@@ -1007,12 +991,7 @@ static __device__ float path_sample(const DevField& F, const PathParams& P, bool
                             TAG_NEE_MASK);
       mn.bits &= allow;
       cnt.rays += 1;
-      float Tl;
-      if constexpr (FF != GF_FLIGHT_DELTA)
-        Tl = expf(-closed_tau(F, mn, x, P.light, 0.f, INFINITY, cnt));
-      else
-        Tl = track<false>(F, mn, x, P.light, 0.f, INFINITY, true, P.seed, pix,
-                          stream_word((uint32_t)s, (uint32_t)b, TAG_NEE), env, cnt, nullptr);
+      const float Tl = expf(-closed_tau(F, mn, x, P.light, 0.f, INFINITY, cnt));
       Lsum += thr * P.irradiance * Tl * (0.25f / 3.14159265358979f);
       const uint4 y = rng4(P.seed, 0, kNoPrim, pix, stream_word((uint32_t)s, (uint32_t)b, TAG_SCATTER));
       const float z = 1.0f - 2.0f * u01(y.x);
