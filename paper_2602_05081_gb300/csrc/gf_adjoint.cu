@@ -173,12 +173,8 @@ struct BackLeaf {
     for (int r = 0; r < 15; ++r) acc[r] = 0.f;
     const float len = ch.dtout - ch.dtin;
     const float m = sqrtf(ch.a) * len + 0.5f * fabsf(ch.B) * len;
-    const int rule = gl_rule(m);
-    int n = gl_n(0), off = 0;
-    for (int r = 0; r <= rule; ++r) {
-      n = gl_n(r);
-      off = gl_off(r);
-    }
+    int n, off;
+    gl_pick(gl_rule(m), n, off);
     const float mid = 0.5f * (ch.dtin + ch.dtout), hl = 0.5f * len;
     for (int k = 0; k < n; ++k) {
       const float dt = fmaf(hl, glx[off + k], mid), wq = hl * glw[off + k];

@@ -162,6 +162,7 @@ __device__ __forceinline__ void coop_tau(const DevField& F, CoopQ& Q, const Mask
     }
     const float len = ch.dtout - ch.dtin;
     if (ok) gl_pick(gl_rule(sqrtf(ch.a) * len + 0.5f * fabsf(ch.B) * len), n, off);
+    cnt.evals += n;
     const int incl = warp_incl_sum(n, lane);
     const int total = __shfl_sync(kFull, incl, 31);
     if (ok) {
@@ -188,7 +189,6 @@ __device__ __forceinline__ void coop_tau(const DevField& F, CoopQ& Q, const Mask
       const float dt = fmaf(C.hl, glx[k], C.mid);
       const float y = fmaf(fmaf(C.y2, dt, C.y1), dt, C.y0);
       neumaier_add(s_acc, c_acc, C.scale * glw[k] * ex2f(y) * cosf(fmaf(C.B, dt, C.delta)));
-      ++cnt.evals;
     }
   });
 }

@@ -70,9 +70,9 @@ __global__ void __launch_bounds__(kBlock, 3)  // at most 168 registers: 12 warps
 // chord integrals), one ray per warp (coop_tau) at every batch size.  Bound by
 // instruction issue.  With one ray per lane the lanes part at every leaf: each
 // runs its own tree walk and its own rule of 8 to 64 nodes.  130,001 rays
-// through 100k kernels (306 chords and 4,092 nodes per ray): 64.8 ms with one
-// ray per lane, 12.2 ms with one per warp; 4,096 rays through 256 kernels: 54.0
-// us over binary nodes, 49.8 us over four-wide ones with the owner table.
+// through 100k kernels (306 chords and 4,092 nodes per ray): 65.0 ms with one
+// ray per lane, 5.6 ms with one per warp; 4,096 rays through 256 kernels: 53.6
+// us over binary nodes, 35.5 us over four-wide ones with the owner table.
 // ---------------------------------------------------------------------------
 template <int MODE>  // GF_TR_DETERMINISTIC or GF_TR_CLOSED_FORM
 __global__ void __launch_bounds__(kBlock, kCoopBlocks)
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kBlock, 3)
 // ---------------------------------------------------------------------------
 // Tomography image: one pixel per warp, its camera rays one after the other
 // (coop_tau), T = exp(-tau) averaged in sample order.  256x256 at 8 samples
-// through 200k kernels: 222 ms with one pixel per lane, 64 ms with one per warp.
+// through 200k kernels: 222 ms with one pixel per lane, 29 ms with one per warp.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kBlock, kCoopBlocks)
     k_tomo(const __grid_constant__ DevField F, const PathParams P, float* out, int* counter) {
