@@ -6,6 +6,28 @@
 
 namespace gf {
 
+struct BlockTables {
+  float glx[kGLTotal], glw[kGLTotal];
+  float env[8];
+};
+
+__device__ __forceinline__ void init_tables(BlockTables& sm, const DevField& F) {
+  for (int i = threadIdx.x; i < kGLTotal; i += blockDim.x) {
+    sm.glx[i] = F.gl[i];
+    sm.glw[i] = F.gl[kGLTotal + i];
+  }
+  if (threadIdx.x < 8) sm.env[threadIdx.x] = F.env[threadIdx.x];
+  __syncthreads();
+}
+
+// the next work item of a persistent grid, the same in every lane (unsigned: the
+// last warps step past a batch of up to 2^31 - 1 items)
+__device__ __forceinline__ uint32_t next_tile(int* counter, uint32_t lane) {
+  uint32_t it = 0;
+  if (lane == 0) it = (uint32_t)atomicAdd(counter, 1);
+  return __shfl_sync(kFull, it, 0);
+}
+
 // Traversal of one ray by a whole warp: a shared stack of four-wide nodes, up to
 // 32 popped per step (one per lane) and their hit children pushed; the leaves
 // reached are queued, and every 32 queued leaves (and the last ones) make a

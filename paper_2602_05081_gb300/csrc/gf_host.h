@@ -149,9 +149,14 @@ struct Field {
   // fixed-point pixel sums of the scattering renderer (grows on demand)
   mutable unsigned long long* acc64 = nullptr;
   mutable size_t acc_bytes = 0;
-  // per-thread primitive lists of the radiance adjoint (grows on demand)
+  // per-thread primitive lists of the radiance adjoint, kept chords of the tomography
+  // adjoint (grows on demand)
   mutable int* rlist = nullptr;
   mutable size_t rlist_bytes = 0;
+  // per primitive in BVH order: the adjoint's gathered parameters (3 float4), then its
+  // gradient sums (4 float4)
+  mutable float4* adj = nullptr;
+  mutable size_t adj_bytes = 0;
 };
 
 // Render server batch (one launch of k_render_server): items of many requests

@@ -14,26 +14,6 @@ constexpr int kBlock = 128;
 constexpr int kTileW = 8, kTileH = 4;
 constexpr int kCoopBlocks = 5;  // resident blocks per SM of the one-ray-per-warp kernels
 
-struct BlockTables {
-  float glx[kGLTotal], glw[kGLTotal];
-  float env[8];
-};
-
-__device__ __forceinline__ void init_tables(BlockTables& sm, const DevField& F) {
-  for (int i = threadIdx.x; i < kGLTotal; i += blockDim.x) {
-    sm.glx[i] = F.gl[i];
-    sm.glw[i] = F.gl[kGLTotal + i];
-  }
-  if (threadIdx.x < 8) sm.env[threadIdx.x] = F.env[threadIdx.x];
-  __syncthreads();
-}
-
-__device__ __forceinline__ int next_tile(int* counter, uint32_t lane) {
-  int it = 0;
-  if (lane == 0) it = atomicAdd(counter, 1);
-  return __shfl_sync(kFull, it, 0);
-}
-
 // ---------------------------------------------------------------------------
 // ratio-tracking transmittance of large batches, one ray per lane
 // ---------------------------------------------------------------------------
@@ -44,7 +24,7 @@ __global__ void __launch_bounds__(kBlock, 3)  // at most 168 registers: 12 warps
   const uint32_t lane = threadIdx.x & 31u;
   Counters cnt;
   for (;;) {
-    const int tile = next_tile(P.counter, lane);
+    const uint32_t tile = next_tile(P.counter, lane);
     if ((int64_t)tile * 32 >= P.n) break;
     const int64_t r = (int64_t)tile * 32 + (int)lane;
     if (r < P.n) {
@@ -257,8 +237,9 @@ __global__ void __launch_bounds__(kBlock, kCoopBlocks)
   Counters cnt;
   const int npix = P.cam.W * P.cam.H;
   for (;;) {
-    const int pix = next_tile(counter, lane);
-    if (pix >= npix) break;
+    const uint32_t tile = next_tile(counter, lane);
+    if (tile >= (uint32_t)npix) break;
+    const int pix = (int)tile;
     float acc = 0.f;
     for (int s = P.s0; s < P.s0 + P.spp; ++s) {
       float3 o, v;
@@ -292,7 +273,7 @@ __global__ void __launch_bounds__(kBlock)
   const int tiles_x = (P.cam.W + kTileW - 1) / kTileW;
   const int tiles_y = (P.cam.H + kTileH - 1) / kTileH;
   for (;;) {
-    const int tile = next_tile(counter, lane);
+    const int tile = (int)next_tile(counter, lane);
     if (tile >= tiles_x * tiles_y) break;
     const int px = (tile % tiles_x) * kTileW + (int)(lane % kTileW);
     const int py = (tile / tiles_x) * kTileH + (int)(lane / kTileW);
@@ -346,7 +327,7 @@ __global__ void __launch_bounds__(kBlock) k_ray_chords(const __grid_constant__ D
                                                        const ChordParams P) {
   const uint32_t lane = threadIdx.x & 31u;
   for (;;) {
-    const int tile = next_tile(P.counter, lane);
+    const uint32_t tile = next_tile(P.counter, lane);
     if ((int64_t)tile * 32 >= P.n) break;
     const int64_t r = (int64_t)tile * 32 + lane;
     if (r >= P.n) continue;  // next_tile below is reached by every lane
