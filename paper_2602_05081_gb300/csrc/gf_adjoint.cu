@@ -43,24 +43,7 @@ struct PrimDeriv {
   float phi;
   bool local, normalized;
 
-  __device__ void init(const BackArgs& B, const Prim& P, int64_t i) {
-    float q[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) q[k] = B.quat[4 * i + k];
-    const float qn = sqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
-    iqn = 1.f / qn;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) qh[k] = q[k] * iqn;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      s[k] = expf(B.ls[3 * i + k]);
-      kin[k] = B.om[3 * i + k];
-    }
-    dAdw = B.wmode == GF_WEIGHT_NORMALIZED ? P.A / B.w[i] : 1.f;
-    derive(B, P);
-  }
-
-  // as init, from the parameters k_adj_prims gathered for sorted primitive j
+  // from the parameters k_adj_prims gathered for sorted primitive j
   __device__ __forceinline__ void load(const BackArgs& B, const Prim& P, int j) {
     const float4* r = B.adj + 3 * (int64_t)j;
     const float4 a = __ldg(r), b = __ldg(r + 1), c = __ldg(r + 2);
@@ -220,18 +203,6 @@ struct PrimDeriv {
     return A * env * cs;
   }
 };
-
-__device__ __forceinline__ void add_grad(const BackArgs& B, int64_t i, const float acc[15],
-                                         float scale) {
-  const int64_t N = B.n;
-  float* g = B.grad;
-  for (int k = 0; k < 3; ++k) atomicAdd(g + 3 * i + k, scale * acc[k]);
-  for (int k = 0; k < 4; ++k) atomicAdd(g + 3 * N + 4 * i + k, scale * acc[3 + k]);
-  for (int k = 0; k < 3; ++k) atomicAdd(g + 7 * N + 3 * i + k, scale * acc[7 + k]);
-  for (int k = 0; k < 3; ++k) atomicAdd(g + 10 * N + 3 * i + k, scale * acc[10 + k]);
-  atomicAdd(g + 13 * N + i, scale * acc[13]);
-  atomicAdd(g + 14 * N + i, scale * acc[14]);
-}
 
 // what PrimDeriv::load needs, gathered once per call in BVH order (48 bytes per
 // primitive instead of 11 scattered words and their arithmetic per chord)
@@ -429,85 +400,6 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
   flush_counters(F, cnt, lane);
 }
 
-// scratch of the adjoints per primitive: gathered parameters, gradient sums
-static cudaError_t ensure_adjoint_prims(const Field& F, cudaStream_t s) {
-  return grow(F, (void**)&F.adj, F.adj_bytes, (size_t)F.n * 7 * sizeof(float4), s);
-}
-static cudaError_t tomo_grid(const Field& F, int64_t& g) {
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tomo_backward, kBackBlock, 0) != cudaSuccess)
-    (void)cudaGetLastError();
-  if (per_sm < 1) per_sm = 1;
-  g = (int64_t)F.ctx.sm_count * per_sm;
-  return cudaSuccess;
-}
-
-// per-primitive inputs gathered and sums cleared, before an adjoint kernel
-static cudaError_t adjoint_begin(const Field& F, BackArgs& B, cudaStream_t s) {
-  cudaError_t e = ensure_adjoint_prims(F, s);
-  if (e != cudaSuccess) return e;
-  B.adj = F.adj;
-  B.acc = F.adj + 3 * F.n;
-  if ((e = cudaMemsetAsync(B.acc, 0, (size_t)F.n * 4 * sizeof(float4), s)) != cudaSuccess) return e;
-  k_adj_prims<<<(unsigned)((F.n + 255) / 256), 256, 0, s>>>(F.dev.rec, B, F.adj);
-  return cudaGetLastError();
-}
-static cudaError_t adjoint_end(const Field& F, const BackArgs& B, cudaStream_t s) {
-  k_adj_finish<<<(unsigned)((F.n + 255) / 256), 256, 0, s>>>(F.dev.rec, B);
-  return cudaGetLastError();
-}
-
-// The primitives whose chords cross a ray under its mask, gathered by one
-// traversal; the replay passes then visit the list instead of the tree.
-constexpr int kRayList = 1024;
-struct RayList {
-  int* idx;    // this thread's first entry; entry k at idx[k * stride] (a warp's
-  int stride;  // lanes hold neighbouring words: coalesced)
-  int n;       // listed primitives; > kRayList: overflow, traverse instead
-  __device__ bool ok() const { return n <= kRayList; }
-  __device__ int at(int k) const { return idx[(int64_t)k * stride]; }
-};
-
-struct ListLeaf {
-  const DevField* F;
-  const Mask* M;
-  float3 o, v;
-  RayList* L;
-  __device__ void operator()(int j) {
-    const Mask& Mk = *M;
-    Chord ch;
-    float w;
-    if (!prim_chord(*F, j, o, v, 0.f, INFINITY, [&](uint32_t c) { return mask_weight(Mk, c); }, w, ch))
-      return;
-    if (L->n < kRayList) L->idx[(int64_t)L->n * L->stride] = j;
-    ++L->n;
-  }
-};
-
-__device__ __forceinline__ void gather_list(const DevField& F, const Mask& M, float3 o, float3 v,
-                                            RayList& L, Counters& cnt) {
-  L.n = 0;
-  const float3 inv = safe_inv(v);
-  float t0, t1;
-  if (M.bits == 0ull || !scene_span(F, o, inv, 0.f, INFINITY, t0, t1)) return;
-  ListLeaf leaf{&F, &M, o, v, &L};
-  SpanTest test{t0, t1};
-  traverse_ray(F, o, inv, M.bits, test, leaf, cnt.nodes, cnt.leaves);
-}
-
-// every primitive of the list, or a traversal with `test` when it overflowed
-template <class Test, class Leaf>
-__device__ __forceinline__ void visit(const DevField& F, const RayList* L, float3 o, float3 inv,
-                                      unsigned long long mask, Test& test, Leaf& leaf,
-                                      Counters& cnt) {
-  if (L && L->ok()) {
-    for (int k = 0; k < L->n; ++k) leaf(L->at(k));
-    cnt.leaves += (unsigned long long)L->n;
-  } else {
-    traverse_ray(F, o, inv, mask, test, leaf, cnt.nodes, cnt.leaves);
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Adjoint of the single-scattering radiance.
 //
@@ -525,136 +417,8 @@ __device__ __forceinline__ void visit(const DevField& F, const RayList* L, float
 //   d/d q_k = -S albedo E/(4 pi) T_light / (1 - q_k)   (NEE points),
 // and d p / d theta = 1[kappa > 0] d kappa/d theta / kappa_bar, where
 // d kappa/d theta sums the mask-weighted derivatives of the kernels covering
-// the point.  Each ray is re-tracked (same Philox streams, same windows) for
-// the derivative passes: nothing per path is stored.
+// the point.
 // ---------------------------------------------------------------------------
-
-// Windows of kPts tentative points, in t order, with kappa and kappa_bar
-// (the windows of track()); win(B, n, kap, kb) returns false to stop.
-template <class Win>
-__device__ void for_windows(const DevField& F, const Mask& M, float3 o, float3 v, uint64_t seed,
-                            uint32_t ray, uint32_t word, const float* env, Counters& cnt,
-                            const RayList* L, Win win) {
-  const unsigned am = __activemask();
-  const float3 inv = safe_inv(v);
-  float t0 = 0.f, t1 = 0.f;
-  bool more = M.bits != 0ull && scene_span(F, o, inv, 0.f, INFINITY, t0, t1);
-  float ta = t0;
-  bool first = true;
-  for (int guard = 0; guard < (1 << 16); ++guard) {
-    if (!__any_sync(am, more)) break;
-    if (!more) continue;
-    PointBuf B;
-#pragma unroll
-    for (int i = 0; i < kPts; ++i) {
-      B.t[i] = INFINITY;
-      B.u[i] = 0.f;
-    }
-    CollectLeaf cl;
-    cl.F = &F;
-    cl.M = &M;
-    cl.o = o;
-    cl.v = v;
-    cl.tmin = 0.f;
-    cl.tmax = INFINITY;
-    cl.ta = ta;
-    cl.first = first;
-    cl.bound = t1;
-    cl.B = &B;
-    cl.seed = seed;
-    cl.ray = ray;
-    cl.word = word;
-    cl.env = env;
-    CollectTest ctest{&cl.ta, &cl.bound};
-    visit(F, L, o, inv, M.bits, ctest, cl, cnt);
-    int n = 0;
-#pragma unroll
-    for (int i = 0; i < kPts; ++i) n += B.t[i] < INFINITY ? 1 : 0;
-    if (n == 0) {
-      more = false;
-      continue;
-    }
-    AccumLeaf al;
-    al.F = &F;
-    al.M = &M;
-    al.o = o;
-    al.v = v;
-    al.tmin = 0.f;
-    al.tmax = INFINITY;
-    al.B = &B;
-    al.n = n;
-    al.env = env;
-#pragma unroll
-    for (int i = 0; i < kPts; ++i) {
-      al.kap[i] = 0.f;
-      al.kb[i] = 0.f;
-    }
-    PointTest ptest{&B, n};
-    visit(F, L, o, inv, M.bits, ptest, al, cnt);
-    cnt.evals += al.nev;
-    if (!win(B, n, al.kap, al.kb) || n < kPts) {
-      more = false;
-      continue;
-    }
-    ta = B.t[kPts - 1];
-    first = false;
-  }
-}
-
-// coef_i * d kappa(x(t_i)) / d theta, scattered over the kernels at the points
-struct RadScatter {
-  const DevField* F;
-  const BackArgs* B;
-  const Mask* M;
-  float3 o, v;
-  const PointBuf* P;
-  const float* coef;
-  int n;
-  __device__ void operator()(int j) {
-    const Prim Pr = load_prim(*F, j);
-    Chord ch;
-    if (!chord_setup(Pr, o, v, 0.f, INFINITY, Pr.k2, ch)) return;
-    const float w = mask_weight(*M, ch.cell);
-    if (w == 0.f) return;
-    const float tin = ch.tc + ch.dtin, tout = ch.tc + ch.dtout;
-    bool any = false;
-#pragma unroll
-    for (int i = 0; i < kPts; ++i)
-      any |= i < n && coef[i] != 0.f && P->t[i] >= tin && P->t[i] <= tout;
-    if (!any) return;
-    PrimDeriv D;
-    D.init(*B, Pr, ch.orig);
-    float acc[15];
-    for (int r = 0; r < 15; ++r) acc[r] = 0.f;
-    for (int i = 0; i < n; ++i) {
-      const float t = P->t[i];
-      if (coef[i] == 0.f || t < tin || t > tout) continue;
-      const float dt = t - ch.tc;
-      const float y[3] = {fmaf(dt, v.x, ch.p.x), fmaf(dt, v.y, ch.p.y), fmaf(dt, v.z, ch.p.z)};
-      float d[15], dq[10];
-      D.at(y, d, dq);
-      for (int r = 0; r < 15; ++r) acc[r] = fmaf(coef[i], d[r], acc[r]);
-    }
-    add_grad(*B, ch.orig, acc, w);
-  }
-};
-
-__device__ __forceinline__ void scatter_window(const DevField& F, const BackArgs& Bk, const Mask& M,
-                                               float3 o, float3 v, const PointBuf& P,
-                                               const float* coef, int n, const RayList* L,
-                                               Counters& cnt) {
-  bool any = false;
-#pragma unroll
-  for (int i = 0; i < kPts; ++i) any |= i < n && coef[i] != 0.f;
-  if (!any) return;
-  RadScatter rs{&F, &Bk, &M, o, v, &P, coef, n};
-  PointTest ptest{&P, n};
-  visit(F, L, o, safe_inv(v), M.bits, ptest, rs, cnt);
-}
-
-struct RadSmem {
-  float env[8];
-};
 
 // ---------------------------------------------------------------------------
 // Adjoint of the multiple-scattering radiance (max_bounces >= 2).
@@ -667,80 +431,771 @@ struct RadSmem {
 //   d E[L] = E[ sum_b S_b d log P_b + sum_b C_b d log T_b ],  S_b = sum_{b'>=b} C_b',
 //   d log P_b = sum_{i<js} -dp_i / (1 - p_i) + dp_js / p_js,
 //   C_b d log T_b = -thr_b E0 sum_k dq_k T_b / (1 - q_k),
-// dp = 1[kappa > 0] d kappa / kappa_bar.  Pass 1 follows the path (the
-// renderer's streams and decisions) and keeps only T_b per collision; pass 2
-// follows it again, scattering each segment's points up to the accepted one
-// and each NEE ray's points with those coefficients.  Nothing per tentative
-// point or per segment ray is stored.
+// dp = 1[kappa > 0] d kappa / kappa_bar.  The path is followed once (the
+// renderer's streams and decisions).  NEE points are scattered as soon as T_b is
+// known.  A segment's coefficients are linear in S_b, which only the end of the path
+// gives: the segment keeps the moments of its chords at S = 1 (32 bytes each), which
+// are scattered at the end; a path with more than kRadKeep of them is followed a
+// second time with its S_b known.
+// ---------------------------------------------------------------------------
+
+// ---------------------------------------------------------------------------
+// The radiance adjoints run one path per warp.  Bound by instruction issue and the
+// latency of tree nodes.  With one pixel per lane 1.8 of 32 lanes ran, every window
+// visited its ray's list three times and paths were followed twice.  Through 200k
+// kernels: 305 -> 9.6 ms (128x128, 2 samples, single scattering), 697 -> 4.2 ms (96x64,
+// 1 sample, 3 bounces).
+//
+// A ray is processed over a window of t, at first all of it:
+//  gather   the warp traverses the binary tree together; chords go to the warp's list
+//           in global scratch, their tentative points to shared memory;
+//  sort     the points by t;
+//  sums     kappa and kappa_bar of four points at a time: the chords covering a point
+//           are collected, their terms computed one per lane and put in the order of a
+//           depth-first walk that visits near children first, in which one lane adds
+//           them up (FP32).  Decisions therefore do not depend on how the work was
+//           shared out: they are those of a single thread walking the tree;
+//  scatter  chords covering a point with a coefficient, one per lane: five moments,
+//           then the gradient.
+// The order of the walk is a 64-bit key per chord: bit 63 - d is set when the path to
+// its leaf takes the second child at depth d.
+// A window with more chords or points than the buffers hold is halved; one that cannot
+// be halved is worked through eight points at a time by one lane that walks the tree.
 // ---------------------------------------------------------------------------
 constexpr int kMaxSeg = 15;
+constexpr int kRadBlocks = 4;     // resident blocks per SM
+constexpr int kRadStack = 384;    // a step adds <= 32; depth first above kRadStack - margin
+constexpr int kRadMargin = 128;   // a full step, then <= 1 entry per level, 64 levels
+constexpr int kRadLeafQ = 96;     // <= 31 left + 64 new
+constexpr int kRadPts = 128;      // tentative points of a window
+constexpr int kRadList = 4096;    // chords of a window (global scratch)
+constexpr int kRadKeep = 4096;    // kept segment moments of a path (global scratch)
+constexpr int kRadGroup = 4;      // points whose sums are formed together
+constexpr int kRadTerms = 256;    // covering chords of a group, 64 per point
+static_assert(32 + 64 <= kRadMargin, "a full step, then a descent");
+static_assert(kStack <= 64, "a key bit per tree level");
+static_assert(kPts <= kRadPts && kRadList <= 1 << 16, "point ids");
 
-// one segment of the path from (o, v): delta tracking to the first accepted
-// point (returns false on escape, else t); with coefficients (S != 0), the
-// points up to the accepted one are scattered, -S/(1 - p) before it, S/p at it
-__device__ __forceinline__ bool path_segment(const DevField& F, const PathParams& P,
-                                             const BackArgs& Bk, float3 o, float3 v,
-                                             uint32_t pix, uint32_t s, int b, float S,
-                                             const float* env, Counters& cnt, RayList& L,
-                                             float& th) {
-  const Mask M = sample_mask_impl<true>(F, P.lod, v, P.seed, pix, s, (uint32_t)b, TAG_MASK);
-  const uint32_t wt = stream_word(s, (uint32_t)b, TAG_TRACK);
-  gather_list(F, M, o, v, L, cnt);
-  bool hit = false;
-  for_windows(F, M, o, v, P.seed, pix, wt, env, cnt, &L,
-              [&](const PointBuf& B, int n, const float* kap, const float* kb) {
-                float coef[kPts];
-                int acc = -1;
+struct RadKept {  // moments of a segment's chord at S = 1, mask weight included
+  float C0, C1, C2, S0, S1;
+  int j, seg, pad;
+};
+static_assert(sizeof(RadKept) == 32, "kept moments of 32 bytes");
+// one warp's chords of a window
+struct RadList {
+  unsigned long long* key;  // order of the depth-first walk
+  float2* span;             // entry and exit
+  float4* rec;              // 3 per chord: (tc, y2, y1, y0), (h, B, delta, sqrt a),
+                            // (peak - tc, exponent at tc without the amplitude, mask
+                            // weight, sorted primitive as bits)
+};
+constexpr size_t kRadListBytes = (size_t)kRadList * (8 + 8 + 48);
+constexpr size_t kRadWarpBytes = 2 * kRadListBytes + (size_t)kRadKeep * sizeof(RadKept);
+
+struct RadTravQ {
+  unsigned long long skey[kRadStack];
+  unsigned long long lkey[kRadLeafQ];
+  int stk[kRadStack];  // node | depth << 26
+  int lq[kRadLeafQ];
+};
+struct RadEvalQ {
+  float4 term[kRadTerms];  // envelope, cos, h, majorant factor
+  unsigned long long key[kRadTerms];
+  int idx[kRadTerms];
+};
+// tentative points of a window in t order; c: acceptance uniform, then coefficient
+struct RadPts {
+  float t[kRadPts], c[kRadPts], kap[kRadPts], kb[kRadPts];
+};
+struct RadRay {  // the ray in work
+  Mask M;
+  float3 o, v, inv;
+  float ta, tb, t1;    // window [ta, tb), or [ta, t1] when tb >= t1
+  uint32_t ray, word;
+  int nch, npts;       // chords and points of the window
+  int c8;              // points since the last multiple of kPts on the ray
+  int listed;          // 0: more chords or points than the buffers hold
+};
+struct RadQ {
+  union {
+    RadTravQ t;
+    RadEvalQ e;
+  };
+  RadPts pts[2];
+  uint32_t id[kRadPts];  // of an unsorted point: chord << 16 | its number on the chord
+  RadRay ray;
+  float3 so[kMaxSeg], sv[kMaxSeg];  // the path's segments
+  float S[kMaxSeg];
+};
+// what a warp carries through a path
+struct RadWarp {
+  const DevField& F;
+  const PathParams& P;
+  const BackArgs& B;
+  RadQ& Q;
+  unsigned char* scratch;
+  const float* env;
+  uint32_t lane;
+  int nkept;    // kept moments (may exceed kRadKeep)
+  bool replay;  // some segment could not be kept
+  Counters cnt;
+  __device__ __forceinline__ RadList list(int which) const {
+    unsigned char* p = scratch + (size_t)which * kRadListBytes;
+    RadList L;
+    L.key = reinterpret_cast<unsigned long long*>(p);
+    L.span = reinterpret_cast<float2*>(p + (size_t)kRadList * 8);
+    L.rec = reinterpret_cast<float4*>(p + (size_t)kRadList * 16);
+    return L;
+  }
+  __device__ __forceinline__ RadKept* kept() const {
+    return reinterpret_cast<RadKept*>(scratch + 2 * kRadListBytes);
+  }
+};
+
+// Chords and tentative points of the window.  The points land unsorted in kap (t),
+// kb (acceptance uniform) and id.
+__device__ __noinline__ void rad_gather(RadWarp& W, int which) {
+  RadQ& Q = W.Q;
+  const DevField& F = W.F;
+  const uint32_t lane = W.lane;
+  const unsigned lt = (1u << lane) - 1u;
+  const RadList L = W.list(which);
+  RadPts& Pt = Q.pts[which];
+  const float3 o = Q.ray.o, v = Q.ray.v, inv = Q.ray.inv;
+  const float ta = Q.ray.ta, t1 = Q.ray.t1;
+  const bool last = Q.ray.tb >= t1;
+  const float tb = last ? t1 : Q.ray.tb;
+  const unsigned long long mask = Q.ray.M.bits;
+  const SpanTest test{ta, tb};
+  const uint32_t ray = Q.ray.ray, word = Q.ray.word;
+  const uint64_t seed = W.P.seed;
+  unsigned nodes = 0, leaves = 0;
+  int nch = 0;
+  int sp = F.root >= 0 ? 1 : 0, lq_n = F.root >= 0 ? 0 : 1;
+  __syncwarp();
+  if (lane == 0) {
+    Q.ray.npts = 0;
+    if (F.root >= 0) {
+      Q.t.stk[0] = F.root;
+      Q.t.skey[0] = 0ull;
+    } else {  // a one-primitive field has no internal node
+      Q.t.lq[0] = 0;
+      Q.t.lkey[0] = 0ull;
+    }
+  }
+  __syncwarp();
+  const long long max_it = F.n + 64;  // every node enters the stack at most once
+  for (long long it = 0;; ++it) {
+    if (it > max_it) {
+      if (lane == 0) set_err(F, ERR_GUARD);
+      break;
+    }
+    int take = sp < 32 ? sp : 32;
+    if (sp > kRadStack - kRadMargin) take = 1;  // near capacity: depth first
+    const bool have = (int)lane < take;
+    const int ent = have ? Q.t.stk[sp - take + (int)lane] : 0;
+    const unsigned long long key = have ? Q.t.skey[sp - take + (int)lane] : 0ull;
+    __syncwarp();
+    sp -= take;
+    int c[2] = {0, 0};
+    bool h[2] = {false, false};
+    unsigned long long kk[2] = {key, key};
+    const int node = ent & (int)kOrigMask, depth = (int)((unsigned)ent >> 26);
+    if (have && (int64_t)node >= F.n - 1) {  // internal nodes 0 .. n-2
+      set_err(F, ERR_INDEX);
+    } else if (have) {
+      const Node* N = F.nodes + node;
+      const float4 a = __ldg(&N->a), b = __ldg(&N->b), cc = __ldg(&N->c);
+      const int4 d = __ldg(&N->d);
+      const uint4 e = __ldg(&N->e);
+      ++nodes;
+      const unsigned long long m0 = (unsigned long long)e.x | ((unsigned long long)e.y << 32);
+      const unsigned long long m1 = (unsigned long long)e.z | ((unsigned long long)e.w << 32);
+      float tn0, tf0, tn1, tf1;
+      slab_interval(o, inv, a.x, a.y, a.z, a.w, b.x, b.y, tn0, tf0);
+      slab_interval(o, inv, b.z, b.w, cc.x, cc.y, cc.z, cc.w, tn1, tf1);
+      c[0] = d.x;
+      c[1] = d.y;
+      h[0] = (m0 & mask) && test(tn0, tf0);
+      h[1] = (m1 & mask) && test(tn1, tf1);
+      // leaves come before internal nodes, then the nearer internal child
+      if (h[0] && h[1]) {
+        const bool first0 = c[0] < 0 || (c[1] >= 0 && tn0 <= tn1);
+        kk[first0 ? 1 : 0] |= 1ull << (63 - depth);
+      }
+    }
+    int np = 0, nl = 0;
 #pragma unroll
-                for (int i = 0; i < kPts; ++i) {
-                  coef[i] = 0.f;
-                  if (i < n && acc < 0) {
-                    const bool take = B.u[i] * kb[i] < fmaxf(kap[i], 0.f);
-                    if (S != 0.f && kap[i] > 0.f && kb[i] > 0.f) {
-                      const float p = kap[i] / kb[i];
-                      coef[i] = (take ? S / p : -S / (1.f - p)) / kb[i];
-                    }
-                    if (take) acc = i;
-                  }
-                }
-                if (S != 0.f) scatter_window(F, Bk, M, o, v, B, coef, n, &L, cnt);
-                if (acc >= 0) {
-                  hit = true;
-                  th = B.t[acc];
-                  return false;
-                }
-                return true;
-              });
-  return hit;
+    for (int k = 0; k < 2; ++k) {
+      const unsigned bp = __ballot_sync(kFull, h[k] && c[k] >= 0);
+      const unsigned bl = __ballot_sync(kFull, h[k] && c[k] < 0);
+      if (h[k] && c[k] >= 0) {
+        const int pos = sp + np + __popc(bp & lt);
+        if (pos < kRadStack) {
+          Q.t.stk[pos] = c[k] | (int)((unsigned)(depth + 1) << 26);
+          Q.t.skey[pos] = kk[k];
+        }
+      }
+      if (h[k] && c[k] < 0) {
+        const int pos = lq_n + nl + __popc(bl & lt);
+        Q.t.lq[pos] = ~c[k];
+        Q.t.lkey[pos] = kk[k];
+      }
+      np += __popc(bp);
+      nl += __popc(bl);
+    }
+    if (sp + np > kRadStack) {
+      if (lane == 0) set_err(F, ERR_STACK);
+      np = kRadStack - sp;
+    }
+    sp += np;
+    lq_n += nl;
+    __syncwarp();
+    const bool more = sp > 0;
+    while (lq_n >= 32 || (!more && lq_n > 0)) {
+      const int tk = lq_n < 32 ? lq_n : 32;
+      int j = -1;
+      unsigned long long lk = 0ull;
+      if ((int)lane < tk) {
+        j = Q.t.lq[lq_n - tk + (int)lane];
+        lk = Q.t.lkey[lq_n - tk + (int)lane];
+      }
+      __syncwarp();
+      lq_n -= tk;
+      if (j >= 0) ++leaves;
+      if ((int64_t)j >= F.n) {  // a leaf beyond the records
+        set_err(F, ERR_INDEX);
+        j = -1;
+      }
+      Chord ch;
+      float w;
+      const bool ok = j >= 0 &&
+                      prim_chord(F, j, o, v, 0.f, INFINITY,
+                                 [&](uint32_t cl) { return mask_weight(Q.ray.M, cl); }, w, ch) &&
+                      ch.tc + ch.dtin <= tb && ch.tc + ch.dtout >= ta;
+      const unsigned bc = __ballot_sync(kFull, ok);
+      const int k = nch + __popc(bc & lt);
+      if (ok && k < kRadList) {
+        const float wa = w * ch.absA;
+        const float y2 = -0.5f * kLog2e * ch.a, y1 = -kLog2e * ch.b;
+        const float y0 = fmaf(-0.5f * kLog2e, ch.g, log2f(wa));
+        const float hh = wa * expf(-0.5f * ch.qmin);
+        const float sa = sqrtf(ch.a);
+        L.span[k] = make_float2(ch.tc + ch.dtin, ch.tc + ch.dtout);
+        L.key[k] = lk;
+        L.rec[3 * k] = make_float4(ch.tc, y2, y1, y0);
+        L.rec[3 * k + 1] = make_float4(hh, ch.B, ch.delta, sa);
+        L.rec[3 * k + 2] = make_float4(ch.dts, -0.5f * kLog2e * ch.g, w, __int_as_float(j));
+        uint32_t num = 0;
+        chord_points(F, ch, hh, seed, ray, word, W.env, [&](float t, float u) {
+          if (t > t1 || (!last && t >= tb)) return false;
+          if (t >= ta) {
+            const int q = atomicAdd(&Q.ray.npts, 1);
+            if (q >= kRadPts) return false;  // too many: the window is halved
+            Pt.kap[q] = t;
+            Pt.kb[q] = u;
+            Q.id[q] = (uint32_t)k << 16 | num;
+          }
+          ++num;
+          return true;
+        });
+      }
+      nch += __popc(bc);
+      __syncwarp();
+    }
+    if (!more && lq_n == 0) break;
+  }
+  if (lane == 0) Q.ray.nch = nch;
+  W.cnt.nodes += nodes;
+  W.cnt.leaves += leaves;
+  __syncwarp();
 }
 
-// NEE ray of collision b from x: returns T = prod (1 - q_k); with cn != 0 the
-// points are scattered with cn / (1 - q_k) / kappa_bar_k
-__device__ __forceinline__ float path_nee(const DevField& F, const PathParams& P,
-                                          const BackArgs& Bk, float3 x, uint32_t pix,
-                                          uint32_t s, int b, float cn, const float* env,
-                                          Counters& cnt, RayList& L) {
-  const Mask Mn = sample_mask_impl<true>(F, P.lod_nee, P.light, P.seed, pix, s, (uint32_t)b,
-                                         TAG_NEE_MASK);
-  const uint32_t wn = stream_word(s, (uint32_t)b, TAG_NEE);
-  gather_list(F, Mn, x, P.light, L, cnt);
-  float Tl = 1.f;
-  for_windows(F, Mn, x, P.light, P.seed, pix, wn, env, cnt, &L,
-              [&](const PointBuf& B, int n, const float* kap, const float* kb) {
-                float coef[kPts];
+// The window's points in t order (equal t: in the order of the walk), in t and c.  The
+// ray's points go in runs of kPts, and a point at the t at which a run ended is left
+// out, as in track().
+__device__ __noinline__ void rad_sort(RadWarp& W, int which) {
+  RadQ& Q = W.Q;
+  RadPts& Pt = Q.pts[which];
+  const unsigned long long* keys = W.list(which).key;
+  const int n = Q.ray.npts;
+  bool tie = false;
+  for (int i = (int)W.lane; i < n; i += 32) {
+    const float t = Pt.kap[i];
+    int rank = 0;
+    for (int k = 0; k < n; ++k) {
+      const float tk = Pt.kap[k];
+      bool before = tk < t;
+      if (tk == t && k != i) {
+        const uint32_t a = Q.id[k], b = Q.id[i];
+        before = (a >> 16) == (b >> 16) ? a < b : keys[a >> 16] < keys[b >> 16];
+        tie = true;
+      }
+      rank += before ? 1 : 0;
+    }
+    Pt.t[rank] = t;
+    Pt.c[rank] = Pt.kb[i];
+  }
+  tie = __any_sync(kFull, tie);
+  __syncwarp();
+  if (W.lane == 0) {
+    if (!tie) {
+      Q.ray.c8 = (Q.ray.c8 + n) % kPts;
+    } else {
+      int m = 0, c8 = Q.ray.c8;
+      float end = -INFINITY;
+      for (int i = 0; i < n; ++i) {
+        const float t = Pt.t[i];
+        if (t == end) continue;
+        Pt.t[m] = t;
+        Pt.c[m] = Pt.c[i];
+        ++m;
+        if (++c8 == kPts) {
+          c8 = 0;
+          end = t;
+        }
+      }
+      Q.ray.c8 = c8;
+      Q.ray.npts = m;
+    }
+  }
+  __syncwarp();
+}
+
+// kappa and kappa_bar at `n` points from g on (n = kRadGroup or 1); false when a point
+// is covered by more chords than its share of the buffers
+__device__ __noinline__ bool rad_sums(RadWarp& W, int which, int g, int n) {
+  RadQ& Q = W.Q;
+  RadPts& Pt = Q.pts[which];
+  const RadList L = W.list(which);
+  const uint32_t lane = W.lane;
+  const unsigned lt = (1u << lane) - 1u;
+  const int nch = Q.ray.nch, cap = kRadTerms / n;
+  n = min(n, Q.ray.npts - g);
+  __syncwarp();
+  float tp[kRadGroup];
+  int c[kRadGroup];
 #pragma unroll
-                for (int i = 0; i < kPts; ++i) {
-                  coef[i] = 0.f;
-                  if (i < n && kb[i] > 0.f) {
-                    const float q = fmaxf(kap[i], 0.f) / kb[i];
-                    Tl *= 1.f - q;
-                    if (cn != 0.f && kap[i] > 0.f && 1.f - q > 0.f) coef[i] = cn / (1.f - q) / kb[i];
-                  }
-                }
-                if (cn != 0.f) scatter_window(F, Bk, Mn, x, P.light, B, coef, n, &L, cnt);
-                return true;
-              });
-  return Tl;
+  for (int p = 0; p < kRadGroup; ++p) {
+    tp[p] = p < n ? Pt.t[g + p] : INFINITY;
+    c[p] = 0;
+  }
+  for (int b = 0; b < nch; b += 32) {
+    const int k = b + (int)lane;
+    const float2 s = k < nch ? L.span[k] : make_float2(INFINITY, -INFINITY);
+#pragma unroll
+    for (int p = 0; p < kRadGroup; ++p) {
+      const bool in = p < n && tp[p] >= s.x && tp[p] <= s.y;
+      const unsigned m = __ballot_sync(kFull, in);
+      const int pos = c[p] + __popc(m & lt);
+      if (in && pos < cap) Q.e.idx[p * cap + pos] = k;
+      c[p] += __popc(m);
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < kRadGroup; ++p)
+    if (c[p] > cap) return false;
+  __syncwarp();
+#pragma unroll
+  for (int p = 0; p < kRadGroup; ++p) {
+    const int base = p * cap;
+    for (int i = (int)lane; i < c[p]; i += 32) Q.e.key[base + i] = L.key[Q.e.idx[base + i]];
+    __syncwarp();
+    for (int i = (int)lane; i < c[p]; i += 32) {
+      const unsigned long long key = Q.e.key[base + i];
+      const float4* r = L.rec + 3 * Q.e.idx[base + i];
+      const float4 a = r[0], b = r[1];
+      const float dts = r[2].x;
+      int rank = 0;
+      for (int k = 0; k < c[p]; ++k) rank += Q.e.key[base + k] < key ? 1 : 0;
+      const float dt = tp[p] - a.x;
+      const float y = fmaf(fmaf(a.y, dt, a.z), dt, a.w);
+      int m = (int)(fabsf(dt - dts) * b.w);
+      m = m > 7 ? 7 : m;
+      Q.e.term[base + rank] = make_float4(ex2f(y), cosf_fast(fmaf(b.y, dt, b.z)), b.x, W.env[m]);
+    }
+    W.cnt.evals += (int)lane < c[p] ? (unsigned)(c[p] - (int)lane + 31) >> 5 : 0u;
+  }
+  __syncwarp();
+  if ((int)lane < n) {
+    const int cl = lane == 0 ? c[0] : lane == 1 ? c[1] : lane == 2 ? c[2] : c[3];
+    const float4* T = Q.e.term + (int)lane * cap;
+    float kap = 0.f, kb = 0.f;
+    for (int i = 0; i < cl; ++i) {
+      const float4 x = T[i];
+      kap = fmaf(x.x, x.y, kap);
+      kb = fmaf(x.z, x.w, kb);
+    }
+    Pt.kap[g + (int)lane] = kap;
+    Pt.kb[g + (int)lane] = kb;
+  }
+  __syncwarp();
+  return true;
+}
+
+// kappa and kappa_bar at points 0 .. n-1 (n <= kPts) by one lane that walks the tree
+__device__ __noinline__ void rad_sums_walk(RadWarp& W, int which, int g, int n) {
+  RadQ& Q = W.Q;
+  RadPts& Pt = Q.pts[which];
+  __syncwarp();
+  if (W.lane == 0) {
+    PointBuf B;
+    AccumLeaf al;
+#pragma unroll
+    for (int i = 0; i < kPts; ++i) {
+      B.t[i] = i < n ? Pt.t[g + i] : INFINITY;
+      al.kap[i] = 0.f;
+      al.kb[i] = 0.f;
+    }
+    al.F = &W.F;
+    al.M = &Q.ray.M;
+    al.o = Q.ray.o;
+    al.v = Q.ray.v;
+    al.tmin = 0.f;
+    al.tmax = INFINITY;
+    al.B = &B;
+    al.n = n;
+    al.env = W.env;
+    PointTest pt{&B, n};
+    traverse_ray(W.F, Q.ray.o, Q.ray.inv, Q.ray.M.bits, pt, al, W.cnt.nodes, W.cnt.leaves);
+#pragma unroll
+    for (int i = 0; i < kPts; ++i)
+      if (i < n) {
+        Pt.kap[g + i] = al.kap[i];
+        Pt.kb[g + i] = al.kb[i];
+      }
+    W.cnt.evals += al.nev;
+  }
+  __syncwarp();
+}
+
+// the next kPts points from ta on by one lane that walks the tree, with their sums
+__device__ __noinline__ void rad_collect_walk(RadWarp& W, int which) {
+  RadQ& Q = W.Q;
+  RadPts& Pt = Q.pts[which];
+  __syncwarp();
+  if (W.lane == 0) {
+    PointBuf B;
+#pragma unroll
+    for (int i = 0; i < kPts; ++i) {
+      B.t[i] = INFINITY;
+      B.u[i] = 0.f;
+    }
+    CollectLeaf cl;
+    cl.F = &W.F;
+    cl.M = &Q.ray.M;
+    cl.o = Q.ray.o;
+    cl.v = Q.ray.v;
+    cl.tmin = 0.f;
+    cl.tmax = INFINITY;
+    cl.ta = Q.ray.ta;
+    cl.first = true;
+    cl.bound = Q.ray.t1;
+    cl.B = &B;
+    cl.seed = W.P.seed;
+    cl.ray = Q.ray.ray;
+    cl.word = Q.ray.word;
+    cl.env = W.env;
+    CollectTest ct{&cl.ta, &cl.bound};
+    traverse_ray(W.F, Q.ray.o, Q.ray.inv, Q.ray.M.bits, ct, cl, W.cnt.nodes, W.cnt.leaves);
+    int n = 0;
+#pragma unroll
+    for (int i = 0; i < kPts; ++i)
+      if (B.t[i] < INFINITY) {
+        Pt.t[i] = B.t[i];
+        Pt.c[i] = B.u[i];
+        ++n;
+      }
+    Q.ray.npts = n;
+    // the next window begins beyond the last point; fewer points: the ray is over
+    Q.ray.tb = n < kPts ? Q.ray.t1 : nextafterf(B.t[kPts - 1], INFINITY);
+    Q.ray.listed = 0;
+  }
+  __syncwarp();
+  rad_sums_walk(W, which, 0, Q.ray.npts);
+}
+
+// start of a ray: false when it misses every kernel
+__device__ __forceinline__ bool rad_begin(RadWarp& W, const Mask& M, float3 o, float3 v, uint32_t ray,
+                                          uint32_t word) {
+  const float3 inv = safe_inv(v);
+  float t0, t1;
+  if (M.bits == 0ull || !scene_span(W.F, o, inv, 0.f, INFINITY, t0, t1)) return false;
+  __syncwarp();
+  if (W.lane == 0) {
+    RadRay& R = W.Q.ray;
+    R.M = M;
+    R.o = o;
+    R.v = v;
+    R.inv = inv;
+    R.ta = t0;
+    R.tb = t1;
+    R.t1 = t1;
+    R.ray = ray;
+    R.word = word;
+    R.c8 = 0;
+  }
+  __syncwarp();
+  return true;
+}
+
+// the window from ta on: its points, sorted; returns their number
+__device__ __noinline__ int rad_window(RadWarp& W, int which) {
+  RadQ& Q = W.Q;
+  for (int it = 0; it < 64; ++it) {
+    rad_gather(W, which);
+    if (Q.ray.nch <= kRadList && Q.ray.npts <= kRadPts) {
+      if (W.lane == 0) Q.ray.listed = 1;
+      rad_sort(W, which);
+      return Q.ray.npts;
+    }
+    const float ta = Q.ray.ta, w = fminf(Q.ray.tb, Q.ray.t1) - ta;
+    if (w <= 1e-6f * (1.0f + fabsf(ta))) break;
+    __syncwarp();
+    if (W.lane == 0) Q.ray.tb = ta + 0.5f * w;
+    __syncwarp();
+  }
+  rad_collect_walk(W, which);
+  return Q.ray.npts;
+}
+
+// on to the next window; false at the end of the ray
+__device__ __forceinline__ bool rad_advance(RadWarp& W) {
+  RadRay& R = W.Q.ray;
+  const float ta = R.ta, tb = R.tb, t1 = R.t1;
+  if (tb >= t1) return false;
+  __syncwarp();
+  if (W.lane == 0) {
+    R.ta = tb;
+    R.tb = R.listed ? fminf(t1, tb + 2.0f * (tb - ta)) : t1;
+  }
+  __syncwarp();
+  return true;
+}
+
+// kappa and kappa_bar at the points of the group from g on
+__device__ __forceinline__ void rad_group(RadWarp& W, int which, int g) {
+  if (!W.Q.ray.listed) return;  // formed when the points were collected
+  if (rad_sums(W, which, g, kRadGroup)) return;
+  const int e = min(g + kRadGroup, W.Q.ray.npts);
+  for (int i = g; i < e; ++i)
+    if (!rad_sums(W, which, i, 1)) rad_sums_walk(W, which, i, 1);
+}
+
+// One kernel's gradient from the points with a coefficient, by a lane on its own
+struct RadScatterLeaf {
+  const RadWarp* W;
+  const RadPts* Pt;
+  int n;
+  float scale;
+  __device__ void operator()(int j) {
+    const RadRay& R = W->Q.ray;
+    const Prim Pr = load_prim(W->F, j);
+    Chord ch;
+    const float w = mask_weight(R.M, Pr.cell);
+    if (w == 0.f || !chord_setup(Pr, R.o, R.v, 0.f, INFINITY, Pr.k2, ch)) return;
+    const float tin = ch.tc + ch.dtin, tout = ch.tc + ch.dtout;
+    float C0 = 0.f, C1 = 0.f, C2 = 0.f, S0 = 0.f, S1 = 0.f;
+    bool any = false;
+    for (int i = 0; i < n; ++i) {
+      const float t = Pt->t[i], c = Pt->c[i];
+      if (c == 0.f || t < tin || t > tout) continue;
+      any = true;
+      const float dt = t - ch.tc;
+      const float e = c * ex2f(-0.5f * kLog2e * fmaf(fmaf(ch.a, dt, 2.f * ch.b), dt, ch.g));
+      float sn, cs;
+      sincosf(fmaf(ch.B, dt, ch.delta), &sn, &cs);
+      C0 += e * cs;
+      C1 = fmaf(e * cs, dt, C1);
+      C2 = fmaf(e * cs * dt, dt, C2);
+      S0 += e * sn;
+      S1 = fmaf(e * sn, dt, S1);
+    }
+    if (!any) return;
+    PrimDeriv D;
+    D.load(W->B, Pr, j);
+    float acc[15];
+    D.from_moments(ch.p, R.v, C0, C1, C2, S0, S1, acc);
+    add_grad4(W->B, j, acc, w * scale);
+  }
+};
+
+// gradients of the chords covering points 0 .. n-1 with a coefficient (c), times scale;
+// seg >= 0: the moments are kept for the end of the path instead
+__device__ __noinline__ void rad_scatter(RadWarp& W, int which, int n, int seg, float scale) {
+  RadQ& Q = W.Q;
+  RadPts& Pt = Q.pts[which];
+  const RadList L = W.list(which);
+  const uint32_t lane = W.lane;
+  const unsigned lt = (1u << lane) - 1u;
+  const int nch = Q.ray.nch;
+  if (n <= 0) return;
+  __syncwarp();
+  if (!Q.ray.listed) {
+    if (seg >= 0) {
+      W.replay = true;  // scattered when the path is followed again
+    } else if (lane == 0) {
+      const RadScatterLeaf leaf_c{&W, &Pt, n, scale};
+      RadScatterLeaf leaf = leaf_c;
+      SpanTest test{Q.ray.ta, fminf(Q.ray.tb, Q.ray.t1)};
+      traverse_ray(W.F, Q.ray.o, Q.ray.inv, Q.ray.M.bits, test, leaf, W.cnt.nodes, W.cnt.leaves);
+    }
+    __syncwarp();
+    return;
+  }
+  int m = 0;  // collected chords
+  for (int b = 0; b < nch || m > 0; b += 32) {
+    if (b < nch) {
+      const int k = b + (int)lane;
+      const float2 s = k < nch ? L.span[k] : make_float2(INFINITY, -INFINITY);
+      bool in = false;
+      for (int i = 0; i < n; ++i) in |= Pt.c[i] != 0.f && Pt.t[i] >= s.x && Pt.t[i] <= s.y;
+      const unsigned bm = __ballot_sync(kFull, in);
+      if (in) Q.e.idx[m + __popc(bm & lt)] = k;
+      m += __popc(bm);
+      __syncwarp();
+      if (m < 32 && b + 32 < nch) continue;
+    }
+    // 32 collected chords (or the last ones)
+    const int tk = m < 32 ? m : 32;
+    const bool have = (int)lane < tk;
+    const int k = have ? Q.e.idx[m - tk + (int)lane] : 0;
+    __syncwarp();
+    m -= tk;
+    const int slot = W.nkept + (int)lane;
+    if (have) {
+      const float2 s = L.span[k];
+      const float4 a = L.rec[3 * k], r1 = L.rec[3 * k + 1], r2 = L.rec[3 * k + 2];
+      const int j = __float_as_int(r2.w);
+      float C0 = 0.f, C1 = 0.f, C2 = 0.f, S0 = 0.f, S1 = 0.f;
+      for (int i = 0; i < n; ++i) {
+        const float t = Pt.t[i], c = Pt.c[i];
+        if (c == 0.f || t < s.x || t > s.y) continue;
+        const float dt = t - a.x;
+        const float e = c * ex2f(fmaf(fmaf(a.y, dt, a.z), dt, r2.y));
+        float sn, cs;
+        sincosf(fmaf(r1.y, dt, r1.z), &sn, &cs);
+        C0 += e * cs;
+        C1 = fmaf(e * cs, dt, C1);
+        C2 = fmaf(e * cs * dt, dt, C2);
+        S0 += e * sn;
+        S1 = fmaf(e * sn, dt, S1);
+      }
+      const float w = r2.z;
+      if (seg >= 0) {
+        if (slot < kRadKeep) {
+          float4* d = reinterpret_cast<float4*>(W.kept() + slot);
+          d[0] = make_float4(w * C0, w * C1, w * C2, w * S0);
+          d[1] = make_float4(w * S1, __int_as_float(j), __int_as_float(seg), 0.f);
+        }
+      } else {
+        const Prim Pr = load_prim(W.F, j);
+        Chord ch;
+        if (chord_setup(Pr, Q.ray.o, Q.ray.v, 0.f, INFINITY, Pr.k2, ch)) {
+          PrimDeriv D;
+          D.load(W.B, Pr, j);
+          float acc[15];
+          D.from_moments(ch.p, Q.ray.v, C0, C1, C2, S0, S1, acc);
+          add_grad4(W.B, j, acc, w * scale);
+        }
+      }
+    }
+    if (seg >= 0) {
+      W.nkept += tk;
+      if (W.nkept > kRadKeep) W.replay = true;
+    }
+  }
+  __syncwarp();
+}
+
+// NEE ray from x: returns T = prod (1 - q_k); windows receives their number.  With one
+// window its points stay in pts[which] for nee_scatter.
+__device__ __forceinline__ float nee_track(RadWarp& W, int which, float3 x, uint32_t pix, uint32_t s,
+                                           int b, int& windows) {
+  const PathParams& P = W.P;
+  const Mask M = sample_mask(W.F, P.lod_nee, P.light, P.seed, pix, s, (uint32_t)b, TAG_NEE_MASK);
+  float T = 1.f;
+  windows = 0;
+  if (!rad_begin(W, M, x, P.light, pix, stream_word(s, (uint32_t)b, TAG_NEE))) return T;
+  const RadPts& Pt = W.Q.pts[which];
+  do {
+    const int n = rad_window(W, which);
+    ++windows;
+    for (int g = 0; g < n; g += kRadGroup) {
+      rad_group(W, which, g);
+      for (int i = g; i < min(g + kRadGroup, n); ++i)
+        if (Pt.kb[i] > 0.f) T *= 1.f - fmaxf(Pt.kap[i], 0.f) / Pt.kb[i];
+    }
+  } while (rad_advance(W));
+  return T;
+}
+// coefficients cn / (1 - q_k) / kappa_bar_k of the ray's NEE points, scattered
+__device__ __forceinline__ void nee_scatter(RadWarp& W, int which, float3 x, uint32_t pix, uint32_t s,
+                                            int b, int windows, float cn) {
+  const PathParams& P = W.P;
+  if (windows == 0 || cn == 0.f) return;
+  RadPts& Pt = W.Q.pts[which];
+  if (windows > 1) {  // the windows again, each scattered in turn
+    const Mask M = sample_mask(W.F, P.lod_nee, P.light, P.seed, pix, s, (uint32_t)b, TAG_NEE_MASK);
+    (void)rad_begin(W, M, x, P.light, pix, stream_word(s, (uint32_t)b, TAG_NEE));
+  }
+  do {
+    const int n = windows > 1 ? rad_window(W, which) : W.Q.ray.npts;
+    if (windows > 1)
+      for (int g = 0; g < n; g += kRadGroup) rad_group(W, which, g);
+    __syncwarp();
+    for (int i = (int)W.lane; i < n; i += 32) {
+      const float kap = Pt.kap[i], kb = Pt.kb[i];
+      float c = 0.f;
+      if (kap > 0.f && kb > 0.f) {
+        const float q = kap / kb;
+        if (1.f - q > 0.f) c = cn / (1.f - q) / kb;
+      }
+      Pt.c[i] = c;
+    }
+    rad_scatter(W, which, n, -1, 1.f);
+  } while (windows > 1 && rad_advance(W));
+}
+
+// One segment of the path from (o, v): delta tracking to the first accepted point
+// (returns false on escape, else its t).  Coefficients at S = 1, -1/(1 - p) before the
+// accepted point and 1/p at it, are kept for segment b (scale == 0) or scattered with
+// scale.
+__device__ __forceinline__ bool path_segment(RadWarp& W, float3 o, float3 v, uint32_t pix, uint32_t s,
+                                             int b, float scale, float& th) {
+  const PathParams& P = W.P;
+  const Mask M = sample_mask(W.F, P.lod, v, P.seed, pix, s, (uint32_t)b, TAG_MASK);
+  if (!rad_begin(W, M, o, v, pix, stream_word(s, (uint32_t)b, TAG_TRACK))) return false;
+  RadPts& Pt = W.Q.pts[0];
+  const int kept0 = W.nkept;
+  const bool replay0 = W.replay;
+  do {
+    const int n = rad_window(W, 0);
+    int acc = -1;
+    for (int g = 0; g < n && acc < 0; g += kRadGroup) {
+      rad_group(W, 0, g);
+      for (int i = g; i < min(g + kRadGroup, n) && acc < 0; ++i) {
+        const float kap = Pt.kap[i], kb = Pt.kb[i], u = Pt.c[i];
+        const bool take = u * kb < fmaxf(kap, 0.f);
+        float c = 0.f;
+        if (kap > 0.f && kb > 0.f) {
+          const float p = kap / kb;
+          c = (take ? 1.f / p : -1.f / (1.f - p)) / kb;
+        }
+        __syncwarp();
+        if (W.lane == 0) Pt.c[i] = c;
+        if (take) acc = i;
+      }
+    }
+    rad_scatter(W, 0, acc >= 0 ? acc + 1 : n, scale == 0.f ? b : -1, scale);
+    if (acc >= 0) {
+      th = Pt.t[acc];
+      return true;
+    }
+  } while (rad_advance(W));
+  W.nkept = kept0;  // an escaping segment has no coefficients
+  W.replay = replay0;
+  return false;
 }
 
 __device__ __forceinline__ float3 path_scatter_dir(const PathParams& P, uint32_t pix, uint32_t s,
@@ -753,162 +1208,186 @@ __device__ __forceinline__ float3 path_scatter_dir(const PathParams& P, uint32_t
   return make_float3(rr * cs, rr * sn, z);
 }
 
-__device__ void path_backward(const DevField& F, const PathParams& P, const BackArgs& Bk,
-                              float3 o0, float3 v0, uint32_t pix, uint32_t s, float base,
-                              const float* env, Counters& cnt, RayList& Lc, RayList& Ln) {
+// multiple scattering: the path of sample s of pixel pix
+__device__ __forceinline__ void path_backward(RadWarp& W, float3 o, float3 v, uint32_t pix, uint32_t s,
+                                              float base) {
+  const PathParams& P = W.P;
+  RadQ& Q = W.Q;
   const float E0 = P.irradiance * (0.25f / 3.14159265358979f);
-  float Tb[kMaxSeg];
+  W.nkept = 0;
+  W.replay = false;
   int nseg = 0;
-  // pass 1: the path, its NEE products
-  {
-    float3 o = o0, v = v0;
-    for (int b = 0; b < P.max_bounces && b < kMaxSeg; ++b) {
-      float th = 0.f;
-      cnt.rays += 1;
-      if (!path_segment(F, P, Bk, o, v, pix, s, b, 0.f, env, cnt, Lc, th)) break;
-      const float3 x = make_float3(fmaf(th, v.x, o.x), fmaf(th, v.y, o.y), fmaf(th, v.z, o.z));
-      cnt.rays += 1;
-      Tb[nseg++] = path_nee(F, P, Bk, x, pix, s, b, 0.f, env, cnt, Ln);
-      o = x;
-      v = path_scatter_dir(P, pix, s, b);
-    }
-  }
-  if (nseg == 0) return;
-  // S_b = sum_{b' >= b} C_b', C_b = albedo^(b+1) E0 T_b
-  float Ssuf = 0.f, thr = 1.f;
-  for (int b = 0; b < nseg; ++b) {
-    thr *= P.albedo;
-    Ssuf += thr * E0 * Tb[b];
-  }
-  // pass 2: the same path again, scattering the coefficients
-  float3 o = o0, v = v0;
-  thr = 1.f;
-  for (int b = 0; b < nseg; ++b) {
+  float thr = 1.f, Ssuf = 0.f;
+  for (int b = 0; b < P.max_bounces && b < kMaxSeg; ++b) {
     float th = 0.f;
-    if (!path_segment(F, P, Bk, o, v, pix, s, b, base * Ssuf, env, cnt, Lc, th)) break;
+    if (W.lane == 0) {
+      W.cnt.rays += 1;
+      Q.so[b] = o;
+      Q.sv[b] = v;
+    }
+    if (!path_segment(W, o, v, pix, s, b, 0.f, th)) break;
     const float3 x = make_float3(fmaf(th, v.x, o.x), fmaf(th, v.y, o.y), fmaf(th, v.z, o.z));
+    if (W.lane == 0) W.cnt.rays += 1;
+    int windows = 0;
+    const float T = nee_track(W, 0, x, pix, s, b, windows);
     thr *= P.albedo;
-    const float Cb = thr * E0 * Tb[b];
-    if (Tb[b] > 0.f) (void)path_nee(F, P, Bk, x, pix, s, b, -base * Cb, env, cnt, Ln);
-    Ssuf -= Cb;
+    const float Cb = thr * E0 * T;
+    if (T > 0.f) nee_scatter(W, 0, x, pix, s, b, windows, -base * Cb);
+    if (W.lane == 0) Q.S[b] = Cb;
+    Ssuf += Cb;
+    ++nseg;
     o = x;
     v = path_scatter_dir(P, pix, s, b);
   }
+  if (nseg == 0) return;
+  // S_b = sum_{b' >= b} C_b'
+  __syncwarp();
+  if (W.lane == 0) {
+    for (int b = 0; b < nseg; ++b) {
+      const float Cb = Q.S[b];
+      Q.S[b] = Ssuf;
+      Ssuf -= Cb;
+    }
+  }
+  __syncwarp();
+  if (W.replay) {
+    // too many chords to keep: the segments again, with their S_b known
+    for (int b = 0; b < nseg; ++b) {
+      const float S = base * Q.S[b];
+      float th = 0.f;
+      if (S == 0.f) continue;
+      if (!path_segment(W, Q.so[b], Q.sv[b], pix, s, b, S, th)) break;
+    }
+    return;
+  }
+  for (int e = (int)W.lane; e < W.nkept; e += 32) {
+    const float4* d = reinterpret_cast<const float4*>(W.kept() + e);
+    const float4 a = d[0], c = d[1];
+    const int j = __float_as_int(c.y), seg = __float_as_int(c.z);
+    const float S = base * Q.S[seg];
+    if (S == 0.f) continue;
+    const float3 so = Q.so[seg], sv = Q.sv[seg];
+    const Prim Pr = load_prim(W.F, j);
+    Chord ch;
+    if (!chord_setup(Pr, so, sv, 0.f, INFINITY, Pr.k2, ch)) continue;
+    PrimDeriv D;
+    D.load(W.B, Pr, j);
+    float acc[15];
+    D.from_moments(ch.p, sv, a.x, a.y, a.z, a.w, c.x, acc);
+    add_grad4(W.B, j, acc, S);
+  }
+  __syncwarp();
 }
 
-// PATH = false: single scattering (the expected-value estimator above);
-// PATH = true: multiple scattering (path_backward), each with its own frame
-template <bool PATH>
-__global__ void __launch_bounds__(kBackBlock)
-    k_radiance_backward(const __grid_constant__ DevField F, const PathParams P, const BackArgs Bk,
-                        const float* dLdI, int* counter, int* lists) {
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int nth = gridDim.x * blockDim.x;
-  RayList Lc{lists + tid, nth, 0}, Ln{lists + (int64_t)kRayList * nth + tid, nth, 0};
-  __shared__ RadSmem sm;
-  if (threadIdx.x < 8) sm.env[threadIdx.x] = F.env[threadIdx.x];
-  __syncthreads();
-  const uint32_t lane = threadIdx.x & 31u;
-  Counters cnt;
+// single scattering: the expected-value estimator of sample s of pixel pix
+__device__ __forceinline__ void single_backward(RadWarp& W, float3 o, float3 v, uint32_t pix,
+                                                uint32_t s, float base) {
+  const PathParams& P = W.P;
+  RadPts& Pt = W.Q.pts[0];
   const float E = P.albedo * P.irradiance * (0.25f / 3.14159265358979f);
-  const int tiles_x = (P.cam.W + 7) / 8, tiles_y = (P.cam.H + 3) / 4;
+  if (W.lane == 0) W.cnt.rays += 1;
+  const Mask M = sample_mask(W.F, P.lod, v, P.seed, pix, s, 0, TAG_MASK);
+  const uint32_t wt = stream_word(s, 0, TAG_TRACK);
+  if (!rad_begin(W, M, o, v, pix, wt)) return;
+  // weights, their sum and the reservoir draw
+  float Pr = 1.f, S = 0.f, pjs = 0.f, tjs = 0.f;
+  int idx = 0, js = -1, windows = 0;
+  do {
+    const int n = rad_window(W, 0);
+    ++windows;
+    for (int g = 0; g < n; g += kRadGroup) {
+      rad_group(W, 0, g);
+      for (int i = g; i < min(g + kRadGroup, n); ++i) {
+        const float kap = Pt.kap[i], kb = Pt.kb[i];
+        const float p = kb > 0.f ? fmaxf(kap, 0.f) / kb : 0.f;
+        const float Wt = Pr * p;
+        S += Wt;
+        if (Wt > 0.f && Pt.c[i] * S < Wt) {
+          js = idx + i;
+          pjs = p;
+          tjs = Pt.t[i];
+        }
+        Pr *= 1.f - p;
+      }
+    }
+    idx += n;
+  } while (rad_advance(W));
+  if (js < 0 || !(S > 0.f)) return;
+  // the camera ray in work, for its scatter after the NEE ray's
+  const int nch = W.Q.ray.nch, npts = W.Q.ray.npts, listed = W.Q.ray.listed;
+  // NEE from the drawn point by ratio tracking, T = prod (1 - kappa+/kappa_bar)
+  const float3 x = make_float3(fmaf(tjs, v.x, o.x), fmaf(tjs, v.y, o.y), fmaf(tjs, v.z, o.z));
+  if (W.lane == 0) W.cnt.rays += 1;
+  int nwin = 0;
+  const float Tl = nee_track(W, 1, x, pix, s, 0, nwin);
+  const float G = E * Tl;
+  if (Tl > 0.f) nee_scatter(W, 1, x, pix, s, 0, nwin, -base * S * E * Tl);
+  // camera points 0 .. js
+  (void)rad_begin(W, M, o, v, pix, wt);
+  idx = 0;
+  do {
+    int n;
+    if (windows > 1) {
+      n = rad_window(W, 0);
+      for (int g = 0; g < n; g += kRadGroup) rad_group(W, 0, g);
+    } else {
+      n = npts;
+      if (W.lane == 0) {
+        W.Q.ray.nch = nch;
+        W.Q.ray.npts = npts;
+        W.Q.ray.listed = listed;
+      }
+    }
+    __syncwarp();
+    const int m = min(n, js + 1 - idx);
+    for (int i = (int)W.lane; i < m; i += 32) {
+      const float kap = Pt.kap[i], kb = Pt.kb[i];
+      float c = 0.f;
+      if (kap > 0.f && kb > 0.f) {
+        const float p = kap / kb;
+        c = base * (idx + i == js ? S * G / pjs : -S * G / (1.f - p)) / kb;
+      }
+      Pt.c[i] = c;
+    }
+    rad_scatter(W, 0, m, -1, 1.f);
+    idx += n;
+  } while (windows > 1 && idx <= js && rad_advance(W));
+}
+
+// PATH = false: single scattering; PATH = true: multiple scattering
+template <bool PATH>
+__global__ void __launch_bounds__(kBackBlock, kRadBlocks)
+    k_radiance_backward(const __grid_constant__ DevField F, const __grid_constant__ PathParams P,
+                        const __grid_constant__ BackArgs Bk, const float* dLdI, int* counter,
+                        int chunk, unsigned char* scratch) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  float* env = reinterpret_cast<float*>(smraw);
+  if (threadIdx.x < 8) env[threadIdx.x] = F.env[threadIdx.x];
+  __syncthreads();
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  RadWarp W{F, P, Bk, reinterpret_cast<RadQ*>(smraw + 32)[warp],
+            scratch + ((size_t)blockIdx.x * (kBackBlock / 32) + warp) * kRadWarpBytes, env, lane, 0,
+            false, Counters()};
+  const uint32_t nchunk = (uint32_t)((P.spp + chunk - 1) / chunk);
+  const uint32_t units = (uint32_t)(P.cam.W * P.cam.H) * nchunk;
   for (;;) {
-    int tile = 0;
-    if (lane == 0) tile = atomicAdd(counter, 1);
-    tile = __shfl_sync(kFull, tile, 0);
-    if (tile >= tiles_x * tiles_y) break;
-    const int px = (tile % tiles_x) * 8 + (int)(lane % 8);
-    const int py = (tile / tiles_x) * 4 + (int)(lane / 8);
-    if (px >= P.cam.W || py >= P.cam.H) continue;  // every lane returns to the tile fetch
-    const uint32_t pix = (uint32_t)(py * P.cam.W + px);
+    const uint32_t u = next_tile(counter, lane);
+    if (u >= units) break;
+    const uint32_t pix = u / nchunk;
     const float gI = dLdI[pix];
     if (gI == 0.f) continue;
     const float base = gI / (float)P.spp;
-    for (int s = P.s0; s < P.s0 + P.spp; ++s) {
+    const int sa = P.s0 + (int)(u % nchunk) * chunk, sb = min(sa + chunk, P.s0 + P.spp);
+    for (int s = sa; s < sb; ++s) {
       float3 o, v;
-      camera_ray(P.cam, P.seed, px, py, s, o, v);
-      if constexpr (PATH) {
-        path_backward(F, P, Bk, o, v, pix, (uint32_t)s, base, sm.env, cnt, Lc, Ln);
-        continue;
-      }
-      cnt.rays += 1;
-      const Mask M = sample_mask_impl<true>(F, P.lod, v, P.seed, pix, (uint32_t)s, 0, TAG_MASK);
-      const uint32_t wt = stream_word((uint32_t)s, 0, TAG_TRACK);
-      gather_list(F, M, o, v, Lc, cnt);
-      // pass 1: weights, their sum and the reservoir draw
-      float Pr = 1.f, S = 0.f, pjs = 0.f, tjs = 0.f;
-      int idx = 0, js = -1;
-      for_windows(F, M, o, v, P.seed, pix, wt, sm.env, cnt, &Lc,
-                  [&](const PointBuf& B, int n, const float* kap, const float* kb) {
-                    for (int i = 0; i < n; ++i) {
-                      const float p = kb[i] > 0.f ? fmaxf(kap[i], 0.f) / kb[i] : 0.f;
-                      const float W = Pr * p;
-                      S += W;
-                      if (W > 0.f && B.u[i] * S < W) {
-                        js = idx + i;
-                        pjs = p;
-                        tjs = B.t[i];
-                      }
-                      Pr *= 1.f - p;
-                    }
-                    idx += n;
-                    return true;
-                  });
-      if (js < 0 || !(S > 0.f)) continue;
-      // NEE from the drawn point by ratio tracking
-      const float3 x = make_float3(fmaf(tjs, v.x, o.x), fmaf(tjs, v.y, o.y), fmaf(tjs, v.z, o.z));
-      const Mask Mn = sample_mask_impl<true>(F, P.lod_nee, P.light, P.seed, pix, (uint32_t)s, 0, TAG_NEE_MASK);
-      const uint32_t wn = stream_word((uint32_t)s, 0, TAG_NEE);
-      cnt.rays += 1;
-      gather_list(F, Mn, x, P.light, Ln, cnt);
-      // ratio tracking of the NEE ray, T = prod (1 - kappa+/kappa_bar)
-      float Tl = 1.f;
-      for_windows(F, Mn, x, P.light, P.seed, pix, wn, sm.env, cnt, &Ln,
-                  [&](const PointBuf& B, int n, const float* kap, const float* kb) {
-                    for (int i = 0; i < n; ++i)
-                      if (kb[i] > 0.f) Tl *= 1.f - fmaxf(kap[i], 0.f) / kb[i];
-                    return true;
-                  });
-      const float G = E * Tl;
-      // pass 2: camera points 0..js
-      idx = 0;
-      for_windows(F, M, o, v, P.seed, pix, wt, sm.env, cnt, &Lc,
-                  [&](const PointBuf& B, int n, const float* kap, const float* kb) {
-                    float coef[kPts];
-#pragma unroll
-                    for (int i = 0; i < kPts; ++i) {
-                      coef[i] = 0.f;
-                      const int gi = idx + i;
-                      if (i < n && gi <= js && kap[i] > 0.f && kb[i] > 0.f) {
-                        const float p = kap[i] / kb[i];
-                        const float c = gi == js ? S * G / pjs : -S * G / (1.f - p);
-                        coef[i] = base * c / kb[i];
-                      }
-                    }
-                    scatter_window(F, Bk, M, o, v, B, coef, n, &Lc, cnt);
-                    idx += n;
-                    return idx <= js;
-                  });
-      // pass 3: NEE points
-      if (Tl > 0.f) {
-        for_windows(F, Mn, x, P.light, P.seed, pix, wn, sm.env, cnt, &Ln,
-                    [&](const PointBuf& B, int n, const float* kap, const float* kb) {
-                      float coef[kPts];
-#pragma unroll
-                      for (int i = 0; i < kPts; ++i) {
-                        coef[i] = 0.f;
-                        if (i < n && kap[i] > 0.f && kb[i] > 0.f) {
-                          const float q = kap[i] / kb[i];
-                          if (1.f - q > 0.f) coef[i] = -base * S * E * Tl / (1.f - q) / kb[i];
-                        }
-                      }
-                      scatter_window(F, Bk, Mn, x, P.light, B, coef, n, &Ln, cnt);
-                      return true;
-                    });
-      }
+      camera_ray(P.cam, P.seed, (int)pix % P.cam.W, (int)pix / P.cam.W, s, o, v);
+      if constexpr (PATH)
+        path_backward(W, o, v, pix, (uint32_t)s, base);
+      else
+        single_backward(W, o, v, pix, (uint32_t)s, base);
     }
   }
-  flush_counters(F, cnt, lane);
+  flush_counters(F, W.cnt, lane);
 }
 
 static BackArgs back_args(const Field& F, float* grad) {
@@ -924,84 +1403,95 @@ static BackArgs back_args(const Field& F, float* grad) {
   return B;
 }
 
-cudaError_t launch_tomo_backward(const Field& F, const PathParams& P, const float* dLdI,
-                                 float* grad, cudaStream_t s) {
+static_assert(sizeof(RadQ) % 16 == 0, "aligned per-warp shared memory");
+constexpr size_t kRadSmem = 32 + sizeof(RadQ) * (kBackBlock / 32);
+static_assert((kRadSmem + 1024) * kRadBlocks <= 233472, "kRadBlocks blocks fit one SM's shared memory");
+
+// blocks of a full persistent grid; the kernel's local frame must fit the context's
+// stack limit as it stands
+template <class K>
+static cudaError_t adjoint_grid(const Field& F, K kernel, size_t smem, int64_t& g) {
+  cudaError_t e;
+  if (smem && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)smem)) != cudaSuccess)
+    return e;
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBackBlock, smem) != cudaSuccess)
+    (void)cudaGetLastError();
+  if (per_sm < 1) per_sm = 1;
+  g = (int64_t)F.ctx.sm_count * per_sm;
+  return cudaSuccess;
+}
+template <class K>
+static cudaError_t adjoint_stack_fits(K kernel) {
+  cudaFuncAttributes fa;
+  size_t limit = 0;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e == cudaSuccess) e = cudaDeviceGetLimit(&limit, cudaLimitStackSize);
+  if (e == cudaSuccess && fa.localSizeBytes > limit) e = cudaErrorLaunchOutOfResources;
+  return e;
+}
+
+// scratch of the adjoints, grown through the field's allocator: per warp of a full
+// persistent grid the chord lists and kept moments (radiance) or the kept chords
+// (tomography) in one buffer, and the arrays per primitive
+cudaError_t ensure_adjoint_lists(const Field& F, cudaStream_t s) {
+  int64_t g = 1;
+  size_t bytes = 0;
+  cudaError_t e;
+  if ((e = adjoint_grid(F, k_tomo_backward, 0, g)) != cudaSuccess) return e;
+  bytes = (size_t)g * (kBackBlock / 32) * kTomoChords * sizeof(TomoChord);
+  if ((e = adjoint_grid(F, k_radiance_backward<false>, kRadSmem, g)) != cudaSuccess) return e;
+  bytes = std::max(bytes, (size_t)g * (kBackBlock / 32) * kRadWarpBytes);
+  if ((e = adjoint_grid(F, k_radiance_backward<true>, kRadSmem, g)) != cudaSuccess) return e;
+  bytes = std::max(bytes, (size_t)g * (kBackBlock / 32) * kRadWarpBytes);
+  if ((e = grow(F, (void**)&F.adj, F.adj_bytes, (size_t)F.n * 7 * sizeof(float4), s)) != cudaSuccess)
+    return e;
+  return grow(F, (void**)&F.rlist, F.rlist_bytes, bytes, s);
+}
+
+// An adjoint kernel over units of `chunk` samples of a pixel (about 16 per warp of the
+// grid at least), between the per-primitive inputs and the copy of the sums to grad
+template <class K, class T>
+static cudaError_t launch_adjoint(const Field& F, const PathParams& P, K kernel, size_t smem,
+                                  const float* dLdI, float* grad, T* scratch_type, cudaStream_t s) {
+  (void)scratch_type;
   (void)cudaGetLastError();  // a stale error of an unrelated call is not ours
   cudaError_t e = cudaMemsetAsync(F.counter, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   BackArgs B = back_args(F, grad);
-  cudaFuncAttributes fa;
-  size_t limit = 0;
-  if ((e = cudaFuncGetAttributes(&fa, k_tomo_backward)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetLimit(&limit, cudaLimitStackSize)) != cudaSuccess) return e;
-  if (fa.localSizeBytes > limit) return cudaErrorLaunchOutOfResources;
   int64_t g = 1;
-  if ((e = tomo_grid(F, g)) != cudaSuccess) return e;
-  // scratch for a full grid (allocated ahead by gf_reserve, else here)
-  if ((e = ensure_adjoint_lists(F, s)) != cudaSuccess) return e;
-  // units of `chunk` samples of a pixel, about 16 per warp of the grid at least
+  if ((e = adjoint_stack_fits(kernel)) != cudaSuccess) return e;
+  if ((e = ensure_adjoint_lists(F, s)) != cudaSuccess) return e;  // unless gf_reserve has
+  if ((e = adjoint_grid(F, kernel, smem, g)) != cudaSuccess) return e;
   const int64_t npix = (int64_t)P.cam.W * P.cam.H, warps = g * (kBackBlock / 32);
   int64_t nchunk = (16 * warps + npix - 1) / npix;
   nchunk = nchunk < 1 ? 1 : (nchunk > P.spp ? P.spp : nchunk);
   const int64_t chunk = (P.spp + nchunk - 1) / nchunk;
   const int64_t units = npix * ((P.spp + chunk - 1) / chunk);
-  const int64_t need = (units + kBackBlock / 32 - 1) / (kBackBlock / 32);
-  if (need < g) g = need;
-  if ((e = adjoint_begin(F, B, s)) != cudaSuccess) return e;
-  k_tomo_backward<<<(unsigned)g, kBackBlock, 0, s>>>(F.dev, P, B, dLdI, F.counter, (int)chunk,
-                                                     reinterpret_cast<TomoChord*>(F.rlist));
+  g = std::min(g, (units + kBackBlock / 32 - 1) / (kBackBlock / 32));
+  B.adj = F.adj;
+  B.acc = F.adj + 3 * F.n;
+  if ((e = cudaMemsetAsync(B.acc, 0, (size_t)F.n * 4 * sizeof(float4), s)) != cudaSuccess) return e;
+  const unsigned pb = (unsigned)((F.n + 255) / 256);
+  k_adj_prims<<<pb, 256, 0, s>>>(F.dev.rec, B, F.adj);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return adjoint_end(F, B, s);
+  kernel<<<(unsigned)g, kBackBlock, smem, s>>>(F.dev, P, B, dLdI, F.counter, (int)chunk,
+                                              reinterpret_cast<T*>(F.rlist));
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  k_adj_finish<<<pb, 256, 0, s>>>(F.dev.rec, B);
+  return cudaGetLastError();
 }
 
-// scratch of the adjoints, grown through the field's allocator: the radiance adjoint's
-// primitive lists (2 per thread of a full persistent grid) or the tomography adjoint's
-// kept chords in the same buffer, and the arrays per primitive
-cudaError_t ensure_adjoint_lists(const Field& F, cudaStream_t s) {
-  int per_sm = 0;
-  for (auto k : {k_radiance_backward<false>, k_radiance_backward<true>}) {
-    int q = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k, kBackBlock, 0) != cudaSuccess)
-      (void)cudaGetLastError();
-    per_sm = q > per_sm ? q : per_sm;
-  }
-  if (per_sm < 1) per_sm = 1;
-  const int64_t threads = (int64_t)F.ctx.sm_count * per_sm * kBackBlock;
-  size_t bytes = (size_t)threads * 2 * kRayList * sizeof(int);
-  int64_t g = 1;
-  cudaError_t e = tomo_grid(F, g);
-  if (e != cudaSuccess) return e;
-  bytes = std::max(bytes, (size_t)g * (kBackBlock / 32) * kTomoChords * sizeof(TomoChord));
-  if ((e = ensure_adjoint_prims(F, s)) != cudaSuccess) return e;
-  return grow(F, (void**)&F.rlist, F.rlist_bytes, bytes, s);
+cudaError_t launch_tomo_backward(const Field& F, const PathParams& P, const float* dLdI,
+                                 float* grad, cudaStream_t s) {
+  return launch_adjoint(F, P, k_tomo_backward, 0, dLdI, grad, (TomoChord*)nullptr, s);
 }
 
 cudaError_t launch_radiance_backward(const Field& F, const PathParams& P, const float* dLdI,
                                      float* grad, cudaStream_t s) {
-  (void)cudaGetLastError();  // a stale error of an unrelated call is not ours
-  cudaError_t e = cudaMemsetAsync(F.counter, 0, sizeof(int), s);
-  if (e != cudaSuccess) return e;
-  const BackArgs B = back_args(F, grad);
-  auto kernel = P.max_bounces >= 2 ? k_radiance_backward<true> : k_radiance_backward<false>;
-  // the kernel's local frame must fit the context's stack limit as it stands
-  cudaFuncAttributes fa;
-  size_t limit = 0;
-  if ((e = cudaFuncGetAttributes(&fa, kernel)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetLimit(&limit, cudaLimitStackSize)) != cudaSuccess) return e;
-  if (fa.localSizeBytes > limit) return cudaErrorLaunchOutOfResources;
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBackBlock, 0) != cudaSuccess)
-    (void)cudaGetLastError();
-  if (per_sm < 1) per_sm = 1;
-  const int64_t tiles = (int64_t)((P.cam.W + 7) / 8) * ((P.cam.H + 3) / 4);
-  const int64_t need = (tiles + kBackBlock / 32 - 1) / (kBackBlock / 32);
-  int64_t g = (int64_t)F.ctx.sm_count * per_sm;
-  if (need < g) g = need;
-  if (g < 1) g = 1;
-  // lists sized for a full grid (allocated ahead by gf_reserve, else here)
-  if ((e = ensure_adjoint_lists(F, s)) != cudaSuccess) return e;
-  kernel<<<(unsigned)g, kBackBlock, 0, s>>>(F.dev, P, B, dLdI, F.counter, F.rlist);
-  return cudaGetLastError();
+  return launch_adjoint(F, P, P.max_bounces >= 2 ? k_radiance_backward<true> : k_radiance_backward<false>,
+                        kRadSmem, dLdI, grad, (unsigned char*)nullptr, s);
 }
 
 }  // namespace gf

@@ -691,12 +691,10 @@ gf_status gf_render_backward(gf_field* h, const gf_camera* camera, const gf_rend
   if ((st = stage(F, dL_dimage, npix * 4, true, s, off, &dl)) ||
       (st = stage(F, grad, gbytes, false, s, off, &gd)))
     return st;
-  if (opts->integrator == GF_INTEG_TOMO) {
+  if (opts->integrator == GF_INTEG_TOMO)
     GF_CUDA(launch_tomo_backward(F, P, (const float*)dl, (float*)gd, s), "backward launch");
-  } else {
-    GF_CUDA(cudaMemsetAsync(gd, 0, gbytes, s), "zero grad");
+  else
     GF_CUDA(launch_radiance_backward(F, P, (const float*)dl, (float*)gd, s), "backward launch");
-  }
   if (gd != grad) {
     GF_CUDA(cudaMemcpyAsync(grad, gd, gbytes, cudaMemcpyDeviceToHost, s), "copy grad");
     GF_CUDA(cudaStreamSynchronize(s), "sync");
