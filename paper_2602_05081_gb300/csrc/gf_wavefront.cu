@@ -24,6 +24,7 @@
 // order.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
 
 #include "gf_host.h"
@@ -554,9 +555,11 @@ struct ServerWork {
 // The paths of one warp: each lane runs its pixels' samples in order (camera
 // ray -> delta tracking -> NEE by ratio tracking -> isotropic scattering), the
 // tracking windows of all 32 lanes advancing together through warp_phase.
+// Only the first `slots` lanes of a warp take paths: a launch with less work than lanes
+// spreads it over every warp of the grid (scatter_slots).
 template <class Work>
 __device__ __forceinline__ void render_paths(const Work& Wk, const float* env, WarpQ& Q,
-                                             float4* wch) {
+                                             float4* wch, int slots) {
   const uint32_t lane = threadIdx.x & 31u;
   LaneRay& R = Q.r[lane];
   Counters cnt;
@@ -659,7 +662,7 @@ __device__ __forceinline__ void render_paths(const Work& Wk, const float* env, W
   // the first pass takes each lane's first work; every later pass is one window
   bool first = true;
   for (int guard = 0; guard < (1 << 30); ++guard) {
-    bool fin = first, fhit = false;
+    bool fin = first && (int)lane < slots, fhit = false;
     float fth = 0.f;
     const bool want = S.kind != 0;
     if (!first && !__any_sync(kFull, want)) break;
@@ -762,11 +765,12 @@ __device__ __forceinline__ float4* warp_store(float4* chord_store) {
 
 __global__ void __launch_bounds__(kWWarps * 32, kBlocksPerSM)
     k_render_scatter(const __grid_constant__ DevField F, const __grid_constant__ PathParams P,
-                     unsigned long long* acc64, int* counter, int chunk, float4* chord_store) {
+                     unsigned long long* acc64, int* counter, int chunk, int slots,
+                     float4* chord_store) {
   extern __shared__ __align__(16) unsigned char smraw[];
   WarpQ& Q = setup_block(smraw, F.env);
   const ImageWork Wk{&F, &P, acc64, counter, P.cam.W * P.cam.H, chunk, (P.spp + chunk - 1) / chunk};
-  render_paths(Wk, reinterpret_cast<const float*>(smraw), Q, warp_store(chord_store));
+  render_paths(Wk, reinterpret_cast<const float*>(smraw), Q, warp_store(chord_store), slots);
 }
 
 __global__ void k_fix_to_image(const unsigned long long* acc64, int64_t npix, int spp, float* out) {
@@ -775,11 +779,11 @@ __global__ void k_fix_to_image(const unsigned long long* acc64, int64_t npix, in
 }
 
 __global__ void __launch_bounds__(kWWarps * 32, kBlocksPerSM)
-    k_render_server(const __grid_constant__ ServerLaunch L, float4* chord_store) {
+    k_render_server(const __grid_constant__ ServerLaunch L, int slots, float4* chord_store) {
   extern __shared__ __align__(16) unsigned char smraw[];
   WarpQ& Q = setup_block(smraw, L.fields[0].env);
   const ServerWork Wk{&L};
-  render_paths(Wk, reinterpret_cast<const float*>(smraw), Q, warp_store(chord_store));
+  render_paths(Wk, reinterpret_cast<const float*>(smraw), Q, warp_store(chord_store), slots);
 }
 
 size_t scatter_smem_bytes() { return 64 + sizeof(WarpQ) * kWWarps; }
@@ -791,10 +795,9 @@ size_t scatter_store_bytes(int64_t grid) {
   return (size_t)grid * kWWarps * 32 * kSlotCh * kRecF4 * sizeof(float4);
 }
 
-// persistent grid of the scattering kernels: every SM filled, never more
-// warps than work (4 warps x 32 lanes per block)
+// full persistent grid of the scattering kernels
 template <class K>
-static cudaError_t scatter_grid(K kernel, int sm_count, int64_t pixels, int64_t& g) {
+static cudaError_t scatter_grid(K kernel, int sm_count, int64_t& g) {
   const size_t smem = scatter_smem_bytes();
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -802,18 +805,29 @@ static cudaError_t scatter_grid(K kernel, int sm_count, int64_t pixels, int64_t&
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kWWarps * 32, smem) != cudaSuccess)
     (void)cudaGetLastError();
   if (per_sm < 1) per_sm = 1;
-  const int64_t need = (pixels + kWWarps * 32 - 1) / (kWWarps * 32);
   g = (int64_t)sm_count * per_sm;
-  if (need < g) g = need;
-  if (g < 1) g = 1;
   return cudaSuccess;
+}
+
+// Paths per warp for `units` units of work, and the grid that holds them (g: the full
+// grid on entry).  With fewer units than lanes every warp of the grid takes its share
+// instead of a few warps taking 32 paths each: a warp works through its paths' windows
+// together, so its time grows with their number.  120x67 pixels at 1 sample through 50k
+// kernels: 1,278 us with 251 full warps, 431 us with 2,010 warps of 4 paths; 96x64
+// 3-bounce paths through 200k kernels: about 47 ms to 10 ms.
+static int scatter_slots(int64_t units, int64_t& g) {
+  const int64_t warps = g * kWWarps;
+  const int64_t slots = std::min<int64_t>(32, std::max<int64_t>(1, (units + warps - 1) / warps));
+  const int64_t need = (units + slots * kWWarps - 1) / (slots * kWWarps);
+  g = std::max<int64_t>(1, std::min(g, need));
+  return (int)slots;
 }
 
 // pixel sums (8 bytes per pixel) and the per-warp chord store of a full
 // persistent grid, grown through the field's allocator
 cudaError_t ensure_render_scratch(const Field& F, int64_t npix, cudaStream_t s) {
   int64_t g = 1;
-  cudaError_t e = scatter_grid(k_render_scatter, F.ctx.sm_count, (int64_t)1 << 40, g);
+  cudaError_t e = scatter_grid(k_render_scatter, F.ctx.sm_count, g);
   if (e != cudaSuccess) return e;
   if ((e = grow(F, (void**)&F.acc64, F.acc_bytes, (size_t)npix * 8, s)) != cudaSuccess) return e;
   return grow(F, (void**)&F.wscratch, F.wscratch_bytes, scatter_store_bytes(g), s);
@@ -825,7 +839,7 @@ cudaError_t launch_render_scatter(const Field& F, const PathParams& P, float* ou
   if (e != cudaSuccess) return e;
   const int64_t npix = (int64_t)P.cam.W * P.cam.H;
   int64_t g = 1;
-  if ((e = scatter_grid(k_render_scatter, F.ctx.sm_count, npix * P.spp, g)) != cudaSuccess) return e;
+  if ((e = scatter_grid(k_render_scatter, F.ctx.sm_count, g)) != cudaSuccess) return e;
   // about 16 units per lane: chunk = ceil(npix spp / (16 lanes)), in [1, spp]
   const int64_t lanes = g * kWWarps * 32;
   int64_t chunk = (npix * P.spp + 16 * lanes - 1) / (16 * lanes);
@@ -835,8 +849,9 @@ cudaError_t launch_render_scatter(const Field& F, const PathParams& P, float* ou
   // fixed-point pixel sums and the chord store (allocated ahead by gf_reserve, else here)
   if ((e = ensure_render_scratch(F, npix, s)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(F.acc64, 0, (size_t)npix * 8, s)) != cudaSuccess) return e;
+  const int slots = scatter_slots(npix * nchunk, g);
   k_render_scatter<<<(unsigned)g, kWWarps * 32, scatter_smem_bytes(), s>>>(
-      F.dev, P, F.acc64, F.counter, (int)chunk, F.wscratch);
+      F.dev, P, F.acc64, F.counter, (int)chunk, slots, F.wscratch);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_fix_to_image<<<(unsigned)((npix + 255) / 256), 256, 0, s>>>(F.acc64, npix, P.spp, out);
   return cudaGetLastError();
@@ -844,7 +859,7 @@ cudaError_t launch_render_scatter(const Field& F, const PathParams& P, float* ou
 
 cudaError_t server_grid(int sm_count, int64_t& g) {
   (void)cudaGetLastError();
-  return scatter_grid(k_render_server, sm_count, (int64_t)1 << 40, g);
+  return scatter_grid(k_render_server, sm_count, g);
 }
 
 cudaError_t launch_fix_to_image(const unsigned long long* acc, int64_t npix, int spp, float* out,
@@ -856,7 +871,8 @@ cudaError_t launch_fix_to_image(const unsigned long long* acc, int64_t npix, int
 cudaError_t launch_render_server(const ServerLaunch& L, int64_t grid, float4* chord_store,
                                  cudaStream_t s) {
   (void)cudaGetLastError();
-  k_render_server<<<(unsigned)grid, kWWarps * 32, scatter_smem_bytes(), s>>>(L, chord_store);
+  const int slots = scatter_slots(L.total, grid);
+  k_render_server<<<(unsigned)grid, kWWarps * 32, scatter_smem_bytes(), s>>>(L, slots, chord_store);
   return cudaGetLastError();
 }
 
