@@ -147,7 +147,7 @@ __device__ __forceinline__ void warp_sum_pair(float& s, float& c) {
 // ---------------------------------------------------------------------------
 // Optical depth of one ray (Eq. 2-3).  A round sets up the chords of 32 leaves,
 // one per lane.  Gauss-Legendre mode: the nodes of those chords are shared out
-// evenly among the lanes (the rule per chord as in det_tau): every chord writes
+// evenly among the lanes (the rule per chord by gl_rule): every chord writes
 // its lane number over its stretch of the round's node list, so that node f of the
 // round finds its chord with one byte load.  Closed form: each lane integrates its
 // own chord.  Every term goes into its lane's compensated sum.
@@ -213,6 +213,246 @@ __device__ __forceinline__ void coop_tau(const DevField& F, CoopQ& Q, const Mask
       neumaier_add(s_acc, c_acc, C.scale * glw[k] * ex2f(y) * cosf(fmaf(C.B, dt, C.delta)));
     }
   });
+}
+
+// ---------------------------------------------------------------------------
+// Analytic free flight of one ray (Sec. 3 Eq. 5, Sec. 4.4 distance sampling).  The
+// optical depth tau(0, t) is the sum of the closed-form chord integrals up to t; with
+// xi the first uniform of the segment's tracking stream, the flight looks for
+// tau(0, t) = -ln(1 - xi).
+//
+// One traversal collects the ray's chords in the warp's list with their full
+// integrals; the bisections then work on the list.  (They used to traverse the tree
+// for every one of up to 33 depths.)  A ray with more chords than the list holds
+// traverses for each depth.
+// ---------------------------------------------------------------------------
+constexpr int kFlightList = 4096;  // chords per warp (global scratch)
+constexpr int kFlightActive = 512; // chords that a bisection still has to clip
+struct FlightRec {
+  float tc, dtin, dtout, a, b, g, B, delta, absA, qmin, dts, w;
+  float full;  // w times the integral over the whole chord
+  float pad[3];
+};
+static_assert(sizeof(FlightRec) == 64, "chord records of 64 bytes");
+struct FlightQ {
+  CoopTrav t;
+  unsigned short act[kFlightActive];
+};
+struct Flight {
+  FlightRec* list;
+  int cap;         // chords the list holds (0: no list)
+  int n;           // chords of the ray (may exceed cap)
+  float tau, tend; // total optical depth and last chord exit
+};
+
+__device__ __forceinline__ Chord flight_chord(const FlightRec& r) {
+  Chord c{};
+  c.tc = r.tc;
+  c.dtin = r.dtin;
+  c.dtout = r.dtout;
+  c.a = r.a;
+  c.b = r.b;
+  c.g = r.g;
+  c.B = r.B;
+  c.delta = r.delta;
+  c.absA = r.absA;
+  c.qmin = r.qmin;
+  c.dts = r.dts;
+  return c;
+}
+
+__device__ __forceinline__ float warp_max(float x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(kFull, x, o));
+  return x;
+}
+
+// chords, total optical depth and last exit of the ray
+static __device__ __noinline__ void flight_gather(const DevField& F, FlightQ& Q, const Mask& M, float3 o,
+                                           float3 v, uint32_t lane, Flight& L, Counters& cnt) {
+  const float3 inv = safe_inv(v);
+  float t0, t1, s = 0.f, c = 0.f, tend = -INFINITY;
+  L.n = 0;
+  L.tau = 0.f;
+  L.tend = -INFINITY;
+  if (M.bits == 0ull || !scene_span(F, o, inv, 0.f, INFINITY, t0, t1)) return;
+  if (lane == 0) cnt.windows += 1;
+  int n = 0;
+  coop_traverse(F, Q.t, M.bits, o, inv, t0, t1, lane, cnt, [&](int j) {
+    Chord ch;
+    float w;
+    const bool ok = j >= 0 && prim_chord(F, j, o, v, 0.f, INFINITY,
+                                         [&](uint32_t cl) { return mask_weight(M, cl); }, w, ch);
+    const unsigned b = __ballot_sync(kFull, ok);
+    if (ok) {
+      ++cnt.chords;
+      const float full = w * chord_closed(F.wd, ch);
+      neumaier_add(s, c, full);
+      tend = fmaxf(tend, ch.tc + ch.dtout);
+      const int k = n + __popc(b & ((1u << lane) - 1u));
+      if (k < L.cap) {
+        float4* d = reinterpret_cast<float4*>(L.list + k);
+        d[0] = make_float4(ch.tc, ch.dtin, ch.dtout, ch.a);
+        d[1] = make_float4(ch.b, ch.g, ch.B, ch.delta);
+        d[2] = make_float4(ch.absA, ch.qmin, ch.dts, w);
+        d[3] = make_float4(full, 0.f, 0.f, 0.f);
+      }
+    }
+    n += __popc(b);
+  });
+  warp_sum_pair(s, c);
+  L.n = n;
+  L.tau = __fadd_rn(s, c);
+  L.tend = warp_max(tend);
+  __syncwarp();
+}
+
+// the part of chord r in [0, mid] added to (s, c)
+__device__ __forceinline__ void flight_part(const DevField& F, const FlightRec& r, float mid, float& s,
+                                            float& c) {
+  const float hi = fminf(r.dtout, mid - r.tc);
+  if (!(r.dtin < hi)) return;
+  if (hi == r.dtout) {
+    neumaier_add(s, c, r.full);
+    return;
+  }
+  Chord ch = flight_chord(r);
+  ch.dtout = hi;
+  neumaier_add(s, c, r.w * chord_closed(F.wd, ch));
+}
+
+// fn(record) for every chord of the ray, each in some lane
+template <class Fn>
+__device__ __forceinline__ void flight_each(const DevField& F, FlightQ& Q, const Mask& M, float3 o,
+                                            float3 v, float tmax, uint32_t lane, const Flight& L,
+                                            Counters& cnt, Fn&& fn) {
+  if (L.n <= L.cap) {
+    for (int k = (int)lane; k < L.n; k += 32) fn(L.list[k]);
+    return;
+  }
+  const float3 inv = safe_inv(v);
+  float t0, t1;
+  if (!scene_span(F, o, inv, 0.f, tmax, t0, t1)) return;
+  coop_traverse(F, Q.t, M.bits, o, inv, t0, t1, lane, cnt, [&](int j) {
+    Chord ch;
+    float w;
+    if (j < 0 || !prim_chord(F, j, o, v, 0.f, INFINITY,
+                             [&](uint32_t cl) { return mask_weight(M, cl); }, w, ch))
+      return;
+    fn(FlightRec{ch.tc, ch.dtin, ch.dtout, ch.a, ch.b, ch.g, ch.B, ch.delta, ch.absA, ch.qmin, ch.dts,
+                 w, w * chord_closed(F.wd, ch), {0.f, 0.f, 0.f}});
+  });
+}
+
+// CDF inversion: 32 bisections of [0, last chord exit].  Chords that end before the
+// bracket keep their full integrals in the lanes' sums, chords that begin behind it
+// leave, so that after a few steps a depth takes the chords around the bracket only.
+// The first crossing needs a non-negative density along the ray.
+static __device__ __noinline__ float cdf_flight(const DevField& F, FlightQ& Q, const Mask& M, float3 o,
+                                         float3 v, float target, uint32_t lane, const Flight& L,
+                                         Counters& cnt) {
+  const unsigned lt = (1u << lane) - 1u;
+  const bool listed = L.n <= L.cap;
+  float lo = 0.f, hi = L.tend;
+  float sb = 0.f, cb = 0.f;  // the lane's chords that end before the bracket
+  int na = -1;               // chords in Q.act; -1: every chord is in play
+  for (int it = 0; it < 32; ++it) {
+    const float mid = 0.5f * (lo + hi);
+    float s = sb, c = cb;
+    if (na < 0)
+      flight_each(F, Q, M, o, v, mid, lane, L, cnt, [&](const FlightRec& r) { flight_part(F, r, mid, s, c); });
+    else
+      for (int k = (int)lane; k < na; k += 32) flight_part(F, L.list[Q.act[k]], mid, s, c);
+    warp_sum_pair(s, c);
+    if (__fadd_rn(s, c) < target) lo = mid;
+    else hi = mid;
+    if (!listed) continue;
+    // the chords a depth inside the bracket still clips
+    const int m = na >= 0 ? na : L.n;
+    int n2 = 0;
+    __syncwarp();
+    for (int b = 0; b < m && n2 <= kFlightActive; b += 32) {
+      const int k = b + (int)lane;
+      const int idx = k < m ? (na >= 0 ? (int)Q.act[k] : k) : 0;
+      bool keep = false;
+      if (k < m) {
+        const FlightRec& r = L.list[idx];
+        const bool before = r.dtout <= lo - r.tc;
+        keep = !before && r.dtin < hi - r.tc;
+        if (before && na >= 0) neumaier_add(sb, cb, r.full);
+      }
+      const unsigned bk = __ballot_sync(kFull, keep);
+      const int pos = n2 + __popc(bk & lt);
+      if (keep && pos < kFlightActive) Q.act[pos] = (unsigned short)idx;
+      n2 += __popc(bk);
+      __syncwarp();
+    }
+    if (na < 0) {
+      if (n2 > kFlightActive) continue;  // too many yet: every chord stays in play
+      for (int k = (int)lane; k < L.n; k += 32) {
+        const FlightRec& r = L.list[k];
+        if (r.dtout <= lo - r.tc) neumaier_add(sb, cb, r.full);
+      }
+    }
+    na = n2;
+  }
+  return 0.5f * (lo + hi);
+}
+
+// Uniform sampling within the crossing segment (Sec. 3: the cheap approximation of the
+// CDF inversion; Sec. 4.4 distance sampling).  The ray is cut into segments at t = 0 and
+// at every chord entry and exit; the segment [e_a, e_b] in which tau(0, t) reaches the
+// target holds the collision e_a + u (e_b - e_a).  It is found by bisection on t that
+// stops once no chord end lies inside the bracket: every step takes tau(0, mid), the
+// chord ends inside both halves of the bracket and the nearest ends around them.
+static __device__ __noinline__ float segment_flight(const DevField& F, FlightQ& Q, const Mask& M, float3 o,
+                                             float3 v, float target, float u, uint32_t lane,
+                                             const Flight& L, Counters& cnt) {
+  float lo = 0.f, hi = L.tend;
+  float ea = 0.f, eb = L.tend;
+  for (int it = 0; it < 48; ++it) {
+    const float mid = 0.5f * (lo + hi);
+    float s = 0.f, c = 0.f;
+    int n_left = 0, n_right = 0;              // chord ends in (lo, mid) and in (mid, hi)
+    float below_lo = 0.f, below_mid = 0.f;    // largest end <= lo, <= mid (or 0)
+    float above_mid = INFINITY, above_hi = INFINITY;  // smallest end >= mid, >= hi
+    auto end = [&](float e) {
+      n_left += (e > lo && e < mid) ? 1 : 0;
+      n_right += (e > mid && e < hi) ? 1 : 0;
+      if (e <= lo) below_lo = fmaxf(below_lo, e);
+      if (e <= mid) below_mid = fmaxf(below_mid, e);
+      if (e >= mid) above_mid = fminf(above_mid, e);
+      if (e >= hi) above_hi = fminf(above_hi, e);
+    };
+    flight_each(F, Q, M, o, v, INFINITY, lane, L, cnt, [&](const FlightRec& r) {
+      const float tin = r.tc + r.dtin, tout = r.tc + r.dtout;
+      end(tin);
+      end(tout);
+      if (tin >= mid) return;
+      if (!(tout > mid)) {
+        neumaier_add(s, c, r.full);
+      } else {  // the chord's part in [0, mid]
+        Chord ch = flight_chord(r);
+        ch.dtout = mid - r.tc;
+        neumaier_add(s, c, r.w * chord_closed(F.wd, ch));
+      }
+    });
+    warp_sum_pair(s, c);
+    if (__fadd_rn(s, c) < target) {
+      lo = mid;
+      ea = warp_max(below_mid);
+      eb = -warp_max(-above_hi);
+      if (__reduce_add_sync(kFull, n_right) == 0) break;
+    } else {
+      hi = mid;
+      ea = warp_max(below_lo);
+      eb = -warp_max(-above_mid);
+      if (__reduce_add_sync(kFull, n_left) == 0) break;
+    }
+    if (!(hi > lo)) break;
+  }
+  if (!(eb < INFINITY)) eb = L.tend;
+  return ea + u * (eb - ea);
 }
 
 }  // namespace gf

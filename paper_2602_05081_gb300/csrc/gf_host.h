@@ -201,6 +201,7 @@ cudaError_t launch_pack(Field& F, const gf_params& P, cudaStream_t s);
 cudaError_t build_bvh(Field& F, cudaStream_t s);
 cudaError_t launch_pack16(Field& F, cudaStream_t s);
 size_t scatter_store_bytes(int64_t grid);
+size_t flight_store_bytes(const Field& F);
 cudaError_t server_grid(int sm_count, int64_t& grid);
 cudaError_t launch_render_server(const ServerLaunch& L, int64_t grid, float4* chord_store,
                                  cudaStream_t s);

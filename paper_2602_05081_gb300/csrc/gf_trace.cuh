@@ -341,11 +341,7 @@ __device__ __forceinline__ Mask sample_mask(const DevField& F, const LodDev& L, 
   return sample_mask_call(F, L, v, seed, ray, sample, bounce, tag);
 }
 
-// ---------------------------------------------------------------------------
-// deterministic optical depth along one ray (Eq. 2-3): every chord is
-// integrated by Gauss-Legendre as soon as its leaf is reached; FP32 with an
-// accurate cosine, Neumaier compensation across chords.
-// ---------------------------------------------------------------------------
+// a box overlaps the span [t0, t1] of the ray
 struct SpanTest {
   float t0, t1;
   __device__ __forceinline__ bool operator()(float tn, float tf) const {
@@ -366,62 +362,6 @@ __device__ __forceinline__ void gl_pick(int r, int& n, int& off) {
   constexpr unsigned long long kN = gl_bytes(false), kOff = gl_bytes(true);
   n = (int)(kN >> (8 * r)) & 0xFF;
   off = (int)(kOff >> (8 * r)) & 0xFF;
-}
-
-struct DetLeaf {
-  const DevField* F;
-  const Mask* M;
-  float3 o, v;
-  float tmin, tmax;
-  const float* glx;
-  const float* glw;
-  float s = 0.f, c = 0.f;
-  unsigned long long nch = 0, nev = 0;
-  __device__ __forceinline__ void operator()(int j) {
-    const Mask& Mk = *M;
-    Chord ch;
-    float w;
-    if (!prim_chord(*F, j, o, v, tmin, tmax, [&](uint32_t c) { return mask_weight(Mk, c); }, w, ch))
-      return;
-    ++nch;
-    const float len = ch.dtout - ch.dtin;
-    int n, off;
-    gl_pick(gl_rule(sqrtf(ch.a) * len + 0.5f * fabsf(ch.B) * len), n, off);
-    const float mid = 0.5f * (ch.dtin + ch.dtout), hl = 0.5f * len;
-    const float y2 = -0.5f * kLog2e * ch.a, y1 = -kLog2e * ch.b, y0 = -0.5f * kLog2e * ch.g;
-    const float scale = w * ch.absA * hl;
-    // every node's term goes into the ray's compensated sum (the node sums of
-    // a chord can cancel as much as the chords of a ray)
-    for (int k = 0; k < n; ++k) {
-      const float dt = fmaf(hl, glx[off + k], mid);
-      const float y = fmaf(fmaf(y2, dt, y1), dt, y0);
-      neumaier_add(s, c, scale * glw[off + k] * ex2f(y) * cosf(fmaf(ch.B, dt, ch.delta)));
-    }
-    nev += (unsigned long long)n;
-  }
-};
-
-__device__ __forceinline__ float det_tau(const DevField& F, const Mask& M, float3 o, float3 v,
-                                         float tmin, float tmax, const float* glx,
-                                         const float* glw, Counters& cnt) {
-  const float3 inv = safe_inv(v);
-  float t0, t1;
-  if (M.bits == 0ull || !scene_span(F, o, inv, tmin, tmax, t0, t1)) return 0.f;
-  DetLeaf leaf;
-  leaf.F = &F;
-  leaf.M = &M;
-  leaf.o = o;
-  leaf.v = v;
-  leaf.tmin = tmin;
-  leaf.tmax = tmax;
-  leaf.glx = glx;
-  leaf.glw = glw;
-  SpanTest test{t0, t1};
-  traverse_ray(F, o, inv, M.bits, test, leaf, cnt.nodes, cnt.leaves);
-  cnt.windows += 1;
-  cnt.chords += leaf.nch;
-  cnt.evals += leaf.nev;
-  return __fadd_rn(leaf.s, leaf.c);
 }
 
 // ---------------------------------------------------------------------------
@@ -468,162 +408,6 @@ __device__ __forceinline__ float chord_closed(const Weideman& W, const Chord& ch
     acc += 2.0f * ex2f(-kLog2e * fmaf(beta, beta, 0.5f * ch.qmin)) *
            cosf(fmaf(ch.B, ch.dts, ch.delta));
   return ch.absA * (0.88622692545275801f / s) * acc;  // sqrt(pi)/2 / s
-}
-
-struct ClosedLeaf {
-  const DevField* F;
-  const Mask* M;
-  float3 o, v;
-  float tmin, tmax;
-  float s = 0.f, c = 0.f;
-  float tend = -INFINITY;  // the last chord exit
-  unsigned long long nch = 0;
-  __device__ __forceinline__ void operator()(int j) {
-    const Mask& Mk = *M;
-    Chord ch;
-    float w;
-    if (!prim_chord(*F, j, o, v, tmin, tmax, [&](uint32_t c) { return mask_weight(Mk, c); }, w, ch))
-      return;
-    ++nch;
-    tend = fmaxf(tend, ch.tc + ch.dtout);
-    neumaier_add(s, c, w * chord_closed(F->wd, ch));
-  }
-};
-
-__device__ __forceinline__ float closed_tau(const DevField& F, const Mask& M, float3 o, float3 v,
-                                            float tmin, float tmax, Counters& cnt,
-                                            float* tend = nullptr) {
-  const float3 inv = safe_inv(v);
-  float t0, t1;
-  if (tend) *tend = -INFINITY;
-  if (M.bits == 0ull || !scene_span(F, o, inv, tmin, tmax, t0, t1)) return 0.f;
-  ClosedLeaf leaf;
-  leaf.F = &F;
-  leaf.M = &M;
-  leaf.o = o;
-  leaf.v = v;
-  leaf.tmin = tmin;
-  leaf.tmax = tmax;
-  SpanTest test{t0, t1};
-  traverse_ray(F, o, inv, M.bits, test, leaf, cnt.nodes, cnt.leaves);
-  cnt.windows += 1;
-  cnt.chords += leaf.nch;
-  if (tend) *tend = leaf.tend;
-  return __fadd_rn(leaf.s, leaf.c);
-}
-
-// Free flight by inversion of the optical-depth CDF (Sec. 3 Eq. 5, segment-based
-// transfer; Sec. 4.4 distance sampling): with xi the first uniform of the
-// segment's tracking stream, the distance solves tau(0, t) = -ln(1 - xi),
-// found by 32 bisections of [0, last chord exit] on the closed-form optical
-// depth (one windowed traversal each).  Returns false when the whole ray's
-// optical depth does not reach the target.  The first crossing needs a
-// non-negative density along the ray.
-__device__ __forceinline__ bool cdf_flight(const DevField& F, const Mask& M, float3 o, float3 v,
-                                           uint64_t seed, uint32_t ray, uint32_t word, float& th,
-                                           Counters& cnt) {
-  const uint4 y = rng4(seed, 0, kNoPrim, ray, word);
-  const float target = -log1pf(-u01(y.x));
-  float tend;
-  const float total = closed_tau(F, M, o, v, 0.f, INFINITY, cnt, &tend);
-  if (!(tend > 0.f) || total < target) return false;
-  float lo = 0.f, hi = tend;
-  for (int it = 0; it < 32; ++it) {
-    const float mid = 0.5f * (lo + hi);
-    if (closed_tau(F, M, o, v, 0.f, mid, cnt) < target) lo = mid;
-    else hi = mid;
-  }
-  th = 0.5f * (lo + hi);
-  return true;
-}
-
-// Free flight by uniform sampling within the crossing segment (Sec. 3: the
-// cheap approximation of the CDF inversion; Sec. 4.4 distance sampling).  The
-// ray is cut into segments at t = 0 and at every chord entry and exit; the
-// segment [e_a, e_b] in which tau(0, t) reaches the target -ln(1 - xi) holds
-// the collision e_a + u (e_b - e_a), xi and u the first two uniforms of the
-// segment's tracking stream.  The crossing segment is found by bisection on t
-// that stops once no chord end lies inside the bracket: every step is one
-// traversal giving tau(0, mid), the chord ends inside both halves of the
-// bracket and the nearest ends around them.
-struct SegLeaf {
-  const DevField* F;
-  const Mask* M;
-  float3 o, v;
-  float lo, mid, hi;  // the bracket and its midpoint
-  float s = 0.f, c = 0.f;  // tau(0, mid), compensated
-  int n_left = 0, n_right = 0;  // chord ends in (lo, mid) and in (mid, hi)
-  float below_lo = 0.f, below_mid = 0.f;             // largest end <= lo, <= mid (or 0)
-  float above_mid = INFINITY, above_hi = INFINITY;   // smallest end >= mid, >= hi
-  __device__ __forceinline__ void end(float e) {
-    n_left += (e > lo && e < mid) ? 1 : 0;
-    n_right += (e > mid && e < hi) ? 1 : 0;
-    if (e <= lo) below_lo = fmaxf(below_lo, e);
-    if (e <= mid) below_mid = fmaxf(below_mid, e);
-    if (e >= mid) above_mid = fminf(above_mid, e);
-    if (e >= hi) above_hi = fminf(above_hi, e);
-  }
-  __device__ __forceinline__ void operator()(int j) {
-    const Mask& Mk = *M;
-    Chord ch;
-    float w;
-    if (!prim_chord(*F, j, o, v, 0.f, INFINITY, [&](uint32_t cc) { return mask_weight(Mk, cc); }, w,
-                    ch))
-      return;
-    end(ch.tc + ch.dtin);
-    end(ch.tc + ch.dtout);
-    if (ch.tc + ch.dtin >= mid) return;
-    // the chord's part in [0, mid]
-    if (ch.tc + ch.dtout > mid) ch.dtout = mid - ch.tc;
-    neumaier_add(s, c, w * chord_closed(F->wd, ch));
-  }
-};
-
-__device__ __forceinline__ bool segment_flight(const DevField& F, const Mask& M, float3 o, float3 v,
-                                               uint64_t seed, uint32_t ray, uint32_t word,
-                                               float& th, Counters& cnt) {
-  const uint4 y = rng4(seed, 0, kNoPrim, ray, word);
-  const float target = -log1pf(-u01(y.x));
-  float tend;
-  const float total = closed_tau(F, M, o, v, 0.f, INFINITY, cnt, &tend);
-  if (!(tend > 0.f) || total < target) return false;
-  const float3 inv = safe_inv(v);
-  float t0, t1;
-  if (!scene_span(F, o, inv, 0.f, INFINITY, t0, t1)) return false;
-  float lo = 0.f, hi = tend;
-  float ea = 0.f, eb = tend;
-  for (int it = 0; it < 48; ++it) {
-    SegLeaf leaf;
-    leaf.F = &F;
-    leaf.M = &M;
-    leaf.o = o;
-    leaf.v = v;
-    leaf.lo = lo;
-    leaf.hi = hi;
-    leaf.mid = 0.5f * (lo + hi);
-    SpanTest test{t0, t1};
-    unsigned long long nodes = 0, leaves = 0;
-    traverse_ray(F, o, inv, M.bits, test, leaf, nodes, leaves);
-    cnt.nodes += nodes;
-    cnt.leaves += leaves;
-    cnt.windows += 1;
-    const bool right = __fadd_rn(leaf.s, leaf.c) < target;
-    if (right) {
-      lo = leaf.mid;
-      ea = leaf.below_mid;
-      eb = leaf.above_hi;
-      if (leaf.n_right == 0) break;
-    } else {
-      hi = leaf.mid;
-      ea = leaf.below_lo;
-      eb = leaf.above_mid;
-      if (leaf.n_left == 0) break;
-    }
-    if (!(hi > lo)) break;
-  }
-  if (!(eb < INFINITY)) eb = tend;
-  th = ea + u01(y.y) * (eb - ea);
-  return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -956,60 +740,6 @@ __device__ __forceinline__ unsigned long long fov_cells(const DevField& F, const
   for (int b = 1; b < 8; ++b)
     if (F.band_wmax[b] <= f) m |= 0xFFull << (1 + kCones * (b - 1));
   return m;
-}
-
-// One sample of pixel (px, py): scattering radiance with the free flight FF
-// (GF_FLIGHT_CDF or GF_FLIGHT_SEGMENT).  Called by all lanes of a warp together
-// (inactive lanes with active = false): every phase (flight, NEE, scattering) runs
-// with the lanes that need it converged, and the lanes regroup after each phase.
-template <int FF>
-static __device__ float path_sample(const DevField& F, const PathParams& P, bool active, int px,
-                                    int py, int s, Counters& cnt) {
-  float3 o = make_float3(0.f, 0.f, 0.f), v = make_float3(0.f, 0.f, 1.f);
-  if (active) camera_ray(P.cam, P.seed, px, py, s, o, v);
-  const uint32_t pix = (uint32_t)py * (uint32_t)P.cam.W + (uint32_t)px;
-  const unsigned long long allow = fov_cells(F, P, v, pix, (uint32_t)s);
-  float thr = 1.f, Lsum = 0.f;
-  bool alive = active;
-  GF_TIC(ct);
-  for (int b = 0; b < P.max_bounces; ++b) {
-    float th = 0.f, hit = 0.f;
-    if (alive) {
-      GF_TIC(cm);
-      Mask m = sample_mask(F, P.lod, v, P.seed, pix, (uint32_t)s, (uint32_t)b, TAG_MASK);
-      m.bits &= allow;
-      GF_TOC(cnt, 3, cm);
-      cnt.rays += 1;
-      const uint32_t tw = stream_word((uint32_t)s, (uint32_t)b, TAG_TRACK);
-      if constexpr (FF == GF_FLIGHT_CDF)
-        hit = cdf_flight(F, m, o, v, P.seed, pix, tw, th, cnt) ? 1.f : 0.f;
-      else
-        hit = segment_flight(F, m, o, v, P.seed, pix, tw, th, cnt) ? 1.f : 0.f;
-    }
-    __syncwarp();
-    alive = alive && hit != 0.f;
-    const float3 x = make_float3(o.x + th * v.x, o.y + th * v.y, o.z + th * v.z);
-    if (alive) {
-      thr *= P.albedo;
-      Mask mn = sample_mask(F, P.lod_nee, P.light, P.seed, pix, (uint32_t)s, (uint32_t)b,
-                            TAG_NEE_MASK);
-      mn.bits &= allow;
-      cnt.rays += 1;
-      const float Tl = expf(-closed_tau(F, mn, x, P.light, 0.f, INFINITY, cnt));
-      Lsum += thr * P.irradiance * Tl * (0.25f / 3.14159265358979f);
-      const uint4 y = rng4(P.seed, 0, kNoPrim, pix, stream_word((uint32_t)s, (uint32_t)b, TAG_SCATTER));
-      const float z = 1.0f - 2.0f * u01(y.x);
-      const float rr = sqrtf(fmaxf(0.0f, 1.0f - z * z));
-      float sn, cs;
-      sincosf(2.0f * 3.14159265358979f * u01(y.y), &sn, &cs);
-      v = make_float3(rr * cs, rr * sn, z);
-      o = x;
-    }
-    __syncwarp();
-    if (!__any_sync(kFull, alive)) break;
-  }
-  GF_TOC(cnt, 4, ct);
-  return Lsum;
 }
 
 }  // namespace gf

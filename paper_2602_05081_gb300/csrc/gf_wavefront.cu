@@ -823,14 +823,15 @@ static int scatter_slots(int64_t units, int64_t& g) {
   return (int)slots;
 }
 
-// pixel sums (8 bytes per pixel) and the per-warp chord store of a full
-// persistent grid, grown through the field's allocator
+// pixel sums (8 bytes per pixel) and the per-warp chord store of a full persistent
+// grid (shared with the analytic flights' lists), grown through the field's allocator
 cudaError_t ensure_render_scratch(const Field& F, int64_t npix, cudaStream_t s) {
   int64_t g = 1;
   cudaError_t e = scatter_grid(k_render_scatter, F.ctx.sm_count, g);
   if (e != cudaSuccess) return e;
   if ((e = grow(F, (void**)&F.acc64, F.acc_bytes, (size_t)npix * 8, s)) != cudaSuccess) return e;
-  return grow(F, (void**)&F.wscratch, F.wscratch_bytes, scatter_store_bytes(g), s);
+  return grow(F, (void**)&F.wscratch, F.wscratch_bytes,
+              std::max(scatter_store_bytes(g), flight_store_bytes(F)), s);
 }
 
 cudaError_t launch_render_scatter(const Field& F, const PathParams& P, float* out, cudaStream_t s) {

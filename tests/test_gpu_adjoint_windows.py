@@ -1,8 +1,9 @@
-"""The adjoints where their per-warp buffers overflow, against the FP64 oracle (GPU).
+"""Adjoints and analytic flights where their per-warp buffers overflow, against the FP64
+oracle (GPU).
 
 A warp holds up to 4,096 chords and 128 tentative points of a ray's window, 64 (then
-256) chords covering a point, and 1,024 chords of a tomography ray.  Each field here
-passes one of these limits, on few pixels.
+256) chords covering a point, 1,024 chords of a tomography ray, 4,096 chords of an
+analytic flight.  Each field here passes one of these limits, on few pixels.
 """
 import numpy as np
 import pytest
@@ -92,3 +93,23 @@ def test_tomography_adjoint_beyond_the_buffers(api, ctx):
     f.sync()
     _, ref = orc.tomo_loss_grad(co, 1, 5, target)
     _check(g.cpu().numpy().astype(np.float64), ref, n, "tomography")
+
+
+@pytest.mark.parametrize("flight", ["cdf", "segment"])
+def test_analytic_flight_beyond_the_list(api, ctx, flight):
+    """About 5,000 chords on a ray (Gaussians, so that the density is positive): every
+    depth traverses the tree.  The radiance is smooth in the collision point, whose FP32
+    depth is within 1e-5 of the target: 1e-3 of a pixel and 1e-4 of the largest."""
+    n, res = 60_000, 4
+    p = synth.octave_field(n, 1, seed=33)
+    f = api.Field(ctx, p)
+    c = synth.DEFAULT_CAMERA
+    cg = api.camera(c["eye"], c["look_at"], c["up"], 30.0, res, res)
+    co = oracle.camera(c["eye"], c["look_at"], c["up"], 30.0, res, res)
+    img = f.render(cg, api.render_opts("scatter", 1, 2, free_flight=flight), seed=3)
+    f.sync()
+    ref = oracle.Field(p, omega_frame="local").render(
+        co, oracle.render_opts("scatter", 1, 2, free_flight=flight), seed=3)
+    a = img.cpu().numpy().astype(np.float64)
+    assert ref.max() > 0
+    assert np.all(np.abs(a - ref) <= 1e-3 * np.abs(ref) + 1e-4 * ref.max())
