@@ -468,7 +468,7 @@ constexpr int kRadStack = 384;    // a step adds <= 32; depth first above kRadSt
 constexpr int kRadMargin = 128;   // a full step, then <= 1 entry per level, 64 levels
 constexpr int kRadLeafQ = 96;     // <= 31 left + 64 new
 constexpr int kRadPts = 128;      // tentative points of a window
-constexpr int kRadList = 4096;    // chords of a window (global scratch)
+constexpr int kRadList = 4096;    // chords of a window at most (global scratch; rad_list_cap)
 constexpr int kRadKeep = 4096;    // kept segment moments of a path (global scratch)
 constexpr int kRadGroup = 4;      // points whose sums are formed together
 constexpr int kRadTerms = 256;    // covering chords of a group, 64 per point
@@ -489,8 +489,14 @@ struct RadList {
                             // (peak - tc, exponent at tc without the amplitude, mask
                             // weight, sorted primitive as bits)
 };
-constexpr size_t kRadListBytes = (size_t)kRadList * (8 + 8 + 48);
-constexpr size_t kRadWarpBytes = 2 * kRadListBytes + (size_t)kRadKeep * sizeof(RadKept);
+// a field of fewer kernels needs no longer lists
+__host__ __device__ __forceinline__ int rad_list_cap(int64_t n) {
+  return (int)(n < kRadList ? (n + 63) / 64 * 64 : kRadList);
+}
+__host__ __device__ __forceinline__ size_t rad_list_bytes(int cap) { return (size_t)cap * (8 + 8 + 48); }
+__host__ __device__ __forceinline__ size_t rad_warp_bytes(int cap) {
+  return 2 * rad_list_bytes(cap) + (size_t)kRadKeep * sizeof(RadKept);
+}
 
 struct RadTravQ {
   unsigned long long skey[kRadStack];
@@ -536,19 +542,20 @@ struct RadWarp {
   unsigned char* scratch;
   const float* env;
   uint32_t lane;
+  int cap;      // chords per list
   int nkept;    // kept moments (may exceed kRadKeep)
   bool replay;  // some segment could not be kept
   Counters cnt;
   __device__ __forceinline__ RadList list(int which) const {
-    unsigned char* p = scratch + (size_t)which * kRadListBytes;
+    unsigned char* p = scratch + (size_t)which * rad_list_bytes(cap);
     RadList L;
     L.key = reinterpret_cast<unsigned long long*>(p);
-    L.span = reinterpret_cast<float2*>(p + (size_t)kRadList * 8);
-    L.rec = reinterpret_cast<float4*>(p + (size_t)kRadList * 16);
+    L.span = reinterpret_cast<float2*>(p + (size_t)cap * 8);
+    L.rec = reinterpret_cast<float4*>(p + (size_t)cap * 16);
     return L;
   }
   __device__ __forceinline__ RadKept* kept() const {
-    return reinterpret_cast<RadKept*>(scratch + 2 * kRadListBytes);
+    return reinterpret_cast<RadKept*>(scratch + 2 * rad_list_bytes(cap));
   }
 };
 
@@ -675,7 +682,7 @@ __device__ __noinline__ void rad_gather(RadWarp& W, int which) {
                       ch.tc + ch.dtin <= tb && ch.tc + ch.dtout >= ta;
       const unsigned bc = __ballot_sync(kFull, ok);
       const int k = nch + __popc(bc & lt);
-      if (ok && k < kRadList) {
+      if (ok && k < W.cap) {
         const float wa = w * ch.absA;
         const float y2 = -0.5f * kLog2e * ch.a, y1 = -kLog2e * ch.b;
         const float y0 = fmaf(-0.5f * kLog2e, ch.g, log2f(wa));
@@ -944,7 +951,7 @@ __device__ __noinline__ int rad_window(RadWarp& W, int which) {
   RadQ& Q = W.Q;
   for (int it = 0; it < 64; ++it) {
     rad_gather(W, which);
-    if (Q.ray.nch <= kRadList && Q.ray.npts <= kRadPts) {
+    if (Q.ray.nch <= W.cap && Q.ray.npts <= kRadPts) {
       if (W.lane == 0) Q.ray.listed = 1;
       rad_sort(W, which);
       return Q.ray.npts;
@@ -1366,8 +1373,8 @@ __global__ void __launch_bounds__(kBackBlock, kRadBlocks)
   __syncthreads();
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   RadWarp W{F, P, Bk, reinterpret_cast<RadQ*>(smraw + 32)[warp],
-            scratch + ((size_t)blockIdx.x * (kBackBlock / 32) + warp) * kRadWarpBytes, env, lane, 0,
-            false, Counters()};
+            scratch + ((size_t)blockIdx.x * (kBackBlock / 32) + warp) * rad_warp_bytes(rad_list_cap(F.n)),
+            env, lane, rad_list_cap(F.n), 0, false, Counters()};
   const uint32_t nchunk = (uint32_t)((P.spp + chunk - 1) / chunk);
   const uint32_t units = (uint32_t)(P.cam.W * P.cam.H) * nchunk;
   for (;;) {
@@ -1432,38 +1439,47 @@ static cudaError_t adjoint_stack_fits(K kernel) {
   return e;
 }
 
-// scratch of the adjoints, grown through the field's allocator: per warp of a full
-// persistent grid the chord lists and kept moments (radiance) or the kept chords
-// (tomography) in one buffer, and the arrays per primitive
+// scratch of an adjoint kernel of a full persistent grid of g blocks: the kept chords
+// (tomography), or the chord lists and kept moments (radiance), in one buffer
+static size_t tomo_scratch(int64_t g) {
+  return (size_t)g * (kBackBlock / 32) * kTomoChords * sizeof(TomoChord);
+}
+static size_t rad_scratch(const Field& F, int64_t g) {
+  return (size_t)g * (kBackBlock / 32) * rad_warp_bytes(rad_list_cap(F.n));
+}
+static cudaError_t grow_adjoint(const Field& F, size_t bytes, cudaStream_t s) {
+  const cudaError_t e = grow(F, (void**)&F.adj, F.adj_bytes, (size_t)F.n * 7 * sizeof(float4), s);
+  return e != cudaSuccess ? e : grow(F, (void**)&F.rlist, F.rlist_bytes, bytes, s);
+}
+
+// the scratch of every adjoint and the arrays per primitive, through the field's allocator
 cudaError_t ensure_adjoint_lists(const Field& F, cudaStream_t s) {
   int64_t g = 1;
   size_t bytes = 0;
   cudaError_t e;
   if ((e = adjoint_grid(F, k_tomo_backward, 0, g)) != cudaSuccess) return e;
-  bytes = (size_t)g * (kBackBlock / 32) * kTomoChords * sizeof(TomoChord);
+  bytes = tomo_scratch(g);
   if ((e = adjoint_grid(F, k_radiance_backward<false>, kRadSmem, g)) != cudaSuccess) return e;
-  bytes = std::max(bytes, (size_t)g * (kBackBlock / 32) * kRadWarpBytes);
+  bytes = std::max(bytes, rad_scratch(F, g));
   if ((e = adjoint_grid(F, k_radiance_backward<true>, kRadSmem, g)) != cudaSuccess) return e;
-  bytes = std::max(bytes, (size_t)g * (kBackBlock / 32) * kRadWarpBytes);
-  if ((e = grow(F, (void**)&F.adj, F.adj_bytes, (size_t)F.n * 7 * sizeof(float4), s)) != cudaSuccess)
-    return e;
-  return grow(F, (void**)&F.rlist, F.rlist_bytes, bytes, s);
+  return grow_adjoint(F, std::max(bytes, rad_scratch(F, g)), s);
 }
 
 // An adjoint kernel over units of `chunk` samples of a pixel (about 16 per warp of the
 // grid at least), between the per-primitive inputs and the copy of the sums to grad
-template <class K, class T>
-static cudaError_t launch_adjoint(const Field& F, const PathParams& P, K kernel, size_t smem,
-                                  const float* dLdI, float* grad, T* scratch_type, cudaStream_t s) {
-  (void)scratch_type;
+template <class T>
+static cudaError_t launch_adjoint(const Field& F, const PathParams& P,
+                                  void (*kernel)(DevField, PathParams, BackArgs, const float*, int*, int, T*),
+                                  size_t smem, const float* dLdI, float* grad, cudaStream_t s) {
   (void)cudaGetLastError();  // a stale error of an unrelated call is not ours
   cudaError_t e = cudaMemsetAsync(F.counter, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   BackArgs B = back_args(F, grad);
   int64_t g = 1;
   if ((e = adjoint_stack_fits(kernel)) != cudaSuccess) return e;
-  if ((e = ensure_adjoint_lists(F, s)) != cudaSuccess) return e;  // unless gf_reserve has
   if ((e = adjoint_grid(F, kernel, smem, g)) != cudaSuccess) return e;
+  // (allocated ahead by gf_reserve, else here)
+  if ((e = grow_adjoint(F, smem ? rad_scratch(F, g) : tomo_scratch(g), s)) != cudaSuccess) return e;
   const int64_t npix = (int64_t)P.cam.W * P.cam.H, warps = g * (kBackBlock / 32);
   int64_t nchunk = (16 * warps + npix - 1) / npix;
   nchunk = nchunk < 1 ? 1 : (nchunk > P.spp ? P.spp : nchunk);
@@ -1485,13 +1501,13 @@ static cudaError_t launch_adjoint(const Field& F, const PathParams& P, K kernel,
 
 cudaError_t launch_tomo_backward(const Field& F, const PathParams& P, const float* dLdI,
                                  float* grad, cudaStream_t s) {
-  return launch_adjoint(F, P, k_tomo_backward, 0, dLdI, grad, (TomoChord*)nullptr, s);
+  return launch_adjoint(F, P, k_tomo_backward, 0, dLdI, grad, s);
 }
 
 cudaError_t launch_radiance_backward(const Field& F, const PathParams& P, const float* dLdI,
                                      float* grad, cudaStream_t s) {
   return launch_adjoint(F, P, P.max_bounces >= 2 ? k_radiance_backward<true> : k_radiance_backward<false>,
-                        kRadSmem, dLdI, grad, (unsigned char*)nullptr, s);
+                        kRadSmem, dLdI, grad, s);
 }
 
 }  // namespace gf

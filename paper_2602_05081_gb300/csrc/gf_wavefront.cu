@@ -36,11 +36,16 @@ constexpr int kWWarps = 4;      // warps per block
 constexpr int kBlocksPerSM = 4; // resident blocks per SM the kernels are built for
 constexpr int kLeafQ = 160;     // queued leaves per warp (<= 31 left + 128 new)
 constexpr int kChordQ = 64;     // queued chords per warp (<= 31 left + 32 new)
-constexpr int kPK = 8;          // tentative points per lane and window
-constexpr int kSlotCh = 256;    // stored chords per lane and window (global scratch)
+// A window with more points or chords than its slot holds is halved and traversed
+// again: with 8 points and 256 chords that took 9 % of the windows of the 1M-kernel
+// benchmark and a third of those through 200k kernels at full detail.  13 points fill
+// the shared memory of 4 blocks per SM.  1024x1024, 8 samples, 1M kernels, stochastic
+// masks: 317 -> 303 ms; 512x512, 16 samples, 100k kernels: 196 -> 183 ms.
+constexpr int kPK = 13;         // tentative points per lane and window
+constexpr int kSlotCh = 448;    // stored chords per lane and window (global scratch)
 constexpr int kRecF4 = 2;       // float4s per stored chord record
 
-// One slot per lane, 47 words: an odd stride keeps same-field accesses of the
+// One slot per lane, 57 words: an odd stride keeps same-field accesses of the
 // 32 slots in distinct shared-memory banks.
 struct LaneRay {
   float o[3], v[3], inv[3];
@@ -57,6 +62,7 @@ struct LaneRay {
   float pt[kPK], pu[kPK];       // the window's tentative points (t, acceptance uniform)
 };
 static_assert(sizeof(LaneRay) % 8 == 4, "odd word stride");
+static_assert(kSlotCh <= 448, "sums of kSlotCh terms below 2^54 (1 + 1e-6) stay below 2^63");
 struct ChordItem {
   float tc;
   float dt;           // where the walk stands (relative to tc): the chord's entry, then
@@ -344,7 +350,8 @@ struct PathState {
   float Lsum, thr, T;
   float3 o, v;    // current ray
   float t0, t1;   // scene span of the current ray
-  float step;     // window length for delta tracking
+  float step;     // window length
+  float fit;      // windows longer than this held too many chords lately
   unsigned long long allow;  // cells the foveation keeps for the sample's path
 };
 
@@ -377,9 +384,13 @@ __device__ __forceinline__ bool start_ray(const DevField& F, LaneRay& R, PathSta
   S.t0 = t0;
   S.t1 = t1;
   if (!hit) return false;
-  S.step = kind == 1 ? fmaxf(0.25f * (t1 - t0), 1e-6f) : (t1 - t0);
+  // first window: a quarter of the span when tracking, all of it for NEE, but not a
+  // length that held too many chords on the lane's last rays
+  const float len = t1 - t0;
+  S.step = kind == 1 ? fmaxf(fminf(0.25f * len, S.fit), 1e-6f) : fminf(len, S.fit);
+  S.fit *= 1.1f;
   R.ta = t0;
-  R.te = kind == 1 ? fminf(t1, t0 + S.step) : t1;
+  R.te = kind == 1 || S.step < len ? fminf(t1, t0 + S.step) : t1;
   if (R.te >= t1) R.te = t1 * (1.0f + 1e-7f) + 1e-30f;  // last window includes t1
   return true;
 }
@@ -389,9 +400,9 @@ __device__ __forceinline__ bool start_ray(const DevField& F, LaneRay& R, PathSta
 // no lane waits on one slot's short list; each pair tests the chord against
 // the slot's points and adds its terms to the slot's sums in shared memory.
 // The sums are exact in 64-bit fixed point: a term is at most the peak h of
-// its chord, so with H the largest peak of the slot's window and at most
-// kSlotCh = 2^8 chords, scaling by 2^(54 - e) (H < 2^e) keeps every partial
-// sum below 2^62.  Each term is rounded once (to 2^(e-54), far below FP32
+// its chord (to ~1e-6), so with H the largest peak of the slot's window and at most
+// kSlotCh < 2^9 chords, scaling by 2^(54 - e) (H < 2^e) keeps every partial
+// sum below 2^63.  Each term is rounded once (to 2^(e-54), far below FP32
 // resolution) and integer addition does not depend on order, so a path's
 // decisions do not depend on which other rays shared its warp or on the order
 // in which its chords were stored or evaluated.
@@ -571,6 +582,7 @@ __device__ __forceinline__ void render_paths(const Work& Wk, const float* env, W
   S.kind = 0;
   S.acc = 0;
   S.allow = ~0ull;
+  S.fit = INFINITY;
 
   // Move the lane's path on from its finished ray (hit: a collision at th on a
   // tracking ray; kind 0: the lane has no path yet) until a new ray starts or
@@ -713,6 +725,7 @@ __device__ __forceinline__ void render_paths(const Work& Wk, const float* env, W
           } else {
             R.te = R.ta + 0.5f * w;
             S.step = 0.5f * w;
+            if (R.nch > kSlotCh) S.fit = 0.5f * w;
           }
         } else if (S.kind == 1) {
           for (int i = 0; i < n && !fhit; ++i) {
