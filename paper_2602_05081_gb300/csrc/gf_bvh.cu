@@ -452,21 +452,26 @@ __global__ void k_collapse4(const Node* nodes, int64_t m, const int* even, const
       lo[a] = fminf(lo[a], box[k][a]);
       hi[a] = fmaxf(hi[a], box[k][3 + a]);
     }
-    // grid step: lo + 255 s >= hi (upward rounding), never zero
-    sc[a] = __fdiv_ru(__fsub_ru(hi[a], lo[a]), 255.0f);
+    // grid step s, never zero, and origin lo - s/64: every child keeps a margin of s/128
+    // between its box and its decoded planes (254.9 s + s/64 + s/128 <= 255 s), which
+    // covers the traversal's rounding of a plane (s/512)
+    sc[a] = __fdiv_ru(__fsub_ru(hi[a], lo[a]), 254.9f);
     const float floor_s = fmaxf(fabsf(lo[a]), fabsf(hi[a])) * 1e-7f + 1e-30f;
     sc[a] = fmaxf(sc[a], floor_s);
+    lo[a] = __fsub_rd(lo[a], 0.015625f * sc[a]);
   }
   uint32_t ql[3] = {0, 0, 0}, qh[3] = {0, 0, 0};
   for (int k = 0; k < nc; ++k) {
     for (int a = 0; a < 3; ++a) {
-      // conservative codes, checked with the decoding formula of the traversal
-      float fl = floorf((box[k][a] - lo[a]) / sc[a]);
+      // conservative codes with the margin
+      const float m = 0.0078125f * sc[a];
+      const float bl = __fsub_rd(box[k][a], m), bh = __fadd_ru(box[k][3 + a], m);
+      float fl = floorf((bl - lo[a]) / sc[a]);
       int cl = (int)fminf(fmaxf(fl, 0.f), 255.f);
-      while (cl > 0 && fmaf((float)cl, sc[a], lo[a]) > box[k][a]) --cl;
-      float fh = ceilf((box[k][3 + a] - lo[a]) / sc[a]);
+      while (cl > 0 && fmaf((float)cl, sc[a], lo[a]) > bl) --cl;
+      float fh = ceilf((bh - lo[a]) / sc[a]);
       int chh = (int)fminf(fmaxf(fh, 0.f), 255.f);
-      while (chh < 255 && fmaf((float)chh, sc[a], lo[a]) < box[k][3 + a]) ++chh;
+      while (chh < 255 && fmaf((float)chh, sc[a], lo[a]) < bh) ++chh;
       ql[a] |= (uint32_t)cl << (8 * k);
       qh[a] |= (uint32_t)chh << (8 * k);
     }

@@ -53,7 +53,6 @@ __device__ __forceinline__ void coop_traverse(const DevField& F, CoopTrav& Q,
                                               unsigned long long mask, float3 o, float3 inv,
                                               float t0, float t1, uint32_t lane, Counters& cnt,
                                               Round&& round) {
-  const unsigned lt = (1u << lane) - 1u;
   // a one-primitive field has no internal node: its leaf is queued at once
   int sp = F.root >= 0 ? 1 : 0, lq_n = F.root >= 0 ? 0 : 1;
   if (lane == 0) {
@@ -81,20 +80,19 @@ __device__ __forceinline__ void coop_traverse(const DevField& F, CoopTrav& Q,
       ++cnt.nodes;
       hit = node4_hits(F.nodes4 + node, o, inv, mask, t0, t1, ch);
     }
-    // push internal children, queue leaves (ballots keep the entries contiguous)
-    int np = 0, nl = 0;
+    // push internal children, queue leaves
+    unsigned leaf = 0u;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) leaf |= ch[k] < 0 ? 1u << k : 0u;
+    int pi, pl, np, nl;
+    hit_places(hit & ~leaf, hit & leaf, lane, pi, pl, np, nl);
+    pi += sp;
+    pl += lq_n;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const bool h = (hit >> k & 1u) != 0u;
-      const unsigned bp = __ballot_sync(kFull, h && ch[k] >= 0);
-      const unsigned bl = __ballot_sync(kFull, h && ch[k] < 0);
-      if (h && ch[k] >= 0) {
-        const int pos = sp + np + __popc(bp & lt);
-        if (pos < kCoopStack) Q.stk[pos] = ch[k];
-      }
-      if (h && ch[k] < 0) Q.lq[lq_n + nl + __popc(bl & lt)] = ~ch[k];
-      np += __popc(bp);
-      nl += __popc(bl);
+      if (!(hit >> k & 1u)) continue;
+      if (ch[k] < 0) Q.lq[pl++] = ~ch[k];
+      else if (pi < kCoopStack) Q.stk[pi++] = ch[k];
     }
     if (sp + np > kCoopStack) {
       if (lane == 0) set_err(F, ERR_STACK);

@@ -624,9 +624,29 @@ __device__ __forceinline__ void traverse_ray(const DevField& F, float3 o, float3
   }
 }
 
-// byte k of x as a float, exactly: 0x4B0000xx is 2^23 + xx
-__device__ __forceinline__ float byte_float(uint32_t x, int k) {
-  return __int_as_float((int)__byte_perm(x, 0x4Bu, (uint32_t)k | 0x4550u)) - 8388608.0f;
+// byte k of x as the float 1 + byte 2^-15, exactly (0x3F80xx00)
+__device__ __forceinline__ float byte_unit(uint32_t x, int k) {
+  return __int_as_float((int)__byte_perm(x, 0x3F800000u, (uint32_t)k << 4 | 0x7604u));
+}
+
+// Places for the hit children of 32 nodes: lane l's internal children (bits of hi) go to
+// oi, oi + 1, ... and its leaves (bits of hl) to ol, ol + 1, ...; ti and tl are the
+// warp's totals.  One scan of both counts.
+__device__ __forceinline__ void hit_places(unsigned hi, unsigned hl, uint32_t lane, int& oi, int& ol,
+                                           int& ti, int& tl) {
+  const int x = __popc(hi) | __popc(hl) << 16;
+  int y = x;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int z = __shfl_up_sync(kFull, y, d);
+    if ((int)lane >= d) y += z;
+  }
+  const int t = __shfl_sync(kFull, y, 31);
+  y -= x;
+  oi = y & 0xFFFF;
+  ol = y >> 16;
+  ti = t & 0xFFFF;
+  tl = t >> 16;
 }
 
 // The children of a four-wide node that overlap [ta, te] of the ray and hold one
@@ -639,9 +659,13 @@ __device__ __forceinline__ unsigned node4_hits(const Node4* N, float3 o, float3 
   const int4 c4 = __ldg(&N->child);
   const uint4 m01 = __ldg(&N->m01), m23 = __ldg(&N->m23);
   const uint32_t qlx = __float_as_uint(v1.z), qly = __float_as_uint(v1.w);
-  // slab distances straight from the codes: t = (lo + c s - o) inv = c (s inv) + (lo - o) inv
-  const float ax = v0.w * inv.x, ay = v1.x * inv.y, az = v1.y * inv.z;
-  const float bx = (v0.x - o.x) * inv.x, by = (v0.y - o.y) * inv.y, bz = (v0.z - o.z) * inv.z;
+  // slab distances straight from the codes: t = (lo + c s - o) inv.  A code byte c is
+  // read as f = 1 + c 2^-15 (one byte permutation), so t = f A + B with A = 2^15 s inv
+  // and B = (lo - o) inv - A; rounding B costs up to s inv / 512, which the margin of
+  // the codes covers (k_collapse4)
+  const float ax = 32768.0f * v0.w * inv.x, ay = 32768.0f * v1.x * inv.y, az = 32768.0f * v1.y * inv.z;
+  const float bx = (v0.x - o.x) * inv.x - ax, by = (v0.y - o.y) * inv.y - ay,
+              bz = (v0.z - o.z) * inv.z - az;
   const unsigned long long mk[4] = {
       (unsigned long long)m01.x | ((unsigned long long)m01.y << 32),
       (unsigned long long)m01.z | ((unsigned long long)m01.w << 32),
@@ -658,9 +682,9 @@ __device__ __forceinline__ unsigned node4_hits(const Node4* N, float3 o, float3 
   unsigned hit = 0u;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const float txn = fmaf(byte_float(nx, k), ax, bx), txf = fmaf(byte_float(fx, k), ax, bx);
-    const float tyn = fmaf(byte_float(ny, k), ay, by), tyf = fmaf(byte_float(fy, k), ay, by);
-    const float tzn = fmaf(byte_float(nz, k), az, bz), tzf = fmaf(byte_float(fz, k), az, bz);
+    const float txn = fmaf(byte_unit(nx, k), ax, bx), txf = fmaf(byte_unit(fx, k), ax, bx);
+    const float tyn = fmaf(byte_unit(ny, k), ay, by), tyf = fmaf(byte_unit(fy, k), ay, by);
+    const float tzn = fmaf(byte_unit(nz, k), az, bz), tzf = fmaf(byte_unit(fz, k), az, bz);
     const float tn = fmaxf(fmaxf(txn, tyn), fmaxf(tzn, ta));
     const float tf = fminf(fminf(txf, tyf), fminf(tzf, te));
     if ((mk[k] & mask) && tn <= tf) hit |= 1u << k;

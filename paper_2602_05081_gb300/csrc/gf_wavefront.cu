@@ -225,22 +225,20 @@ __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, c
       ++cnt.nodes;
       hit = node4_hits(Wk.field(R.asset).nodes4 + node, o, inv, slot_mask(R), R.ta, R.te, ch);
     }
-    // ---------------- push internal children, queue leaves: per child slot k a
-    // ballot places the lanes' entries contiguously (no bank conflicts)
+    // ---------------- push internal children, queue leaves
     {
-      int np = 0, nl = 0;
+      unsigned leaf = 0u;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) leaf |= ch[k] < 0 ? 1u << k : 0u;
+      int pi, pl, np, nl;
+      hit_places(hit & ~leaf, hit & leaf, lane, pi, pl, np, nl);
+      pi += sp;
+      pl += lq_n;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const bool h = (hit >> k & 1u) != 0u;
-        const unsigned bp = __ballot_sync(kFull, h && ch[k] >= 0);
-        const unsigned bl = __ballot_sync(kFull, h && ch[k] < 0);
-        if (h && ch[k] >= 0) {
-          const int pos = sp + np + __popc(bp & lt);
-          if (pos < kWStack) Q.t.stk[pos] = (ch[k] << 5) | slot;
-        }
-        if (h && ch[k] < 0) Q.t.lq[lq_n + nl + __popc(bl & lt)] = (~ch[k] << 5) | slot;
-        np += __popc(bp);
-        nl += __popc(bl);
+        if (!(hit >> k & 1u)) continue;
+        if (ch[k] < 0) Q.t.lq[pl++] = (~ch[k] << 5) | slot;
+        else if (pi < kWStack) Q.t.stk[pi++] = (ch[k] << 5) | slot;
       }
       if (sp + np > kWStack) {
         if (lane == 0) set_err(Wk.err_field(), ERR_STACK);
