@@ -129,6 +129,10 @@ cudaError_t dev_alloc(const Ctx& c, void** p, size_t bytes, cudaStream_t s) {
   if (!c.alloc.alloc) return cudaMalloc(p, bytes);
   void* q = c.alloc.alloc(c.alloc.user, bytes, (gf_stream)s);
   if (!q) return cudaErrorMemoryAllocation;
+  if (reinterpret_cast<uintptr_t>(q) & 31u) {  // (gf_allocator promises 256)
+    if (c.alloc.free) c.alloc.free(c.alloc.user, q, bytes, (gf_stream)s);
+    return cudaErrorMisalignedAddress;
+  }
   *p = q;
   return cudaSuccess;
 }
