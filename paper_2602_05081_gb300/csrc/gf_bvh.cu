@@ -3,7 +3,10 @@
 // prefix, radix sort, Karras's binary radix tree, bottom-up box/mask refit.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cstdint>
 #include <cstring>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -237,7 +240,9 @@ __device__ __forceinline__ unsigned int spread10(unsigned int x) {
   return x;
 }
 
-__global__ void k_morton(const float4* rec, int64_t n, const unsigned int* bounds,
+// sort keys: the cell (or, by_band, its band) above 30 Morton bits of the mean
+__device__ __forceinline__ uint32_t cell_band(uint32_t cell) { return cell == 0 ? 0u : ((cell - 1u) >> 3) + 1u; }
+__global__ void k_morton(const float4* rec, int64_t n, const unsigned int* bounds, bool by_band,
                          unsigned long long* keys, int* idx) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -257,7 +262,7 @@ __global__ void k_morton(const float4* rec, int64_t n, const unsigned int* bound
     c[j] = (unsigned int)fminf(u * 1024.f, 1023.f);
   }
   unsigned int mc = (spread10(c[0]) << 2) | (spread10(c[1]) << 1) | spread10(c[2]);
-  keys[i] = ((unsigned long long)cell << 30) | mc;
+  keys[i] = ((unsigned long long)(by_band ? cell_band(cell) : cell) << 30) | mc;
   idx[i] = (int)i;
 }
 
@@ -362,14 +367,18 @@ __device__ __forceinline__ void write_slot(Node* nd, int slot, const float* b, u
   }
 }
 
-// bottom-up refit: the second child to arrive at a node merges both slots
-__global__ void k_refit(const float* box, const float4* rec, int64_t n, Node* nodes,
-                        const int* leaf_parent, int* flags) {
+// bottom-up refit: the second child to arrive at a node merges both slots.  Leaf j of
+// the tree is the sorted primitive of[j] (j itself without of); masks hold cells, or
+// bands when by_band.
+__global__ void k_refit(const float* box, const float4* rec, const int* of, bool by_band, int64_t n,
+                        Node* nodes, const int* leaf_parent, int* flags) {
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
+  const int64_t pj = of ? of[j] : j;
   float b[6];
-  for (int k = 0; k < 6; ++k) b[k] = box[6 * j + k];
-  unsigned long long m = 1ull << (__float_as_uint(rec[4 * j + 3].w) >> 26);
+  for (int k = 0; k < 6; ++k) b[k] = box[6 * pj + k];
+  const uint32_t cell = __float_as_uint(rec[4 * pj + 3].w) >> 26;
+  unsigned long long m = 1ull << (by_band ? cell_band(cell) : cell);
   int child = ~(int)j;
   int node = leaf_parent[j];
   for (int guard = 0; node >= 0 && guard < 4096; ++guard) {
@@ -391,20 +400,33 @@ __global__ void k_refit(const float* box, const float4* rec, int64_t n, Node* no
 }
 
 // ---------------------------------------------------------------------------
-// Four-wide collapse: binary nodes at even depth become Node4s whose children
-// are their children's children (a leaf child stays a leaf).
+// Four-wide trees.  Keys begin with the class (cell, or band), so the primitives of a
+// class are one subtree of the binary tree (or one leaf).  Within it, binary nodes at
+// even depth below its root become Node4s whose children are their children's children
+// (a leaf child stays a leaf).
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned long long node_mask(const Node& N) {
+  return (unsigned long long)(N.e.x | N.e.z) | ((unsigned long long)(N.e.y | N.e.w) << 32);
+}
+__device__ __forceinline__ bool one_class(unsigned long long m) { return (m & (m - 1ull)) == 0ull; }
+
 __global__ void k_depth_parity(const Node* nodes, int64_t m, int* even, unsigned int* max_depth) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m) return;
-  int d = 0;
+  int d = 0, dc = 0;  // depth, depth below the class's root
+  bool in = one_class(node_mask(nodes[i]));
+  even[i] = in ? 1 : 0;
   int v = (int)i;
   for (int g = 0; g < 4096 && v > 0; ++g) {  // node 0 is the root
     v = nodes[v].d.z;
     ++d;
+    in = in && one_class(node_mask(nodes[v]));
+    dc += in ? 1 : 0;
   }
-  even[i] = (d & 1) == 0 ? 1 : 0;
-  atomicMax(max_depth, (unsigned int)d);
+  if (dc & 1) even[i] = 0;
+  const unsigned am = __activemask();
+  const unsigned dm = __reduce_max_sync(am, (unsigned)d);
+  if ((int)(threadIdx.x & 31u) == __ffs((int)am) - 1) atomicMax(max_depth, dm);
 }
 
 __device__ __forceinline__ void node_slot(const Node& N, int slot, float* b, unsigned long long& m,
@@ -417,33 +439,7 @@ __device__ __forceinline__ void node_slot(const Node& N, int slot, float* b, uns
   child = slot == 0 ? N.d.x : N.d.y;
 }
 
-__global__ void k_collapse4(const Node* nodes, int64_t m, const int* even, const int* map,
-                            Node4* out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m || !even[i]) return;
-  float box[4][6];
-  unsigned long long mk[4] = {0, 0, 0, 0};
-  int ch[4] = {0, 0, 0, 0};
-  int nc = 0;
-  const Node& N = nodes[i];
-  for (int s = 0; s < 2; ++s) {
-    float b[6];
-    unsigned long long mm;
-    int c;
-    node_slot(N, s, b, mm, c);
-    if (c < 0) {
-      for (int k = 0; k < 6; ++k) box[nc][k] = b[k];
-      mk[nc] = mm;
-      ch[nc++] = c;
-      continue;
-    }
-    const Node& C = nodes[c];
-    for (int t = 0; t < 2; ++t) {
-      int cc;
-      node_slot(C, t, box[nc], mk[nc], cc);
-      ch[nc++] = cc < 0 ? cc : map[cc];
-    }
-  }
+__device__ __forceinline__ Node4 emit_node4(int nc, const float box[4][6], const int ch[4]) {
   float lo[3], hi[3], sc[3];
   for (int a = 0; a < 3; ++a) {
     lo[a] = box[0][a];
@@ -480,10 +476,76 @@ __global__ void k_collapse4(const Node* nodes, int64_t m, const int* even, const
   o.v0 = make_float4(lo[0], lo[1], lo[2], sc[0]);
   o.v1 = make_float4(sc[1], sc[2], __uint_as_float(ql[0]), __uint_as_float(ql[1]));
   o.q = make_uint4(ql[2], qh[0], qh[1], qh[2]);
-  o.child = make_int4(ch[0], ch[1], ch[2], ch[3]);
-  o.m01 = make_uint4((uint32_t)mk[0], (uint32_t)(mk[0] >> 32), (uint32_t)mk[1], (uint32_t)(mk[1] >> 32));
-  o.m23 = make_uint4((uint32_t)mk[2], (uint32_t)(mk[2] >> 32), (uint32_t)mk[3], (uint32_t)(mk[3] >> 32));
-  out[map[i]] = o;
+  o.child = make_int4(ch[0], nc > 1 ? ch[1] : kNoChild, nc > 2 ? ch[2] : kNoChild,
+                      nc > 3 ? ch[3] : kNoChild);
+  return o;
+}
+
+// out[base + map[i]]: Node4 of the marked binary node i; out[base + m4 + class]: the
+// root of a class with one primitive.  roots[class] receives the class's root.
+struct CollapseArgs {
+  const Node* nodes;
+  int64_t m;
+  const int *even, *map, *of;
+  Node4* out;
+  int base, m4;
+  int* roots;
+};
+__global__ void k_collapse4(const CollapseArgs A) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= A.m) return;
+  auto leaf = [&](int c) { return A.of ? ~A.of[~c] : c; };
+  const Node& N = A.nodes[i];
+  const unsigned long long mi = node_mask(N);
+  float box[4][6];
+  unsigned long long mm;
+  int ch[4] = {kNoChild, kNoChild, kNoChild, kNoChild};
+  if (!one_class(mi)) {
+    // a class of one primitive hangs below as a leaf
+    for (int s = 0; s < 2; ++s) {
+      int c;
+      node_slot(N, s, box[0], mm, c);
+      if (c >= 0) continue;
+      const int cls = __ffsll((long long)mm) - 1, at = A.base + A.m4 + cls;
+      ch[0] = leaf(c);
+      A.out[at] = emit_node4(1, box, ch);
+      A.roots[cls] = at;
+    }
+    return;
+  }
+  if (!A.even[i]) return;
+  int nc = 0;
+  for (int s = 0; s < 2; ++s) {
+    float b[6];
+    int c;
+    node_slot(N, s, b, mm, c);
+    if (c < 0) {
+      for (int k = 0; k < 6; ++k) box[nc][k] = b[k];
+      ch[nc++] = leaf(c);
+      continue;
+    }
+    const Node& C = A.nodes[c];
+    for (int t = 0; t < 2; ++t) {
+      int cc;
+      node_slot(C, t, box[nc], mm, cc);
+      ch[nc++] = cc < 0 ? leaf(cc) : A.base + A.map[cc];
+    }
+  }
+  const int at = A.base + A.map[i];
+  A.out[at] = emit_node4(nc, box, ch);
+  if (i == 0 || !one_class(node_mask(A.nodes[N.d.z]))) A.roots[__ffsll((long long)mi) - 1] = at;
+}
+
+// the tree of a one-primitive field
+__global__ void k_single4(const float* box, const float4* rec, bool by_band, Node4* out, int base,
+                          int* roots) {
+  float b[4][6];
+  for (int k = 0; k < 6; ++k) b[0][k] = box[k];
+  const int ch[4] = {~0, kNoChild, kNoChild, kNoChild};
+  const uint32_t cell = __float_as_uint(rec[3].w) >> 26;
+  const int cls = (int)(by_band ? cell_band(cell) : cell);
+  out[base + cls] = emit_node4(1, b, ch);
+  roots[cls] = base + cls;
 }
 
 // reduced-precision records: the decoded mean moves by up to half a u16 step of
@@ -504,23 +566,49 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
   (void)cudaGetLastError();  // a stale error of an unrelated call is not ours
   const int64_t n = F.n;
   cudaError_t e = cudaSuccess;
-  unsigned int* bounds = nullptr;
+  // temporaries, in one block
+  unsigned int* bounds = nullptr;  // boxes (12), the two trees' depths
+  int* roots = nullptr;            // of cells, then of bands
   unsigned long long *keys = nullptr, *keys2 = nullptr;
-  int *idx = nullptr, *idx2 = nullptr, *leaf_parent = nullptr, *flags = nullptr;
+  int *idx = nullptr, *idx2 = nullptr, *leaf_parent = nullptr, *flags = nullptr, *leaf_parent_b = nullptr,
+      *flags_b = nullptr;
   float* box_sorted = nullptr;
-  void* tmp = nullptr;
-  size_t tmp_bytes = 0;
-  unsigned int hb[13];
+  Node* nodes_b = nullptr;  // binary tree by bands
+  void *tmp = nullptr, *block = nullptr;
+  size_t tmp_bytes = 0, sort_bytes = 0;
+  const int64_t m = n - 1;
+  const unsigned pn = (unsigned)((n + 255) / 256), pm = (unsigned)((m + 255) / 256);
+  unsigned int hb[14];
+  int hroots[kMaxCells + 8];
 #define GF_TRY(x) do { e = (x); if (e != cudaSuccess) goto done; } while (0)
-  GF_TRY(F.mem.alloc((void**)&bounds, 13 * sizeof(unsigned int), s));  // boxes, then the depth
-  GF_TRY(cudaMemsetAsync(bounds + 12, 0, sizeof(unsigned int), s));
-  GF_TRY(F.mem.alloc((void**)&keys, n * sizeof(unsigned long long), s));
-  GF_TRY(F.mem.alloc((void**)&keys2, n * sizeof(unsigned long long), s));
-  GF_TRY(F.mem.alloc((void**)&idx, n * sizeof(int), s));
-  GF_TRY(F.mem.alloc((void**)&idx2, n * sizeof(int), s));
-  GF_TRY(F.mem.alloc((void**)&leaf_parent, n * sizeof(int), s));
-  GF_TRY(F.mem.alloc((void**)&flags, n * sizeof(int), s));
-  GF_TRY(F.mem.alloc((void**)&box_sorted, n * 6 * sizeof(float), s));
+  GF_TRY(cub::DeviceRadixSort::SortPairs(nullptr, sort_bytes, keys, keys2, idx, idx2, (int)n, 0, 36, s));
+  GF_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tmp_bytes, flags, leaf_parent, (int)n, s));
+  if (sort_bytes > tmp_bytes) tmp_bytes = sort_bytes;
+  for (int pass = 0; pass < 2; ++pass) {  // sizes, then places
+    uintptr_t at = reinterpret_cast<uintptr_t>(block);
+    auto take = [&](auto*& p, size_t bytes) {
+      p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(at);
+      at += (bytes + 255) & ~size_t(255);
+    };
+    char* tp = nullptr;
+    take(bounds, sizeof(hb));
+    take(roots, sizeof(hroots));
+    take(keys, n * sizeof(unsigned long long));
+    take(keys2, n * sizeof(unsigned long long));
+    take(idx, n * sizeof(int));
+    take(idx2, n * sizeof(int));
+    take(leaf_parent, n * sizeof(int));
+    take(flags, n * sizeof(int));
+    take(leaf_parent_b, n * sizeof(int));
+    take(flags_b, n * sizeof(int));
+    take(box_sorted, n * 6 * sizeof(float));
+    take(nodes_b, n * sizeof(Node));
+    take(tp, tmp_bytes);
+    tmp = tp;
+    if (pass == 0) GF_TRY(F.mem.alloc(&block, (size_t)at, s));
+  }
+  GF_TRY(cudaMemsetAsync(bounds + 12, 0, 2 * sizeof(unsigned int), s));
+  GF_TRY(cudaMemsetAsync(roots, 0xFF, sizeof(hroots), s));
   {
     unsigned int init[12];
     for (int j = 0; j < 12; ++j) {
@@ -544,49 +632,58 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
       k_bounds<<<blocks, 256, 0, s>>>(F.box_orig, F.rec_orig, n, bounds);
       GF_TRY(cudaGetLastError());
     }
-    k_morton<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(F.rec_orig, n, bounds, keys, idx);
+    k_morton<<<pn, 256, 0, s>>>(F.rec_orig, n, bounds, false, keys, idx);
     GF_TRY(cudaGetLastError());
   }
-  GF_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tmp_bytes, keys, keys2, idx, idx2, (int)n, 0, 36, s));
-  GF_TRY(F.mem.alloc(&tmp, tmp_bytes, s));
   GF_TRY(cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, keys, keys2, idx, idx2, (int)n, 0, 36, s));
   k_gather<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(F.rec_orig, F.box_orig, F.ext2_orig, idx2,
                                                       n, F.rec, box_sorted, F.ext2, F.muw,
                                                       F.sorted_orig);
   GF_TRY(cudaGetLastError());
-  if (n >= 2) {
-    GF_TRY(cudaMemsetAsync(F.nodes, 0, (n - 1) * sizeof(Node), s));
-    GF_TRY(cudaMemsetAsync(flags, 0, n * sizeof(int), s));
-    k_karras<<<(unsigned)((n - 1 + 255) / 256), 256, 0, s>>>(keys2, n, F.nodes, leaf_parent);
-    GF_TRY(cudaGetLastError());
-    k_refit<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(box_sorted, F.rec, n, F.nodes, leaf_parent, flags);
-    GF_TRY(cudaGetLastError());
-    // four-wide collapse (flags become even-depth markers, leaf_parent their scan)
-    const int64_t m = n - 1;
-    k_depth_parity<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(F.nodes, m, flags, bounds + 12);
-    GF_TRY(cudaGetLastError());
-    size_t sb = 0;
-    GF_TRY(cub::DeviceScan::ExclusiveSum(nullptr, sb, flags, leaf_parent, (int)m, s));
-    if (sb > tmp_bytes) {
-      GF_TRY(cudaStreamSynchronize(s));
-      F.mem.release(tmp, s);
-      tmp = nullptr;
-      GF_TRY(F.mem.alloc(&tmp, sb, s));
-      tmp_bytes = sb;
+  {
+    // the binary trees by cells (kept) and by bands, each with its boxes, the marks of its
+    // four-wide nodes (flags, then their scan in leaf_parent)
+    int last[4] = {0, 0, 0, 0};
+    for (int t = 0; t < 2 && n >= 2; ++t) {
+      const bool band = t == 1;
+      Node* nd = band ? nodes_b : F.nodes;
+      int *lp = band ? leaf_parent_b : leaf_parent, *fl = band ? flags_b : flags;
+      const int* of = band ? idx2 : nullptr;
+      if (band) {
+        k_morton<<<pn, 256, 0, s>>>(F.rec, n, bounds, true, keys, idx);
+        GF_TRY(cudaGetLastError());
+        GF_TRY(cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, keys, keys2, idx, idx2, (int)n, 0, 33, s));
+      }
+      GF_TRY(cudaMemsetAsync(nd, 0, m * sizeof(Node), s));
+      GF_TRY(cudaMemsetAsync(fl, 0, n * sizeof(int), s));
+      k_karras<<<pm, 256, 0, s>>>(keys2, n, nd, lp);
+      GF_TRY(cudaGetLastError());
+      k_refit<<<pn, 256, 0, s>>>(box_sorted, F.rec, of, band, n, nd, lp, fl);
+      GF_TRY(cudaGetLastError());
+      k_depth_parity<<<pm, 256, 0, s>>>(nd, m, fl, bounds + 12 + t);
+      GF_TRY(cudaGetLastError());
+      GF_TRY(cub::DeviceScan::ExclusiveSum(tmp, tmp_bytes, fl, lp, (int)m, s));
+      GF_TRY(cudaMemcpyAsync(&last[2 * t], lp + (m - 1), sizeof(int), cudaMemcpyDeviceToHost, s));
+      GF_TRY(cudaMemcpyAsync(&last[2 * t + 1], fl + (m - 1), sizeof(int), cudaMemcpyDeviceToHost, s));
     }
-    GF_TRY(cub::DeviceScan::ExclusiveSum(tmp, sb, flags, leaf_parent, (int)m, s));
-    int last[2] = {0, 0};
-    GF_TRY(cudaMemcpyAsync(&last[0], leaf_parent + (m - 1), sizeof(int), cudaMemcpyDeviceToHost, s));
-    GF_TRY(cudaMemcpyAsync(&last[1], flags + (m - 1), sizeof(int), cudaMemcpyDeviceToHost, s));
     GF_TRY(cudaStreamSynchronize(s));
-    const int64_t m4 = (int64_t)last[0] + last[1];
-    F.n_nodes4 = m4;
+    const int ma = last[0] + last[1], mb = last[2] + last[3];
+    const int base_b = ma + kMaxCells;
+    F.n_nodes4 = (int64_t)base_b + mb + 8;
     F.mem.release(F.nodes4, s);  // a rebuild (the stream was synchronised above)
     F.nodes4 = nullptr;
-    GF_TRY(F.mem.alloc((void**)&F.nodes4, (size_t)m4 * sizeof(Node4), s));
-    k_collapse4<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(F.nodes, m, flags, leaf_parent, F.nodes4);
+    GF_TRY(F.mem.alloc((void**)&F.nodes4, (size_t)F.n_nodes4 * sizeof(Node4), s));
+    if (n >= 2) {
+      k_collapse4<<<pm, 256, 0, s>>>(CollapseArgs{F.nodes, m, flags, leaf_parent, nullptr, F.nodes4, 0, ma, roots});
+      k_collapse4<<<pm, 256, 0, s>>>(
+          CollapseArgs{nodes_b, m, flags_b, leaf_parent_b, idx2, F.nodes4, base_b, mb, roots + kMaxCells});
+    } else {
+      k_single4<<<1, 1, 0, s>>>(box_sorted, F.rec, false, F.nodes4, 0, roots);
+      k_single4<<<1, 1, 0, s>>>(box_sorted, F.rec, true, F.nodes4, base_b, roots + kMaxCells);
+    }
     GF_TRY(cudaGetLastError());
   }
+  GF_TRY(cudaMemcpyAsync(hroots, roots, sizeof(hroots), cudaMemcpyDeviceToHost, s));
   GF_TRY(cudaMemcpyAsync(hb, bounds, sizeof(hb), cudaMemcpyDeviceToHost, s));
   GF_TRY(cudaStreamSynchronize(s));
   {
@@ -596,7 +693,9 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
       memcpy(&f, &b, 4);
       return f;
     };
-    F.depth = (int)hb[12] + 1;  // levels of internal nodes (0 for a single primitive)
+    // levels of internal nodes (0 for a single primitive) of the deeper tree.  (By bands
+    // the keys are 3 bits shorter and runs of equal keys below 2^26 primitives.)
+    F.depth = (int)std::max(hb[12], hb[13]) + 1;
     if (n < 2) F.depth = 0;
     F.dev.lo = make_float3(dec(hb[0]), dec(hb[1]), dec(hb[2]));
     F.dev.hi = make_float3(dec(hb[3]), dec(hb[4]), dec(hb[5]));
@@ -611,14 +710,15 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
   F.dev.ext2 = F.opts.clamp_eps > 0.f ? F.ext2 : nullptr;
   F.dev.nodes = F.nodes;
   F.dev.nodes4 = F.nodes4;
-  F.dev.n_nodes4 = n >= 2 ? F.n_nodes4 : 0;
+  F.dev.n_nodes4 = F.n_nodes4;
+  // an empty class's root is never started from; node 0 stands in
+  for (int c = 0; c < kMaxCells; ++c) F.dev.croot[c] = std::max(0, hroots[c]);
+  for (int b = 0; b < 8; ++b) F.dev.broot[b] = std::max(0, hroots[kMaxCells + b]);
   F.dev.root = n >= 2 ? 0 : -1;
 done:
 #undef GF_TRY
   cudaStreamSynchronize(s);  // the temporaries are no longer read
-  for (void* t : {(void*)bounds, (void*)keys, (void*)keys2, (void*)idx, (void*)idx2,
-                  (void*)leaf_parent, (void*)flags, (void*)box_sorted, tmp})
-    F.mem.release(t, s);
+  F.mem.release(block, s);
   return e;
 }
 

@@ -28,8 +28,8 @@ __device__ __forceinline__ uint32_t next_tile(int* counter, uint32_t lane) {
   return __shfl_sync(kFull, it, 0);
 }
 
-// Traversal of one ray by a whole warp: a shared stack of four-wide nodes, up to
-// 32 popped per step (one per lane) and their hit children pushed; the leaves
+// Traversal of one ray by a whole warp, from the roots of the trees its mask needs: a
+// shared stack of four-wide nodes, up to 32 popped per step (one per lane) and their hit children pushed; the leaves
 // reached are queued, and every 32 queued leaves (and the last ones) make a
 // round, in which round(j) is called by every lane, j the sorted primitive of the
 // lane's leaf or -1.
@@ -53,11 +53,16 @@ __device__ __forceinline__ void coop_traverse(const DevField& F, CoopTrav& Q,
                                               unsigned long long mask, float3 o, float3 inv,
                                               float t0, float t1, uint32_t lane, Counters& cnt,
                                               Round&& round) {
-  // a one-primitive field has no internal node: its leaf is queued at once
-  int sp = F.root >= 0 ? 1 : 0, lq_n = F.root >= 0 ? 0 : 1;
-  if (lane == 0) {
-    if (F.root >= 0) Q.stk[0] = 0;
-    else Q.lq[0] = 0;
+  int sp = 0, lq_n = 0;
+  {
+    unsigned long long cm;
+    unsigned bm;
+    tree_roots(mask, cm, bm);
+    while (cm | bm) {
+      const int r = next_root(F, cm, bm);
+      if (lane == 0) Q.stk[sp] = r;
+      ++sp;
+    }
   }
   __syncwarp();
   // every node enters the stack at most once
@@ -78,7 +83,7 @@ __device__ __forceinline__ void coop_traverse(const DevField& F, CoopTrav& Q,
       set_err(F, ERR_INDEX);  // a node beyond the tree: skipped
     } else if (node >= 0) {
       ++cnt.nodes;
-      hit = node4_hits(F.nodes4 + node, o, inv, mask, t0, t1, ch);
+      hit = node4_hits(F.nodes4 + node, o, inv, t0, t1, ch);
     }
     // push internal children, queue leaves
     unsigned leaf = 0u;

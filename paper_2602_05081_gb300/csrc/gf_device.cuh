@@ -40,22 +40,21 @@ struct __align__(16) Node {
   uint4 e;   // cell mask of child0 (lo, hi), child1 (lo, hi)
 };
 
-// Four-wide node of the scattering renderer's BVH, collapsed from the binary
-// tree (every even-depth binary node with its children's children).  Child
-// boxes are 8-bit codes on a per-node grid: box = lo + code * s per axis,
-// floor/ceil rounded on the builder and checked with the decoding formula so
-// that each decoded box contains the exact child box.  Unused children have
-// an empty code box and a zero cell mask.  child >= 0: four-wide node;
-// child < 0: leaf of the sorted primitive ~child.
+// Four-wide node of the warp traversals' trees, collapsed from a binary tree (every
+// even-depth binary node with its children's children).  Child boxes are 8-bit codes
+// on a per-node grid: box = lo + code * s per axis, rounded outwards on the builder
+// with a margin for the traversal's arithmetic.  child >= 0: four-wide node; child
+// < 0: leaf of the sorted primitive ~child; kNoChild: unused.  Nodes carry no cell
+// masks: there is one tree per cell and one per band, and a ray starts at the roots
+// of the trees it needs (tree_roots).  64 bytes: two 32-byte loads.
 struct __align__(32) Node4 {
   float4 v0;  // lo.xyz, s.x
   float4 v1;  // s.yz, bits: qlo.x (4 children x u8), qlo.y
   uint4 q;    // qlo.z, qhi.x, qhi.y, qhi.z (4 children x u8 each)
   int4 child;
-  uint4 m01;  // cell masks of children 0, 1 (lo, hi)
-  uint4 m23;  // cell masks of children 2, 3
 };
-static_assert(sizeof(Node4) == 96, "three 32-byte loads per node");
+static_assert(sizeof(Node4) == 64, "two 32-byte loads per node");
+constexpr int kNoChild = -2147483647 - 1;
 
 struct LodDev {
   int freq_policy, max_band, cone_policy;
@@ -78,12 +77,14 @@ struct DevField {
   const float4* rec;       // FP32 records: 4 x float4 per primitive, BVH order
   const uint4* rec16;      // FP16/BF16 records: 2 x uint4 per primitive, BVH order
   const Node* nodes;
-  const Node4* nodes4;     // four-wide collapse of nodes (root 0 when n >= 2)
+  const Node4* nodes4;     // four-wide trees: one per cell, one per band
   int64_t n;
   int64_t n_nodes4;        // four-wide nodes
   int root;                // internal root node, -1 when n == 1
   int precision;           // 0 FP32, 1 FP16, 2 BF16
   float ksig, k2;
+  int croot[kMaxCells];    // root of each occupied cell's tree in nodes4
+  int broot[8];            // root of each occupied band's tree (all its cones)
   float3 lo, hi;           // scene bounds (union of all ellipsoid boxes)
   unsigned long long occupied;
   float kbar[kMaxCells];   // mean |k_W| per cell
@@ -673,29 +674,62 @@ __device__ __forceinline__ void hit_places(unsigned hi, unsigned hl, uint32_t la
   tl = t >> 16;
 }
 
-// The children of a four-wide node that overlap [ta, te] of the ray and hold one
-// of the ray's cells (bit k: child k); ch receives the children.
-__device__ __forceinline__ unsigned node4_hits(const Node4* N, float3 o, float3 inv,
-                                               unsigned long long mask, float ta, float te,
-                                               int ch[4]) {
+// The trees a ray with the cell mask `mask` (occupied cells) walks: bits of cm are
+// cells, bits of bm bands.  A band of at most 3 selected cones takes the cones' own
+// trees, more take the band's tree, whose kernels of all cones lie together (a leaf of
+// an unselected cone has weight 0).  Counted on full rays through 100k kernels in 4
+// octaves: 41 node visits per cone's tree and 163 per band's; all cones 1,045 by cells,
+// 654 by bands; one cone of one band and the Gaussians 175 by cells, 254 by bands.
+// Never more than 14 trees: beyond, bands of 2 and 3 cones take the band's tree too.
+constexpr int kMaxRoots = 14;
+__device__ __forceinline__ void tree_roots(unsigned long long mask, unsigned long long& cm,
+                                           unsigned& bm) {
+  cm = mask & 1ull;
+  bm = 0u;
+  unsigned two = 0u;  // bands of 2 or 3 cones
+#pragma unroll
+  for (int b = 1; b < 8; ++b) {
+    const unsigned c = (unsigned)(mask >> (1 + kCones * (b - 1))) & 0xFFu;
+    const int k = __popc(c);
+    if (k > 3) bm |= 1u << b;
+    else cm |= (unsigned long long)c << (1 + kCones * (b - 1));
+    if (k == 2 || k == 3) two |= 1u << b;
+  }
+  if (__popcll(cm) + __popc(bm) > kMaxRoots) {
+    bm |= two;
+#pragma unroll
+    for (int b = 1; b < 8; ++b)
+      if (two >> b & 1u) cm &= ~(0xFFull << (1 + kCones * (b - 1)));
+  }
+}
+// the next of those trees' roots (cm or bm not empty)
+__device__ __forceinline__ int next_root(const DevField& F, unsigned long long& cm, unsigned& bm) {
+  if (cm) {
+    const int c = __ffsll((long long)cm) - 1;
+    cm &= cm - 1ull;
+    return F.croot[c];
+  }
+  const int b = __ffs((int)bm) - 1;
+  bm &= bm - 1u;
+  return F.broot[b];
+}
+
+// The children of a four-wide node that overlap [ta, te] of the ray (bit k: child k);
+// ch receives the children.
+__device__ __forceinline__ unsigned node4_hits(const Node4* N, float3 o, float3 inv, float ta,
+                                               float te, int ch[4]) {
   float4 v0, v1;
-  uint4 q, c4, m01, m23;
+  uint4 q, c4;
   ldg32(&N->v0, v0, v1);
   ldg32(&N->q, q, c4);
-  ldg32(&N->m01, m01, m23);
   const uint32_t qlx = __float_as_uint(v1.z), qly = __float_as_uint(v1.w);
   // slab distances straight from the codes: t = (lo + c s - o) inv.  A code byte c is
   // read as f = 1 + c 2^-15 (one byte permutation), so t = f A + B with A = 2^15 s inv
   // and B = (lo - o) inv - A; rounding B costs up to s inv / 512, which the margin of
-  // the codes covers (k_collapse4)
+  // the codes covers (emit_node4)
   const float ax = 32768.0f * v0.w * inv.x, ay = 32768.0f * v1.x * inv.y, az = 32768.0f * v1.y * inv.z;
   const float bx = (v0.x - o.x) * inv.x - ax, by = (v0.y - o.y) * inv.y - ay,
               bz = (v0.z - o.z) * inv.z - az;
-  const unsigned long long mk[4] = {
-      (unsigned long long)m01.x | ((unsigned long long)m01.y << 32),
-      (unsigned long long)m01.z | ((unsigned long long)m01.w << 32),
-      (unsigned long long)m23.x | ((unsigned long long)m23.y << 32),
-      (unsigned long long)m23.z | ((unsigned long long)m23.w << 32)};
   ch[0] = (int)c4.x;
   ch[1] = (int)c4.y;
   ch[2] = (int)c4.z;
@@ -712,7 +746,7 @@ __device__ __forceinline__ unsigned node4_hits(const Node4* N, float3 o, float3 
     const float tzn = fmaf(byte_unit(nz, k), az, bz), tzf = fmaf(byte_unit(fz, k), az, bz);
     const float tn = fmaxf(fmaxf(txn, tyn), fmaxf(tzn, ta));
     const float tf = fminf(fminf(txf, tyf), fminf(tzf, te));
-    if ((mk[k] & mask) && tn <= tf) hit |= 1u << k;
+    if (ch[k] != kNoChild && tn <= tf) hit |= 1u << k;
   }
   return hit;
 }

@@ -72,12 +72,11 @@ struct ChordItem {
   uint32_t orig_own;  // original primitive index | owning slot << 26
 };
 static_assert(sizeof(ChordItem) == 32, "chord items of 32 bytes");
-// Shared (node, slot) stack entries per warp.  A step pushes at most 128
-// entries (32 four-wide nodes); above kWStack - kStackMargin the warp goes
-// depth first (one entry per step, net growth <= 3 per tree level), so the
-// stack holds a full step plus 40 levels of descent.
+// Shared (node, slot) stack entries per warp: the first roots (32 slots of up to
+// kMaxRoots), and a margin of 3 entries per level of a descent (32 four-wide levels).
 constexpr int kWStack = 640;
-constexpr int kStackMargin = 248;
+constexpr int kStackMargin = 96;
+static_assert(32 * kMaxRoots + 96 <= kWStack - kStackMargin, "full steps on the first roots");
 struct TravQ {
   int stk[kWStack];   // (node << 5) | slot
   int lq[kLeafQ];     // (sorted primitive << 5) | slot
@@ -187,14 +186,18 @@ __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, c
   const unsigned lt = (1u << lane) - 1u;
   int sp = 0, lq_n = 0, cq_n = 0;  // warp-uniform sizes
   {
-    // a one-primitive field has no internal node: its leaf is queued instead
-    const int root = want ? Wk.field(Q.r[lane].asset).root : -1;
-    const unsigned bs = __ballot_sync(kFull, want && root >= 0);
-    const unsigned bl = __ballot_sync(kFull, want && root < 0);
-    if (want && root >= 0) Q.t.stk[__popc(bs & lt)] = (root << 5) | (int)lane;
-    if (want && root < 0) Q.t.lq[__popc(bl & lt)] = (0 << 5) | (int)lane;
-    sp = __popc(bs);
-    lq_n = __popc(bl);
+    // the roots of the trees each slot's mask needs, at most 32 kMaxRoots in all
+    unsigned long long cm = 0ull;
+    unsigned bm = 0u;
+    if (want) tree_roots(slot_mask(Q.r[lane]), cm, bm);
+    for (;;) {
+      const bool has = (cm | bm) != 0ull;
+      const unsigned b = __ballot_sync(kFull, has);
+      if (b == 0u) break;
+      if (has)
+        Q.t.stk[sp + __popc(b & lt)] = (next_root(Wk.field(Q.r[lane].asset), cm, bm) << 5) | (int)lane;
+      sp += __popc(b);
+    }
     __syncwarp();
   }
   const long long max_it = 4 * (Wk.max_n() + 64) + 4096;
@@ -206,7 +209,9 @@ __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, c
     // ---------------- one traversal step: up to 32 (four-wide node, slot) entries
     GF_TIC(t_step);
     int take = sp < 32 ? sp : 32;
-    if (sp > kWStack - kStackMargin) take = 1;  // near capacity: depth first
+    // near capacity fewer, down to one: a node leaves room for three more entries, and
+    // a descent adds at most three per level
+    take = min(take, max(1, (kWStack - kStackMargin - sp) / 3));
     const int ent = (int)lane < take ? Q.t.stk[sp - take + (int)lane] : -1;
     __syncwarp();
     sp -= take;
@@ -223,7 +228,7 @@ __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, c
       const float3 o = make_float3(R.o[0], R.o[1], R.o[2]);
       const float3 inv = make_float3(R.inv[0], R.inv[1], R.inv[2]);
       ++cnt.nodes;
-      hit = node4_hits(Wk.field(R.asset).nodes4 + node, o, inv, slot_mask(R), R.ta, R.te, ch);
+      hit = node4_hits(Wk.field(R.asset).nodes4 + node, o, inv, R.ta, R.te, ch);
     }
     // ---------------- push internal children, queue leaves
     {
