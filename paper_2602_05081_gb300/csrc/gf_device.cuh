@@ -188,6 +188,18 @@ __device__ __forceinline__ void ldg32(const void* p, uint4& a, uint4& b) {
   a = make_uint4((uint32_t)r0, (uint32_t)(r0 >> 32), (uint32_t)r1, (uint32_t)(r1 >> 32));
   b = make_uint4((uint32_t)r2, (uint32_t)(r2 >> 32), (uint32_t)r3, (uint32_t)(r3 >> 32));
 }
+// the same of memory that this warp has written
+__device__ __forceinline__ void ld32(const void* p, float4& a, float4& b) {
+  unsigned long long r0, r1, r2, r3;
+  asm volatile("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(r0), "=l"(r1), "=l"(r2), "=l"(r3)
+               : "l"(p)
+               : "memory");
+  a = make_float4(__uint_as_float((uint32_t)r0), __uint_as_float((uint32_t)(r0 >> 32)),
+                  __uint_as_float((uint32_t)r1), __uint_as_float((uint32_t)(r1 >> 32)));
+  b = make_float4(__uint_as_float((uint32_t)r2), __uint_as_float((uint32_t)(r2 >> 32)),
+                  __uint_as_float((uint32_t)r3), __uint_as_float((uint32_t)(r3 >> 32)));
+}
 __device__ __forceinline__ float4 as_float4(uint4 x) {
   return make_float4(__uint_as_float(x.x), __uint_as_float(x.y), __uint_as_float(x.z),
                      __uint_as_float(x.w));

@@ -13,9 +13,8 @@
 // from its own Philox stream (chords that may hold more points go back to the
 // queue, so the lanes stay busy).  Points land in
 // the owner's buffer through shared-memory atomics.  kappa and kappa_bar at
-// the points are then summed from the stored records (the lanes share out the
-// (slot, chord) pairs of all slots and add into per-point sums in shared
-// memory), after which each lane takes its delta-tracking or
+// the points are then summed from the stored records, a lane (or several) per
+// point, after which each lane takes its delta-tracking or
 // ratio-tracking decision and moves its path on (camera ray -> collision ->
 // NEE -> scattering).
 //
@@ -43,7 +42,15 @@ constexpr int kChordQ = 64;     // queued chords per warp (<= 31 left + 32 new)
 // masks: 317 -> 303 ms; 512x512, 16 samples, 100k kernels: 196 -> 183 ms.
 constexpr int kPK = 13;         // tentative points per lane and window
 constexpr int kSlotCh = 448;    // stored chords per lane and window (global scratch)
-constexpr int kRecF4 = 2;       // float4s per stored chord record
+constexpr int kHits = 40;         // covering chords a lane collects before it evaluates them
+static_assert(kSlotCh % 4 == 0, "spans are read four at a time");
+// A warp's stored chords, per slot: entry and exit (8 bytes each, read by themselves
+// while points look for the chords that cover them), and the records.
+struct ChordStore {
+  float2 span[32][kSlotCh];
+  float4 rec[32][kSlotCh][2];  // (t*, t_in, t_out, B), (-a log2(e) / 2, log2 h, phase at t*, sqrt(a))
+};
+static_assert(sizeof(float2) * 32 * kSlotCh % 32 == 0, "records on 32-byte boundaries");
 
 // One slot per lane, 57 words: an odd stride keeps same-field accesses of the
 // 32 slots in distinct shared-memory banks.
@@ -82,12 +89,11 @@ struct TravQ {
   int lq[kLeafQ];     // (sorted primitive << 5) | slot
   ChordItem cq[kChordQ];
 };
-// The point evaluation that follows a traversal phase reuses the queues' space:
-// 64-bit fixed-point sums of kappa and kappa_bar per (slot, point), and the
-// running ends of the slots' chord lists.
+// The point evaluation that follows a traversal phase reuses the queues' space.
 struct EvalQ {
-  unsigned long long kap[32 * kPK], kb[32 * kPK];
-  int end[33];  // chords of slots 0..s-1 to evaluate: end[s]
+  float kap[kPK][32], kb[kPK][32];     // kappa and kappa_bar of every slot's points
+  unsigned short own[32 * kPK];        // point of the phase -> slot | index << 5
+  unsigned short hit[kHits][32];       // per lane: chords that cover its point
 };
 struct WarpQ {
   LaneRay r[32];
@@ -182,7 +188,7 @@ __device__ __forceinline__ bool walk_step(const DevField& F, WarpQ& Q, ChordItem
 // window's chords for their evaluation.
 template <class Work>
 __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, const float* env,
-                           float4* wch, Counters& cnt) {
+                           ChordStore* wch, Counters& cnt) {
   const unsigned lt = (1u << lane) - 1u;
   int sp = 0, lq_n = 0, cq_n = 0;  // warp-uniform sizes
   {
@@ -293,7 +299,8 @@ __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, c
             if (k < kSlotCh) {
               // centred on the envelope peak t* = tc + dts: exponent y2 dt^2 + log2 h,
               // phase B dt + delta*, majorant piece floor(|dt| sqrt(a))
-              float4* dst = wch + ((size_t)own * kSlotCh + k) * kRecF4;
+              wch->span[own][k] = make_float2(tin, tout);
+              float4* dst = wch->rec[own][k];
               dst[0] = make_float4(ch.tc + ch.dts, tin, tout, ch.B);
               dst[1] = make_float4(-0.5f * kLog2e * ch.a, __log2f(h),
                                    reduce_2pi(fmaf(ch.B, ch.dts, ch.delta)), sa);
@@ -398,10 +405,12 @@ __device__ __forceinline__ bool start_ray(const DevField& F, LaneRay& R, PathSta
   return true;
 }
 
-// kappa and kappa_bar at the points of every slot, from the chords pass 1
-// stored.  The lanes share out the (slot, chord) pairs of all slots evenly, so
-// no lane waits on one slot's short list; each pair tests the chord against
-// the slot's points and adds its terms to the slot's sums in shared memory.
+// kappa and kappa_bar at the points of every slot, from the chords pass 1 stored.
+// A lane takes one point of the phase (with few points left, 2, 4, ... 32 lanes share
+// one): it runs through the entries and exits of its slot's chords, four per load, and
+// notes the chords that cover the point; then it evaluates those, so that the
+// evaluations run with the lanes full.  (Adding every covering chord to 64-bit sums in
+// shared memory as it was found kept 34 % of the renderer's cycles busy.)
 // The sums are exact in 64-bit fixed point: a term is at most the peak h of
 // its chord (to ~1e-6), so with H the largest peak of the slot's window and at most
 // kSlotCh < 2^9 chords, scaling by 2^(54 - e) (H < 2^e) keeps every partial
@@ -413,81 +422,77 @@ __device__ __forceinline__ int slot_exp(const LaneRay& R) {
   const int ex = ((R.hmax >> 23) & 0xFF) - 126;  // H < 2^ex
   return ex < -70 ? -70 : ex;
 }
-__device__ void eval_stored(WarpQ& Q, const float4* wch, const float* env, uint32_t lane,
+__device__ void eval_stored(WarpQ& Q, const ChordStore* wch, const float* env, uint32_t lane,
                             Counters& cnt) {
-  LaneRay& Rl = Q.r[lane];
-  const int ns_l = Rl.npts;  // 0: no points (or an overflowed window)
-  const int m = ns_l > 0 ? Rl.nch : 0;
-  int incl = m;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(kFull, incl, o);
-    if ((int)lane >= o) incl += y;
-  }
-  const int total = __shfl_sync(kFull, incl, 31);
   EvalQ& E = Q.e;
-  E.end[lane + 1] = incl;
-  if (lane == 0) E.end[0] = 0;
+  int left;  // points of the phase
+  {
+    const int n = Q.r[lane].npts;  // 0: no points (or an overflowed window)
+    int incl = n;
 #pragma unroll
-  for (int i = 0; i < kPK; ++i) {
-    E.kap[i * 32 + lane] = 0ull;
-    E.kb[i * 32 + lane] = 0ull;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kFull, incl, o);
+      if ((int)lane >= o) incl += y;
+    }
+    left = __shfl_sync(kFull, incl, 31);
+    for (int i = 0; i < n; ++i) E.own[incl - n + i] = (unsigned short)(lane | (uint32_t)i << 5);
   }
   __syncwarp();
-  // lane l takes the pairs [l per, (l + 1) per): a lane stays within one slot
-  // for most of its pairs, and lanes of a long list sit in different slots at
-  // any moment, so the atomics below rarely meet on one address.  Each pair's
-  // record is loaded one pair ahead, so that its latency overlaps the work on
-  // the pair before.
-  const int per = (total + 31) >> 5;
-  int f = (int)lane * per;
-  const int fe = min(f + per, total);
-  int s = 0;  // the slot of pair f: the number of slot ends at or below f
-  float4 an = make_float4(0.f, 0.f, 0.f, 0.f), bn = an;
-  if (f < fe) {
-#pragma unroll
-    for (int w = 16; w > 0; w >>= 1)
-      if (E.end[s + w] <= f) s += w;
-    const float4* rec = wch + ((size_t)s * kSlotCh + (f - E.end[s])) * kRecF4;
-    an = rec[0];
-    bn = rec[1];
-  }
-  for (; f < fe; ++f) {
-    const float4 a = an, b = bn;
-    const int sc = s;
-    if (f + 1 < fe) {
-      while (E.end[s + 1] <= f + 1) ++s;  // the next slot with chords (f + 1 < end[32])
-      const float4* rec = wch + ((size_t)s * kSlotCh + (f + 1 - E.end[s])) * kRecF4;
-      an = rec[0];
-      bn = rec[1];
-    }
-    const LaneRay& R = Q.r[sc];
-    const int ex = slot_exp(R);
+  for (int q0 = 0; left > 0;) {
+    int sh = 0;  // 2^sh lanes per point
+    while (sh < 5 && left << (sh + 1) <= 32) ++sh;
+    const int pts = min(left, 32 >> sh);
+    const bool act = (int)(lane >> sh) < pts;
+    const uint32_t own = act ? E.own[q0 + (int)(lane >> sh)] : 0u;
+    const int sl = (int)(own & 31u), i = (int)(own >> 5);
+    const LaneRay& R = Q.r[sl];
+    const float t = R.pt[i];
+    const int m = act ? R.nch : 0, ex = slot_exp(R);
     const float S = __int_as_float((127 + 54 - ex) << 23);  // 2^(54 - ex)
-    const int ns = R.npts;
-    for (int i = 0; i < ns; ++i) {
-      const float t = R.pt[i];
-      if (t > a.z) break;  // the points are sorted by t
-      if (t >= a.y) {
+    const float2* span = wch->span[sl];
+    long long kap = 0, kb = 0;
+    int k = 4 * (int)(lane & ((1u << sh) - 1u));
+    for (;;) {
+      int h = 0;
+      for (; k < m && h <= kHits - 4; k += 4 << sh) {
+        float4 a, b;
+        ld32(span + k, a, b);
+        if (t >= a.x && t <= a.y) E.hit[h++][lane] = (unsigned short)k;
+        if (t >= a.z && t <= a.w && k + 1 < m) E.hit[h++][lane] = (unsigned short)(k + 1);
+        if (t >= b.x && t <= b.y && k + 2 < m) E.hit[h++][lane] = (unsigned short)(k + 2);
+        if (t >= b.z && t <= b.w && k + 3 < m) E.hit[h++][lane] = (unsigned short)(k + 3);
+      }
+      __syncwarp();
+      for (int x = 0; x < h; ++x) {
+        float4 a, b;
+        ld32(wch->rec[sl][E.hit[x][lane]], a, b);
         const float dt = t - a.x;
-        const long long k1 =
-            __float2ll_rn(ex2f(fmaf(b.x, dt * dt, b.y)) * cosf_fast(fmaf(a.w, dt, b.z)) * S);
+        kap += __float2ll_rn(ex2f(fmaf(b.x, dt * dt, b.y)) * cosf_fast(fmaf(a.w, dt, b.z)) * S);
         int mm = (int)(fabsf(dt) * b.w);
         mm = mm > 7 ? 7 : mm;
-        const long long k2 = __float2ll_rn(ex2f(b.y + env[8 + mm]) * S);  // h exp(-m^2/2)
-        atomicAdd(&E.kap[i * 32 + sc], (unsigned long long)k1);
-        atomicAdd(&E.kb[i * 32 + sc], (unsigned long long)k2);
-        ++cnt.evals;
+        kb += __float2ll_rn(ex2f(b.y + env[8 + mm]) * S);  // h exp(-m^2/2)
       }
+      cnt.evals += (unsigned)h;
+      if (!__any_sync(kFull, k < m)) break;
     }
+    for (int o = 1; o < 1 << sh; o <<= 1) {
+      kap += __shfl_xor_sync(kFull, kap, o);
+      kb += __shfl_xor_sync(kFull, kb, o);
+    }
+    if (act && (lane & ((1u << sh) - 1u)) == 0u) {
+      const float u = __int_as_float((127 - 54 + ex) << 23);
+      E.kap[i][sl] = __ll2float_rn(kap) * u;
+      E.kb[i][sl] = __ll2float_rn(kb) * u;
+    }
+    q0 += pts;
+    left -= pts;
+    __syncwarp();
   }
-  __syncwarp();
 }
-// kappa (k = 0) or kappa_bar (k = 1) at point i of the calling lane's slot,
-// from the sums eval_stored left
+// kappa (k = 0) or kappa_bar (k = 1) at point i of the calling lane's slot, as
+// eval_stored left them
 __device__ __forceinline__ float slot_sum(const WarpQ& Q, uint32_t lane, int i, int k) {
-  const unsigned long long v = (k ? Q.e.kb : Q.e.kap)[i * 32 + lane];
-  return __ll2float_rn((long long)v) * __int_as_float((127 - 54 + slot_exp(Q.r[lane])) << 23);
+  return k ? Q.e.kb[i][lane] : Q.e.kap[i][lane];
 }
 
 // ---------------------------------------------------------------------------
@@ -573,7 +578,7 @@ struct ServerWork {
 // spreads it over every warp of the grid (scatter_slots).
 template <class Work>
 __device__ __forceinline__ void render_paths(const Work& Wk, const float* env, WarpQ& Q,
-                                             float4* wch, int slots) {
+                                             ChordStore* wch, int slots) {
   const uint32_t lane = threadIdx.x & 31u;
   LaneRay& R = Q.r[lane];
   Counters cnt;
@@ -775,8 +780,8 @@ __device__ __forceinline__ WarpQ& setup_block(unsigned char* smraw, const float*
   return Qs[threadIdx.x >> 5];
 }
 
-__device__ __forceinline__ float4* warp_store(float4* chord_store) {
-  return chord_store + ((size_t)blockIdx.x * kWWarps + (threadIdx.x >> 5)) * 32 * kSlotCh * kRecF4;
+__device__ __forceinline__ ChordStore* warp_store(float4* chord_store) {
+  return reinterpret_cast<ChordStore*>(chord_store) + (size_t)blockIdx.x * kWWarps + (threadIdx.x >> 5);
 }
 
 __global__ void __launch_bounds__(kWWarps * 32, kBlocksPerSM)
@@ -808,7 +813,7 @@ static_assert((64 + sizeof(WarpQ) * kWWarps + 1024) * kBlocksPerSM <= 233472,
               "kBlocksPerSM blocks fit one SM's shared memory");
 
 size_t scatter_store_bytes(int64_t grid) {
-  return (size_t)grid * kWWarps * 32 * kSlotCh * kRecF4 * sizeof(float4);
+  return (size_t)grid * kWWarps * sizeof(ChordStore);
 }
 
 // full persistent grid of the scattering kernels
