@@ -213,18 +213,21 @@ __device__ __forceinline__ Mask sample_mask_impl(const DevField& F, const LodDev
     }
   }
 #pragma unroll
-  for (int b = 0; b < 8; ++b) {
-    M.bw[b] = bw[b];
-    if (!(sel >> b & 1u)) continue;
+  for (int b = 0; b < 8; ++b) M.bw[b] = bw[b];
+  if (sel & 1u) M.bits |= (unsigned long long)band_cells8(F.occupied, 0);
+  // The selected Gabor bands one after the other, whatever their numbers: lanes that
+  // draw in different bands then run the cone choice together (unrolled over the bands
+  // they took it in turn).
+  for (unsigned rest = sel & ~1u; rest != 0u; rest &= rest - 1u) {
+    const int b = __ffs((int)rest) - 1;
     const unsigned cells = band_cells8(F.occupied, b);
-    if (b == 0) {
-      M.bits |= (unsigned long long)cells;
-      continue;
-    }
     if (L.cone_policy == 0) {
       M.bits |= (unsigned long long)cells << (1 + kCones * (b - 1));
       continue;
     }
+    float bwb = bw[0];
+#pragma unroll
+    for (int q = 1; q < 8; ++q) bwb = (q == b) ? bw[q] : bwb;
     const uint32_t y = rng4(seed, (uint32_t)(1 + b), kNoPrim, ray, word).x;
     const int nc = __popc(cells);
     int k;
@@ -256,9 +259,10 @@ __device__ __forceinline__ Mask sample_mask_impl(const DevField& F, const LodDev
         const int na = __popc(above);
         const int c = nth_bit(above, (int)(((unsigned long long)(y >> 8) * (unsigned)na) >> 24));
         below |= 1u << c;
-        M.cx[b >> 2] |= ((uint32_t)c | ((uint32_t)na << 3)) << (8 * (b & 3));
+        const uint32_t cx = ((uint32_t)c | ((uint32_t)na << 3)) << (8 * (b & 3));
+        M.cx[0] |= b < 4 ? cx : 0u;
+        M.cx[1] |= b < 4 ? 0u : cx;
       }
-      M.bw[b] = bw[b];
       M.bits |= (unsigned long long)below << (1 + kCones * (b - 1));
       continue;
     }
@@ -302,7 +306,9 @@ __device__ __forceinline__ Mask sample_mask_impl(const DevField& F, const LodDev
       }
       cf = W / wk;
     }
-    M.bw[b] = bw[b] * cf;
+    const float wcf = bwb * cf;
+#pragma unroll
+    for (int q = 1; q < 8; ++q) M.bw[q] = (q == b) ? wcf : M.bw[q];
     M.bits |= 1ull << (1 + kCones * (b - 1) + k);
   }
   M.bits &= F.cells_on;  // cells the camera selection emptied are not traversed
