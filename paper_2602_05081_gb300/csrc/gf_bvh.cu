@@ -473,8 +473,8 @@ __device__ __forceinline__ Node4 emit_node4(int nc, const float box[4][6], const
     }
   }
   Node4 o;
-  o.v0 = make_float4(lo[0], lo[1], lo[2], sc[0]);
-  o.v1 = make_float4(sc[1], sc[2], __uint_as_float(ql[0]), __uint_as_float(ql[1]));
+  o.v0 = make_float4(lo[0], lo[1], lo[2], 32768.0f * sc[0]);
+  o.v1 = make_float4(32768.0f * sc[1], 32768.0f * sc[2], __uint_as_float(ql[0]), __uint_as_float(ql[1]));
   o.q = make_uint4(ql[2], qh[0], qh[1], qh[2]);
   o.child = make_int4(ch[0], nc > 1 ? ch[1] : kNoChild, nc > 2 ? ch[2] : kNoChild,
                       nc > 3 ? ch[3] : kNoChild);

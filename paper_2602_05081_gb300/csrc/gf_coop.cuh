@@ -1,6 +1,8 @@
 // gf_coop.cuh -- one ray per warp: the warp traverses the ray's tree together
 // and shares out its chords.
 #pragma once
+#include <cstddef>
+
 #include "gf_device.cuh"
 #include "gf_trace.cuh"
 
@@ -45,8 +47,9 @@ constexpr int kCoopLeafQ = 160;  // <= 31 left + 128 new
 static_assert(kCoopStack - kCoopMargin + 96 + 3 * 32 <= kCoopStack, "a full step, then a descent");
 struct CoopTrav {
   int stk[kCoopStack];
-  int lq[kCoopLeafQ];
+  int lq[kCoopLeafQ];  // directly behind the stack (push_hits)
 };
+static_assert(offsetof(CoopTrav, lq) == kCoopStack * sizeof(int), "queue behind the stack");
 
 template <class Round>
 __device__ __forceinline__ void coop_traverse(const DevField& F, CoopTrav& Q,
@@ -85,26 +88,8 @@ __device__ __forceinline__ void coop_traverse(const DevField& F, CoopTrav& Q,
       ++cnt.nodes;
       hit = node4_hits(F.nodes4 + node, o, inv, t0, t1, ch);
     }
-    // push internal children, queue leaves
-    unsigned leaf = 0u;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) leaf |= ch[k] < 0 ? 1u << k : 0u;
-    int pi, pl, np, nl;
-    hit_places(hit & ~leaf, hit & leaf, lane, pi, pl, np, nl);
-    pi += sp;
-    pl += lq_n;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (!(hit >> k & 1u)) continue;
-      if (ch[k] < 0) Q.lq[pl++] = ~ch[k];
-      else if (pi < kCoopStack) Q.stk[pi++] = ch[k];
-    }
-    if (sp + np > kCoopStack) {
-      if (lane == 0) set_err(F, ERR_STACK);
-      np = kCoopStack - sp;
-    }
-    sp += np;
-    lq_n += nl;
+    if (!push_hits(Q.stk, kCoopStack, hit, ch, lane, sp, lq_n, [](int c) { return c; }) && lane == 0)
+      set_err(F, ERR_STACK);
     __syncwarp();
     const bool more = sp > 0;
     while (lq_n >= 32 || (!more && lq_n > 0)) {

@@ -48,8 +48,8 @@ struct __align__(16) Node {
 // masks: there is one tree per cell and one per band, and a ray starts at the roots
 // of the trees it needs (tree_roots).  64 bytes: two 32-byte loads.
 struct __align__(32) Node4 {
-  float4 v0;  // lo.xyz, s.x
-  float4 v1;  // s.yz, bits: qlo.x (4 children x u8), qlo.y
+  float4 v0;  // lo.xyz, 2^15 s.x
+  float4 v1;  // 2^15 s.yz, bits: qlo.x (4 children x u8), qlo.y
   uint4 q;    // qlo.z, qhi.x, qhi.y, qhi.z (4 children x u8 each)
   int4 child;
 };
@@ -666,6 +666,35 @@ __device__ __forceinline__ float byte_unit(uint32_t x, int k) {
   return __int_as_float((int)__byte_perm(x, 0x3F800000u, (uint32_t)k << 4 | 0x7604u));
 }
 
+__device__ __forceinline__ void hit_places(unsigned hi, unsigned hl, uint32_t lane, int& oi, int& ol,
+                                           int& ti, int& tl);
+
+// Children of 32 nodes to the warp's stack (internal ones, from sp on) and leaf queue
+// (from lq_n on), which lie one behind the other: stk[stack_words], then the queue.
+// word(c) packs an internal child or, for a leaf, its primitive.  The stack's size is
+// checked once for the warp; returns false when it would overflow (nothing is pushed).
+template <class Word>
+__device__ __forceinline__ bool push_hits(int* stk, int stack_words, unsigned hit, const int ch[4],
+                                          uint32_t lane, int& sp, int& lq_n, Word&& word) {
+  const unsigned leaf = (unsigned)ch[0] >> 31 | ((unsigned)ch[1] >> 31) << 1 |
+                        ((unsigned)ch[2] >> 31) << 2 | ((unsigned)ch[3] >> 31) << 3;
+  int pi, pl, np, nl;
+  hit_places(hit & ~leaf, hit & leaf, lane, pi, pl, np, nl);
+  if (sp + np > stack_words) return false;
+  pi += sp;
+  pl += stack_words + lq_n;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const bool lf = ch[k] < 0, h = (hit >> k & 1u) != 0u;
+    if (h) stk[lf ? pl : pi] = word(lf ? ~ch[k] : ch[k]);
+    pi += h && !lf ? 1 : 0;
+    pl += h && lf ? 1 : 0;
+  }
+  sp += np;
+  lq_n += nl;
+  return true;
+}
+
 // Places for the hit children of 32 nodes: lane l's internal children (bits of hi) go to
 // oi, oi + 1, ... and its leaves (bits of hl) to ol, ol + 1, ...; ti and tl are the
 // warp's totals.  One scan of both counts.
@@ -739,7 +768,7 @@ __device__ __forceinline__ unsigned node4_hits(const Node4* N, float3 o, float3 
   // read as f = 1 + c 2^-15 (one byte permutation), so t = f A + B with A = 2^15 s inv
   // and B = (lo - o) inv - A; rounding B costs up to s inv / 512, which the margin of
   // the codes covers (emit_node4)
-  const float ax = 32768.0f * v0.w * inv.x, ay = 32768.0f * v1.x * inv.y, az = 32768.0f * v1.y * inv.z;
+  const float ax = v0.w * inv.x, ay = v1.x * inv.y, az = v1.y * inv.z;
   const float bx = (v0.x - o.x) * inv.x - ax, by = (v0.y - o.y) * inv.y - ay,
               bz = (v0.z - o.z) * inv.z - az;
   ch[0] = (int)c4.x;

@@ -25,6 +25,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <cstddef>
 
 #include "gf_host.h"
 #include "gf_trace.cuh"
@@ -86,9 +87,10 @@ constexpr int kStackMargin = 96;
 static_assert(32 * kMaxRoots + 96 <= kWStack - kStackMargin, "full steps on the first roots");
 struct TravQ {
   int stk[kWStack];   // (node << 5) | slot
-  int lq[kLeafQ];     // (sorted primitive << 5) | slot
+  int lq[kLeafQ];     // (sorted primitive << 5) | slot; directly behind the stack
   ChordItem cq[kChordQ];
 };
+static_assert(offsetof(TravQ, lq) == kWStack * sizeof(int), "queue behind the stack");
 // The point evaluation that follows a traversal phase reuses the queues' space.
 struct EvalQ {
   float kap[kPK][32], kb[kPK][32];     // kappa and kappa_bar of every slot's points
@@ -237,28 +239,10 @@ __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, c
       hit = node4_hits(Wk.field(R.asset).nodes4 + node, o, inv, R.ta, R.te, ch);
     }
     // ---------------- push internal children, queue leaves
-    {
-      unsigned leaf = 0u;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) leaf |= ch[k] < 0 ? 1u << k : 0u;
-      int pi, pl, np, nl;
-      hit_places(hit & ~leaf, hit & leaf, lane, pi, pl, np, nl);
-      pi += sp;
-      pl += lq_n;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (!(hit >> k & 1u)) continue;
-        if (ch[k] < 0) Q.t.lq[pl++] = (~ch[k] << 5) | slot;
-        else if (pi < kWStack) Q.t.stk[pi++] = (ch[k] << 5) | slot;
-      }
-      if (sp + np > kWStack) {
-        if (lane == 0) set_err(Wk.err_field(), ERR_STACK);
-        np = kWStack - sp;
-      }
-      sp += np;
-      lq_n += nl;
-      __syncwarp();
-    }
+    if (!push_hits(Q.t.stk, kWStack, hit, ch, lane, sp, lq_n, [&](int c) { return (c << 5) | slot; }) &&
+        lane == 0)
+      set_err(Wk.err_field(), ERR_STACK);
+    __syncwarp();
     const bool any_trav = sp > 0;
     if (lane == 0) GF_TOC(cnt, 0, t_step);
     // ---------------- leaf rounds: 32 leaves of any slots' rays at a time; once
@@ -394,10 +378,12 @@ __device__ __forceinline__ bool start_ray(const DevField& F, LaneRay& R, PathSta
   S.t0 = t0;
   S.t1 = t1;
   if (!hit) return false;
-  // first window: a quarter of the span when tracking, all of it for NEE, but not a
-  // length that held too many chords on the lane's last rays
+  // first window: 0.3 of the span when tracking, all of it for NEE, but not a length that
+  // held too many chords on the lane's last rays.  Shares of 0.25, 0.35 and 0.5: 201, 197
+  // and 203 ms (1024x1024, 8 samples, 1M kernels, one-cone masks), 6.4, 6.8 and 6.9 ms
+  // (333x217, 4 samples, FP16), 99, 99 and 107 ms (512x512, 16 samples, every cone).
   const float len = t1 - t0;
-  S.step = kind == 1 ? fmaxf(fminf(0.25f * len, S.fit), 1e-6f) : fminf(len, S.fit);
+  S.step = kind == 1 ? fmaxf(fminf(0.3f * len, S.fit), 1e-6f) : fminf(len, S.fit);
   S.fit *= 1.1f;
   R.ta = t0;
   R.te = kind == 1 || S.step < len ? fminf(t1, t0 + S.step) : t1;
