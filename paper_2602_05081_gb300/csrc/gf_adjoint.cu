@@ -254,8 +254,9 @@ __device__ __forceinline__ void add_grad4(const BackArgs& B, int j, const float 
 //
 // d tau / d theta needs the five moments of the chord's envelope (from_moments) and
 // the two chord ends; the first of them, A C0, is the chord's part of tau.  So one
-// traversal gives both: each lane integrates its own chord, keeps its moments
-// (24 bytes) and adds to tau; then the warp goes through the kept chords, 32 at a
+// traversal gives both: chords are queued, so that 32 at a time are integrated, one per
+// lane (about half of the leaves reached have none), their moments kept (24 bytes) and
+// their integrals added to tau; then the warp goes through the kept chords, 32 at a
 // time, and scatters dL/dtau times their gradients.  A ray with more chords than
 // kTomoChords is traversed again with its tau known.  Bound by instruction issue.
 // Every lane used to carry its own pixel, with 15 derivatives formed at every
@@ -270,22 +271,39 @@ struct TomoChord {
 };
 static_assert(sizeof(TomoChord) == 24, "kept chords of 24 bytes");
 
-// moments of a chord's envelope in t - tc, and its terms of tau into (s, c)
-__device__ __forceinline__ TomoChord tomo_moments(const Chord& ch, const float* glx,
-                                                  const float* glw, float& s_acc, float& c_acc,
-                                                  Counters& cnt) {
+// a chord to integrate
+struct TomoItem {
+  float mid, hl, y2, y1, y0, B, delta, absA;
+  int j;
+  int rule;  // node count | table offset << 8
+};
+constexpr int kTomoQ = 64;  // queued chords per warp (<= 31 left + 32 new)
+struct TomoQ {
+  CoopTrav t;
+  float f[8][kTomoQ];
+  int j[kTomoQ], rule[kTomoQ];
+};
+__device__ __forceinline__ TomoItem tomo_item(const Chord& ch, int j) {
   const float len = ch.dtout - ch.dtin;
   int n, off;
   gl_pick(gl_rule(sqrtf(ch.a) * len + 0.5f * fabsf(ch.B) * len), n, off);
+  return TomoItem{0.5f * (ch.dtin + ch.dtout), 0.5f * len, -0.5f * kLog2e * ch.a, -kLog2e * ch.b,
+                  -0.5f * kLog2e * ch.g, ch.B, ch.delta, ch.absA, j, n | off << 8};
+}
+
+// moments of a chord's envelope in t - tc, and its terms of tau into (s, c)
+__device__ __forceinline__ TomoChord tomo_moments(const TomoItem& q, const float* glx,
+                                                  const float* glw, float& s_acc, float& c_acc,
+                                                  Counters& cnt) {
+  const int n = q.rule & 0xFF, off = q.rule >> 8;
   cnt.evals += 2 * n;
-  const float mid = 0.5f * (ch.dtin + ch.dtout), hl = 0.5f * len;
-  const float y2 = -0.5f * kLog2e * ch.a, y1 = -kLog2e * ch.b, y0 = -0.5f * kLog2e * ch.g;
-  const float scale = ch.absA * hl;
-  TomoChord m{0.f, 0.f, 0.f, 0.f, 0.f, 0};
+  const float scale = q.absA * q.hl;
+  TomoChord m{0.f, 0.f, 0.f, 0.f, 0.f, q.j};
   for (int k = off; k < off + n; ++k) {
-    const float dt = fmaf(hl, glx[k], mid), e = glw[k] * ex2f(fmaf(fmaf(y2, dt, y1), dt, y0));
+    const float dt = fmaf(q.hl, glx[k], q.mid),
+                e = glw[k] * ex2f(fmaf(fmaf(q.y2, dt, q.y1), dt, q.y0));
     float sn, cs;
-    sincosf(fmaf(ch.B, dt, ch.delta), &sn, &cs);
+    sincosf(fmaf(q.B, dt, q.delta), &sn, &cs);
     const float ec = e * cs, es = e * sn, ect = ec * dt;
     neumaier_add(s_acc, c_acc, scale * ec);
     m.C0 += ec;
@@ -294,11 +312,11 @@ __device__ __forceinline__ TomoChord tomo_moments(const Chord& ch, const float* 
     m.S0 += es;
     m.S1 = fmaf(es, dt, m.S1);
   }
-  m.C0 *= hl;
-  m.C1 *= hl;
-  m.C2 *= hl;
-  m.S0 *= hl;
-  m.S1 *= hl;
+  m.C0 *= q.hl;
+  m.C1 *= q.hl;
+  m.C2 *= q.hl;
+  m.S0 *= q.hl;
+  m.S1 *= q.hl;
   return m;
 }
 
@@ -330,10 +348,10 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
     k_tomo_backward(const __grid_constant__ DevField F, const PathParams P, const BackArgs Bk,
                     const float* dLdI, int* counter, int chunk, TomoChord* store) {
   __shared__ BlockTables sm;
-  __shared__ CoopTrav qs[kBackBlock / 32];
+  __shared__ TomoQ qs[kBackBlock / 32];
   init_tables(sm, F);
   const uint32_t lane = threadIdx.x & 31u;
-  CoopTrav& Q = qs[threadIdx.x >> 5];
+  TomoQ& Q = qs[threadIdx.x >> 5];
   store += ((size_t)blockIdx.x * (kBackBlock / 32) + (threadIdx.x >> 5)) * kTomoChords;
   Counters cnt;
   const uint32_t nchunk = (uint32_t)((P.spp + chunk - 1) / chunk);
@@ -354,8 +372,24 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
       if (!scene_span(F, o, inv, 0.f, INFINITY, t0, t1)) continue;
       if (lane == 0) cnt.windows += 1;
       float s_acc = 0.f, c_acc = 0.f;
-      int nch = 0;
-      coop_traverse(F, Q, F.occupied, o, inv, t0, t1, lane, cnt, [&](int j) {
+      int nch = 0, nq = 0;  // integrated and queued chords
+      auto integrate = [&](int tk) {
+        const bool have = (int)lane < tk;
+        const int at = nq - tk + (int)lane;
+        TomoItem q{};
+        if (have)
+          q = TomoItem{Q.f[0][at], Q.f[1][at], Q.f[2][at], Q.f[3][at], Q.f[4][at],
+                       Q.f[5][at], Q.f[6][at], Q.f[7][at], Q.j[at],    Q.rule[at]};
+        __syncwarp();
+        nq -= tk;
+        if (have) {
+          ++cnt.chords;
+          const TomoChord m = tomo_moments(q, sm.glx, sm.glw, s_acc, c_acc, cnt);
+          if (nch + (int)lane < kTomoChords) store[nch + (int)lane] = m;
+        }
+        nch += tk;
+      };
+      coop_traverse(F, Q.t, F.occupied, o, inv, t0, t1, lane, cnt, [&](int j) {
         Chord ch;
         // the support radius is a constant of the differentiation (adaptive extents too)
         bool ok = false;
@@ -365,14 +399,24 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
         }
         const unsigned b = __ballot_sync(kFull, ok);
         if (ok) {
-          ++cnt.chords;
-          TomoChord m = tomo_moments(ch, sm.glx, sm.glw, s_acc, c_acc, cnt);
-          m.j = j;
-          const int k = nch + __popc(b & ((1u << lane) - 1u));
-          if (k < kTomoChords) store[k] = m;
+          const TomoItem q = tomo_item(ch, j);
+          const int at = nq + __popc(b & ((1u << lane) - 1u));
+          Q.f[0][at] = q.mid;
+          Q.f[1][at] = q.hl;
+          Q.f[2][at] = q.y2;
+          Q.f[3][at] = q.y1;
+          Q.f[4][at] = q.y0;
+          Q.f[5][at] = q.B;
+          Q.f[6][at] = q.delta;
+          Q.f[7][at] = q.absA;
+          Q.j[at] = q.j;
+          Q.rule[at] = q.rule;
         }
-        nch += __popc(b);
+        nq += __popc(b);
+        __syncwarp();
+        if (nq >= 32) integrate(32);
       });
+      if (nq > 0) integrate(nq);
       warp_sum_pair(s_acc, c_acc);
       const float dLdtau = -gI * expf(-__fadd_rn(s_acc, c_acc)) / (float)P.spp;
       __syncwarp();  // the kept chords are read by other lanes
@@ -384,13 +428,13 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
           if (chord_setup(Pr, o, v, 0.f, INFINITY, Pr.k2, ch)) tomo_scatter(Bk, Pr, ch, m, v, m.j, dLdtau);
         }
       } else {
-        coop_traverse(F, Q, F.occupied, o, inv, t0, t1, lane, cnt, [&](int j) {
+        coop_traverse(F, Q.t, F.occupied, o, inv, t0, t1, lane, cnt, [&](int j) {
           if (j < 0) return;
           const Prim Pr = load_prim(F, j);
           Chord ch;
           if (!chord_setup(Pr, o, v, 0.f, INFINITY, Pr.k2, ch)) return;
           float s2 = 0.f, c2 = 0.f;
-          const TomoChord m = tomo_moments(ch, sm.glx, sm.glw, s2, c2, cnt);
+          const TomoChord m = tomo_moments(tomo_item(ch, j), sm.glx, sm.glw, s2, c2, cnt);
           tomo_scatter(Bk, Pr, ch, m, v, j, dLdtau);
         });
       }
