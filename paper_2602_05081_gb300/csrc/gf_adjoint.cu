@@ -33,14 +33,13 @@ struct BackArgs {
 
 // Derivatives of one kernel g = A exp(-q/2) cos(theta) with respect to its 15
 // raw parameters (mu 3, quaternion 4 through qhat = q/|q|, log scale 3, omega 3
-// in the input frame, phase, weight), at offsets y = x - mu.
+// in the input frame, phase, weight) along a ray, at offsets y = x - mu.
 struct PrimDeriv {
   float R[3][3];
   float qh[4], iqn;    // unit quaternion (w, x, y, z) and 1/|q| of the raw one
   float s[3], is2[3], kin[3];
   float A, dAdw;
   float3 om;
-  float phi;
   bool local, normalized;
 
   // from the parameters k_adj_prims gathered for sorted primitive j
@@ -69,7 +68,6 @@ struct PrimDeriv {
     normalized = B.wmode == GF_WEIGHT_NORMALIZED;
     A = P.A;
     om = P.om;
-    phi = P.phi;
   }
 
   // dz/dq of the raw quaternion at offset y (linear in y): dz/d(qhat_l) =
@@ -103,9 +101,10 @@ struct PrimDeriv {
   // the envelope: C_k of e cos(theta) t^k and S_k of e sin(theta) t^k (e the weighted
   // envelope without the amplitude, theta the phase with the sign of the amplitude
   // folded in).  q is quadratic and theta linear in t, so every derivative is a
-  // combination of five moments.
+  // combination of five moments.  qt receives half of dq/dquaternion as a quadratic in t.
   __device__ __forceinline__ void from_moments(float3 pp, float3 vv, float C0, float C1, float C2,
-                                               float S0, float S1, float acc[15]) const {
+                                               float S0, float S1, float acc[15],
+                                               float qt[4][3]) const {
     const float p[3] = {pp.x, pp.y, pp.z}, v[3] = {vv.x, vv.y, vv.z};
     const float aA = fabsf(A), sgn = A < 0.f ? -1.f : 1.f;
     float zp[3], zv[3];
@@ -138,6 +137,9 @@ struct PrimDeriv {
         h1 += kos[k] * gv[m][k];
       }
       acc[3 + m] = -aA * (q0 * C0 + q1 * C1 + q2 * C2 + h0 * S0 + h1 * S1);
+      qt[m][0] = q0;
+      qt[m][1] = q1;
+      qt[m][2] = q2;
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -150,57 +152,31 @@ struct PrimDeriv {
     acc[14] = sgn * dAdw * C0;
   }
 
-  // value g at y; d[15] = dg/dparam; dq[10] = dq/dparam (mu, quaternion, log scale)
-  __device__ float at(const float y[3], float d[15], float dq[10]) const {
-    float z[3];
+  // The Leibniz term of a chord end at dt (relative to the chord's tc), added to acc:
+  // the end moves as dt/dtheta = -(dq/dtheta)/(dq/dt), g sgn times that enters the
+  // integral.  dq/dt is formed from dq/dmu at the end's position (grazing chords divide
+  // by little, so its rounding matters); dq/dquaternion is the quadratic qt.
+  __device__ __forceinline__ void end_term(const Chord& ch, float3 v, float dt, float sgn,
+                                           const float qt[4][3], float acc[15]) const {
+    const float y[3] = {fmaf(dt, v.x, ch.p.x), fmaf(dt, v.y, ch.p.y), fmaf(dt, v.z, ch.p.z)};
+    float z[3], dm[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) z[k] = R[0][k] * y[0] + R[1][k] * y[1] + R[2][k] * y[2];
-    const float qq = z[0] * z[0] * is2[0] + z[1] * z[1] * is2[1] + z[2] * z[2] * is2[2];
-    const float env = expf(-0.5f * qq);
-    const float th = om.x * y[0] + om.y * y[1] + om.z * y[2] + phi;
-    float sn, cs;
-    sincosf(th, &sn, &cs);
-    float dth[15], dA[15];
-#pragma unroll
-    for (int r = 0; r < 15; ++r) {
-      dth[r] = 0.f;
-      dA[r] = 0.f;
-    }
 #pragma unroll
     for (int a = 0; a < 3; ++a)
-      dq[a] = -2.f * (R[a][0] * z[0] * is2[0] + R[a][1] * z[1] * is2[1] + R[a][2] * z[2] * is2[2]);
-    dth[0] = -om.x;
-    dth[1] = -om.y;
-    dth[2] = -om.z;
-    float g[4][3];
-    dz_dq(y, g);
+      dm[a] = -2.f * (R[a][0] * z[0] * is2[0] + R[a][1] * z[1] * is2[1] + R[a][2] * z[2] * is2[2]);
+    const float dqdt = -(v.x * dm[0] + v.y * dm[1] + v.z * dm[2]);
+    if (dqdt == 0.f) return;
+    const float q = fmaf(fmaf(ch.a, dt, 2.f * ch.b), dt, ch.g);
+    const float g = ch.absA * ex2f(-0.5f * kLog2e * q) * cosf(fmaf(ch.B, dt, ch.delta));
+    const float w = -sgn * g / dqdt;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      float dqm = 0.f, dthm = 0.f;
+    for (int a = 0; a < 3; ++a) acc[a] = fmaf(w, dm[a], acc[a]);
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        dqm += 2.f * z[k] * g[m][k] * is2[k];
-        if (local) dthm += kin[k] / s[k] * g[m][k];
-      }
-      dq[3 + m] = dqm;
-      dth[3 + m] = dthm;
-    }
+    for (int m = 0; m < 4; ++m)
+      acc[3 + m] = fmaf(w, 2.f * fmaf(fmaf(qt[m][2], dt, qt[m][1]), dt, qt[m][0]), acc[3 + m]);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      dq[7 + k] = -2.f * z[k] * z[k] * is2[k];
-      if (local) dth[7 + k] = -kin[k] * z[k] / s[k];
-      if (normalized) dA[7 + k] = -A;
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) dth[10 + k] = local ? z[k] / s[k] : y[k];
-    dth[13] = 1.f;
-    dA[14] = dAdw;
-#pragma unroll
-    for (int r = 0; r < 15; ++r) {
-      const float dqr = r < 10 ? dq[r] : 0.f;
-      d[r] = A * env * (-0.5f * dqr * cs - sn * dth[r]) + dA[r] * env * cs;
-    }
-    return A * env * cs;
+    for (int k = 0; k < 3; ++k) acc[7 + k] = fmaf(w, -2.f * z[k] * z[k] * is2[k], acc[7 + k]);
   }
 };
 
@@ -325,22 +301,11 @@ __device__ __forceinline__ void tomo_scatter(const BackArgs& B, const Prim& P, c
                                              const TomoChord& m, float3 v, int j, float dLdtau) {
   PrimDeriv D;
   D.load(B, P, j);
-  float acc[15];
-  D.from_moments(ch.p, v, m.C0, m.C1, m.C2, m.S0, m.S1, acc);
-  // Leibniz terms where a chord end lies on the ellipsoid (not on t = 0): the end
-  // moves as dt/dtheta = -(dq/dtheta)/(dq/dt)
-  const bool on_in = ch.dts - ch.hw > 0.f - ch.tc;
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    if (e == 0 && !on_in) continue;
-    const float dt = e == 0 ? ch.dtin : ch.dtout, sgn = e == 0 ? -1.f : 1.f;
-    const float y[3] = {fmaf(dt, v.x, ch.p.x), fmaf(dt, v.y, ch.p.y), fmaf(dt, v.z, ch.p.z)};
-    float d[15], dq[10];
-    const float g = D.at(y, d, dq);
-    const float dqdt = -(v.x * dq[0] + v.y * dq[1] + v.z * dq[2]);
-    if (dqdt != 0.f)
-      for (int r = 0; r < 10; ++r) acc[r] += sgn * g * (-dq[r] / dqdt);
-  }
+  float acc[15], qt[4][3];
+  D.from_moments(ch.p, v, m.C0, m.C1, m.C2, m.S0, m.S1, acc, qt);
+  // chord ends that lie on the ellipsoid (not on t = 0)
+  if (ch.dts - ch.hw > 0.f - ch.tc) D.end_term(ch, v, ch.dtin, -1.f, qt, acc);
+  D.end_term(ch, v, ch.dtout, 1.f, qt, acc);
   add_grad4(B, j, acc, dLdtau);
 }
 
@@ -1065,8 +1030,8 @@ struct RadScatterLeaf {
     if (!any) return;
     PrimDeriv D;
     D.load(W->B, Pr, j);
-    float acc[15];
-    D.from_moments(ch.p, R.v, C0, C1, C2, S0, S1, acc);
+    float acc[15], qt[4][3];
+    D.from_moments(ch.p, R.v, C0, C1, C2, S0, S1, acc, qt);
     add_grad4(W->B, j, acc, w * scale);
   }
 };
@@ -1145,8 +1110,8 @@ __device__ __noinline__ void rad_scatter(RadWarp& W, int which, int n, int seg, 
         if (chord_setup(Pr, Q.ray.o, Q.ray.v, 0.f, INFINITY, Pr.k2, ch)) {
           PrimDeriv D;
           D.load(W.B, Pr, j);
-          float acc[15];
-          D.from_moments(ch.p, Q.ray.v, C0, C1, C2, S0, S1, acc);
+          float acc[15], qt[4][3];
+          D.from_moments(ch.p, Q.ray.v, C0, C1, C2, S0, S1, acc, qt);
           add_grad4(W.B, j, acc, w * scale);
         }
       }
@@ -1323,8 +1288,8 @@ __device__ __forceinline__ void path_backward(RadWarp& W, float3 o, float3 v, ui
     if (!chord_setup(Pr, so, sv, 0.f, INFINITY, Pr.k2, ch)) continue;
     PrimDeriv D;
     D.load(W.B, Pr, j);
-    float acc[15];
-    D.from_moments(ch.p, sv, a.x, a.y, a.z, a.w, c.x, acc);
+    float acc[15], qt[4][3];
+    D.from_moments(ch.p, sv, a.x, a.y, a.z, a.w, c.x, acc, qt);
     add_grad4(W.B, j, acc, S);
   }
   __syncwarp();
