@@ -452,14 +452,14 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
 // The radiance adjoints run one path per warp.  Bound by instruction issue and the
 // latency of tree nodes.  With one pixel per lane 1.8 of 32 lanes ran, every window
 // visited its ray's list three times and paths were followed twice.  Through 200k
-// kernels: 305 -> 9.6 ms (128x128, 2 samples, single scattering), 697 -> 4.2 ms (96x64,
+// kernels: 305 -> 8.3 ms (128x128, 2 samples, single scattering), 697 -> 3.5 ms (96x64,
 // 1 sample, 3 bounces).
 //
 // A ray is processed over a window of t, at first all of it:
 //  gather   the warp traverses the binary tree together; chords go to the warp's list
 //           in global scratch, their tentative points to shared memory;
 //  sort     the points by t;
-//  sums     kappa and kappa_bar of four points at a time: the chords covering a point
+//  sums     kappa and kappa_bar of two points at a time: the chords covering a point
 //           are collected, their terms computed one per lane and put in the order of a
 //           depth-first walk that visits near children first, in which one lane adds
 //           them up (FP32).  Decisions therefore do not depend on how the work was
@@ -473,15 +473,17 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
 // ---------------------------------------------------------------------------
 constexpr int kMaxSeg = 15;
 constexpr int kRadBlocks = 4;     // resident blocks per SM
-constexpr int kRadStack = 384;    // a step adds <= 32; depth first above kRadStack - margin
-constexpr int kRadMargin = 128;   // a full step, then <= 1 entry per level, 64 levels
+constexpr int kRadStack = 256;
+constexpr int kRadMargin = 64;    // a descent adds <= 1 entry per level, 64 levels
 constexpr int kRadLeafQ = 96;     // <= 31 left + 64 new
-constexpr int kRadPts = 128;      // tentative points of a window
+// (The buffers are kept small: beside 28 KB of them per warp's block the L1 holds the
+// tree's upper nodes.  With 384 stack entries, 128 points and groups of 4 the blocks
+// took 215 KB of an SM: 9.7 and 4.4 ms for the cases above, 8.3 and 3.5 now.)
+constexpr int kRadPts = 64;       // tentative points of a window
 constexpr int kRadList = 4096;    // chords of a window at most (global scratch; rad_list_cap)
 constexpr int kRadKeep = 4096;    // kept segment moments of a path (global scratch)
-constexpr int kRadGroup = 4;      // points whose sums are formed together
-constexpr int kRadTerms = 256;    // covering chords of a group, 64 per point
-static_assert(32 + 64 <= kRadMargin, "a full step, then a descent");
+constexpr int kRadGroup = 2;      // points whose sums are formed together
+constexpr int kRadTerms = 128;    // covering chords of a group, 64 per point
 static_assert(kStack <= 64, "a key bit per tree level");
 static_assert(kPts <= kRadPts && kRadList <= 1 << 16, "point ids");
 
@@ -607,7 +609,8 @@ __device__ __noinline__ void rad_gather(RadWarp& W, int which) {
       break;
     }
     int take = sp < 32 ? sp : 32;
-    if (sp > kRadStack - kRadMargin) take = 1;  // near capacity: depth first
+    // near capacity fewer, down to one: a node leaves room for one more entry
+    take = min(take, max(1, kRadStack - kRadMargin - sp));
     const bool have = (int)lane < take;
     const int ent = have ? Q.t.stk[sp - take + (int)lane] : 0;
     const unsigned long long key = have ? Q.t.skey[sp - take + (int)lane] : 0ull;
@@ -834,7 +837,9 @@ __device__ __noinline__ bool rad_sums(RadWarp& W, int which, int g, int n) {
   }
   __syncwarp();
   if ((int)lane < n) {
-    const int cl = lane == 0 ? c[0] : lane == 1 ? c[1] : lane == 2 ? c[2] : c[3];
+    int cl = c[0];
+#pragma unroll
+    for (int p = 1; p < kRadGroup; ++p) cl = (int)lane == p ? c[p] : cl;
     const float4* T = Q.e.term + (int)lane * cap;
     float kap = 0.f, kb = 0.f;
     for (int i = 0; i < cl; ++i) {

@@ -265,10 +265,10 @@ __global__ void __launch_bounds__(kBlock, kCoopBlocks)
 // GF_FLIGHT_SEGMENT): one pixel per warp, its samples in order; every flight works on
 // the ray's collected chords, the NEE transmittance is exp(-tau) in closed form.
 // 160x120 at 2 samples through 50k kernels: 260 ms with one pixel per lane and a
-// traversal for each of up to 33 depths of a flight, 3.6 ms now.  Bound by instruction
+// traversal for each of up to 33 depths of a flight, 2.9 ms now.  Bound by instruction
 // issue: two traversals per collision, then the Faddeeva sums of the chord ends.
 // ---------------------------------------------------------------------------
-constexpr int kFlightBlocks = 4;  // resident blocks per SM
+constexpr int kFlightBlocks = 5;  // resident blocks per SM (3.02 ms with 4, 2.85 with 5)
 template <int FF>
 __global__ void __launch_bounds__(kBlock, kFlightBlocks)
     k_flight(const __grid_constant__ DevField F, const __grid_constant__ PathParams P, float* out,

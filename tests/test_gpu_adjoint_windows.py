@@ -1,8 +1,8 @@
 """Adjoints and analytic flights where their per-warp buffers overflow, against the FP64
 oracle (GPU).
 
-A warp holds up to 4,096 chords and 128 tentative points of a ray's window, 64 (then
-256) chords covering a point, 1,024 chords of a tomography ray, 4,096 chords of an
+A warp holds up to 4,096 chords and 64 tentative points of a ray's window, 64 (then
+128) chords covering a point, 1,024 chords of a tomography ray, 4,096 chords of an
 analytic flight.  Each field here passes one of these limits, on few pixels.
 """
 import numpy as np
@@ -58,8 +58,8 @@ def _check(g, g_ref, n, what):
 @pytest.mark.parametrize("n,tau,res,bounces", [
     (6_000, 5.0, 6, 1),      # about 140 chords cover a point: more than 64
     (6_000, 5.0, 6, 2),
-    (14_000, 5.0, 5, 1),     # about 320: more than 256
-    (3_000, 300.0, 5, 1),    # more than 128 tentative points on a ray
+    (14_000, 5.0, 5, 1),     # about 320: more than 128
+    (3_000, 300.0, 5, 1),    # more than 64 tentative points on a ray
     (3_000, 300.0, 5, 3),
     # about 18,000 chords on a ray, 5,000 covering a point: no window holds them
     (220_000, 80.0, 3, 2),
