@@ -66,6 +66,8 @@ struct TrParams {
   float* out_T;
   float* out_tau;
   int* counter;
+  bool dealt = false;  // rays dealt out to the warps instead of fetched (set by the launcher)
+  bool exact = false;  // ratio tracking: terms in the per-thread tracker's form (rt_coop)
 };
 
 struct ChordParams {

@@ -1,8 +1,6 @@
 // gf_kernels.cu -- render, transmittance and test kernels of the Gabor-field
 // renderer.  Persistent warps pull work from a global counter: one ray per warp
-// (gf_coop.cuh) for optical depths, analytic free flights and small ratio-tracking
-// batches; 32 rays per warp, each lane owning one (gf_trace.cuh), for large
-// ratio-tracking batches.
+// (gf_coop.cuh).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -16,35 +14,14 @@ namespace gf {
 constexpr int kBlock = 128;
 constexpr int kCoopBlocks = 5;  // resident blocks per SM of the one-ray-per-warp kernels
 
-// ---------------------------------------------------------------------------
-// ratio-tracking transmittance of large batches, one ray per lane
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kBlock, 3)  // at most 168 registers: 12 warps per SM
-    k_transmittance_rt(const __grid_constant__ DevField F, const TrParams P) {
-  __shared__ BlockTables sm;
-  init_tables(sm, F);
-  const uint32_t lane = threadIdx.x & 31u;
-  Counters cnt;
-  for (;;) {
-    const uint32_t tile = next_tile(P.counter, lane);
-    if ((int64_t)tile * 32 >= P.n) break;
-    const int64_t r = (int64_t)tile * 32 + (int)lane;
-    if (r < P.n) {
-      const float3 o = make_float3(P.o[3 * r], P.o[3 * r + 1], P.o[3 * r + 2]);
-      const float3 v = unit_dir(make_float3(P.d[3 * r], P.d[3 * r + 1], P.d[3 * r + 2]));
-      const float tmin = P.trange ? P.trange[2 * r] : 0.f;
-      const float tmax = P.trange ? P.trange[2 * r + 1] : INFINITY;
-      float acc = 0.f;
-      for (int s = 0; s < P.spp; ++s) {
-        const Mask m = sample_mask(F, P.lod, v, P.seed, (uint32_t)r, (uint32_t)s, 0, TAG_MASK);
-        cnt.rays += 1;
-        acc += track<false>(F, m, o, v, tmin, tmax, false, P.seed, (uint32_t)r,
-                            stream_word((uint32_t)s, 0, TAG_TRACK), sm.env, cnt, nullptr);
-      }
-      P.out_T[r] = acc / (float)P.spp;
-    }
-  }
-  flush_counters(F, cnt, lane);
+// The rays of a warp: a small batch is dealt out (no counter to clear, no atomic per
+// ray), larger ones are fetched one by one (launch_transmittance).
+__device__ __forceinline__ int64_t first_ray(const TrParams& P, uint32_t lane) {
+  return P.dealt ? (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)
+                 : (int64_t)next_tile(P.counter, lane);
+}
+__device__ __forceinline__ int64_t next_ray(const TrParams& P, uint32_t lane, int64_t r) {
+  return P.dealt ? r + (int64_t)gridDim.x * (blockDim.x >> 5) : (int64_t)next_tile(P.counter, lane);
 }
 
 // ---------------------------------------------------------------------------
@@ -66,9 +43,7 @@ __global__ void __launch_bounds__(kBlock, kCoopBlocks)
   CoopQ& Q = qs[threadIdx.x >> 5];
   Counters cnt;
   const int spp = lod_is_deterministic(P.lod) ? 1 : P.spp;
-  for (;;) {
-    const int64_t r = next_tile(P.counter, lane);
-    if (r >= P.n) break;
+  for (int64_t r = first_ray(P, lane); r < P.n; r = next_ray(P, lane, r)) {
     const float3 o = make_float3(P.o[3 * r], P.o[3 * r + 1], P.o[3 * r + 2]);
     const float3 v = unit_dir(make_float3(P.d[3 * r], P.d[3 * r + 1], P.d[3 * r + 2]));
     const float tmin = P.trange ? P.trange[2 * r] : 0.f;
@@ -90,108 +65,172 @@ __global__ void __launch_bounds__(kBlock, kCoopBlocks)
 }
 
 // ---------------------------------------------------------------------------
-// Ratio tracking of small batches, one ray per warp.  The warp traverses the
-// ray's tree together; each round's chords (one per lane) store their
-// evaluation records in shared memory and draw all their tentative points in
-// [t0, t1] (chord_points: the per-chord streams of the per-thread tracker, so
-// the same points), written in lane order after a counting pass.  Then each
-// lane takes points i = lane, lane + 32, ..., sums kappa and kappa_bar at them
-// over all stored chords in order, and multiplies its factors 1 - kappa /
-// kappa_bar; the lanes' products are combined in a fixed butterfly order.  A
-// ray with more chords or points than the buffers hold is tracked by the
-// per-thread tracker instead (lane 0).
+// Ratio tracking, one ray per warp, over a window of t, at first all of the ray.  The
+// warp traverses the trees together; each round's chords (one per lane) store their
+// evaluation records in shared memory and draw their tentative points in the window
+// (chord_points: the per-chord streams of the per-thread tracker, so the same points).
+// The points are put in t order; then 1, 2, ... 32 lanes per point sum kappa and
+// kappa_bar over the window's chords and multiply the factors 1 - kappa / kappa_bar;
+// the lanes' products are combined in a fixed butterfly order.  A window with more
+// chords or points than the buffers hold is halved.  Bound by instruction issue and the
+// latency of tree nodes.  30,000 rays through 100k kernels: 38 ms with one ray per lane
+// (the per-thread tracker traverses twice per eight points, its lanes parted), 4.3 ms now;
+// 4,096 rays through 256 kernels: 32 -> 27 us (rays dealt out).
+//
+// Terms come in two forms.  Rays of a small batch that fit one window take records
+// centred on the envelope's peak; large batches and rays of several windows take the
+// per-thread tracker's own form (`exact`), which differs by up to 2e-4 of T where
+// carriers of ~1e3 rad run over a chord (fast cosine of an unreduced phase).
+// Left to the per-thread tracker (one lane): windows that cannot be halved, and in the
+// exact form a ray on which two points coincide (the tracker goes through its points in
+// runs of kPts and leaves out a point at the t at which a run ended).
 // ---------------------------------------------------------------------------
-constexpr int kRtChords = 256;  // chords of one ray held in shared memory
-constexpr int kRtPts = 128;     // tentative points of one ray
+constexpr int kRtRec = 512;    // float4s of chord records of a window in shared memory
+constexpr int kRtPts = 128;    // tentative points of a window
 struct RtQ {
   CoopTrav t;
-  float4 rec[kRtChords][2];  // centred on the envelope peak t*: (t*, t_in, t_out, B),
-                             // (-a log2(e) / 2, log2 h, phase at t*, sqrt(a))
-  float pt[kRtPts], pu[kRtPts];
+  // centred, 2 per chord: (t*, t_in, t_out, B), (-a log2(e) / 2, log2 h, phase at t*,
+  // sqrt(a)); exact, 3 per chord: (tc, t_in, t_out, B), exponent's y2, y1, y0 and the phase
+  // at tc, (h, t* - tc, sqrt(a), -)
+  float4 rec[kRtRec];
+  float raw[kRtPts], pt[kRtPts];  // points as drawn, and in t order
+  int npts;
 };
 
-__device__ float rt_coop(const DevField& F, RtQ& Q, const Mask& M, float3 o, float3 v, float3 inv,
-                         float tmin, float tmax, float t0, float t1, uint64_t seed, uint32_t ray,
-                         uint32_t word, const float* env, uint32_t lane, Counters& cnt) {
+// chords and points of the window [ta, tb), or [ta, t1] when last; returns the chords
+__device__ __forceinline__ int rt_gather(const DevField& F, RtQ& Q, const Mask& M, float3 o, float3 v,
+                                         float3 inv, float tmin, float tmax, float ta, float tb,
+                                         bool last, uint64_t seed, uint32_t ray, uint32_t word,
+                                         const float* env, uint32_t lane, bool exact, Counters& cnt) {
   const unsigned lt = (1u << lane) - 1u;
-  int nch = 0, npts = 0;  // warp-uniform
-  coop_traverse(F, Q.t, M.bits, o, inv, t0, t1, lane, cnt, [&](int j) {
+  const int cap = exact ? kRtRec / 3 : kRtRec / 2;
+  int nch = 0;
+  __syncwarp();
+  if (lane == 0) Q.npts = 0;
+  coop_traverse(F, Q.t, M.bits, o, inv, ta, tb, lane, cnt, [&](int j) {
     Chord ch;
-    float w, h = 0.f;
-    bool ok = false;
-    if (j >= 0 &&
-        prim_chord(F, j, o, v, tmin, tmax, [&](uint32_t cl) { return mask_weight(M, cl); }, w, ch) &&
-        ch.tc + ch.dtin <= t1 && ch.tc + ch.dtout >= t0) {
-      ok = true;
-      h = w * ch.absA * expf(-0.5f * ch.qmin);
-    }
+    float w;
+    const bool ok = j >= 0 &&
+                    prim_chord(F, j, o, v, tmin, tmax,
+                               [&](uint32_t cl) { return mask_weight(M, cl); }, w, ch) &&
+                    ch.tc + ch.dtin <= tb && ch.tc + ch.dtout >= ta;
     const unsigned bc = __ballot_sync(kFull, ok);
-    if (ok) {
+    const int k = nch + __popc(bc & lt);
+    if (ok && k < cap) {
+      const float wa = w * ch.absA, h = wa * expf(-0.5f * ch.qmin);
       ++cnt.chords;
-      const int k = nch + __popc(bc & lt);
-      if (k < kRtChords) {
-        Q.rec[k][0] = make_float4(ch.tc + ch.dts, ch.tc + ch.dtin, ch.tc + ch.dtout, ch.B);
-        Q.rec[k][1] = make_float4(-0.5f * kLog2e * ch.a, __log2f(h),
-                                  reduce_2pi(fmaf(ch.B, ch.dts, ch.delta)), sqrtf(ch.a));
+      if (exact) {
+        Q.rec[3 * k] = make_float4(ch.tc, ch.tc + ch.dtin, ch.tc + ch.dtout, ch.B);
+        Q.rec[3 * k + 1] = make_float4(-0.5f * kLog2e * ch.a, -kLog2e * ch.b,
+                                       fmaf(-0.5f * kLog2e, ch.g, log2f(wa)), ch.delta);
+        Q.rec[3 * k + 2] = make_float4(h, ch.dts, sqrtf(ch.a), 0.f);
+      } else {
+        Q.rec[2 * k] = make_float4(ch.tc + ch.dts, ch.tc + ch.dtin, ch.tc + ch.dtout, ch.B);
+        Q.rec[2 * k + 1] = make_float4(-0.5f * kLog2e * ch.a, __log2f(h),
+                                       reduce_2pi(fmaf(ch.B, ch.dts, ch.delta)), sqrtf(ch.a));
       }
-    }
-    nch += __popc(bc);
-    // the round's points in lane order: count, then write at the prefix offsets
-    int m = 0;
-    if (ok)
       chord_points(F, ch, h, seed, ray, word, env, [&](float t, float) {
-        if (t > t1) return false;
-        if (t >= t0) ++m;
-        return true;
-      });
-    const int incl = warp_incl_sum(m, lane);
-    if (ok && m > 0) {
-      int q = npts + incl - m;
-      chord_points(F, ch, h, seed, ray, word, env, [&](float t, float u) {
-        if (t > t1) return false;
-        if (t >= t0) {
-          if (q < kRtPts) {
-            Q.pt[q] = t;
-            Q.pu[q] = u;
-          }
-          ++q;
+        if (last ? t > tb : t >= tb) return false;
+        if (t >= ta) {
+          const int q = atomicAdd(&Q.npts, 1);
+          if (q >= kRtPts) return false;  // too many: the window is halved
+          Q.raw[q] = t;
         }
         return true;
       });
     }
-    npts += __shfl_sync(kFull, incl, 31);
+    nch += __popc(bc);
   });
-  if (lane == 0) cnt.points += (unsigned long long)npts;
   __syncwarp();
-  if (nch > kRtChords || npts > kRtPts) {  // too many for the buffers: per-thread tracker
+  return nch;
+}
+
+__device__ float rt_coop(const DevField& F, RtQ& Q, const Mask& M, float3 o, float3 v, float3 inv,
+                         float tmin, float tmax, float t0, float t1, uint64_t seed, uint32_t ray,
+                         uint32_t word, const float* env, uint32_t lane, bool exact, Counters& cnt) {
+  float prod = 1.f, ta = t0, tb = t1;
+  bool alone = false;  // to the per-thread tracker
+  while (!alone) {
+    const bool last = tb >= t1;
+    const int nch =
+        rt_gather(F, Q, M, o, v, inv, tmin, tmax, ta, tb, last, seed, ray, word, env, lane, exact,
+                  cnt);
+    const int npts = Q.npts;
+    __syncwarp();
+    const float w = tb - ta;
+    if (nch > (exact ? kRtRec / 3 : kRtRec / 2) || npts > kRtPts) {
+      if (w > 1e-6f * (1.0f + fabsf(ta))) tb = ta + 0.5f * w;
+      else alone = true;
+      exact = true;
+      continue;
+    }
+    if (lane == 0) cnt.points += (unsigned long long)npts;
+    // t order (so that the product does not depend on which lane drew first)
+    bool tie = false;
+    for (int i = (int)lane; i < npts; i += 32) {
+      const float t = Q.raw[i];
+      int rank = 0;
+      for (int k = 0; k < npts; ++k) {
+        const float x = Q.raw[k];
+        rank += x < t || (x == t && k < i) ? 1 : 0;
+        tie = tie || (x == t && k != i);
+      }
+      Q.pt[rank] = t;
+    }
+    alone = __any_sync(kFull, exact && tie);
+    __syncwarp();
+    if (alone) break;
+    for (int q0 = 0; q0 < npts;) {
+      const int left = npts - q0;
+      int sh = 0;  // 2^sh lanes per point
+      while (sh < 5 && left << (sh + 1) <= 32) ++sh;
+      const int pts = min(left, 32 >> sh), sub = (int)(lane & ((1u << sh) - 1u));
+      const bool act = (int)(lane >> sh) < pts;
+      const float t = act ? Q.pt[q0 + (int)(lane >> sh)] : 0.f;
+      float kap = 0.f, kb = 0.f;
+      for (int c = act ? sub : nch; c < nch; c += 1 << sh) {
+        const float4 a = Q.rec[exact ? 3 * c : 2 * c];
+        if (!(t >= a.y && t <= a.z)) continue;
+        const float dt = t - a.x;
+        ++cnt.evals;
+        if (exact) {
+          const float4 b = Q.rec[3 * c + 1], d = Q.rec[3 * c + 2];
+          kap = fmaf(ex2f(fmaf(fmaf(b.x, dt, b.y), dt, b.z)), cosf_fast(fmaf(a.w, dt, b.w)), kap);
+          int mm = (int)(fabsf(dt - d.y) * d.z);
+          mm = mm > 7 ? 7 : mm;
+          kb = fmaf(d.x, env[mm], kb);
+        } else {
+          const float4 b = Q.rec[2 * c + 1];
+          kap = fmaf(ex2f(fmaf(b.x, dt * dt, b.y)), cosf_fast(fmaf(a.w, dt, b.z)), kap);
+          int mm = (int)(fabsf(dt) * b.w);
+          mm = mm > 7 ? 7 : mm;
+          kb = fmaf(ex2f(b.y), env[mm], kb);  // h exp(-m^2/2)
+        }
+      }
+      __syncwarp();
+      for (int o2 = 1; o2 < 1 << sh; o2 <<= 1) {
+        kap += __shfl_xor_sync(kFull, kap, o2);
+        kb += __shfl_xor_sync(kFull, kb, o2);
+      }
+      if (act && sub == 0 && kb > 0.f) prod *= 1.f - kap / kb;
+      q0 += pts;
+    }
+    if (last) break;
+    ta = tb;
+    tb = fminf(t1, ta + 2.0f * w);
+  }
+  if (alone) {
     float T = 1.f;
     if (lane == 0) T = track<false>(F, M, o, v, tmin, tmax, false, seed, ray, word, env, cnt, nullptr);
+    __syncwarp();
     return __shfl_sync(kFull, T, 0);
-  }
-  float prod = 1.f;
-  for (int i = (int)lane; i < npts; i += 32) {
-    const float t = Q.pt[i];
-    float kap = 0.f, kb = 0.f;
-    for (int c = 0; c < nch; ++c) {
-      const float4 a = Q.rec[c][0];
-      if (t >= a.y && t <= a.z) {
-        const float4 b = Q.rec[c][1];
-        const float dt = t - a.x;
-        kap = fmaf(ex2f(fmaf(b.x, dt * dt, b.y)), cosf_fast(fmaf(a.w, dt, b.z)), kap);
-        int mm = (int)(fabsf(dt) * b.w);
-        mm = mm > 7 ? 7 : mm;
-        kb = fmaf(ex2f(b.y), env[mm], kb);  // h exp(-m^2/2)
-        ++cnt.evals;
-      }
-    }
-    if (kb > 0.f) prod *= 1.f - kap / kb;
   }
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) prod *= __shfl_xor_sync(kFull, prod, off);
   return prod;
 }
 
-__global__ void __launch_bounds__(kBlock, 3)
+__global__ void __launch_bounds__(kBlock, 4)
     k_transmittance_rt_coop(const __grid_constant__ DevField F, const TrParams P) {
   __shared__ BlockTables sm;
   __shared__ RtQ qs[kBlock / 32];
@@ -199,9 +238,7 @@ __global__ void __launch_bounds__(kBlock, 3)
   const uint32_t lane = threadIdx.x & 31u;
   RtQ& Q = qs[threadIdx.x >> 5];
   Counters cnt;
-  for (;;) {
-    const int64_t r = next_tile(P.counter, lane);  // one ray per warp
-    if (r >= P.n) break;
+  for (int64_t r = first_ray(P, lane); r < P.n; r = next_ray(P, lane, r)) {
     const float3 o = make_float3(P.o[3 * r], P.o[3 * r + 1], P.o[3 * r + 2]);
     const float3 v = unit_dir(make_float3(P.d[3 * r], P.d[3 * r + 1], P.d[3 * r + 2]));
     const float tmin = P.trange ? P.trange[2 * r] : 0.f;
@@ -215,7 +252,7 @@ __global__ void __launch_bounds__(kBlock, 3)
       if (m.bits != 0ull && scene_span(F, o, inv, tmin, tmax, t0, t1)) {
         if (lane == 0) cnt.windows += 1;
         T = rt_coop(F, Q, m, o, v, inv, tmin, tmax, t0, t1, P.seed, (uint32_t)r,
-                    stream_word((uint32_t)s, 0, TAG_TRACK), sm.env, lane, cnt);
+                    stream_word((uint32_t)s, 0, TAG_TRACK), sm.env, lane, P.exact, cnt);
       }
       acc += T;
     }
@@ -436,26 +473,28 @@ static int persistent_grid(const Field& F, K kernel, int64_t warps_of_work) {
   return (int)(g < 1 ? 1 : g);
 }
 
+template <class K>
+static cudaError_t launch_rays(const Field& F, K kernel, TrParams P, cudaStream_t s) {
+  const int64_t g = persistent_grid(F, kernel, P.n);
+  // up to four rays per warp are dealt out: 4,096 rays through 256 kernels take 32.4 us with
+  // the counter (its clearing is a launch of its own), 29.1 us without
+  P.dealt = P.n <= 4 * g * (kBlock / 32);
+  if (!P.dealt) {
+    const cudaError_t e = cudaMemsetAsync(P.counter, 0, sizeof(int), s);
+    if (e != cudaSuccess) return e;
+  }
+  kernel<<<(unsigned)g, kBlock, 0, s>>>(F.dev, P);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_transmittance(const Field& F, const TrParams& P, cudaStream_t s) {
   (void)cudaGetLastError();  // a stale error of an unrelated call is not ours
-  cudaError_t e = cudaMemsetAsync(P.counter, 0, sizeof(int), s);
-  if (e != cudaSuccess) return e;
-  if (P.mode == GF_TR_DETERMINISTIC) {
-    auto k = k_transmittance_coop<GF_TR_DETERMINISTIC>;
-    k<<<persistent_grid(F, k, P.n), kBlock, 0, s>>>(F.dev, P);
-  } else if (P.mode == GF_TR_CLOSED_FORM) {
-    auto k = k_transmittance_coop<GF_TR_CLOSED_FORM>;
-    k<<<persistent_grid(F, k, P.n), kBlock, 0, s>>>(F.dev, P);
-  } else if (P.n * 8 <= (int64_t)F.ctx.sm_count * 16 * 32) {
-    // few rays: the whole warp on each ray (k_transmittance_rt_coop)
-    auto k = k_transmittance_rt_coop;
-    k<<<persistent_grid(F, k, P.n), kBlock, 0, s>>>(F.dev, P);
-  } else {
-    const int64_t tiles = (P.n + 31) / 32;
-    auto k = k_transmittance_rt;
-    k<<<persistent_grid(F, k, tiles), kBlock, 0, s>>>(F.dev, P);
-  }
-  return cudaGetLastError();
+  if (P.mode == GF_TR_DETERMINISTIC) return launch_rays(F, k_transmittance_coop<GF_TR_DETERMINISTIC>, P, s);
+  if (P.mode == GF_TR_CLOSED_FORM) return launch_rays(F, k_transmittance_coop<GF_TR_CLOSED_FORM>, P, s);
+  if (!stack_fits(k_transmittance_rt_coop)) return cudaErrorLaunchOutOfResources;
+  TrParams Q = P;
+  Q.exact = P.n * 8 > (int64_t)F.ctx.sm_count * 16 * 32;
+  return launch_rays(F, k_transmittance_rt_coop, Q, s);
 }
 
 // bytes of the analytic flights' chord lists of a full persistent grid
