@@ -88,7 +88,7 @@ __device__ __forceinline__ void coop_traverse(const DevField& F, CoopTrav& Q,
       ++cnt.nodes;
       hit = node4_hits(F.nodes4 + node, o, inv, t0, t1, ch);
     }
-    if (!push_hits(Q.stk, kCoopStack, hit, ch, lane, sp, lq_n, [](int c) { return c; }) && lane == 0)
+    if (!push_hits(Q.stk, kCoopStack, hit, ch, lane, sp, lq_n, [](int, int c) { return c; }) && lane == 0)
       set_err(F, ERR_STACK);
     __syncwarp();
     const bool more = sp > 0;

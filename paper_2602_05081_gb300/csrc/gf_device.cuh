@@ -671,22 +671,23 @@ __device__ __forceinline__ void hit_places(unsigned hi, unsigned hl, uint32_t la
 
 // Children of 32 nodes to the warp's stack (internal ones, from sp on) and leaf queue
 // (from lq_n on), which lie one behind the other: stk[stack_words], then the queue.
-// word(c) packs an internal child or, for a leaf, its primitive.  The stack's size is
+// word(k, c) packs child k, c the internal child or, for a leaf, its primitive.  The stack's size is
 // checked once for the warp; returns false when it would overflow (nothing is pushed).
-template <class Word>
-__device__ __forceinline__ bool push_hits(int* stk, int stack_words, unsigned hit, const int ch[4],
+template <int NC, class Word>
+__device__ __forceinline__ bool push_hits(int* stk, int stack_words, unsigned hit, const int (&ch)[NC],
                                           uint32_t lane, int& sp, int& lq_n, Word&& word) {
-  const unsigned leaf = (unsigned)ch[0] >> 31 | ((unsigned)ch[1] >> 31) << 1 |
-                        ((unsigned)ch[2] >> 31) << 2 | ((unsigned)ch[3] >> 31) << 3;
+  unsigned leaf = 0u;
+#pragma unroll
+  for (int k = 0; k < NC; ++k) leaf |= ((unsigned)ch[k] >> 31) << k;
   int pi, pl, np, nl;
   hit_places(hit & ~leaf, hit & leaf, lane, pi, pl, np, nl);
   if (sp + np > stack_words) return false;
   pi += sp;
   pl += stack_words + lq_n;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < NC; ++k) {
     const bool lf = ch[k] < 0, h = (hit >> k & 1u) != 0u;
-    if (h) stk[lf ? pl : pi] = word(lf ? ~ch[k] : ch[k]);
+    if (h) stk[lf ? pl : pi] = word(k, lf ? ~ch[k] : ch[k]);
     pi += h && !lf ? 1 : 0;
     pl += h && lf ? 1 : 0;
   }
@@ -758,7 +759,7 @@ __device__ __forceinline__ int next_root(const DevField& F, unsigned long long& 
 // The children of a four-wide node that overlap [ta, te] of the ray (bit k: child k);
 // ch receives the children.
 __device__ __forceinline__ unsigned node4_hits(const Node4* N, float3 o, float3 inv, float ta,
-                                               float te, int ch[4]) {
+                                               float te, int* ch) {
   float4 v0, v1;
   uint4 q, c4;
   ldg32(&N->v0, v0, v1);

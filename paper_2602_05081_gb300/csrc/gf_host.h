@@ -205,8 +205,9 @@ cudaError_t launch_pack16(Field& F, cudaStream_t s);
 size_t scatter_store_bytes(int64_t grid);
 size_t flight_store_bytes(const Field& F);
 cudaError_t server_grid(int sm_count, int64_t& grid);
-cudaError_t launch_render_server(const ServerLaunch& L, int64_t grid, float4* chord_store,
-                                 cudaStream_t s);
+// reqs: the batch's requests on the host (as L.reqs on the device, one per item)
+cudaError_t launch_render_server(const ServerLaunch& L, const ServerReqDev* reqs, int64_t grid,
+                                 float4* chord_store, cudaStream_t s);
 // image = fixed-point sums / spp
 cudaError_t launch_fix_to_image(const unsigned long long* acc, int64_t npix, int spp, float* out,
                                 cudaStream_t s);

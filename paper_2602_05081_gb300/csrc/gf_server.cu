@@ -208,7 +208,7 @@ struct gf_server {
     L.counter = reinterpret_cast<int*>(b.dev);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b.dev, b.host, up, cudaMemcpyHostToDevice, b.stream);
     if (e == cudaSuccess) e = cudaEventRecord(b.start, b.stream);
-    if (e == cudaSuccess) e = launch_render_server(L, grid, b.store, b.stream);
+    if (e == cudaSuccess) e = launch_render_server(L, rq, grid, b.store, b.stream);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(b.host + kErrOff, b.dev + kErrOff, kHead - kErrOff, cudaMemcpyDeviceToHost,
                           b.stream);

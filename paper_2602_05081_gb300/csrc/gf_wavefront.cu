@@ -34,7 +34,7 @@ namespace gf {
 
 constexpr int kWWarps = 4;      // warps per block
 constexpr int kBlocksPerSM = 4; // resident blocks per SM the kernels are built for
-constexpr int kLeafQ = 160;     // queued leaves per warp (<= 31 left + 128 new)
+constexpr int kLeafQ = 288;     // queued leaves per warp (<= 31 left + 256 new)
 constexpr int kChordQ = 64;     // queued chords per warp (<= 31 left + 32 new)
 // A window with more points or chords than its slot holds is halved and traversed
 // again: with 8 points and 256 chords that took 9 % of the windows of the 1M-kernel
@@ -126,6 +126,17 @@ __device__ __forceinline__ bool slot_chord(const DevField& F, const LaneRay& R, 
                     0.f, INFINITY, [&](uint32_t c) { return ray_weight(R, c); }, w, ch);
 }
 
+// Nodes per lane and traversal step.  Two hide each other's latency where rays visit many
+// nodes: with every cone selected, 512x512, 16 samples, 100k kernels take 98.4 ms with
+// one and 93.1 with two.  With one-cone masks (100 nodes per ray) a step seldom holds 64
+// entries and the longer code costs more: 1M kernels, 1024x1024, 8 samples 198 and 216 ms.
+static int nodes_per_step(const LodDev& a, const LodDev& b) {
+  return a.cone_policy == GF_CONE_ALL && b.cone_policy == GF_CONE_ALL && a.freq_policy <= GF_FREQ_CUTOFF &&
+                 b.freq_policy <= GF_FREQ_CUTOFF
+             ? 2
+             : 1;
+}
+
 // One draw of a queued chord's walk: the next tentative point of its majorant
 // (Sec. 3) from the chord's own Philox stream, recorded for the owner when it
 // falls in the window [ta, te).  Returns true when the chord may hold further
@@ -188,7 +199,7 @@ __device__ __forceinline__ bool walk_step(const DevField& F, WarpQ& Q, ChordItem
 // frontiers of all its rays, so lanes stay busy while 32 rays are in flight.
 // It collects the tentative points of each slot's window and stores the
 // window's chords for their evaluation.
-template <class Work>
+template <int kPerStep, class Work>
 __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, const float* env,
                            ChordStore* wch, Counters& cnt) {
   const unsigned lt = (1u << lane) - 1u;
@@ -214,32 +225,42 @@ __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, c
       if (lane == 0) set_err(Wk.err_field(), ERR_GUARD);
       break;
     }
-    // ---------------- one traversal step: up to 32 (four-wide node, slot) entries
+    // ---------------- one traversal step: up to kPerStep (four-wide node, slot) entries
+    // per lane
     GF_TIC(t_step);
-    int take = sp < 32 ? sp : 32;
+    int take = min(sp, 32 * kPerStep);
     // near capacity fewer, down to one: a node leaves room for three more entries, and
     // a descent adds at most three per level
     take = min(take, max(1, (kWStack - kStackMargin - sp) / 3));
-    const int ent = (int)lane < take ? Q.t.stk[sp - take + (int)lane] : -1;
+    int ent[kPerStep];
+#pragma unroll
+    for (int u = 0; u < kPerStep; ++u)
+      ent[u] = 32 * u + (int)lane < take ? Q.t.stk[sp - take + 32 * u + (int)lane] : -1;
     __syncwarp();
     sp -= take;
     if (lane == 0) ++cnt.steps;
-    int slot = 0;
-    int ch[4] = {0, 0, 0, 0};
-    unsigned hit = 0u;  // bit k: child k overlaps the window and the ray's cells
-    if (ent >= 0 && (int64_t)(ent >> 5) >= Wk.field(Q.r[ent & 31].asset).n_nodes4) {
-      set_err(Wk.err_field(), ERR_INDEX);  // a node beyond the tree: skipped
-    } else if (ent >= 0) {
-      const int node = ent >> 5;
-      slot = ent & 31;
-      const LaneRay& R = Q.r[slot];
+    int ch[4 * kPerStep];
+    unsigned hit = 0u;  // bit k: child k overlaps the window
+#pragma unroll
+    for (int k = 0; k < 4 * kPerStep; ++k) ch[k] = 0;
+#pragma unroll
+    for (int u = 0; u < kPerStep; ++u) {
+      if (u > 0 && take <= 32 * u) break;  // (the same in every lane)
+      if (ent[u] < 0) continue;
+      const LaneRay& R = Q.r[ent[u] & 31];
+      const DevField& F = Wk.field(R.asset);
+      if ((int64_t)(ent[u] >> 5) >= F.n_nodes4) {
+        set_err(Wk.err_field(), ERR_INDEX);  // a node beyond the tree: skipped
+        continue;
+      }
       const float3 o = make_float3(R.o[0], R.o[1], R.o[2]);
       const float3 inv = make_float3(R.inv[0], R.inv[1], R.inv[2]);
       ++cnt.nodes;
-      hit = node4_hits(Wk.field(R.asset).nodes4 + node, o, inv, R.ta, R.te, ch);
+      hit |= node4_hits(F.nodes4 + (ent[u] >> 5), o, inv, R.ta, R.te, ch + 4 * u) << (4 * u);
     }
     // ---------------- push internal children, queue leaves
-    if (!push_hits(Q.t.stk, kWStack, hit, ch, lane, sp, lq_n, [&](int c) { return (c << 5) | slot; }) &&
+    if (!push_hits(Q.t.stk, kWStack, hit, ch, lane, sp, lq_n,
+                   [&](int k, int c) { return (c << 5) | (ent[k >> 2] & 31); }) &&
         lane == 0)
       set_err(Wk.err_field(), ERR_STACK);
     __syncwarp();
@@ -562,7 +583,7 @@ struct ServerWork {
 // tracking windows of all 32 lanes advancing together through warp_phase.
 // Only the first `slots` lanes of a warp take paths: a launch with less work than lanes
 // spreads it over every warp of the grid (scatter_slots).
-template <class Work>
+template <int kPerStep, class Work>
 __device__ __forceinline__ void render_paths(const Work& Wk, const float* env, WarpQ& Q,
                                              ChordStore* wch, int slots) {
   const uint32_t lane = threadIdx.x & 31u;
@@ -678,7 +699,7 @@ __device__ __forceinline__ void render_paths(const Work& Wk, const float* env, W
       R.nch = 0;
       R.hmax = 0;
       __syncwarp();
-      warp_phase(Wk, Q, want, lane, env, wch, cnt);
+      warp_phase<kPerStep>(Wk, Q, want, lane, env, wch, cnt);
       // owner: a window whose points overflowed the slots is halved and redone;
       // otherwise its points are sorted by t for the decisions
       int n = 0;
@@ -770,6 +791,7 @@ __device__ __forceinline__ ChordStore* warp_store(float4* chord_store) {
   return reinterpret_cast<ChordStore*>(chord_store) + (size_t)blockIdx.x * kWWarps + (threadIdx.x >> 5);
 }
 
+template <int kPerStep>
 __global__ void __launch_bounds__(kWWarps * 32, kBlocksPerSM)
     k_render_scatter(const __grid_constant__ DevField F, const __grid_constant__ PathParams P,
                      unsigned long long* acc64, int* counter, int chunk, int slots,
@@ -777,7 +799,7 @@ __global__ void __launch_bounds__(kWWarps * 32, kBlocksPerSM)
   extern __shared__ __align__(16) unsigned char smraw[];
   WarpQ& Q = setup_block(smraw, F.env);
   const ImageWork Wk{&F, &P, acc64, counter, P.cam.W * P.cam.H, chunk, (P.spp + chunk - 1) / chunk};
-  render_paths(Wk, reinterpret_cast<const float*>(smraw), Q, warp_store(chord_store), slots);
+  render_paths<kPerStep>(Wk, reinterpret_cast<const float*>(smraw), Q, warp_store(chord_store), slots);
 }
 
 __global__ void k_fix_to_image(const unsigned long long* acc64, int64_t npix, int spp, float* out) {
@@ -785,12 +807,13 @@ __global__ void k_fix_to_image(const unsigned long long* acc64, int64_t npix, in
   if (i < npix) out[i] = fix_mean((long long)acc64[i], spp);
 }
 
+template <int kPerStep>
 __global__ void __launch_bounds__(kWWarps * 32, kBlocksPerSM)
     k_render_server(const __grid_constant__ ServerLaunch L, int slots, float4* chord_store) {
   extern __shared__ __align__(16) unsigned char smraw[];
   WarpQ& Q = setup_block(smraw, L.fields[0].env);
   const ServerWork Wk{&L};
-  render_paths(Wk, reinterpret_cast<const float*>(smraw), Q, warp_store(chord_store), slots);
+  render_paths<kPerStep>(Wk, reinterpret_cast<const float*>(smraw), Q, warp_store(chord_store), slots);
 }
 
 size_t scatter_smem_bytes() { return 64 + sizeof(WarpQ) * kWWarps; }
@@ -816,6 +839,15 @@ static cudaError_t scatter_grid(K kernel, int sm_count, int64_t& g) {
   return cudaSuccess;
 }
 
+// the grid that both variants of a kernel fit
+static cudaError_t render_grid(int sm_count, int64_t& g) {
+  int64_t h = 1;
+  cudaError_t e = scatter_grid(k_render_scatter<1>, sm_count, g);
+  if (e == cudaSuccess) e = scatter_grid(k_render_scatter<2>, sm_count, h);
+  g = std::min(g, h);
+  return e;
+}
+
 // Paths per warp for `units` units of work, and the grid that holds them (g: the full
 // grid on entry).  With fewer units than lanes every warp of the grid takes its share
 // instead of a few warps taking 32 paths each: a warp works through its paths' windows
@@ -834,7 +866,7 @@ static int scatter_slots(int64_t units, int64_t& g) {
 // grid (shared with the analytic flights' lists), grown through the field's allocator
 cudaError_t ensure_render_scratch(const Field& F, int64_t npix, cudaStream_t s) {
   int64_t g = 1;
-  cudaError_t e = scatter_grid(k_render_scatter, F.ctx.sm_count, g);
+  cudaError_t e = render_grid(F.ctx.sm_count, g);
   if (e != cudaSuccess) return e;
   if ((e = grow(F, (void**)&F.acc64, F.acc_bytes, (size_t)npix * 8, s)) != cudaSuccess) return e;
   return grow(F, (void**)&F.wscratch, F.wscratch_bytes,
@@ -847,7 +879,7 @@ cudaError_t launch_render_scatter(const Field& F, const PathParams& P, float* ou
   if (e != cudaSuccess) return e;
   const int64_t npix = (int64_t)P.cam.W * P.cam.H;
   int64_t g = 1;
-  if ((e = scatter_grid(k_render_scatter, F.ctx.sm_count, g)) != cudaSuccess) return e;
+  if ((e = render_grid(F.ctx.sm_count, g)) != cudaSuccess) return e;
   // about 16 units per lane: chunk = ceil(npix spp / (16 lanes)), in [1, spp]
   const int64_t lanes = g * kWWarps * 32;
   int64_t chunk = (npix * P.spp + 16 * lanes - 1) / (16 * lanes);
@@ -858,8 +890,9 @@ cudaError_t launch_render_scatter(const Field& F, const PathParams& P, float* ou
   if ((e = ensure_render_scratch(F, npix, s)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(F.acc64, 0, (size_t)npix * 8, s)) != cudaSuccess) return e;
   const int slots = scatter_slots(npix * nchunk, g);
-  k_render_scatter<<<(unsigned)g, kWWarps * 32, scatter_smem_bytes(), s>>>(
-      F.dev, P, F.acc64, F.counter, (int)chunk, slots, F.wscratch);
+  auto kernel = nodes_per_step(P.lod, P.lod_nee) == 2 ? k_render_scatter<2> : k_render_scatter<1>;
+  kernel<<<(unsigned)g, kWWarps * 32, scatter_smem_bytes(), s>>>(F.dev, P, F.acc64, F.counter, (int)chunk,
+                                                                 slots, F.wscratch);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_fix_to_image<<<(unsigned)((npix + 255) / 256), 256, 0, s>>>(F.acc64, npix, P.spp, out);
   return cudaGetLastError();
@@ -867,7 +900,11 @@ cudaError_t launch_render_scatter(const Field& F, const PathParams& P, float* ou
 
 cudaError_t server_grid(int sm_count, int64_t& g) {
   (void)cudaGetLastError();
-  return scatter_grid(k_render_server, sm_count, g);
+  int64_t h = 1;
+  cudaError_t e = scatter_grid(k_render_server<1>, sm_count, g);
+  if (e == cudaSuccess) e = scatter_grid(k_render_server<2>, sm_count, h);
+  g = std::min(g, h);
+  return e;
 }
 
 cudaError_t launch_fix_to_image(const unsigned long long* acc, int64_t npix, int spp, float* out,
@@ -876,11 +913,15 @@ cudaError_t launch_fix_to_image(const unsigned long long* acc, int64_t npix, int
   return cudaGetLastError();
 }
 
-cudaError_t launch_render_server(const ServerLaunch& L, int64_t grid, float4* chord_store,
-                                 cudaStream_t s) {
+cudaError_t launch_render_server(const ServerLaunch& L, const ServerReqDev* reqs, int64_t grid,
+                                 float4* chord_store, cudaStream_t s) {
   (void)cudaGetLastError();
   const int slots = scatter_slots(L.total, grid);
-  k_render_server<<<(unsigned)grid, kWWarps * 32, scatter_smem_bytes(), s>>>(L, slots, chord_store);
+  // two nodes per step when every request of the batch gains by it
+  bool two = true;
+  for (int i = 0; i < L.n_items; ++i) two = two && nodes_per_step(reqs[i].P.lod, reqs[i].P.lod_nee) == 2;
+  auto kernel = two ? k_render_server<2> : k_render_server<1>;
+  kernel<<<(unsigned)grid, kWWarps * 32, scatter_smem_bytes(), s>>>(L, slots, chord_store);
   return cudaGetLastError();
 }
 
