@@ -150,20 +150,43 @@ __global__ void k_pack(const __grid_constant__ PackArgs A) {
   A.labels[2 * A.p.n + i] = (uint8_t)cell;
   // largest |k_W| and largest world carrier |omega| per band (the per-cell sums
   // follow in k_cell_sums, on the scale the first one sets)
-  atomicMax(&A.cell_acc->kw_max, __float_as_uint(kn));
-  atomicMax(&A.cell_acc->band_wmax[band],
-            __float_as_uint(sqrtf(om[0] * om[0] + om[1] * om[1] + om[2] * om[2])));
+  // one atomic per warp (and band): 200k atomics on one word took most of this kernel's
+  // 78 us
+  const unsigned am = __activemask();
+  const int me = (int)(threadIdx.x & 31u);
+  const unsigned km = __reduce_max_sync(am, __float_as_uint(kn));
+  if (me == __ffs((int)am) - 1) atomicMax(&A.cell_acc->kw_max, km);
+  const unsigned same = __match_any_sync(am, band);
+  const unsigned wm = __reduce_max_sync(
+      same, __float_as_uint(sqrtf(om[0] * om[0] + om[1] * om[1] + om[2] * om[2])));
+  if (me == __ffs((int)same) - 1) atomicMax(&A.cell_acc->band_wmax[band], wm);
 }
 
-// per cell: the sum of |k_W| in exact fixed point and the member count
-__global__ void k_cell_sums(const float* kw, const uint8_t* cell, int64_t n, CellAcc* acc) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// per cell: the sum of |k_W| in exact fixed point and the member count.  A block sums
+// kCellBlock kernels in shared memory first, each term (at most 2^36) as a low and a high
+// part of 18 bits (400k 64-bit atomics on a few dozen words took 50 to 98 us).
+constexpr int kCellBlock = 1024;
+__global__ void __launch_bounds__(256) k_cell_sums(const float* kw, const uint8_t* cell, int64_t n,
+                                                   CellAcc* acc) {
+  __shared__ unsigned lo[64], hi[64], cnt[64];
+  if (threadIdx.x < 64) lo[threadIdx.x] = hi[threadIdx.x] = cnt[threadIdx.x] = 0u;
+  __syncthreads();
   const int e = cell_fix_exp(acc->kw_max);
   const float sc = __int_as_float((127 + 36 - e) << 23);  // 2^(36 - e)
-  const unsigned c = cell[i] & 63u;
-  atomicAdd(&acc->kw_fix[c], (unsigned long long)__float2ull_rn(kw[i] * sc));
-  atomicAdd(&acc->count[c], 1ull);
+  const int64_t i0 = (int64_t)blockIdx.x * kCellBlock;
+  for (int k = (int)threadIdx.x; k < kCellBlock && i0 + k < n; k += 256) {
+    const unsigned c = cell[i0 + k] & 63u;
+    const unsigned long long v = (unsigned long long)__float2ull_rn(kw[i0 + k] * sc);
+    atomicAdd(&lo[c], (unsigned)(v & 0x3FFFFull));
+    atomicAdd(&hi[c], (unsigned)(v >> 18));
+    atomicAdd(&cnt[c], 1u);
+  }
+  __syncthreads();
+  if (threadIdx.x < 64 && cnt[threadIdx.x]) {
+    const unsigned c = threadIdx.x;
+    atomicAdd(&acc->kw_fix[c], ((unsigned long long)hi[c] << 18) + lo[c]);
+    atomicAdd(&acc->count[c], (unsigned long long)cnt[c]);
+  }
 }
 
 cudaError_t launch_pack(Field& F, const gf_params& P, cudaStream_t s) {
@@ -186,7 +209,8 @@ cudaError_t launch_pack(Field& F, const gf_params& P, cudaStream_t s) {
   A.err = F.err;
   int64_t blocks = (P.n + 127) / 128;
   k_pack<<<(unsigned)blocks, 128, 0, s>>>(A);
-  k_cell_sums<<<(unsigned)((P.n + 255) / 256), 256, 0, s>>>(A.kw, A.labels + 2 * P.n, P.n, A.cell_acc);
+  k_cell_sums<<<(unsigned)((P.n + kCellBlock - 1) / kCellBlock), 256, 0, s>>>(A.kw, A.labels + 2 * P.n,
+                                                                             P.n, A.cell_acc);
   return cudaGetLastError();
 }
 
@@ -217,17 +241,22 @@ __global__ void k_bounds(const float* box, const float4* rec, int64_t n, unsigne
       v[9 + j] = fmaxf(v[9 + j], m[j]);
     }
   }
+  // warp, block, then one atomic per block and bound
+  __shared__ unsigned int part[12][8];
   for (int j = 0; j < 12; ++j) {
-    float x = v[j];
-    bool mn = (j < 3) || (j >= 6 && j < 9);
-    for (int o = 16; o > 0; o >>= 1) {
-      float y = __shfl_xor_sync(kFull, x, o);
-      x = mn ? fminf(x, y) : fmaxf(x, y);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      if (mn) atomicMin(bounds + j, ord_enc(x));
-      else atomicMax(bounds + j, ord_enc(x));
-    }
+    const bool mn = (j < 3) || (j >= 6 && j < 9);
+    const unsigned x = ord_enc(v[j]);
+    const unsigned r = mn ? __reduce_min_sync(kFull, x) : __reduce_max_sync(kFull, x);
+    if ((threadIdx.x & 31) == 0) part[j][threadIdx.x >> 5] = r;
+  }
+  __syncthreads();
+  if (threadIdx.x < 12) {
+    const int j = (int)threadIdx.x;
+    const bool mn = (j < 3) || (j >= 6 && j < 9);
+    unsigned r = part[j][0];
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = mn ? min(r, part[j][w]) : max(r, part[j][w]);
+    if (mn) atomicMin(bounds + j, r);
+    else atomicMax(bounds + j, r);
   }
 }
 
@@ -240,9 +269,11 @@ __device__ __forceinline__ unsigned int spread10(unsigned int x) {
   return x;
 }
 
-// sort keys: the cell (or, by_band, its band) above 30 Morton bits of the mean
+// sort keys of both trees: the cell, or its band, above 30 Morton bits of the mean; the
+// second tree's n entries follow the first's, with bit 36 set, so that one sort orders
+// both
 __device__ __forceinline__ uint32_t cell_band(uint32_t cell) { return cell == 0 ? 0u : ((cell - 1u) >> 3) + 1u; }
-__global__ void k_morton(const float4* rec, int64_t n, const unsigned int* bounds, bool by_band,
+__global__ void k_morton(const float4* rec, int64_t n, const unsigned int* bounds,
                          unsigned long long* keys, int* idx) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -262,13 +293,15 @@ __global__ void k_morton(const float4* rec, int64_t n, const unsigned int* bound
     c[j] = (unsigned int)fminf(u * 1024.f, 1023.f);
   }
   unsigned int mc = (spread10(c[0]) << 2) | (spread10(c[1]) << 1) | spread10(c[2]);
-  keys[i] = ((unsigned long long)(by_band ? cell_band(cell) : cell) << 30) | mc;
+  keys[i] = ((unsigned long long)cell << 30) | mc;
+  keys[n + i] = 1ull << 36 | ((unsigned long long)cell_band(cell) << 30) | mc;
   idx[i] = (int)i;
+  idx[n + i] = (int)i;
 }
 
 __global__ void k_gather(const float4* rec_in, const float* box_in, const float* ext2_in,
                          const int* idx, int64_t n, float4* rec_out, float* box_out,
-                         float* ext2_out, float4* muw_out, int* sorted_orig) {
+                         float* ext2_out, float4* muw_out, int* sorted_orig, int* pos) {
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   int i = idx[j];
@@ -281,7 +314,30 @@ __global__ void k_gather(const float4* rec_in, const float* box_in, const float*
                                         __fmul_rn(r3.z, r3.z)));
   muw_out[j] = make_float4(r0.x, r0.y, r0.z, wn);
   sorted_orig[j] = i;
+  pos[i] = (int)j;
 }
+
+// leaves of the tree by bands: the sorted primitive of each
+__global__ void k_band_leaves(const int* idx, const int* pos, int64_t n, int* of) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p < n) of[p] = pos[idx[n + p]];
+}
+
+// One of the two binary trees in the making (by cells, by bands).  The kernels below
+// build both in one launch (blockIdx.y): each is bound by the latency of its chains, not
+// by its size.
+struct TreeBuild {
+  const unsigned long long* keys;
+  Node* nodes;
+  int* above;               // node above each leaf
+  int* flags;               // refit counters, then marks of four-wide nodes
+  const int* of;            // sorted primitive of each leaf (null: the leaf itself)
+  unsigned int* max_depth;
+  bool band;
+};
+struct TreePair {
+  TreeBuild t[2];
+};
 
 // camera LoD selection (Supp. A): primitive j stays in the mixture iff
 // |omega| d <= c, d the distance from the eye to its mean, c = pi H / (2 tan(phi/2))
@@ -326,7 +382,10 @@ __device__ __forceinline__ int delta_key(const unsigned long long* k, int64_t n,
 }
 
 // Karras (HPG 2012): internal node i covers [min(i,j), max(i,j)], split at gamma
-__global__ void k_karras(const unsigned long long* keys, int64_t n, Node* nodes, int* leaf_parent) {
+__global__ void k_karras(const __grid_constant__ TreePair T, int64_t n) {
+  const unsigned long long* keys = T.t[blockIdx.y].keys;
+  Node* nodes = T.t[blockIdx.y].nodes;
+  int* leaf_parent = T.t[blockIdx.y].above;
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n - 1) return;
   int d = (delta_key(keys, n, i, i + 1) - delta_key(keys, n, i, i - 1)) >= 0 ? 1 : -1;
@@ -370,8 +429,14 @@ __device__ __forceinline__ void write_slot(Node* nd, int slot, const float* b, u
 // bottom-up refit: the second child to arrive at a node merges both slots.  Leaf j of
 // the tree is the sorted primitive of[j] (j itself without of); masks hold cells, or
 // bands when by_band.
-__global__ void k_refit(const float* box, const float4* rec, const int* of, bool by_band, int64_t n,
-                        Node* nodes, const int* leaf_parent, int* flags) {
+__global__ void k_refit(const float* box, const float4* rec, const __grid_constant__ TreePair T,
+                        int64_t n) {
+  const TreeBuild& B = T.t[blockIdx.y];
+  const int* of = B.of;
+  const bool by_band = B.band;
+  Node* nodes = B.nodes;
+  const int* leaf_parent = B.above;
+  int* flags = B.flags;
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   const int64_t pj = of ? of[j] : j;
@@ -410,7 +475,10 @@ __device__ __forceinline__ unsigned long long node_mask(const Node& N) {
 }
 __device__ __forceinline__ bool one_class(unsigned long long m) { return (m & (m - 1ull)) == 0ull; }
 
-__global__ void k_depth_parity(const Node* nodes, int64_t m, int* even, unsigned int* max_depth) {
+__global__ void k_depth_parity(const __grid_constant__ TreePair T, int64_t m) {
+  const Node* nodes = T.t[blockIdx.y].nodes;
+  int* even = T.t[blockIdx.y].flags;
+  unsigned int* max_depth = T.t[blockIdx.y].max_depth;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m) return;
   int d = 0, dc = 0;  // depth, depth below the class's root
@@ -481,17 +549,21 @@ __device__ __forceinline__ Node4 emit_node4(int nc, const float box[4][6], const
   return o;
 }
 
-// out[base + map[i]]: Node4 of the marked binary node i; out[base + m4 + class]: the
-// root of a class with one primitive.  roots[class] receives the class's root.
+// out[base + map[i]]: Node4 of the marked binary node i; out[single + class]: the root of
+// a class with one primitive.  roots[class] receives the class's root.
 struct CollapseArgs {
   const Node* nodes;
   int64_t m;
   const int *even, *map, *of;
   Node4* out;
-  int base, m4;
+  int base, single;  // out index of map 0, and of class 0's one-primitive root
   int* roots;
 };
-__global__ void k_collapse4(const CollapseArgs A) {
+struct CollapsePair {
+  CollapseArgs a[2];
+};
+__global__ void k_collapse4(const __grid_constant__ CollapsePair C2) {
+  const CollapseArgs& A = C2.a[blockIdx.y];
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.m) return;
   auto leaf = [&](int c) { return A.of ? ~A.of[~c] : c; };
@@ -506,7 +578,7 @@ __global__ void k_collapse4(const CollapseArgs A) {
       int c;
       node_slot(N, s, box[0], mm, c);
       if (c >= 0) continue;
-      const int cls = __ffsll((long long)mm) - 1, at = A.base + A.m4 + cls;
+      const int cls = __ffsll((long long)mm) - 1, at = A.single + cls;
       ch[0] = leaf(c);
       A.out[at] = emit_node4(1, box, ch);
       A.roots[cls] = at;
@@ -570,8 +642,8 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
   unsigned int* bounds = nullptr;  // boxes (12), the two trees' depths
   int* roots = nullptr;            // of cells, then of bands
   unsigned long long *keys = nullptr, *keys2 = nullptr;
-  int *idx = nullptr, *idx2 = nullptr, *leaf_parent = nullptr, *flags = nullptr, *leaf_parent_b = nullptr,
-      *flags_b = nullptr;
+  int *idx = nullptr, *idx2 = nullptr, *above = nullptr, *above_b = nullptr, *flags = nullptr, *map = nullptr,
+      *pos = nullptr, *of = nullptr;
   float* box_sorted = nullptr;
   Node* nodes_b = nullptr;  // binary tree by bands
   void *tmp = nullptr, *block = nullptr;
@@ -581,8 +653,8 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
   unsigned int hb[14];
   int hroots[kMaxCells + 8];
 #define GF_TRY(x) do { e = (x); if (e != cudaSuccess) goto done; } while (0)
-  GF_TRY(cub::DeviceRadixSort::SortPairs(nullptr, sort_bytes, keys, keys2, idx, idx2, (int)n, 0, 36, s));
-  GF_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tmp_bytes, flags, leaf_parent, (int)n, s));
+  GF_TRY(cub::DeviceRadixSort::SortPairs(nullptr, sort_bytes, keys, keys2, idx, idx2, (int)(2 * n), 0, 37, s));
+  GF_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tmp_bytes, flags, map, (int)(2 * n), s));
   if (sort_bytes > tmp_bytes) tmp_bytes = sort_bytes;
   for (int pass = 0; pass < 2; ++pass) {  // sizes, then places
     uintptr_t at = reinterpret_cast<uintptr_t>(block);
@@ -593,14 +665,16 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
     char* tp = nullptr;
     take(bounds, sizeof(hb));
     take(roots, sizeof(hroots));
-    take(keys, n * sizeof(unsigned long long));
-    take(keys2, n * sizeof(unsigned long long));
-    take(idx, n * sizeof(int));
-    take(idx2, n * sizeof(int));
-    take(leaf_parent, n * sizeof(int));
-    take(flags, n * sizeof(int));
-    take(leaf_parent_b, n * sizeof(int));
-    take(flags_b, n * sizeof(int));
+    take(keys, 2 * n * sizeof(unsigned long long));
+    take(keys2, 2 * n * sizeof(unsigned long long));
+    take(idx, 2 * n * sizeof(int));
+    take(idx2, 2 * n * sizeof(int));
+    take(above, n * sizeof(int));
+    take(above_b, n * sizeof(int));
+    take(flags, 2 * n * sizeof(int));  // marks of both trees, m each
+    take(map, 2 * n * sizeof(int));    // their scan
+    take(pos, n * sizeof(int));
+    take(of, n * sizeof(int));
     take(box_sorted, n * 6 * sizeof(float));
     take(nodes_b, n * sizeof(Node));
     take(tp, tmp_bytes);
@@ -618,8 +692,7 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
     GF_TRY(cudaMemcpyAsync(bounds, init, sizeof(init), cudaMemcpyHostToDevice, s));
   }
   {
-    int blocks = (int)((n + 255) / 256);
-    if (blocks > 4096) blocks = 4096;
+    const int blocks = (int)std::min<int64_t>((n + 255) / 256, 2 * F.ctx.sm_count);
     k_bounds<<<blocks, 256, 0, s>>>(F.box_orig, F.rec_orig, n, bounds);
     GF_TRY(cudaGetLastError());
     if (F.opts.precision != GF_PREC_FP32) {
@@ -632,54 +705,51 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
       k_bounds<<<blocks, 256, 0, s>>>(F.box_orig, F.rec_orig, n, bounds);
       GF_TRY(cudaGetLastError());
     }
-    k_morton<<<pn, 256, 0, s>>>(F.rec_orig, n, bounds, false, keys, idx);
+    k_morton<<<pn, 256, 0, s>>>(F.rec_orig, n, bounds, keys, idx);
     GF_TRY(cudaGetLastError());
   }
-  GF_TRY(cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, keys, keys2, idx, idx2, (int)n, 0, 36, s));
+  GF_TRY(cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, keys, keys2, idx, idx2, (int)(2 * n), 0, 37, s));
   k_gather<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(F.rec_orig, F.box_orig, F.ext2_orig, idx2,
                                                       n, F.rec, box_sorted, F.ext2, F.muw,
-                                                      F.sorted_orig);
+                                                      F.sorted_orig, pos);
   GF_TRY(cudaGetLastError());
   {
-    // the binary trees by cells (kept) and by bands, each with its boxes, the marks of its
-    // four-wide nodes (flags, then their scan in leaf_parent)
-    int last[4] = {0, 0, 0, 0};
-    for (int t = 0; t < 2 && n >= 2; ++t) {
-      const bool band = t == 1;
-      Node* nd = band ? nodes_b : F.nodes;
-      int *lp = band ? leaf_parent_b : leaf_parent, *fl = band ? flags_b : flags;
-      const int* of = band ? idx2 : nullptr;
-      if (band) {
-        k_morton<<<pn, 256, 0, s>>>(F.rec, n, bounds, true, keys, idx);
-        GF_TRY(cudaGetLastError());
-        GF_TRY(cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, keys, keys2, idx, idx2, (int)n, 0, 33, s));
-      }
-      GF_TRY(cudaMemsetAsync(nd, 0, m * sizeof(Node), s));
-      GF_TRY(cudaMemsetAsync(fl, 0, n * sizeof(int), s));
-      k_karras<<<pm, 256, 0, s>>>(keys2, n, nd, lp);
+    // the binary trees by cells (kept) and by bands with their boxes, the marks of their
+    // four-wide nodes (flags) and the marks' scan (map)
+    int last[3] = {0, 0, 0};  // marks before the second tree's; of the last node, scan and mark
+    const dim3 gn(pn, 2), gm(pm, 2);
+    if (n >= 2) {
+      k_band_leaves<<<pn, 256, 0, s>>>(idx2, pos, n, of);
       GF_TRY(cudaGetLastError());
-      k_refit<<<pn, 256, 0, s>>>(box_sorted, F.rec, of, band, n, nd, lp, fl);
+      const TreePair T{{{keys2, F.nodes, above, flags, nullptr, bounds + 12, false},
+                        {keys2 + n, nodes_b, above_b, flags + m, of, bounds + 13, true}}};
+      GF_TRY(cudaMemsetAsync(flags, 0, 2 * m * sizeof(int), s));
+      k_karras<<<gm, 256, 0, s>>>(T, n);
       GF_TRY(cudaGetLastError());
-      k_depth_parity<<<pm, 256, 0, s>>>(nd, m, fl, bounds + 12 + t);
+      k_refit<<<gn, 256, 0, s>>>(box_sorted, F.rec, T, n);
       GF_TRY(cudaGetLastError());
-      GF_TRY(cub::DeviceScan::ExclusiveSum(tmp, tmp_bytes, fl, lp, (int)m, s));
-      GF_TRY(cudaMemcpyAsync(&last[2 * t], lp + (m - 1), sizeof(int), cudaMemcpyDeviceToHost, s));
-      GF_TRY(cudaMemcpyAsync(&last[2 * t + 1], fl + (m - 1), sizeof(int), cudaMemcpyDeviceToHost, s));
+      k_depth_parity<<<gm, 256, 0, s>>>(T, m);
+      GF_TRY(cudaGetLastError());
+      GF_TRY(cub::DeviceScan::ExclusiveSum(tmp, tmp_bytes, flags, map, (int)(2 * m), s));
+      GF_TRY(cudaMemcpyAsync(&last[0], map + m, sizeof(int), cudaMemcpyDeviceToHost, s));
+      GF_TRY(cudaMemcpyAsync(&last[1], map + 2 * m - 1, sizeof(int), cudaMemcpyDeviceToHost, s));
+      GF_TRY(cudaMemcpyAsync(&last[2], flags + 2 * m - 1, sizeof(int), cudaMemcpyDeviceToHost, s));
     }
     GF_TRY(cudaStreamSynchronize(s));
-    const int ma = last[0] + last[1], mb = last[2] + last[3];
-    const int base_b = ma + kMaxCells;
-    F.n_nodes4 = (int64_t)base_b + mb + 8;
+    // nodes4: the cells' trees, the cells' one-primitive roots, then the same of the bands
+    const int ma = last[0], mb = last[1] + last[2] - last[0];
+    const int single_b = ma + kMaxCells + mb;
+    F.n_nodes4 = (int64_t)single_b + 8;
     F.mem.release(F.nodes4, s);  // a rebuild (the stream was synchronised above)
     F.nodes4 = nullptr;
     GF_TRY(F.mem.alloc((void**)&F.nodes4, (size_t)F.n_nodes4 * sizeof(Node4), s));
     if (n >= 2) {
-      k_collapse4<<<pm, 256, 0, s>>>(CollapseArgs{F.nodes, m, flags, leaf_parent, nullptr, F.nodes4, 0, ma, roots});
-      k_collapse4<<<pm, 256, 0, s>>>(
-          CollapseArgs{nodes_b, m, flags_b, leaf_parent_b, idx2, F.nodes4, base_b, mb, roots + kMaxCells});
+      k_collapse4<<<gm, 256, 0, s>>>(
+          CollapsePair{{{F.nodes, m, flags, map, nullptr, F.nodes4, 0, ma, roots},
+                        {nodes_b, m, flags + m, map + m, of, F.nodes4, kMaxCells, single_b, roots + kMaxCells}}});
     } else {
       k_single4<<<1, 1, 0, s>>>(box_sorted, F.rec, false, F.nodes4, 0, roots);
-      k_single4<<<1, 1, 0, s>>>(box_sorted, F.rec, true, F.nodes4, base_b, roots + kMaxCells);
+      k_single4<<<1, 1, 0, s>>>(box_sorted, F.rec, true, F.nodes4, single_b, roots + kMaxCells);
     }
     GF_TRY(cudaGetLastError());
   }
