@@ -182,7 +182,7 @@ enum { GF_INTEG_TOMO = 0, GF_INTEG_SCATTER = 1 };
    segment-based transfer; Sec. 4.4 distance sampling), by 32 bisections on the
    closed-form optical depth (see GF_TR_CLOSED_FORM), and the NEE transmittance
    is exp(-tau) in closed form; it assumes a non-negative mixture along each
-   ray (the first crossing) and is rendered per thread.
+   ray (the first crossing).
    SEGMENT: the cheap approximation of CDF (Sec. 3: uniform sampling within
    segments): the ray is cut into segments at t = 0 and every chord entry and
    exit, and the collision is drawn uniformly (second uniform of the stream)
@@ -270,9 +270,9 @@ gf_status gf_load_field(gf_ctx* ctx, const gf_params* params, const gf_field_opt
 gf_status gf_field_free(gf_field* field);
 
 /* Build the BVH over the k-sigma ellipsoid bounds (Sec. 3; the per-level
-   acceleration structures of Sec. 4.6 become one radix tree whose top levels
-   split by cell, every node carrying the 64-bit OR of its cells).
-   Reorders the packed records along the tree.  GF_EOVERFLOW if the tree is
+   acceleration structures of Sec. 4.6: one tree per cell and one per band, of
+   which a ray starts in those that its mask selects).
+   Reorders the packed records along the trees by cell.  GF_EOVERFLOW if the tree is
    deeper than the per-thread traversal stack (64 levels; clustered inputs
    whose keys share long prefixes); the field then stays unbuilt. */
 gf_status gf_build_bvh(gf_field* field, gf_stream stream);
@@ -283,7 +283,7 @@ gf_status gf_build_bvh(gf_field* field, gf_stream stream);
    chords each for gf_ray_chords), max_pixels pixels of gf_render (the pixel
    sums of the scattering renderer and the staging of a host image), and
    the per-warp chord store of the scattering renderer when render != 0, and
-   the per-thread lists of the radiance adjoint when adjoint != 0.  Sizes only
+   the adjoints' chord lists when adjoint != 0.  Sizes only
    grow; zeros leave a part as it is.  GF_ESTATE before gf_build_bvh. */
 typedef struct gf_reserve_opts {
   int64_t max_rays;
@@ -349,7 +349,8 @@ gf_status gf_render(gf_field* field, const gf_camera* camera, const gf_render_op
 /* Adjoint of a rendered image: given dL/dI (float[W*H]), write dL/dparam to
    grad (float[15 N], SoA like gf_params: mu[3N], quat[4N], log_scale[3N],
    omega[3N] in the input frame, phase[N], weight[N]); grad is overwritten.
-   Nothing per path is stored: every ray is re-traced.  FP32 records only.
+   Nothing is kept from the forward render: every ray is re-traced.  FP32 records
+   only.
    TOMO (all cells): dtau/dtheta = integral of d(integrand)/dtheta plus the
    Leibniz terms of the chord ends on the ellipsoid (Eq. 2-3).
    SCATTER with max_bounces = 1 (LoD masks as set by gf_set_lod_mask): per
@@ -362,7 +363,7 @@ gf_status gf_render(gf_field* field, const gf_camera* camera, const gf_render_op
    is unbiased for the derivative of the expected image (the derivative of
    the k-sigma cut itself is not included).
    SCATTER with max_bounces >= 2: the renderer's delta-tracking path (same
-   streams and decisions) is followed twice.  Segment b's accepted point has
+   streams and decisions) is followed.  Segment b's accepted point has
    probability prod_{i<js}(1 - p_i) p_js, collision b adds C_b = albedo^(b+1)
    E/(4 pi) T_b (T_b the ratio-tracked NEE product); the gradient is that of
    sum_b S_b log P_b + sum_b C_b log T_b with S_b = sum_{b' >= b} C_b', the

@@ -1,4 +1,5 @@
-// gf_adjoint.cu -- hand-written adjoint of the tomography renderer.
+// gf_adjoint.cu -- hand-written adjoints of the tomography renderer and (further below)
+// of the scattering renderer.
 //
 // Image I_p = (1/spp) sum_s exp(-tau_s) (Sec. 4.6 tomography), tau_s the
 // optical depth of Eq. 2-3 along the jittered camera ray.  Given dL/dI:
@@ -6,9 +7,10 @@
 //   dtau/dtheta = int_chord d(integrand)/dtheta dt
 //               + g(t_out) dt_out/dtheta - g(t_in) dt_in/dtheta,
 // with the ellipsoid ends moving as dt/dtheta = -(dq/dtheta)/(dq/dt)
-// (Leibniz rule for the k-sigma-truncated kernel).  Each ray is traversed
-// twice (forward optical depth, then the adjoint pass): nothing is stored
-// per path.  Gradients are accumulated with atomics in SoA layout.
+// (Leibniz rule for the k-sigma-truncated kernel).  A ray is traversed
+// once: its chords' moments are kept until its optical depth is known.  Gradients are
+// summed by vector atomics, 16 floats per primitive in BVH order, and copied to the
+// caller's layout at the end.
 #include <cuda_runtime.h>
 
 #include <algorithm>

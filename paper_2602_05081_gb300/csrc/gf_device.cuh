@@ -29,7 +29,8 @@ enum : int {
   ERR_STACK = 1, ERR_WINDOW = 2, ERR_POINTS = 4, ERR_GUARD = 8, ERR_INPUT = 16, ERR_INDEX = 32
 };
 
-// Binary BVH node holding the boxes, children and cell masks of both children
+// Binary BVH node of the tree by cells (the radiance adjoints and the walks of one
+// lane, traverse_ray), holding the boxes, children and cell masks of both children
 // (one 80-byte fetch tests two boxes).  child >= 0: internal node; child < 0:
 // leaf of the sorted primitive ~child.
 struct __align__(16) Node {
@@ -212,18 +213,8 @@ __device__ __forceinline__ void ldg32(const void* p, float4& a, float4& b) {
 }
 
 // ---------------------------------------------------------------------------
-// warp helpers
+// compensated sums
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float warp_sum(float x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-  return x;
-}
-__device__ __forceinline__ long long warp_sum_ll(long long x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-  return x;
-}
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
   float bb = __fsub_rn(s, a);
@@ -237,18 +228,6 @@ __device__ __forceinline__ void neumaier_add(float& s, float& c, float x) {
   else
     c = __fadd_rn(c, __fadd_rn(__fsub_rn(x, t), s));
   s = t;
-}
-// compensated warp sum of (s + c) pairs; every lane receives the total
-__device__ __forceinline__ float warp_sum_comp(float s, float c) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    float so = __shfl_xor_sync(kFull, s, o), co = __shfl_xor_sync(kFull, c, o);
-    float t, e;
-    two_sum(s, so, t, e);
-    s = t;
-    c = __fadd_rn(__fadd_rn(c, co), e);
-  }
-  return __fadd_rn(s, c);
 }
 
 // ---------------------------------------------------------------------------
@@ -469,17 +448,6 @@ __device__ __forceinline__ bool prim_chord(const DevField& F, int j, float3 o, f
   return chord_setup16(F, r0, r1, j, o, v, tmin, tmax, ch);
 }
 
-// ray-box slab test over [t0, t1]
-__device__ __forceinline__ bool slab(float3 o, float3 inv, float lx, float ly, float lz, float hx,
-                                     float hy, float hz, float t0, float t1) {
-  float tx0 = (lx - o.x) * inv.x, tx1 = (hx - o.x) * inv.x;
-  float ty0 = (ly - o.y) * inv.y, ty1 = (hy - o.y) * inv.y;
-  float tz0 = (lz - o.z) * inv.z, tz1 = (hz - o.z) * inv.z;
-  float tn = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), t0));
-  float tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fminf(fmaxf(tz0, tz1), t1));
-  return tn <= tf;
-}
-
 // Unit direction of a caller's ray, d / |d| rounded once to FP32 (FP32
 // arithmetic only).  The argument is scaled by a power of two (exact), |d|^2
 // is formed as an unevaluated sum hi + lo of error-free products and sums,
@@ -541,8 +509,9 @@ __device__ __forceinline__ bool scene_span(const DevField& F, float3 o, float3 i
 __device__ __forceinline__ void set_err(const DevField& F, int code) { atomicOr(F.err, code); }
 
 // ---------------------------------------------------------------------------
-// Per-thread traversal of one ray under a cell mask: every lane of a warp owns
-// its own ray, so a warp advances 32 independent rays per step.  One 80-byte
+// Per-thread traversal of one ray under a cell mask, for what the traversals of a
+// whole warp leave over (windows with more chords or points than their buffers hold)
+// and for the chord lists of gf_ray_chords.  One 80-byte
 // fetch gives both child boxes of a node; test(tn, tf) decides whether a child
 // whose box spans [tn, tf] along the ray can matter (the test may tighten as
 // the traversal proceeds); hit leaves go to leaf(j) at once; the nearer

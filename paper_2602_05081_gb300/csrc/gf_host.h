@@ -127,7 +127,7 @@ struct Field {
   float4* rec = nullptr;        // FP32 records in BVH order
   uint4* rec16 = nullptr;       // reduced-precision records in BVH order
   Node* nodes = nullptr;
-  Node4* nodes4 = nullptr;      // four-wide collapse (built by gf_build_bvh)
+  Node4* nodes4 = nullptr;      // four-wide trees by cells, then by bands (gf_build_bvh)
   int* sorted_orig = nullptr;   // BVH position -> original index
   uint8_t* labels = nullptr;    // band, cone, cell per primitive (3N, original order)
   int* err = nullptr;
@@ -151,8 +151,8 @@ struct Field {
   // fixed-point pixel sums of the scattering renderer (grows on demand)
   mutable unsigned long long* acc64 = nullptr;
   mutable size_t acc_bytes = 0;
-  // per-thread primitive lists of the radiance adjoint, kept chords of the tomography
-  // adjoint (grows on demand)
+  // per-warp chord lists and kept moments of the radiance adjoints, kept chords of the
+  // tomography adjoint (grows on demand)
   mutable int* rlist = nullptr;
   mutable size_t rlist_bytes = 0;
   // per primitive in BVH order: the adjoint's gathered parameters (3 float4), then its
@@ -212,7 +212,7 @@ cudaError_t launch_render_server(const ServerLaunch& L, const ServerReqDev* reqs
 cudaError_t launch_fix_to_image(const unsigned long long* acc, int64_t npix, int spp, float* out,
                                 cudaStream_t s);
 // scratch of the compute calls, grown through the field's allocator: the pixel sums and
-// chord store of the scattering renderer, the radiance adjoint's primitive lists
+// chord store of the scattering renderer, the adjoints' chord lists
 cudaError_t ensure_render_scratch(const Field& F, int64_t npix, cudaStream_t s);
 cudaError_t ensure_adjoint_lists(const Field& F, cudaStream_t s);
 // grow a field-owned buffer to at least `bytes` (synchronises the device before

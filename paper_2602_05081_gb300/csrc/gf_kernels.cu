@@ -221,7 +221,7 @@ __device__ float rt_coop(const DevField& F, RtQ& Q, const Mask& M, float3 o, flo
   }
   if (alone) {
     float T = 1.f;
-    if (lane == 0) T = track<false>(F, M, o, v, tmin, tmax, false, seed, ray, word, env, cnt, nullptr);
+    if (lane == 0) T = track(F, M, o, v, tmin, tmax, seed, ray, word, env, cnt);
     __syncwarp();
     return __shfl_sync(kFull, T, 0);
   }

@@ -1,8 +1,7 @@
-// gf_trace.cuh -- per-ray work shared by the render, transmittance and server
-// kernels: LoD mask sampling, deterministic optical depth (Gauss-Legendre and
-// closed-form chord integrals), tentative points, ratio and delta tracking,
-// CDF-inversion free flight, path samples.  One thread owns one ray (or one
-// pixel's paths); a warp advances 32 rays, or 32/G rays with G lanes each.
+// gf_trace.cuh -- per-ray work shared by the render, transmittance, adjoint and
+// server kernels: LoD mask sampling, quadrature rules and closed-form chord
+// integrals, tentative points, ratio tracking of a ray by one lane (for the windows
+// that the one-ray-per-warp kernels cannot hold), camera rays.
 #pragma once
 #include "../../include/gf.h"
 #include "gf_device.cuh"
@@ -578,17 +577,15 @@ struct AccumLeaf {
   }
 };
 
-// Ratio tracking (DELTA = false): returns prod (1 - kappa/kappa_bar).
-// Delta tracking (DELTA = true): returns 1 and *t_hit at the first accepted
-// point (probability max(kappa,0)/kappa_bar), else 0.
-template <bool DELTA>
-__device__ float track(const DevField& F, const Mask& M, float3 o, float3 v, float tmin,
-                       float tmax, bool clamp_neg, uint64_t seed, uint32_t ray, uint32_t word,
-                       const float* env, Counters& cnt, float* t_hit) {
+// Ratio tracking of one ray by one lane: prod (1 - kappa / kappa_bar) over the ray's
+// tentative points.
+inline __device__ float track(const DevField& F, const Mask& M, float3 o, float3 v, float tmin,
+                       float tmax, uint64_t seed, uint32_t ray, uint32_t word, const float* env,
+                       Counters& cnt) {
   const unsigned am = __activemask();
   const float3 inv = safe_inv(v);
   float t0 = 0.f, t1 = 0.f;
-  float Tr = 1.f, hit = 0.f;
+  float Tr = 1.f;
   // `more`: this lane still has windows to process; all lanes that entered
   // iterate together until none has
   bool more = M.bits != 0ull && scene_span(F, o, inv, tmin, tmax, t0, t1);
@@ -603,7 +600,6 @@ __device__ float track(const DevField& F, const Mask& M, float3 o, float3 v, flo
       B.t[i] = INFINITY;
       B.u[i] = 0.f;
     }
-    GF_TIC(c0);
     CollectLeaf cl;
     cl.F = &F;
     cl.M = &M;
@@ -621,7 +617,6 @@ __device__ float track(const DevField& F, const Mask& M, float3 o, float3 v, flo
     cl.env = env;
     CollectTest ctest{&cl.ta, &cl.bound};
     traverse_ray(F, o, inv, M.bits, ctest, cl, cnt.nodes, cnt.leaves);
-    GF_TOC(cnt, 0, c0);
     cnt.windows += 1;
     cnt.chords += cl.nch;
     int n = 0;
@@ -632,7 +627,6 @@ __device__ float track(const DevField& F, const Mask& M, float3 o, float3 v, flo
       more = false;
       continue;
     }
-    GF_TIC(c1);
     AccumLeaf al;
     al.F = &F;
     al.M = &M;
@@ -650,32 +644,11 @@ __device__ float track(const DevField& F, const Mask& M, float3 o, float3 v, flo
     }
     PointTest ptest{&B, n};
     traverse_ray(F, o, inv, M.bits, ptest, al, cnt.nodes, cnt.leaves);
-    GF_TOC(cnt, 1, c1);
     cnt.windows += 1;
     cnt.evals += al.nev;
-    if (DELTA) {
-      bool found = false;
 #pragma unroll
-      for (int i = 0; i < kPts; ++i) {
-        if (!found && i < n && B.u[i] * al.kb[i] < fmaxf(al.kap[i], 0.f)) {
-          *t_hit = B.t[i];
-          found = true;
-        }
-      }
-      if (found) {
-        hit = 1.f;
-        more = false;
-        continue;
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < kPts; ++i) {
-        if (i < n && al.kb[i] > 0.f) {
-          const float k = clamp_neg ? fmaxf(al.kap[i], 0.f) : al.kap[i];
-          Tr *= 1.f - k / al.kb[i];
-        }
-      }
-    }
+    for (int i = 0; i < kPts; ++i)
+      if (i < n && al.kb[i] > 0.f) Tr *= 1.f - al.kap[i] / al.kb[i];
     if (n < kPts) {  // every point of the ray has been used
       more = false;
       continue;
@@ -683,7 +656,7 @@ __device__ float track(const DevField& F, const Mask& M, float3 o, float3 v, flo
     ta = B.t[kPts - 1];
     first = false;
   }
-  return DELTA ? hit : Tr;
+  return Tr;
 }
 
 // ---------------------------------------------------------------------------
