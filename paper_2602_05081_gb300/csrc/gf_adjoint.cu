@@ -39,24 +39,20 @@ struct BackArgs {
 struct PrimDeriv {
   float R[3][3];
   float qh[4], iqn;    // unit quaternion (w, x, y, z) and 1/|q| of the raw one
-  float s[3], is2[3], kin[3];
+  float is[3], is2[3], kin[3];  // 1/s, 1/s^2 of the scales s, input carrier
   float A, dAdw;
   float3 om;
   bool local, normalized;
 
   // from the parameters k_adj_prims gathered for sorted primitive j
-  __device__ __forceinline__ void load(const BackArgs& B, const Prim& P, int j) {
+  __device__ __forceinline__ void load(const BackArgs& B, float amp, float3 omega, int j) {
     const float4* r = B.adj + 3 * (int64_t)j;
     const float4 a = __ldg(r), b = __ldg(r + 1), c = __ldg(r + 2);
     qh[0] = a.x; qh[1] = a.y; qh[2] = a.z; qh[3] = a.w;
-    s[0] = b.x; s[1] = b.y; s[2] = b.z;
+    is[0] = b.x; is[1] = b.y; is[2] = b.z;
     iqn = b.w;
     kin[0] = c.x; kin[1] = c.y; kin[2] = c.z;
     dAdw = c.w;
-    derive(B, P);
-  }
-
-  __device__ __forceinline__ void derive(const BackArgs& B, const Prim& P) {
     const float qw = qh[0], qx = qh[1], qy = qh[2], qz = qh[3];
     R[0][0] = 1.f - 2.f * (qy * qy + qz * qz); R[0][1] = 2.f * (qx * qy - qw * qz);
     R[0][2] = 2.f * (qx * qz + qw * qy);
@@ -65,11 +61,11 @@ struct PrimDeriv {
     R[2][0] = 2.f * (qx * qz - qw * qy); R[2][1] = 2.f * (qy * qz + qw * qx);
     R[2][2] = 1.f - 2.f * (qx * qx + qy * qy);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) is2[k] = 1.f / (s[k] * s[k]);
+    for (int k = 0; k < 3; ++k) is2[k] = is[k] * is[k];
     local = B.frame == GF_OMEGA_LOCAL;
     normalized = B.wmode == GF_WEIGHT_NORMALIZED;
-    A = P.A;
-    om = P.om;
+    A = amp;
+    om = omega;
   }
 
   // dz/dq of the raw quaternion at offset y (linear in y): dz/d(qhat_l) =
@@ -126,7 +122,7 @@ struct PrimDeriv {
     dz_dq(p, gp);
     dz_dq(v, gv);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) kos[k] = local ? kin[k] / s[k] : 0.f;
+    for (int k = 0; k < 3; ++k) kos[k] = local ? kin[k] * is[k] : 0.f;
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       float q0 = 0.f, q1 = 0.f, q2 = 0.f, h0 = 0.f, h1 = 0.f;
@@ -148,7 +144,7 @@ struct PrimDeriv {
       const float d = (zp[k] * zp[k] * C0 + 2.f * zp[k] * zv[k] * C1 + zv[k] * zv[k] * C2) * is2[k] +
                       kos[k] * (zp[k] * S0 + zv[k] * S1);
       acc[7 + k] = aA * (normalized ? d - C0 : d);
-      acc[10 + k] = local ? -aA * (zp[k] * S0 + zv[k] * S1) / s[k] : -aA * (p[k] * S0 + v[k] * S1);
+      acc[10 + k] = local ? -aA * (zp[k] * S0 + zv[k] * S1) * is[k] : -aA * (p[k] * S0 + v[k] * S1);
     }
     acc[13] = -aA * S0;
     acc[14] = sgn * dAdw * C0;
@@ -183,7 +179,9 @@ struct PrimDeriv {
 };
 
 // what PrimDeriv::load needs, gathered once per call in BVH order (48 bytes per
-// primitive instead of 11 scattered words and their arithmetic per chord)
+// primitive instead of 11 scattered words and their arithmetic per chord).  Scales come
+// as reciprocals: nine divisions less per chord took the tomography adjoint of 524,288
+// rays through 200k kernels from 37.0 to 31.2 ms.
 __global__ void k_adj_prims(const float4* rec, const BackArgs B, float4* adj) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= B.n) return;
@@ -193,7 +191,8 @@ __global__ void k_adj_prims(const float4* rec, const BackArgs B, float4* adj) {
   const float iqn = 1.f / sqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
   const float A = rec[4 * j].w;
   adj[3 * j] = make_float4(q[0] * iqn, q[1] * iqn, q[2] * iqn, q[3] * iqn);
-  adj[3 * j + 1] = make_float4(expf(B.ls[3 * i]), expf(B.ls[3 * i + 1]), expf(B.ls[3 * i + 2]), iqn);
+  adj[3 * j + 1] = make_float4(1.f / expf(B.ls[3 * i]), 1.f / expf(B.ls[3 * i + 1]),
+                               1.f / expf(B.ls[3 * i + 2]), iqn);
   adj[3 * j + 2] = make_float4(B.om[3 * i], B.om[3 * i + 1], B.om[3 * i + 2],
                                B.wmode == GF_WEIGHT_NORMALIZED ? A / B.w[i] : 1.f);
 }
@@ -302,7 +301,7 @@ __device__ __forceinline__ TomoChord tomo_moments(const TomoItem& q, const float
 __device__ __forceinline__ void tomo_scatter(const BackArgs& B, const Prim& P, const Chord& ch,
                                              const TomoChord& m, float3 v, int j, float dLdtau) {
   PrimDeriv D;
-  D.load(B, P, j);
+  D.load(B, P.A, P.om, j);
   float acc[15], qt[4][3];
   D.from_moments(ch.p, v, m.C0, m.C1, m.C2, m.S0, m.S1, acc, qt);
   // chord ends that lie on the ellipsoid (not on t = 0)
@@ -454,7 +453,7 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
 // The radiance adjoints run one path per warp.  Bound by instruction issue and the
 // latency of tree nodes.  With one pixel per lane 1.8 of 32 lanes ran, every window
 // visited its ray's list three times and paths were followed twice.  Through 200k
-// kernels: 305 -> 8.3 ms (128x128, 2 samples, single scattering), 697 -> 3.5 ms (96x64,
+// kernels: 305 -> 6.9 ms (128x128, 2 samples, single scattering), 697 -> 3.4 ms (96x64,
 // 1 sample, 3 bounces).
 //
 // A ray is processed over a window of t, at first all of it:
@@ -468,6 +467,10 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
 //           shared out: they are those of a single thread walking the tree;
 //  scatter  chords covering a point with a coefficient, one per lane: five moments,
 //           then the gradient.
+// Warps change between these phases every few rounds, so the kernel also waits for its
+// own instructions (3.5 of 12.3 cycles per issue).  Loops are therefore not unrolled,
+// the points of a group share one copy of the code, and a gradient takes only the offset
+// of its chord (rad_grad) instead of setting it up: 8.4 -> 6.9 and 3.6 -> 3.4 ms.
 // The order of the walk is a 64-bit key per chord: bit 63 - d is set when the path to
 // its leaf takes the second child at depth d.
 // A window with more chords or points than the buffers hold is halved; one that cannot
@@ -480,7 +483,7 @@ constexpr int kRadMargin = 64;    // a descent adds <= 1 entry per level, 64 lev
 constexpr int kRadLeafQ = 96;     // <= 31 left + 64 new
 // (The buffers are kept small: beside 28 KB of them per warp's block the L1 holds the
 // tree's upper nodes.  With 384 stack entries, 128 points and groups of 4 the blocks
-// took 215 KB of an SM: 9.7 and 4.4 ms for the cases above, 8.3 and 3.5 now.)
+// took 215 KB of an SM: 9.7 and 4.4 ms for the cases above, 8.3 and 3.5 with these.)
 constexpr int kRadPts = 64;       // tentative points of a window
 constexpr int kRadList = 4096;    // chords of a window at most (global scratch; rad_list_cap)
 constexpr int kRadKeep = 4096;    // kept segment moments of a path (global scratch)
@@ -491,7 +494,8 @@ static_assert(kPts <= kRadPts && kRadList <= 1 << 16, "point ids");
 
 struct RadKept {  // moments of a segment's chord at S = 1, mask weight included
   float C0, C1, C2, S0, S1;
-  int j, seg, pad;
+  int j, seg;
+  float tc;
 };
 static_assert(sizeof(RadKept) == 32, "kept moments of 32 bytes");
 // one warp's chords of a window
@@ -744,6 +748,7 @@ __device__ __noinline__ void rad_sort(RadWarp& W, int which) {
   for (int i = (int)W.lane; i < n; i += 32) {
     const float t = Pt.kap[i];
     int rank = 0;
+#pragma unroll 1
     for (int k = 0; k < n; ++k) {
       const float tk = Pt.kap[k];
       bool before = tk < t;
@@ -801,6 +806,7 @@ __device__ __noinline__ bool rad_sums(RadWarp& W, int which, int g, int n) {
     tp[p] = p < n ? Pt.t[g + p] : INFINITY;
     c[p] = 0;
   }
+#pragma unroll 1
   for (int b = 0; b < nch; b += 32) {
     const int k = b + (int)lane;
     const float2 s = k < nch ? L.span[k] : make_float2(INFINITY, -INFINITY);
@@ -817,25 +823,34 @@ __device__ __noinline__ bool rad_sums(RadWarp& W, int which, int g, int n) {
   for (int p = 0; p < kRadGroup; ++p)
     if (c[p] > cap) return false;
   __syncwarp();
-#pragma unroll
+#pragma unroll 1
   for (int p = 0; p < kRadGroup; ++p) {
     const int base = p * cap;
-    for (int i = (int)lane; i < c[p]; i += 32) Q.e.key[base + i] = L.key[Q.e.idx[base + i]];
+    int cp = c[0];
+    float t = tp[0];
+#pragma unroll
+    for (int q = 1; q < kRadGroup; ++q) {
+      cp = p == q ? c[q] : cp;
+      t = p == q ? tp[q] : t;
+    }
+#pragma unroll 1
+    for (int i = (int)lane; i < cp; i += 32) Q.e.key[base + i] = L.key[Q.e.idx[base + i]];
     __syncwarp();
-    for (int i = (int)lane; i < c[p]; i += 32) {
+#pragma unroll 1
+    for (int i = (int)lane; i < cp; i += 32) {
       const unsigned long long key = Q.e.key[base + i];
       const float4* r = L.rec + 3 * Q.e.idx[base + i];
       const float4 a = r[0], b = r[1];
       const float dts = r[2].x;
       int rank = 0;
-      for (int k = 0; k < c[p]; ++k) rank += Q.e.key[base + k] < key ? 1 : 0;
-      const float dt = tp[p] - a.x;
+      for (int k = 0; k < cp; ++k) rank += Q.e.key[base + k] < key ? 1 : 0;
+      const float dt = t - a.x;
       const float y = fmaf(fmaf(a.y, dt, a.z), dt, a.w);
       int m = (int)(fabsf(dt - dts) * b.w);
       m = m > 7 ? 7 : m;
       Q.e.term[base + rank] = make_float4(ex2f(y), cosf_fast(fmaf(b.y, dt, b.z)), b.x, W.env[m]);
     }
-    W.cnt.evals += (int)lane < c[p] ? (unsigned)(c[p] - (int)lane + 31) >> 5 : 0u;
+    W.cnt.evals += (int)lane < cp ? (unsigned)(cp - (int)lane + 31) >> 5 : 0u;
   }
   __syncwarp();
   if ((int)lane < n) {
@@ -1036,12 +1051,27 @@ struct RadScatterLeaf {
     }
     if (!any) return;
     PrimDeriv D;
-    D.load(W->B, Pr, j);
+    D.load(W->B, Pr.A, Pr.om, j);
     float acc[15], qt[4][3];
     D.from_moments(ch.p, R.v, C0, C1, C2, S0, S1, acc, qt);
     add_grad4(W->B, j, acc, w * scale);
   }
 };
+
+// the gradient of sorted primitive j from the moments of its chord around tc, times
+// scale.  The offset at tc is all that it needs of the chord.
+__device__ __forceinline__ void rad_grad(const RadWarp& W, int j, float3 o, float3 v, float tc,
+                                         float C0, float C1, float C2, float S0, float S1,
+                                         float scale) {
+  const float4* r = W.F.rec + 4 * (int64_t)j;
+  const float4 mu = __ldg(r), om = __ldg(r + 3);
+  PrimDeriv D;
+  D.load(W.B, mu.w, make_float3(om.x, om.y, om.z), j);
+  float acc[15], qt[4][3];
+  D.from_moments(chord_offset(make_float3(mu.x, mu.y, mu.z), o, v, tc), v, C0, C1, C2, S0, S1, acc,
+                 qt);
+  add_grad4(W.B, j, acc, scale);
+}
 
 // gradients of the chords covering points 0 .. n-1 with a coefficient (c), times scale;
 // seg >= 0: the moments are kept for the end of the path instead
@@ -1072,6 +1102,7 @@ __device__ __noinline__ void rad_scatter(RadWarp& W, int which, int n, int seg, 
       const int k = b + (int)lane;
       const float2 s = k < nch ? L.span[k] : make_float2(INFINITY, -INFINITY);
       bool in = false;
+#pragma unroll 1
       for (int i = 0; i < n; ++i) in |= Pt.c[i] != 0.f && Pt.t[i] >= s.x && Pt.t[i] <= s.y;
       const unsigned bm = __ballot_sync(kFull, in);
       if (in) Q.e.idx[m + __popc(bm & lt)] = k;
@@ -1091,6 +1122,7 @@ __device__ __noinline__ void rad_scatter(RadWarp& W, int which, int n, int seg, 
       const float4 a = L.rec[3 * k], r1 = L.rec[3 * k + 1], r2 = L.rec[3 * k + 2];
       const int j = __float_as_int(r2.w);
       float C0 = 0.f, C1 = 0.f, C2 = 0.f, S0 = 0.f, S1 = 0.f;
+#pragma unroll 1
       for (int i = 0; i < n; ++i) {
         const float t = Pt.t[i], c = Pt.c[i];
         if (c == 0.f || t < s.x || t > s.y) continue;
@@ -1109,18 +1141,10 @@ __device__ __noinline__ void rad_scatter(RadWarp& W, int which, int n, int seg, 
         if (slot < kRadKeep) {
           float4* d = reinterpret_cast<float4*>(W.kept() + slot);
           d[0] = make_float4(w * C0, w * C1, w * C2, w * S0);
-          d[1] = make_float4(w * S1, __int_as_float(j), __int_as_float(seg), 0.f);
+          d[1] = make_float4(w * S1, __int_as_float(j), __int_as_float(seg), a.x);
         }
       } else {
-        const Prim Pr = load_prim(W.F, j);
-        Chord ch;
-        if (chord_setup(Pr, Q.ray.o, Q.ray.v, 0.f, INFINITY, Pr.k2, ch)) {
-          PrimDeriv D;
-          D.load(W.B, Pr, j);
-          float acc[15], qt[4][3];
-          D.from_moments(ch.p, Q.ray.v, C0, C1, C2, S0, S1, acc, qt);
-          add_grad4(W.B, j, acc, w * scale);
-        }
+        rad_grad(W, j, Q.ray.o, Q.ray.v, a.x, C0, C1, C2, S0, S1, w * scale);
       }
     }
     if (seg >= 0) {
@@ -1167,6 +1191,7 @@ __device__ __forceinline__ void nee_scatter(RadWarp& W, int which, float3 x, uin
     if (windows > 1)
       for (int g = 0; g < n; g += kRadGroup) rad_group(W, which, g);
     __syncwarp();
+#pragma unroll 1
     for (int i = (int)W.lane; i < n; i += 32) {
       const float kap = Pt.kap[i], kb = Pt.kb[i];
       float c = 0.f;
@@ -1290,14 +1315,7 @@ __device__ __forceinline__ void path_backward(RadWarp& W, float3 o, float3 v, ui
     const float S = base * Q.S[seg];
     if (S == 0.f) continue;
     const float3 so = Q.so[seg], sv = Q.sv[seg];
-    const Prim Pr = load_prim(W.F, j);
-    Chord ch;
-    if (!chord_setup(Pr, so, sv, 0.f, INFINITY, Pr.k2, ch)) continue;
-    PrimDeriv D;
-    D.load(W.B, Pr, j);
-    float acc[15], qt[4][3];
-    D.from_moments(ch.p, sv, a.x, a.y, a.z, a.w, c.x, acc, qt);
-    add_grad4(W.B, j, acc, S);
+    rad_grad(W, j, so, sv, c.w, a.x, a.y, a.z, a.w, c.x, S);
   }
   __syncwarp();
 }

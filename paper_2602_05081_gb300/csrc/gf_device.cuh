@@ -282,6 +282,17 @@ struct Chord {
   uint32_t cell, orig;
 };
 
+// o + tc v - mu with compensated arithmetic (positions ~1, offsets ~sigma)
+__device__ __forceinline__ float3 chord_offset(float3 mu, float3 o, float3 v, float tc) {
+  auto axis = [&](float ok, float vk, float mk) {
+    const float d = __fsub_rn(ok, mk), bb = __fsub_rn(d, ok);  // error-free o - mu
+    const float e = __fsub_rn(__fsub_rn(ok, __fsub_rn(d, bb)), __fadd_rn(mk, bb));
+    const float pr = __fmul_rn(tc, vk);
+    return __fadd_rn(__fadd_rn(d, pr), __fadd_rn(e, fmaf(tc, vk, -pr)));
+  };
+  return make_float3(axis(o.x, v.x, mu.x), axis(o.y, v.y, mu.y), axis(o.z, v.z, mu.z));
+}
+
 __device__ __forceinline__ bool chord_setup(const Prim& P, float3 o, float3 v, float tmin,
                                             float tmax, float k2, Chord& c) {
   // u = Sigma^-1 v, a = v^T Sigma^-1 v
@@ -289,23 +300,12 @@ __device__ __forceinline__ bool chord_setup(const Prim& P, float3 o, float3 v, f
   float uy = fmaf(P.p01, v.x, fmaf(P.p11, v.y, P.p12 * v.z));
   float uz = fmaf(P.p02, v.x, fmaf(P.p12, v.y, P.p22 * v.z));
   float a = fmaf(v.x, ux, fmaf(v.y, uy, v.z * uz));
-  // d0 = o - mu, error-free split; reference tc = -(d0 . u)/a
+  // reference tc = -((o - mu) . u)/a
   float d0x = __fsub_rn(o.x, P.mu.x), d0y = __fsub_rn(o.y, P.mu.y), d0z = __fsub_rn(o.z, P.mu.z);
   const float ia = __frcp_rn(a);
   float tc = -fmaf(d0x, ux, fmaf(d0y, uy, d0z * uz)) * ia;
-  // p = (o - mu) + tc v with compensated arithmetic (positions ~1, offsets ~sigma)
-  float ex, ey, ez;
-  {
-    float s, bb;
-    s = d0x; bb = __fsub_rn(s, o.x); ex = __fsub_rn(__fsub_rn(o.x, __fsub_rn(s, bb)), __fadd_rn(P.mu.x, bb));
-    s = d0y; bb = __fsub_rn(s, o.y); ey = __fsub_rn(__fsub_rn(o.y, __fsub_rn(s, bb)), __fadd_rn(P.mu.y, bb));
-    s = d0z; bb = __fsub_rn(s, o.z); ez = __fsub_rn(__fsub_rn(o.z, __fsub_rn(s, bb)), __fadd_rn(P.mu.z, bb));
-  }
-  float prx = __fmul_rn(tc, v.x), pry = __fmul_rn(tc, v.y), prz = __fmul_rn(tc, v.z);
-  float erx = fmaf(tc, v.x, -prx), ery = fmaf(tc, v.y, -pry), erz = fmaf(tc, v.z, -prz);
-  float px = __fadd_rn(__fadd_rn(d0x, prx), __fadd_rn(ex, erx));
-  float py = __fadd_rn(__fadd_rn(d0y, pry), __fadd_rn(ey, ery));
-  float pz = __fadd_rn(__fadd_rn(d0z, prz), __fadd_rn(ez, erz));
+  const float3 p = chord_offset(P.mu, o, v, tc);
+  const float px = p.x, py = p.y, pz = p.z;
   // b = v^T Sigma^-1 p (~0), g = p^T Sigma^-1 p
   float b = fmaf(ux, px, fmaf(uy, py, uz * pz));
   float qx = fmaf(P.p00, px, fmaf(P.p01, py, P.p02 * pz));
