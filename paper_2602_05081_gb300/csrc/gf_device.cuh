@@ -284,13 +284,20 @@ struct Chord {
 
 // o + tc v - mu with compensated arithmetic (positions ~1, offsets ~sigma)
 __device__ __forceinline__ float3 chord_offset(float3 mu, float3 o, float3 v, float tc) {
-  auto axis = [&](float ok, float vk, float mk) {
-    const float d = __fsub_rn(ok, mk), bb = __fsub_rn(d, ok);  // error-free o - mu
-    const float e = __fsub_rn(__fsub_rn(ok, __fsub_rn(d, bb)), __fadd_rn(mk, bb));
-    const float pr = __fmul_rn(tc, vk);
-    return __fadd_rn(__fadd_rn(d, pr), __fadd_rn(e, fmaf(tc, vk, -pr)));
-  };
-  return make_float3(axis(o.x, v.x, mu.x), axis(o.y, v.y, mu.y), axis(o.z, v.z, mu.z));
+  // o - mu, error-free split
+  const float dx = __fsub_rn(o.x, mu.x), dy = __fsub_rn(o.y, mu.y), dz = __fsub_rn(o.z, mu.z);
+  float ex, ey, ez;
+  {
+    float bb;
+    bb = __fsub_rn(dx, o.x); ex = __fsub_rn(__fsub_rn(o.x, __fsub_rn(dx, bb)), __fadd_rn(mu.x, bb));
+    bb = __fsub_rn(dy, o.y); ey = __fsub_rn(__fsub_rn(o.y, __fsub_rn(dy, bb)), __fadd_rn(mu.y, bb));
+    bb = __fsub_rn(dz, o.z); ez = __fsub_rn(__fsub_rn(o.z, __fsub_rn(dz, bb)), __fadd_rn(mu.z, bb));
+  }
+  const float prx = __fmul_rn(tc, v.x), pry = __fmul_rn(tc, v.y), prz = __fmul_rn(tc, v.z);
+  const float erx = fmaf(tc, v.x, -prx), ery = fmaf(tc, v.y, -pry), erz = fmaf(tc, v.z, -prz);
+  return make_float3(__fadd_rn(__fadd_rn(dx, prx), __fadd_rn(ex, erx)),
+                     __fadd_rn(__fadd_rn(dy, pry), __fadd_rn(ey, ery)),
+                     __fadd_rn(__fadd_rn(dz, prz), __fadd_rn(ez, erz)));
 }
 
 __device__ __forceinline__ bool chord_setup(const Prim& P, float3 o, float3 v, float tmin,

@@ -452,12 +452,10 @@ __device__ __forceinline__ void chord_points(const DevField& F, const Chord& ch,
     if (bp <= dt) ++p;
     else break;
   }
-#pragma unroll 1
   for (uint32_t draw = 0; draw < (1u << 16); ++draw) {
     const uint4 x = rng4(seed, draw, ch.orig, ray, word);
     float z = -__logf(1.0f - u01(x.x));
     bool more = false;
-#pragma unroll 1
     for (int q = 0; q < 2 * J + 2; ++q) {
       const float bp = p < J ? dts - (float)(J - p) * invs : dts + (float)(p - J + 1) * invs;
       const float end = p < 2 * J ? fminf(bp, dtout) : dtout;
