@@ -1471,12 +1471,14 @@ static size_t tomo_scratch(int64_t g) {
 static size_t rad_scratch(const Field& F, int64_t g) {
   return (size_t)g * (kBackBlock / 32) * rad_warp_bytes(rad_list_cap(F.n));
 }
-static cudaError_t grow_adjoint(const Field& F, size_t bytes, cudaStream_t s) {
+// the arrays per primitive and `bytes` of scratch for a grid of g blocks, through the
+// field's allocator; g comes back smaller when less scratch is to be had
+static cudaError_t grow_adjoint(const Field& F, size_t bytes, int64_t& g, cudaStream_t s) {
   const cudaError_t e = grow(F, (void**)&F.adj, F.adj_bytes, (size_t)F.n * 7 * sizeof(float4), s);
-  return e != cudaSuccess ? e : grow(F, (void**)&F.rlist, F.rlist_bytes, bytes, s);
+  return e != cudaSuccess ? e : grow_shares(F, (void**)&F.rlist, F.rlist_bytes, bytes / g, g, s);
 }
 
-// the scratch of every adjoint and the arrays per primitive, through the field's allocator
+// the scratch of every adjoint
 cudaError_t ensure_adjoint_lists(const Field& F, cudaStream_t s) {
   int64_t g = 1;
   size_t bytes = 0;
@@ -1486,7 +1488,8 @@ cudaError_t ensure_adjoint_lists(const Field& F, cudaStream_t s) {
   if ((e = adjoint_grid(F, k_radiance_backward<false>, kRadSmem, g)) != cudaSuccess) return e;
   bytes = std::max(bytes, rad_scratch(F, g));
   if ((e = adjoint_grid(F, k_radiance_backward<true>, kRadSmem, g)) != cudaSuccess) return e;
-  return grow_adjoint(F, std::max(bytes, rad_scratch(F, g)), s);
+  bytes = std::max(bytes, rad_scratch(F, g));
+  return grow_adjoint(F, (bytes + g - 1) / g * g, g, s);
 }
 
 // An adjoint kernel over units of `chunk` samples of a pixel (about 16 per warp of the
@@ -1503,7 +1506,7 @@ static cudaError_t launch_adjoint(const Field& F, const PathParams& P,
   if ((e = adjoint_stack_fits(kernel)) != cudaSuccess) return e;
   if ((e = adjoint_grid(F, kernel, smem, g)) != cudaSuccess) return e;
   // (allocated ahead by gf_reserve, else here)
-  if ((e = grow_adjoint(F, smem ? rad_scratch(F, g) : tomo_scratch(g), s)) != cudaSuccess) return e;
+  if ((e = grow_adjoint(F, smem ? rad_scratch(F, g) : tomo_scratch(g), g, s)) != cudaSuccess) return e;
   const int64_t npix = (int64_t)P.cam.W * P.cam.H, warps = g * (kBackBlock / 32);
   int64_t nchunk = (16 * warps + npix - 1) / npix;
   nchunk = nchunk < 1 ? 1 : (nchunk > P.spp ? P.spp : nchunk);

@@ -162,6 +162,15 @@ cudaError_t grow(const Field& F, void** p, size_t& have, size_t bytes, cudaStrea
   return e;
 }
 
+cudaError_t grow_shares(const Field& F, void** p, size_t& have, size_t share, int64_t& shares,
+                        cudaStream_t s) {
+  for (;; shares = (shares + 1) / 2) {
+    const cudaError_t e = grow(F, p, have, share * (size_t)shares, s);
+    if (e != cudaErrorMemoryAllocation || shares <= 1) return e;
+    (void)cudaGetLastError();
+  }
+}
+
 // The field's device error word, read after the stream has been synchronised
 // (host-buffer paths): mapped to a status and cleared, as gf_sync does.
 gf_status take_device_error(Field& F) {

@@ -218,6 +218,10 @@ cudaError_t ensure_adjoint_lists(const Field& F, cudaStream_t s);
 // grow a field-owned buffer to at least `bytes` (synchronises the device before
 // returning the old one)
 cudaError_t grow(const Field& F, void** p, size_t& have, size_t bytes, cudaStream_t s);
+// the same for `shares` equal shares (the blocks of a persistent grid); when the memory is
+// refused, half as many and so on down to one: a kernel of fewer blocks, same results
+cudaError_t grow_shares(const Field& F, void** p, size_t& have, size_t share, int64_t& shares,
+                        cudaStream_t s);
 cudaError_t launch_radiance_backward(const Field& F, const PathParams& P, const float* dLdI,
                                      float* grad, cudaStream_t s);
 cudaError_t launch_tomo_backward(const Field& F, const PathParams& P, const float* dLdI,

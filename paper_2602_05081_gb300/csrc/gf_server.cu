@@ -414,8 +414,6 @@ gf_status gf_server_create(gf_ctx* ctx, gf_field* const* fields, int n_fields,
     free_server(S);
     return fail_cuda(e, "occupancy");
   }
-  // about four units of kUnitSamples samples per resident lane
-  if (S->opts.batch_samples == 0) S->opts.batch_samples = S->grid * 128 * 4 * kUnitSamples;
   if ((e = S->mem.get(&S->pool_mem, S->opts.mem_budget, nullptr)) != cudaSuccess) {
     free_server(S);
     return fail_cuda(e, "framebuffer pool");
@@ -435,8 +433,7 @@ gf_status gf_server_create(gf_ctx* ctx, gf_field* const* fields, int n_fields,
         (e = cudaEventCreate(&b.start)) != cudaSuccess || (e = cudaEventCreate(&b.done)) != cudaSuccess ||
         (e = cudaHostAlloc((void**)&b.host, bytes, cudaHostAllocDefault)) != cudaSuccess ||
         (e = S->mem.get(&b.dev, bytes, b.stream)) != cudaSuccess ||
-        (e = S->mem.get(&b.fields, sizeof(DevField) * n_fields, b.stream)) != cudaSuccess ||
-        (e = S->mem.get(&b.store, scatter_store_bytes(S->grid), b.stream)) != cudaSuccess) {
+        (e = S->mem.get(&b.fields, sizeof(DevField) * n_fields, b.stream)) != cudaSuccess) {
       free_server(S);
       return fail_cuda(e, "server buffers");
     }
@@ -451,6 +448,24 @@ gf_status gf_server_create(gf_ctx* ctx, gf_field* const* fields, int n_fields,
       return fail_cuda(e, "field views");
     }
   }
+  // the chord stores of the batches in flight, of a smaller grid when memory is short
+  for (;; S->grid = (S->grid + 1) / 2) {
+    e = cudaSuccess;
+    for (Batch& b : S->batches)
+      if (e == cudaSuccess) e = S->mem.get(&b.store, scatter_store_bytes(S->grid), b.stream);
+    if (e == cudaSuccess) break;
+    (void)cudaGetLastError();
+    if (e != cudaErrorMemoryAllocation || S->grid <= 1) {
+      free_server(S);
+      return fail_cuda(e, "server buffers");
+    }
+    for (Batch& b : S->batches) {
+      S->mem.release(b.store, b.stream);
+      b.store = nullptr;
+    }
+  }
+  // about four units of kUnitSamples samples per resident lane
+  if (S->opts.batch_samples == 0) S->opts.batch_samples = S->grid * 128 * 4 * kUnitSamples;
   S->t0 = std::chrono::steady_clock::now();
   S->worker = std::thread([S] { S->run(); });
   for (const Field* f : S->fields) ++const_cast<Field*>(f)->server_refs;

@@ -873,14 +873,18 @@ static int scatter_slots(int64_t units, int64_t& g) {
 }
 
 // pixel sums (8 bytes per pixel) and the per-warp chord store of a full persistent
-// grid (shared with the analytic flights' lists), grown through the field's allocator
-cudaError_t ensure_render_scratch(const Field& F, int64_t npix, cudaStream_t s) {
-  int64_t g = 1;
+// grid of g blocks (shared with the analytic flights' lists), grown through the field's
+// allocator; g comes back smaller when less memory is to be had
+static cudaError_t render_scratch(const Field& F, int64_t npix, int64_t& g, cudaStream_t s) {
   cudaError_t e = render_grid(F.ctx.sm_count, g);
   if (e != cudaSuccess) return e;
   if ((e = grow(F, (void**)&F.acc64, F.acc_bytes, (size_t)npix * 8, s)) != cudaSuccess) return e;
-  return grow(F, (void**)&F.wscratch, F.wscratch_bytes,
-              std::max(scatter_store_bytes(g), flight_store_bytes(F)), s);
+  const size_t share = std::max(scatter_store_bytes(1), (flight_store_bytes(F) + g - 1) / g);
+  return grow_shares(F, (void**)&F.wscratch, F.wscratch_bytes, share, g, s);
+}
+cudaError_t ensure_render_scratch(const Field& F, int64_t npix, cudaStream_t s) {
+  int64_t g = 1;
+  return render_scratch(F, npix, g, s);
 }
 
 cudaError_t launch_render_scatter(const Field& F, const PathParams& P, float* out, cudaStream_t s) {
@@ -889,15 +893,14 @@ cudaError_t launch_render_scatter(const Field& F, const PathParams& P, float* ou
   if (e != cudaSuccess) return e;
   const int64_t npix = (int64_t)P.cam.W * P.cam.H;
   int64_t g = 1;
-  if ((e = render_grid(F.ctx.sm_count, g)) != cudaSuccess) return e;
+  // fixed-point pixel sums and the chord store (allocated ahead by gf_reserve, else here)
+  if ((e = render_scratch(F, npix, g, s)) != cudaSuccess) return e;
   // about 16 units per lane: chunk = ceil(npix spp / (16 lanes)), in [1, spp]
   const int64_t lanes = g * kWWarps * 32;
   int64_t chunk = (npix * P.spp + 16 * lanes - 1) / (16 * lanes);
   chunk = chunk < 1 ? 1 : (chunk > P.spp ? P.spp : chunk);
   const int64_t nchunk = (P.spp + chunk - 1) / chunk;
   if (npix * nchunk >= (int64_t)INT_MAX) return cudaErrorInvalidValue;
-  // fixed-point pixel sums and the chord store (allocated ahead by gf_reserve, else here)
-  if ((e = ensure_render_scratch(F, npix, s)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(F.acc64, 0, (size_t)npix * 8, s)) != cudaSuccess) return e;
   const int slots = scatter_slots(npix * nchunk, g);
   auto kernel = nodes_per_step(P.lod, P.lod_nee) == 2 ? k_render_scatter<2> : k_render_scatter<1>;
