@@ -169,7 +169,7 @@ struct PrimDeriv {
 // what PrimDeriv::load needs, gathered once per call in BVH order (48 bytes per
 // primitive instead of 11 scattered words and their arithmetic per chord).  Scales come
 // as reciprocals: nine divisions less per chord took the tomography adjoint of 524,288
-// rays through 200k kernels from 37.0 to 31.2 ms.
+// rays through 200k kernels from 37.0 to 31.3 ms.
 __global__ void k_adj_prims(const float4* rec, const BackArgs B, float4* adj) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= B.n) return;
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
 // The radiance adjoints run one path per warp.  Bound by instruction issue and the
 // latency of tree nodes.  With one pixel per lane 1.8 of 32 lanes ran, every window
 // visited its ray's list three times and paths were followed twice.  Through 200k
-// kernels: 305 -> 6.9 ms (128x128, 2 samples, single scattering), 697 -> 3.4 ms (96x64,
+// kernels: 305 -> 6.8 ms (128x128, 2 samples, single scattering), 697 -> 3.4 ms (96x64,
 // 1 sample, 3 bounces).
 //
 // A ray is processed over a window of t, at first all of it:
@@ -457,10 +457,10 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
 //           shared out: they are those of a single thread walking the tree;
 //  scatter  chords covering a point with a coefficient, one per lane: five moments,
 //           then the gradient.
-// Warps change between these phases every few rounds, so the kernel also waits for its
-// own instructions (3.5 of 12.3 cycles per issue).  Loops are therefore not unrolled,
-// the points of a group share one copy of the code, and a gradient takes only the offset
-// of its chord (rad_grad) instead of setting it up: 8.4 -> 6.9 and 3.6 -> 3.4 ms.
+// Warps change between these phases every few rounds, so code size counts: 3.5 of 12.3
+// cycles per issued instruction were waits for instructions.  Loops are not unrolled, the
+// points of a group share one copy of the code, and a gradient takes only the offset of
+// its chord (rad_grad) instead of setting it up: 0.3 of 10.1, 8.4 -> 6.8 and 3.6 -> 3.4 ms.
 // The order of the walk is a 64-bit key per chord: bit 63 - d is set when the path to
 // its leaf takes the second child at depth d.
 // A window with more chords or points than the buffers hold is halved; one that cannot
