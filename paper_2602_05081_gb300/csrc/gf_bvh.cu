@@ -273,9 +273,32 @@ __device__ __forceinline__ unsigned int spread10(unsigned int x) {
 // second tree's n entries follow the first's, with bit 36 set, so that one sort orders
 // both
 __device__ __forceinline__ uint32_t cell_band(uint32_t cell) { return cell == 0 ? 0u : ((cell - 1u) >> 3) + 1u; }
-__global__ void k_morton(const float4* rec, int64_t n, const unsigned int* bounds,
-                         unsigned long long* keys, int* idx) {
+// face areas of a box, summed over the three axes
+__host__ __device__ __forceinline__ float face_areas(float x, float y, float z) { return x * y + y * z + z * x; }
+// unit of the summed shares of the scene's face areas that the kernels' boxes take: a
+// share is at most 1, so 256 of them stay below 2^32
+constexpr float kAreaUnit = 1.0f / 2097152.0f;
+
+__global__ void __launch_bounds__(256) k_morton(const float4* rec, const float* box, int64_t n,
+                                                const unsigned int* bounds, unsigned long long* keys,
+                                                int* idx, unsigned long long* area) {
+  // per band: the boxes' shares of the scene's face areas (sums of integers, the same in
+  // any order)
+  __shared__ unsigned int part[8];
+  if (threadIdx.x < 8) part[threadIdx.x] = 0u;
+  __syncthreads();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) {
+    const float* b = box + 6 * i;
+    const float s = face_areas(ord_dec(bounds[3]) - ord_dec(bounds[0]), ord_dec(bounds[4]) - ord_dec(bounds[1]),
+                               ord_dec(bounds[5]) - ord_dec(bounds[2]));
+    const float q = face_areas(b[3] - b[0], b[4] - b[1], b[5] - b[2]) / s;
+    if (q > 0.f)  // (not for boxes without faces)
+      atomicAdd(&part[cell_band(__float_as_uint(rec[4 * i + 3].w) >> 26)],
+                (unsigned)__float2uint_rn(fminf(q, 1.0f) * (1.0f / kAreaUnit)));
+  }
+  __syncthreads();
+  if (threadIdx.x < 8 && part[threadIdx.x]) atomicAdd(area + threadIdx.x, (unsigned long long)part[threadIdx.x]);
   if (i >= n) return;
   float lo[3], hi[3];
   for (int j = 0; j < 3; ++j) {
@@ -634,11 +657,18 @@ __global__ void k_pad_mean_step(float* box, int64_t n, const unsigned int* bound
 }
 
 
+// results of the build that the host reads
+struct BuildHead {
+  unsigned int bounds[16];     // boxes (12), the two trees' depths
+  unsigned long long area[8];  // per band: summed face areas (k_morton)
+};
+
 cudaError_t build_bvh(Field& F, cudaStream_t s) {
   (void)cudaGetLastError();  // a stale error of an unrelated call is not ours
   const int64_t n = F.n;
   cudaError_t e = cudaSuccess;
   // temporaries, in one block
+  BuildHead* head = nullptr;
   unsigned int* bounds = nullptr;  // boxes (12), the two trees' depths
   int* roots = nullptr;            // of cells, then of bands
   unsigned long long *keys = nullptr, *keys2 = nullptr;
@@ -650,7 +680,8 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
   size_t tmp_bytes = 0, sort_bytes = 0;
   const int64_t m = n - 1;
   const unsigned pn = (unsigned)((n + 255) / 256), pm = (unsigned)((m + 255) / 256);
-  unsigned int hb[14];
+  BuildHead hh;
+  const unsigned int* hb = hh.bounds;
   int hroots[kMaxCells + 8];
 #define GF_TRY(x) do { e = (x); if (e != cudaSuccess) goto done; } while (0)
   GF_TRY(cub::DeviceRadixSort::SortPairs(nullptr, sort_bytes, keys, keys2, idx, idx2, (int)(2 * n), 0, 37, s));
@@ -663,7 +694,7 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
       at += (bytes + 255) & ~size_t(255);
     };
     char* tp = nullptr;
-    take(bounds, sizeof(hb));
+    take(head, sizeof(BuildHead));
     take(roots, sizeof(hroots));
     take(keys, 2 * n * sizeof(unsigned long long));
     take(keys2, 2 * n * sizeof(unsigned long long));
@@ -681,7 +712,8 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
     tmp = tp;
     if (pass == 0) GF_TRY(F.mem.alloc(&block, (size_t)at, s));
   }
-  GF_TRY(cudaMemsetAsync(bounds + 12, 0, 2 * sizeof(unsigned int), s));
+  bounds = head->bounds;
+  GF_TRY(cudaMemsetAsync(bounds + 12, 0, sizeof(BuildHead) - 12 * sizeof(unsigned int), s));
   GF_TRY(cudaMemsetAsync(roots, 0xFF, sizeof(hroots), s));
   {
     unsigned int init[12];
@@ -705,7 +737,7 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
       k_bounds<<<blocks, 256, 0, s>>>(F.box_orig, F.rec_orig, n, bounds);
       GF_TRY(cudaGetLastError());
     }
-    k_morton<<<pn, 256, 0, s>>>(F.rec_orig, n, bounds, keys, idx);
+    k_morton<<<pn, 256, 0, s>>>(F.rec_orig, F.box_orig, n, bounds, keys, idx, head->area);
     GF_TRY(cudaGetLastError());
   }
   GF_TRY(cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, keys, keys2, idx, idx2, (int)(2 * n), 0, 37, s));
@@ -754,7 +786,7 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
     GF_TRY(cudaGetLastError());
   }
   GF_TRY(cudaMemcpyAsync(hroots, roots, sizeof(hroots), cudaMemcpyDeviceToHost, s));
-  GF_TRY(cudaMemcpyAsync(hb, bounds, sizeof(hb), cudaMemcpyDeviceToHost, s));
+  GF_TRY(cudaMemcpyAsync(&hh, head, sizeof(hh), cudaMemcpyDeviceToHost, s));
   GF_TRY(cudaStreamSynchronize(s));
   {
     auto dec = [](unsigned int u) {
@@ -769,6 +801,18 @@ cudaError_t build_bvh(Field& F, cudaStream_t s) {
     if (n < 2) F.depth = 0;
     F.dev.lo = make_float3(dec(hb[0]), dec(hb[1]), dec(hb[2]));
     F.dev.hi = make_float3(dec(hb[3]), dec(hb[4]), dec(hb[5]));
+    // a convex body of mean projected area a in a volume V is crossed a / V times per unit
+    // length; an ellipsoid's is about pi / 12 of its box's face areas.  V: the box of the
+    // means, which holds the bodies but for the margins around it
+    const float x = F.dev.hi.x - F.dev.lo.x, y = F.dev.hi.y - F.dev.lo.y, z = F.dev.hi.z - F.dev.lo.z;
+    const double V = (double)fmaxf(dec(hb[9]) - dec(hb[6]), 0.5f * x) * fmaxf(dec(hb[10]) - dec(hb[7]), 0.5f * y) *
+                     fmaxf(dec(hb[11]) - dec(hb[8]), 0.5f * z);
+    const double per = 3.14159265358979323846 / 12.0 * kAreaUnit * face_areas(x, y, z) / V;
+    for (int b = 0; b < 8; ++b) {
+      const unsigned long long cones = b == 0 ? F.dev.occupied & 1ull : F.dev.occupied >> (1 + kCones * (b - 1)) & 0xFFull;
+      const int k = __builtin_popcountll(cones);
+      F.dev.chords[b] = k && hh.area[b] ? (float)(per * (double)hh.area[b] / k) : 0.f;
+    }
     for (int k = 0; k < 3; ++k) {
       F.mu_lo[k] = dec(hb[6 + k]);
       F.mu_hi[k] = dec(hb[9 + k]);

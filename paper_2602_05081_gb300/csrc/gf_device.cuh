@@ -89,6 +89,8 @@ struct DevField {
   float3 lo, hi;           // scene bounds (union of all ellipsoid boxes)
   unsigned long long occupied;
   float kbar[kMaxCells];   // mean |k_W| per cell
+  float chords[8];         // per band: chords of one occupied cone per unit length of a ray
+                           // through the scene, on average
   float band_wmax[8];      // largest world carrier |omega| (rad/unit) per band
   float axes[kCones][3];   // orientation-bin axes
   float env[8];            // exp(-n^2/2), n = 0..7

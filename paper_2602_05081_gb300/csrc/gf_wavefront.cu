@@ -29,6 +29,7 @@
 
 #include "gf_host.h"
 #include "gf_trace.cuh"
+#include "gf_window.h"
 
 namespace gf {
 
@@ -43,6 +44,7 @@ constexpr int kChordQ = 64;     // queued chords per warp (<= 31 left + 32 new)
 // masks: 317 -> 303 ms; 512x512, 16 samples, 100k kernels: 196 -> 183 ms.
 constexpr int kPK = 13;         // tentative points per lane and window
 constexpr int kSlotCh = 448;    // stored chords per lane and window (global scratch)
+constexpr float kFill = 0.7f;     // share of them that a ray's windows aim at (0.5 to 0.9: within 4 %)
 constexpr int kHits = 40;         // covering chords a lane collects before it evaluates them
 static_assert(kSlotCh % 4 == 0, "spans are read four at a time");
 // A warp's stored chords, per slot: entry and exit (8 bytes each, read by themselves
@@ -376,7 +378,7 @@ struct PathState {
   float3 o, v;    // current ray
   float t0, t1;   // scene span of the current ray
   float step;     // window length
-  float fit;      // windows longer than this held too many chords lately
+  float lim;      // length that holds kFill of a window's chords on average
   unsigned long long allow;  // cells the foveation keeps for the sample's path
 };
 
@@ -396,6 +398,15 @@ __device__ __forceinline__ void set_slot(LaneRay& R, float3 o, float3 v, const M
   R.cx[1] = m.cx[1];
 }
 
+// chords per unit length that rays with the cell mask `mask` have on average
+__device__ __forceinline__ float chords_per_length(const DevField& F, unsigned long long mask) {
+  float r = (mask & 1ull) ? F.chords[0] : 0.f;
+#pragma unroll
+  for (int b = 1; b < 8; ++b)
+    r = fmaf(F.chords[b], (float)__popc((unsigned)(mask >> (1 + kCones * (b - 1))) & 0xFFu), r);
+  return r;
+}
+
 // Start a tracking ray: returns false if it misses the scene (nothing to do).
 __device__ __forceinline__ bool start_ray(const DevField& F, LaneRay& R, PathState& S, int kind,
                                           float3 o, float3 v, const Mask& m, uint32_t ray,
@@ -409,16 +420,11 @@ __device__ __forceinline__ bool start_ray(const DevField& F, LaneRay& R, PathSta
   S.t0 = t0;
   S.t1 = t1;
   if (!hit) return false;
-  // first window: 0.3 of the span when tracking, all of it for NEE, but not a length that
-  // held too many chords on the lane's last rays.  Shares of 0.25, 0.35 and 0.5: 201, 197
-  // and 203 ms (1024x1024, 8 samples, 1M kernels, one-cone masks), 6.4, 6.8 and 6.9 ms
-  // (333x217, 4 samples, FP16), 99, 99 and 107 ms (512x512, 16 samples, every cone).
-  const float len = t1 - t0;
-  S.step = kind == 1 ? fmaxf(fminf(0.3f * len, S.fit), 1e-6f) : fminf(len, S.fit);
-  S.fit *= 1.1f;
-  R.ta = t0;
-  R.te = kind == 1 || S.step < len ? fminf(t1, t0 + S.step) : t1;
-  if (R.te >= t1) R.te = t1 * (1.0f + 1e-7f) + 1e-30f;  // last window includes t1
+  S.lim = kFill * (float)kSlotCh / chords_per_length(F, m.bits);
+  const Window w = window_first(kind == 1, t0, t1, S.lim);
+  R.ta = w.ta;
+  R.te = w.te;
+  S.step = w.step;
   return true;
 }
 
@@ -607,7 +613,6 @@ __device__ __forceinline__ void render_paths(const Work& Wk, const float* env, W
   S.kind = 0;
   S.acc = 0;
   S.allow = ~0ull;
-  S.fit = INFINITY;
 
   // Move the lane's path on from its finished ray (hit: a collision at th on a
   // tracking ray; kind 0: the lane has no path yet) until a new ray starts or
@@ -740,41 +745,33 @@ __device__ __forceinline__ void render_paths(const Work& Wk, const float* env, W
       GF_TIC(t_dec);
       if (want) {
         const bool last = R.te >= S.t1;
-        bool next_window = false;
+        Window w{R.ta, R.te, S.step};
         if (ovf) {
-          const float w = R.te - R.ta;
-          if (w <= 1e-6f * (1.0f + fabsf(R.ta))) {
-            // more than kPK points at one t: give up on this ray
+          if (!window_halve(w)) {
+            // more points or chords at one t than a window holds: give up on this ray
             set_err(Wk.err_field(), ERR_POINTS);
             fin = true;
-          } else {
-            R.te = R.ta + 0.5f * w;
-            S.step = 0.5f * w;
-            if (R.nch > kSlotCh) S.fit = 0.5f * w;
           }
-        } else if (S.kind == 1) {
-          for (int i = 0; i < n && !fhit; ++i) {
-            if (R.pu[i] * slot_sum(Q, lane, i, 1) < fmaxf(slot_sum(Q, lane, i, 0), 0.f)) {
-              fhit = true;
-              fth = R.pt[i];
+        } else {
+          if (S.kind == 1) {
+            for (int i = 0; i < n && !fhit; ++i) {
+              if (R.pu[i] * slot_sum(Q, lane, i, 1) < fmaxf(slot_sum(Q, lane, i, 0), 0.f)) {
+                fhit = true;
+                fth = R.pt[i];
+              }
+            }
+          } else {
+            for (int i = 0; i < n; ++i) {
+              const float kb = slot_sum(Q, lane, i, 1);
+              if (kb > 0.f) S.T *= 1.f - fmaxf(slot_sum(Q, lane, i, 0), 0.f) / kb;
             }
           }
           fin = fhit || last;
-          next_window = !fin;
-        } else {
-          for (int i = 0; i < n; ++i) {
-            const float kb = slot_sum(Q, lane, i, 1);
-            if (kb > 0.f) S.T *= 1.f - fmaxf(slot_sum(Q, lane, i, 0), 0.f) / kb;
-          }
-          if (!last) S.step *= 2.0f;
-          fin = last;
-          next_window = !last;
+          if (!fin) window_next(w, S.kind == 1, S.lim, S.t1);
         }
-        if (next_window) {
-          R.ta = R.te;
-          R.te = fminf(S.t1, R.ta + S.step);
-          if (R.te >= S.t1) R.te = S.t1 * (1.0f + 1e-7f) + 1e-30f;
-        }
+        R.ta = w.ta;
+        R.te = w.te;
+        S.step = w.step;
       }
       if (lane == 0) GF_TOC(cnt, 4, t_dec);
     }
@@ -782,6 +779,7 @@ __device__ __forceinline__ void render_paths(const Work& Wk, const float* env, W
     if (fin) advance(fhit, fth);
     __syncwarp();
   }
+  if (S.kind != 0) set_err(Wk.err_field(), ERR_GUARD);  // paths left over
   flush_counters(Wk.err_field(), cnt, lane);
 }
 
