@@ -12,6 +12,7 @@
 
 #include "gf_host.h"
 #include "gf_trace.cuh"
+#include "gf_words.h"
 
 using namespace gf;
 
@@ -380,8 +381,8 @@ gf_status gf_load_field(gf_ctx* ctx, const gf_params* p, const gf_field_opts* op
                         gf_stream stream, gf_field** out) {
   if (!ctx || !p || !opts || !out) return fail(GF_EINVAL, "null argument");
   *out = nullptr;
-  // node and primitive indices share a 32-bit word with a 5-bit lane index
-  if (p->n < 1 || p->n >= (1ll << 26)) return fail(GF_EINVAL, "n must be in [1, 2^26)");
+  // node and primitive indices share a 32-bit word with a 5-bit lane index (gf_words.h)
+  if (p->n < 1 || p->n >= kMaxPrims) return fail(GF_EINVAL, "n must be in [1, 2^26)");
   if (!p->mu || !p->quat || !p->log_scale || !p->omega || !p->phase || !p->weight)
     return fail(GF_EINVAL, "parameter array null");
   if (!(opts->k_sigma > 0.f && opts->k_sigma <= 6.f)) return fail(GF_EINVAL, "k_sigma in (0,6]");

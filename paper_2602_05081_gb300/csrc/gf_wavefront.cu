@@ -30,6 +30,7 @@
 #include "gf_host.h"
 #include "gf_trace.cuh"
 #include "gf_window.h"
+#include "gf_words.h"
 
 namespace gf {
 
@@ -88,8 +89,8 @@ constexpr int kWStack = 640;
 constexpr int kStackMargin = 96;
 static_assert(32 * kMaxRoots + 96 <= kWStack - kStackMargin, "full steps on the first roots");
 struct TravQ {
-  int stk[kWStack];   // (node << 5) | slot
-  int lq[kLeafQ];     // (sorted primitive << 5) | slot; directly behind the stack
+  int stk[kWStack];   // index_word(node, slot)
+  int lq[kLeafQ];     // index_word(sorted primitive, slot); directly behind the stack
   ChordItem cq[kChordQ];
 };
 static_assert(offsetof(TravQ, lq) == kWStack * sizeof(int), "queue behind the stack");
@@ -226,7 +227,8 @@ __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, c
       const unsigned b = __ballot_sync(kFull, has);
       if (b == 0u) break;
       if (has)
-        Q.t.stk[sp + __popc(b & lt)] = (next_root(Wk.field(Q.r[lane].asset), cm, bm) << 5) | (int)lane;
+        Q.t.stk[sp + __popc(b & lt)] =
+            (int)index_word((uint32_t)next_root(Wk.field(Q.r[lane].asset), cm, bm), lane);
       sp += __popc(b);
     }
     __syncwarp();
@@ -244,10 +246,10 @@ __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, c
     // near capacity fewer, down to one: a node leaves room for three more entries, and
     // a descent adds at most three per level
     take = min(take, max(1, (kWStack - kStackMargin - sp) / 3));
-    int ent[kPerStep];
+    uint32_t ent[kPerStep];
 #pragma unroll
     for (int u = 0; u < kPerStep; ++u)
-      ent[u] = 32 * u + (int)lane < take ? Q.t.stk[sp - take + 32 * u + (int)lane] : -1;
+      ent[u] = 32 * u + (int)lane < take ? (uint32_t)Q.t.stk[sp - take + 32 * u + (int)lane] : kNoWord;
     __syncwarp();
     sp -= take;
     if (lane == 0) ++cnt.steps;
@@ -258,21 +260,21 @@ __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, c
 #pragma unroll
     for (int u = 0; u < kPerStep; ++u) {
       if (u > 0 && take <= 32 * u) break;  // (the same in every lane)
-      if (ent[u] < 0) continue;
-      const LaneRay& R = Q.r[ent[u] & 31];
+      if (ent[u] == kNoWord) continue;
+      const LaneRay& R = Q.r[word_slot(ent[u])];
       const DevField& F = Wk.field(R.asset);
-      if ((int64_t)(ent[u] >> 5) >= F.n_nodes4) {
+      if ((int64_t)word_index(ent[u]) >= F.n_nodes4) {
         set_err(Wk.err_field(), ERR_INDEX);  // a node beyond the tree: skipped
         continue;
       }
       const float3 o = make_float3(R.o[0], R.o[1], R.o[2]);
       const float3 inv = make_float3(R.inv[0], R.inv[1], R.inv[2]);
       ++cnt.nodes;
-      hit |= node4_hits(F.nodes4 + (ent[u] >> 5), o, inv, R.ta, R.te, ch + 4 * u) << (4 * u);
+      hit |= node4_hits(F.nodes4 + word_index(ent[u]), o, inv, R.ta, R.te, ch + 4 * u) << (4 * u);
     }
     // ---------------- push internal children, queue leaves
     if (!push_hits(Q.t.stk, kWStack, hit, ch, lane, sp, lq_n,
-                   [&](int k, int c) { return (c << 5) | (ent[k >> 2] & 31); }) &&
+                   [&](int k, int c) { return (int)index_word((uint32_t)c, word_slot(ent[k >> 2])); }) &&
         lane == 0)
       set_err(Wk.err_field(), ERR_STACK);
     __syncwarp();
@@ -286,9 +288,9 @@ __device__ void warp_phase(const Work& Wk, WarpQ& Q, bool want, uint32_t lane, c
       bool have = (int)lane < tk;
       int j = 0, own = 0;
       if (have) {
-        const int e = Q.t.lq[lq_n - tk + (int)lane];
-        j = e >> 5;
-        own = e & 31;
+        const uint32_t e = (uint32_t)Q.t.lq[lq_n - tk + (int)lane];
+        j = (int)word_index(e);
+        own = (int)word_slot(e);
         if ((int64_t)j >= Wk.field(Q.r[own].asset).n) {  // a leaf beyond the records
           set_err(Wk.err_field(), ERR_INDEX);
           have = false;

@@ -12,10 +12,12 @@
 #pragma once
 #include <math.h>
 
+#ifndef GF_HD
 #ifdef __CUDACC__
 #define GF_HD __host__ __device__ __forceinline__
 #else
 #define GF_HD inline
+#endif
 #endif
 
 namespace gf {
