@@ -283,7 +283,10 @@ gf_status gf_build_bvh(gf_field* field, gf_stream stream);
    chords each for gf_ray_chords), max_pixels pixels of gf_render (the pixel
    sums of the scattering renderer and the staging of a host image), and
    the per-warp chord store of the scattering renderer when render != 0, and
-   the adjoints' chord lists when adjoint != 0.  Sizes only
+   the adjoints' chord lists when adjoint != 0.  Where the
+   chord store or the lists are refused, half as much is asked for, and so on:
+   GF_OK with less, calls then run on fewer blocks with the same results and
+   still allocate nothing (a further gf_reserve asks again).  Sizes only
    grow; zeros leave a part as it is.  GF_ESTATE before gf_build_bvh. */
 typedef struct gf_reserve_opts {
   int64_t max_rays;

@@ -1476,7 +1476,7 @@ static size_t rad_scratch(const Field& F, int64_t g) {
 // field's allocator; g comes back smaller when less scratch is to be had
 static cudaError_t grow_adjoint(const Field& F, size_t bytes, int64_t& g, cudaStream_t s) {
   const cudaError_t e = grow(F, (void**)&F.adj, F.adj_bytes, (size_t)F.n * 7 * sizeof(float4), s);
-  return e != cudaSuccess ? e : grow_shares(F, (void**)&F.rlist, F.rlist_bytes, bytes / g, g, s);
+  return e != cudaSuccess ? e : grow_shares(F, F.rlist, bytes / g, g, s);
 }
 
 // the scratch of every adjoint
@@ -1521,7 +1521,7 @@ static cudaError_t launch_adjoint(const Field& F, const PathParams& P,
   k_adj_prims<<<pb, 256, 0, s>>>(F.dev.rec, B, F.adj);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   kernel<<<(unsigned)g, kBackBlock, smem, s>>>(F.dev, P, B, dLdI, F.counter, (int)chunk,
-                                              reinterpret_cast<T*>(F.rlist));
+                                              static_cast<T*>(F.rlist.p));
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_adj_finish<<<pb, 256, 0, s>>>(F.dev.rec, B);
   return cudaGetLastError();

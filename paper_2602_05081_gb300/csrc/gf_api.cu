@@ -163,13 +163,35 @@ cudaError_t grow(const Field& F, void** p, size_t& have, size_t bytes, cudaStrea
   return e;
 }
 
-cudaError_t grow_shares(const Field& F, void** p, size_t& have, size_t share, int64_t& shares,
-                        cudaStream_t s) {
-  for (;; shares = (shares + 1) / 2) {
-    const cudaError_t e = grow(F, p, have, share * (size_t)shares, s);
-    if (e != cudaErrorMemoryAllocation || shares <= 1) return e;
-    (void)cudaGetLastError();
+cudaError_t grow_shares(const Field& F, ShareBuf& b, size_t share, int64_t& shares, cudaStream_t s) {
+  const int64_t held = b.p ? (int64_t)(b.bytes / share) : 0;
+  if (held >= shares) return cudaSuccess;
+  if (held > 0) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    (void)cudaStreamIsCapturing(s, &cap);
+    if (b.scarce || cap != cudaStreamCaptureStatusNone) {
+      shares = held;
+      return cudaSuccess;
+    }
   }
+  for (int64_t k = shares; k > held; k /= 2) {
+    void* q = nullptr;
+    const cudaError_t e = F.mem.alloc(&q, share * (size_t)k, s);
+    if (e == cudaSuccess) {
+      // (the buffer before it stays until the field is freed: work in flight and captured
+      // graphs may use it)
+      b.p = q;
+      b.bytes = share * (size_t)k;
+      shares = k;
+      return e;
+    }
+    if (e != cudaErrorMemoryAllocation) return e;
+    (void)cudaGetLastError();
+    b.scarce = true;
+  }
+  if (held == 0) return cudaErrorMemoryAllocation;
+  shares = held;
+  return cudaSuccess;
 }
 
 // The field's device error word, read after the stream has been synchronised
@@ -590,6 +612,7 @@ gf_status gf_reserve(gf_field* h, const gf_reserve_opts* o, gf_stream stream) {
   if (npix && o->adjoint) stage = std::max(stage, npix * 4 + (size_t)F.n * 60 + 512);
   gf_status st;
   if (stage && (st = ensure_stage(F, stage, s))) return st;
+  F.wscratch.scarce = F.rlist.scarce = false;  // more may be had by now
   if (o->render && npix) GF_CUDA(ensure_render_scratch(F, (int64_t)npix, s), "render scratch");
   if (o->adjoint) GF_CUDA(ensure_adjoint_lists(F, s), "adjoint lists");
   return GF_OK;

@@ -102,6 +102,12 @@ inline __host__ __device__ int cell_fix_exp(unsigned int mb) {
   int e = (int)((mb >> 23) & 0xFFu) - 126;
   return e < -60 ? -60 : (e > 100 ? 100 : e);
 }
+// A buffer of equal shares, one per block of a persistent grid (grow_shares)
+struct ShareBuf {
+  void* p = nullptr;
+  size_t bytes = 0;
+  bool scarce = false;  // more was refused: calls make do with what there is
+};
 struct Field {
   Ctx ctx;                     // copy: a field outlives the gf_ctx it came from
   mutable DevMem mem;          // every device buffer of the field, through ctx.alloc
@@ -146,15 +152,13 @@ struct Field {
   void* stage = nullptr;
   size_t stage_bytes = 0;
   // per-warp chord store of the scattering renderer (grows on demand)
-  mutable float4* wscratch = nullptr;
-  mutable size_t wscratch_bytes = 0;
+  mutable ShareBuf wscratch;
   // fixed-point pixel sums of the scattering renderer (grows on demand)
   mutable unsigned long long* acc64 = nullptr;
   mutable size_t acc_bytes = 0;
   // per-warp chord lists and kept moments of the radiance adjoints, kept chords of the
   // tomography adjoint (grows on demand)
-  mutable int* rlist = nullptr;
-  mutable size_t rlist_bytes = 0;
+  mutable ShareBuf rlist;
   // per primitive in BVH order: the adjoint's gathered parameters (3 float4), then its
   // gradient sums (4 float4)
   mutable float4* adj = nullptr;
@@ -218,10 +222,11 @@ cudaError_t ensure_adjoint_lists(const Field& F, cudaStream_t s);
 // grow a field-owned buffer to at least `bytes` (synchronises the device before
 // returning the old one)
 cudaError_t grow(const Field& F, void** p, size_t& have, size_t bytes, cudaStream_t s);
-// the same for `shares` equal shares (the blocks of a persistent grid); when the memory is
-// refused, half as many and so on down to one: a kernel of fewer blocks, same results
-cudaError_t grow_shares(const Field& F, void** p, size_t& have, size_t share, int64_t& shares,
-                        cudaStream_t s);
+// `shares` equal shares in b; when the memory is refused, half as many and so on down to one:
+// a kernel of fewer blocks, same results.  Once refused, what is held serves every later
+// call (gf_reserve asks again), and under a stream capture what is held serves anyway; a
+// buffer is never given up for one that might be refused.
+cudaError_t grow_shares(const Field& F, ShareBuf& b, size_t share, int64_t& shares, cudaStream_t s);
 cudaError_t launch_radiance_backward(const Field& F, const PathParams& P, const float* dLdI,
                                      float* grad, cudaStream_t s);
 cudaError_t launch_tomo_backward(const Field& F, const PathParams& P, const float* dLdI,

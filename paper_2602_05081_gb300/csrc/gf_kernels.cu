@@ -519,17 +519,17 @@ cudaError_t launch_render(const Field& F, const PathParams& P, float* out, cudaS
     // memory (refused, or not reserved before a stream capture) each depth traverses
     int cap = kFlightList;
     const size_t need = flight_store_bytes(F);
-    if (F.wscratch_bytes < need) {
+    if (F.wscratch.bytes < need) {
       cudaStreamCaptureStatus cap_st = cudaStreamCaptureStatusNone;
       (void)cudaStreamIsCapturing(s, &cap_st);
       if (cap_st != cudaStreamCaptureStatusNone ||
-          grow(F, (void**)&F.wscratch, F.wscratch_bytes, need, s) != cudaSuccess) {
+          grow(F, &F.wscratch.p, F.wscratch.bytes, need, s) != cudaSuccess) {
         (void)cudaGetLastError();
         cap = 0;
       }
     }
     k<<<(unsigned)g, kBlock, 0, s>>>(F.dev, P, out, F.counter,
-                                     reinterpret_cast<FlightRec*>(cap ? F.wscratch : nullptr), cap);
+                                     static_cast<FlightRec*>(cap ? F.wscratch.p : nullptr), cap);
   } else {
     if (!stack_fits(k_tomo)) return cudaErrorLaunchOutOfResources;
     k_tomo<<<persistent_grid(F, k_tomo, npix), kBlock, 0, s>>>(F.dev, P, out, F.counter);

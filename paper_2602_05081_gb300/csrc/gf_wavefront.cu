@@ -880,7 +880,7 @@ static cudaError_t render_scratch(const Field& F, int64_t npix, int64_t& g, cuda
   if (e != cudaSuccess) return e;
   if ((e = grow(F, (void**)&F.acc64, F.acc_bytes, (size_t)npix * 8, s)) != cudaSuccess) return e;
   const size_t share = std::max(scatter_store_bytes(1), (flight_store_bytes(F) + g - 1) / g);
-  return grow_shares(F, (void**)&F.wscratch, F.wscratch_bytes, share, g, s);
+  return grow_shares(F, F.wscratch, share, g, s);
 }
 cudaError_t ensure_render_scratch(const Field& F, int64_t npix, cudaStream_t s) {
   int64_t g = 1;
@@ -905,7 +905,7 @@ cudaError_t launch_render_scatter(const Field& F, const PathParams& P, float* ou
   const int slots = scatter_slots(npix * nchunk, g);
   auto kernel = nodes_per_step(P.lod, P.lod_nee) == 2 ? k_render_scatter<2> : k_render_scatter<1>;
   kernel<<<(unsigned)g, kWWarps * 32, scatter_smem_bytes(), s>>>(F.dev, P, F.acc64, F.counter, (int)chunk,
-                                                                 slots, F.wscratch);
+                                                                 slots, static_cast<float4*>(F.wscratch.p));
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_fix_to_image<<<(unsigned)((npix + 255) / 256), 256, 0, s>>>(F.acc64, npix, P.spp, out);
   return cudaGetLastError();

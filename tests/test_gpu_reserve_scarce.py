@@ -1,0 +1,89 @@
+"""gf_reserve under an allocator that refuses large blocks (GPU).
+
+Later calls within the reserved sizes ask the allocator for nothing, whatever it refused,
+and so run under stream capture; a further gf_reserve asks again.
+"""
+import pytest
+
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2602_05081_gb300 import api as _api
+    return _api
+
+
+class _Limited:
+    """A context whose allocator refuses blocks above `limit` bytes and counts its calls."""
+
+    def __init__(self, api, limit):
+        from paper_2602_05081_gb300 import _abi
+        self.limit, self.asked, self.refused = limit, 0, 0
+        al = api.TorchAllocator(0)
+        inner = al._on_alloc
+
+        def on_alloc(user, nbytes, stream):
+            self.asked += 1
+            if nbytes > self.limit:
+                self.refused += 1
+                return None
+            return inner(user, nbytes, stream)
+
+        al._alloc = _abi.ALLOC_FN(on_alloc)
+        al.c = _abi.gf_allocator(al._alloc, al._free, None)
+        self.ctx = api.Context(0, allocator=al)
+        self.freed = lambda: al.calls_free
+
+
+def test_calls_after_a_refused_reserve_allocate_nothing(api):
+    L = _Limited(api, 48 << 20)
+    c = synth.DEFAULT_CAMERA
+    cam = api.camera(c["eye"], c["look_at"], c["up"], c["vfov_deg"], 48, 40)
+    f = api.Field(L.ctx, synth.octave_field(2000, 4, seed=4))
+    f.reserve(max_pixels=48 * 40, render=True, adjoint=True)
+    assert L.refused > 0
+    asked, freed = L.asked, L.freed()
+    dL = torch.ones(40, 48, device="cuda")
+    out = torch.empty(40, 48, device="cuda")
+    opts = {"single": api.render_opts("scatter", 2, 1), "path": api.render_opts("scatter", 1, 3),
+            "tomo": api.render_opts("tomo", 2)}
+    images = {}
+    for k, o in opts.items():
+        images[k] = f.render(cam, o, 3, out=out).clone()
+        f.render_backward(cam, o, 4, dL)
+    f.sync()
+    assert (L.asked, L.freed()) == (asked, freed)
+    # captured, and the same image
+    g = torch.cuda.CUDAGraph()
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(g, stream=s):
+        f.render(cam, opts["path"], 3, out=out, stream=s.cuda_stream)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, images["path"])
+    assert (L.asked, L.freed()) == (asked, freed)
+    # asked again, more is had, and the captured render still has its memory
+    L.limit = 1 << 40
+    f.reserve(max_pixels=48 * 40, render=True, adjoint=True)
+    assert L.asked > asked
+    asked, freed = L.asked, L.freed()
+    for k, o in opts.items():
+        assert torch.equal(images[k], f.render(cam, o, 3, out=out)), k
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, images["path"])
+    assert (L.asked, L.freed()) == (asked, freed)
+    del g
+    f.free()
+    L.ctx.close()
