@@ -87,3 +87,50 @@ def test_calls_after_a_refused_reserve_allocate_nothing(api):
     del g
     f.free()
     L.ctx.close()
+
+
+@pytest.mark.parametrize("ff", ["cdf", "segment"])
+def test_flights_take_what_is_held(api, ff):
+    """The chord lists of an analytic flight: within the reserved store, by the launch's own
+    grid, and with the same image from fewer blocks or without lists."""
+    c = synth.DEFAULT_CAMERA
+    cam = api.camera(c["eye"], c["look_at"], c["up"], c["vfov_deg"], 120, 80)
+    o = api.render_opts("scatter", 1, 2, free_flight=ff)
+    p = synth.octave_field(2000, 4, seed=4)
+    images = []
+    for limit in (1 << 40, 200 << 20, 8 << 20):  # lists for every block, for a quarter, for none
+        L = _Limited(api, limit)
+        f = api.Field(L.ctx, p)
+        if limit == 200 << 20:
+            f.reserve(max_pixels=120 * 80, render=True)
+        asked, freed = L.asked, L.freed()
+        images.append(f.render(cam, o, 3).clone())
+        f.sync()
+        if limit == 200 << 20:
+            assert (L.asked, L.freed()) == (asked, freed)
+        f.free()
+        L.ctx.close()
+    assert torch.equal(images[0], images[1]) and torch.equal(images[0], images[2])
+    # a small image needs few lists, and a captured flight keeps them when the field's
+    # store grows
+    L = _Limited(api, 1 << 40)
+    f = api.Field(L.ctx, p)
+    small = api.camera(c["eye"], c["look_at"], c["up"], c["vfov_deg"], 16, 8)
+    out = torch.empty(8, 16, device="cuda")
+    live = L.ctx.allocator.live_bytes
+    want = f.render(small, o, 3, out=out).clone()
+    assert L.ctx.allocator.live_bytes - live <= 64 << 20
+    g = torch.cuda.CUDAGraph()
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(g, stream=s):
+        f.render(small, o, 3, out=out, stream=s.cuda_stream)
+    f.render(cam, api.render_opts("scatter", 1, 2), 3)
+    f.render(cam, o, 3)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    del g
+    f.free()
+    L.ctx.close()
