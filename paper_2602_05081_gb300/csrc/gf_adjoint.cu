@@ -29,9 +29,28 @@ struct BackArgs {
   int frame, wmode;
   int64_t n;
   float* grad;
+  // null where the memory is not to be had (tomography): parameters are then read in the
+  // caller's order and gradients added to grad itself
   const float4* adj;  // per primitive (BVH order): what PrimDeriv::load needs, 3 float4
   float4* acc;        // gradient sums per primitive (BVH order), 4 float4 each
 };
+
+// what the gradient of a primitive needs besides its record
+struct AdjPrim {
+  float4 q;      // unit quaternion
+  float4 is;     // 1 / scales, 1 / |q|
+  float4 carry;  // input carrier, dA/dweight
+};
+// of original primitive i with amplitude A
+__device__ __forceinline__ AdjPrim adj_prim(const BackArgs& B, int64_t i, float A) {
+  float q[4];
+  for (int k = 0; k < 4; ++k) q[k] = B.quat[4 * i + k];
+  const float iqn = 1.f / sqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
+  return AdjPrim{make_float4(q[0] * iqn, q[1] * iqn, q[2] * iqn, q[3] * iqn),
+                 make_float4(1.f / expf(B.ls[3 * i]), 1.f / expf(B.ls[3 * i + 1]), 1.f / expf(B.ls[3 * i + 2]), iqn),
+                 make_float4(B.om[3 * i], B.om[3 * i + 1], B.om[3 * i + 2],
+                             B.wmode == GF_WEIGHT_NORMALIZED ? A / B.w[i] : 1.f)};
+}
 
 // Derivatives of one kernel g = A exp(-q/2) cos(theta) with respect to its 15
 // raw parameters (mu 3, quaternion 4 through qhat = q/|q|, log scale 3, omega 3
@@ -47,7 +66,10 @@ struct PrimDeriv {
   // from the parameters k_adj_prims gathered for sorted primitive j
   __device__ __forceinline__ void load(const BackArgs& B, float amp, float3 omega, int j) {
     const float4* r = B.adj + 3 * (int64_t)j;
-    const float4 a = __ldg(r), b = __ldg(r + 1), c = __ldg(r + 2);
+    load(B, amp, omega, AdjPrim{__ldg(r), __ldg(r + 1), __ldg(r + 2)});
+  }
+  __device__ __forceinline__ void load(const BackArgs& B, float amp, float3 omega, const AdjPrim& p) {
+    const float4 a = p.q, b = p.is, c = p.carry;
     qh[0] = a.x; qh[1] = a.y; qh[2] = a.z; qh[3] = a.w;
     is[0] = b.x; is[1] = b.y; is[2] = b.z;
     iqn = b.w;
@@ -174,15 +196,10 @@ __global__ void k_adj_prims(const float4* rec, const BackArgs B, float4* adj) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= B.n) return;
   const int64_t i = __float_as_uint(rec[4 * j + 3].w) & kOrigMask;
-  float q[4];
-  for (int k = 0; k < 4; ++k) q[k] = B.quat[4 * i + k];
-  const float iqn = 1.f / sqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
-  const float A = rec[4 * j].w;
-  adj[3 * j] = make_float4(q[0] * iqn, q[1] * iqn, q[2] * iqn, q[3] * iqn);
-  adj[3 * j + 1] = make_float4(1.f / expf(B.ls[3 * i]), 1.f / expf(B.ls[3 * i + 1]),
-                               1.f / expf(B.ls[3 * i + 2]), iqn);
-  adj[3 * j + 2] = make_float4(B.om[3 * i], B.om[3 * i + 1], B.om[3 * i + 2],
-                               B.wmode == GF_WEIGHT_NORMALIZED ? A / B.w[i] : 1.f);
+  const AdjPrim p = adj_prim(B, i, rec[4 * j].w);
+  adj[3 * j] = p.q;
+  adj[3 * j + 1] = p.is;
+  adj[3 * j + 2] = p.carry;
 }
 
 // the sums of every primitive to the caller's layout and order
@@ -212,6 +229,22 @@ __device__ __forceinline__ void add_grad4(const BackArgs& B, int j, const float 
   red_add4(p + 1, scale * acc[4], scale * acc[5], scale * acc[6], scale * acc[7]);
   red_add4(p + 2, scale * acc[8], scale * acc[9], scale * acc[10], scale * acc[11]);
   red_add4(p + 3, scale * acc[12], scale * acc[13], scale * acc[14], 0.f);
+}
+
+// straight to the caller's gradient of original primitive i
+__device__ __forceinline__ void add_grad(const BackArgs& B, int64_t i, const float acc[15], float scale) {
+  const int64_t N = B.n;
+  float* g = B.grad;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    atomicAdd(g + 3 * i + k, scale * acc[k]);
+    atomicAdd(g + 7 * N + 3 * i + k, scale * acc[7 + k]);
+    atomicAdd(g + 10 * N + 3 * i + k, scale * acc[10 + k]);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) atomicAdd(g + 3 * N + 4 * i + k, scale * acc[3 + k]);
+  atomicAdd(g + 13 * N + i, scale * acc[13]);
+  atomicAdd(g + 14 * N + i, scale * acc[14]);
 }
 
 // ---------------------------------------------------------------------------
@@ -287,10 +320,12 @@ __device__ __forceinline__ TomoChord tomo_moments(const TomoItem& q, const float
 }
 
 // dL/dtau times the gradient of one chord's integral
+template <bool SCRATCH>
 __device__ __forceinline__ void tomo_scatter(const BackArgs& B, const Prim& P, const Chord& ch,
                                              const TomoChord& m, float3 v, int j, float dLdtau) {
   PrimDeriv D;
-  D.load(B, P.A, P.om, j);
+  if (SCRATCH) D.load(B, P.A, P.om, j);
+  else D.load(B, P.A, P.om, adj_prim(B, P.orig, P.A));
   PrimDeriv::Moments M = D.moments(ch.p, v, m.C0, m.C1, m.C2, m.S0, m.S1);
   // chord ends that lie on the ellipsoid (not on t = 0)
 #pragma unroll 1
@@ -298,9 +333,13 @@ __device__ __forceinline__ void tomo_scatter(const BackArgs& B, const Prim& P, c
     D.end(ch, v, e ? ch.dtout : ch.dtin, e ? 1.f : -1.f, M);
   float acc[15];
   D.grad(ch.p, v, M, acc);
-  add_grad4(B, j, acc, dLdtau);
+  if (SCRATCH) add_grad4(B, j, acc, dLdtau);
+  else add_grad(B, P.orig, acc, dLdtau);
 }
 
+// SCRATCH: with the arrays per primitive and kept chords (store); without, every ray is
+// traversed twice
+template <bool SCRATCH>
 __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
     k_tomo_backward(const __grid_constant__ DevField F, const PathParams P, const BackArgs Bk,
                     const float* dLdI, int* counter, int chunk, TomoChord* store) {
@@ -342,7 +381,7 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
         if (have) {
           ++cnt.chords;
           const TomoChord m = tomo_moments(q, sm.glx, sm.glw, s_acc, c_acc, cnt);
-          if (nch + (int)lane < kTomoChords) store[nch + (int)lane] = m;
+          if (SCRATCH && nch + (int)lane < kTomoChords) store[nch + (int)lane] = m;
         }
         nch += tk;
       };
@@ -377,12 +416,12 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
       warp_sum_pair(s_acc, c_acc);
       const float dLdtau = -gI * expf(-__fadd_rn(s_acc, c_acc)) / (float)P.spp;
       __syncwarp();  // the kept chords are read by other lanes
-      if (nch <= kTomoChords) {
+      if (SCRATCH && nch <= kTomoChords) {
         for (int k = (int)lane; k < nch; k += 32) {
           const TomoChord m = store[k];
           const Prim Pr = load_prim(F, m.j);
           Chord ch;
-          if (chord_setup(Pr, o, v, 0.f, INFINITY, Pr.k2, ch)) tomo_scatter(Bk, Pr, ch, m, v, m.j, dLdtau);
+          if (chord_setup(Pr, o, v, 0.f, INFINITY, Pr.k2, ch)) tomo_scatter<SCRATCH>(Bk, Pr, ch, m, v, m.j, dLdtau);
         }
       } else {
         coop_traverse(F, Q.t, F.occupied, o, inv, t0, t1, lane, cnt, [&](int j) {
@@ -392,7 +431,7 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
           if (!chord_setup(Pr, o, v, 0.f, INFINITY, Pr.k2, ch)) return;
           float s2 = 0.f, c2 = 0.f;
           const TomoChord m = tomo_moments(tomo_item(ch, j), sm.glx, sm.glw, s2, c2, cnt);
-          tomo_scatter(Bk, Pr, ch, m, v, j, dLdtau);
+          tomo_scatter<SCRATCH>(Bk, Pr, ch, m, v, j, dLdtau);
         });
       }
       __syncwarp();  // before the next ray's chords overwrite the store
@@ -1484,7 +1523,7 @@ cudaError_t ensure_adjoint_lists(const Field& F, cudaStream_t s) {
   int64_t g = 1;
   size_t bytes = 0;
   cudaError_t e;
-  if ((e = adjoint_grid(F, k_tomo_backward, 0, g)) != cudaSuccess) return e;
+  if ((e = adjoint_grid(F, k_tomo_backward<true>, 0, g)) != cudaSuccess) return e;
   bytes = tomo_scratch(g);
   if ((e = adjoint_grid(F, k_radiance_backward<false>, kRadSmem, g)) != cudaSuccess) return e;
   bytes = std::max(bytes, rad_scratch(F, g));
@@ -1494,11 +1533,14 @@ cudaError_t ensure_adjoint_lists(const Field& F, cudaStream_t s) {
 }
 
 // An adjoint kernel over units of `chunk` samples of a pixel (about 16 per warp of the
-// grid at least), between the per-primitive inputs and the copy of the sums to grad
+// grid at least), between the per-primitive inputs and the copy of the sums to grad; bare: a
+// kernel that goes without scratch, where it is not to be had (null: the call fails)
 template <class T>
-static cudaError_t launch_adjoint(const Field& F, const PathParams& P,
-                                  void (*kernel)(DevField, PathParams, BackArgs, const float*, int*, int, T*),
-                                  size_t smem, const float* dLdI, float* grad, cudaStream_t s) {
+using AdjointKernel = void (*)(DevField, PathParams, BackArgs, const float*, int*, int, T*);
+template <class T>
+static cudaError_t launch_adjoint(const Field& F, const PathParams& P, AdjointKernel<T> kernel,
+                                  AdjointKernel<T> bare, size_t smem, const float* dLdI, float* grad,
+                                  cudaStream_t s) {
   (void)cudaGetLastError();  // a stale error of an unrelated call is not ours
   cudaError_t e = cudaMemsetAsync(F.counter, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
@@ -1507,35 +1549,54 @@ static cudaError_t launch_adjoint(const Field& F, const PathParams& P,
   if ((e = adjoint_stack_fits(kernel)) != cudaSuccess) return e;
   if ((e = adjoint_grid(F, kernel, smem, g)) != cudaSuccess) return e;
   // (allocated ahead by gf_reserve, else here)
-  if ((e = grow_adjoint(F, smem ? rad_scratch(F, g) : tomo_scratch(g), g, s)) != cudaSuccess) return e;
+  bool scratch = true;
+  if (bare && (!F.adj || !F.rlist.p)) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    (void)cudaStreamIsCapturing(s, &cap);
+    scratch = cap == cudaStreamCaptureStatusNone;
+  }
+  if (scratch && (e = grow_adjoint(F, smem ? rad_scratch(F, g) : tomo_scratch(g), g, s)) != cudaSuccess) {
+    if (!bare || e != cudaErrorMemoryAllocation) return e;
+    (void)cudaGetLastError();
+    scratch = false;
+  }
+  if (!scratch) {
+    kernel = bare;
+    if ((e = adjoint_stack_fits(kernel)) != cudaSuccess) return e;
+    if ((e = adjoint_grid(F, kernel, smem, g)) != cudaSuccess) return e;
+  }
   const int64_t npix = (int64_t)P.cam.W * P.cam.H, warps = g * (kBackBlock / 32);
   int64_t nchunk = (16 * warps + npix - 1) / npix;
   nchunk = nchunk < 1 ? 1 : (nchunk > P.spp ? P.spp : nchunk);
   const int64_t chunk = (P.spp + nchunk - 1) / nchunk;
   const int64_t units = npix * ((P.spp + chunk - 1) / chunk);
   g = std::min(g, (units + kBackBlock / 32 - 1) / (kBackBlock / 32));
-  B.adj = F.adj;
-  B.acc = F.adj + 3 * F.n;
-  if ((e = cudaMemsetAsync(B.acc, 0, (size_t)F.n * 4 * sizeof(float4), s)) != cudaSuccess) return e;
   const unsigned pb = (unsigned)((F.n + 255) / 256);
-  k_adj_prims<<<pb, 256, 0, s>>>(F.dev.rec, B, F.adj);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (scratch) {
+    B.adj = F.adj;
+    B.acc = F.adj + 3 * F.n;
+    if ((e = cudaMemsetAsync(B.acc, 0, (size_t)F.n * 4 * sizeof(float4), s)) != cudaSuccess) return e;
+    k_adj_prims<<<pb, 256, 0, s>>>(F.dev.rec, B, F.adj);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  } else if ((e = cudaMemsetAsync(grad, 0, (size_t)F.n * 15 * sizeof(float), s)) != cudaSuccess) {
+    return e;
+  }
   kernel<<<(unsigned)g, kBackBlock, smem, s>>>(F.dev, P, B, dLdI, F.counter, (int)chunk,
-                                              static_cast<T*>(F.rlist.p));
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_adj_finish<<<pb, 256, 0, s>>>(F.dev.rec, B);
-  return cudaGetLastError();
+                                              scratch ? static_cast<T*>(F.rlist.p) : nullptr);
+  if (scratch && (e = cudaGetLastError()) == cudaSuccess) k_adj_finish<<<pb, 256, 0, s>>>(F.dev.rec, B);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_tomo_backward(const Field& F, const PathParams& P, const float* dLdI,
                                  float* grad, cudaStream_t s) {
-  return launch_adjoint(F, P, k_tomo_backward, 0, dLdI, grad, s);
+  return launch_adjoint<TomoChord>(F, P, k_tomo_backward<true>, k_tomo_backward<false>, 0, dLdI, grad, s);
 }
 
 cudaError_t launch_radiance_backward(const Field& F, const PathParams& P, const float* dLdI,
                                      float* grad, cudaStream_t s) {
-  return launch_adjoint(F, P, P.max_bounces >= 2 ? k_radiance_backward<true> : k_radiance_backward<false>,
-                        kRadSmem, dLdI, grad, s);
+  return launch_adjoint<unsigned char>(
+      F, P, P.max_bounces >= 2 ? k_radiance_backward<true> : k_radiance_backward<false>, nullptr, kRadSmem,
+      dLdI, grad, s);
 }
 
 }  // namespace gf

@@ -3,6 +3,7 @@
 Later calls within the reserved sizes ask the allocator for nothing, whatever it refused,
 and so run under stream capture; a further gf_reserve asks again.
 """
+import numpy as np
 import pytest
 
 import synth
@@ -134,3 +135,53 @@ def test_flights_take_what_is_held(api, ff):
     del g
     f.free()
     L.ctx.close()
+
+
+def test_tomography_adjoint_without_scratch(api):
+    """Refused its arrays, or captured before they exist, the tomography adjoint runs without
+    them.  Gradients are FP32 atomics of the same terms in another order: at most 48 * 40 *
+    2 = 3,840 per entry, each rounding to 2^-24 of a partial sum of at most twice the largest
+    entry: 2 * 3,840 * 2^-24 = 4.6e-4 of it."""
+    c = synth.DEFAULT_CAMERA
+    cam = api.camera(c["eye"], c["look_at"], c["up"], c["vfov_deg"], 48, 40)
+    o = api.render_opts("tomo", 2)
+    dL = torch.ones(40, 48, device="cuda")
+    n = 2000
+    for mode in ("peak", "normalized"):
+        for frame in ("local", "world"):
+            p = {**synth.octave_field(n, 4, seed=4), "weight_mode": mode, "omega_frame": frame}
+            if mode == "normalized":  # the weights that give the same amplitudes
+                s3 = np.exp(np.asarray(p["log_scale"], np.float64)).prod(1)
+                p["weight"] = (p["weight"] * (2 * np.pi) ** 1.5 * s3).astype(np.float32)
+            L = _Limited(api, 1 << 40)
+            f = api.Field(L.ctx, p)
+            # staging reserved by another call, nothing of the adjoint's
+            f.reserve(max_pixels=48 * 40 + 16 * n)
+            asked = L.asked
+            grad = torch.full((15 * n,), 7.0, device="cuda")
+            L.limit = 0
+            f.render_backward(cam, o, 4, dL, grad=grad)
+            f.sync()
+            bare = grad.clone()
+            L.limit = 1 << 40
+            refused = L.asked
+            g = torch.cuda.CUDAGraph()
+            s = torch.cuda.Stream()
+            s.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.graph(g, stream=s):
+                f.render_backward(cam, o, 4, dL, grad=grad, stream=s.cuda_stream)
+            assert L.asked == refused > asked
+            grad.fill_(7.0)
+            g.replay()
+            torch.cuda.synchronize()
+            captured = grad.clone()
+            full = f.render_backward(cam, o, 4, dL)
+            f.sync()
+            assert L.asked > refused and float(full.abs().max()) > 0.0
+            for k, v in api.split_grad(full, n).items():
+                for other in (bare, captured):
+                    d = (v - api.split_grad(other, n)[k]).abs().max() / v.abs().max()
+                    assert float(d) <= 4.6e-4, (mode, frame, k, float(d))
+            del g
+            f.free()
+            L.ctx.close()
