@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kBlock, kCoopBlocks)
 // (the per-thread tracker traverses twice per eight points, its lanes parted), 4.3 ms now;
 // 4,096 rays through 256 kernels: 27 us (rays dealt out).  With 445 kernels over a point
 // (14k in all), 130,000 rays: 135 ms with one ray per lane, 742 when windows were halved
-// for their chords and the rest left to one lane, 26 now.
+// for their chords and the rest left to one lane, 22 now.
 //
 // Terms come in two forms.  Rays of a small batch that fit one window take records
 // centred on the envelope's peak; large batches and other rays take the
@@ -96,32 +96,70 @@ struct RtQ {
   // sqrt(a)); exact, 3 per chord: (tc, t_in, t_out, B), exponent's y2, y1, y0 and the phase
   // at tc, (h, t* - tc, sqrt(a), -)
   float4 rec[kRtRec];
-  float raw[kRtPts], pt[kRtPts];  // points as drawn, and in t order
+  float raw[kRtPts], pt[kRtPts];  // points as drawn (then kappa, with many chords), in t order
+  float kb[kRtPts];               // kappa_bar, with many chords
   int npts;
 };
 
-// the record of a chord in the exact form, and its terms at t (inside the chord)
-__device__ __forceinline__ void rt_record(float4* r, const Chord& ch, float wa, float h) {
-  r[0] = make_float4(ch.tc, ch.tc + ch.dtin, ch.tc + ch.dtout, ch.B);
-  r[1] = make_float4(-0.5f * kLog2e * ch.a, -kLog2e * ch.b, fmaf(-0.5f * kLog2e, ch.g, log2f(wa)), ch.delta);
-  r[2] = make_float4(h, ch.dts, sqrtf(ch.a), 0.f);
-}
-__device__ __forceinline__ void rt_terms(const float4* r, float4 a, float t, const float* env, float& kap,
-                                         float& kb) {
-  const float4 b = r[1], d = r[2];
-  const float dt = t - a.x;
-  kap = fmaf(ex2f(fmaf(fmaf(b.x, dt, b.y), dt, b.z)), cosf_fast(fmaf(a.w, dt, b.w)), kap);
-  int mm = (int)(fabsf(dt - d.y) * d.z);
-  mm = mm > 7 ? 7 : mm;
-  kb = fmaf(d.x, env[mm], kb);
+// The factors of the sorted points from the stored chords: the lane's share of their
+// product; or (add) their sums added to raw and kb.
+__device__ __forceinline__ float rt_points(RtQ& Q, int npts, int nch, bool exact, bool add, const float* env,
+                                           uint32_t lane, Counters& cnt) {
+  float prod = 1.f;
+  for (int q0 = 0; q0 < npts;) {
+    const int left = npts - q0;
+    int sh = 0;  // 2^sh lanes per point
+    while (sh < 5 && left << (sh + 1) <= 32) ++sh;
+    const int pts = min(left, 32 >> sh), sub = (int)(lane & ((1u << sh) - 1u));
+    const bool act = (int)(lane >> sh) < pts;
+    const int i = q0 + (int)(lane >> sh);
+    const float t = act ? Q.pt[i] : 0.f;
+    float kap = 0.f, kb = 0.f;
+    for (int c = act ? sub : nch; c < nch; c += 1 << sh) {
+      const float4 a = Q.rec[exact ? 3 * c : 2 * c];
+      if (!(t >= a.y && t <= a.z)) continue;
+      const float dt = t - a.x;
+      ++cnt.evals;
+      if (exact) {
+        const float4 b = Q.rec[3 * c + 1], d = Q.rec[3 * c + 2];
+        kap = fmaf(ex2f(fmaf(fmaf(b.x, dt, b.y), dt, b.z)), cosf_fast(fmaf(a.w, dt, b.w)), kap);
+        int mm = (int)(fabsf(dt - d.y) * d.z);
+        mm = mm > 7 ? 7 : mm;
+        kb = fmaf(d.x, env[mm], kb);
+      } else {
+        const float4 b = Q.rec[2 * c + 1];
+        kap = fmaf(ex2f(fmaf(b.x, dt * dt, b.y)), cosf_fast(fmaf(a.w, dt, b.z)), kap);
+        int mm = (int)(fabsf(dt) * b.w);
+        mm = mm > 7 ? 7 : mm;
+        kb = fmaf(ex2f(b.y), env[mm], kb);  // h exp(-m^2/2)
+      }
+    }
+    __syncwarp();
+    for (int o2 = 1; o2 < 1 << sh; o2 <<= 1) {
+      kap += __shfl_xor_sync(kFull, kap, o2);
+      kb += __shfl_xor_sync(kFull, kb, o2);
+    }
+    if (act && sub == 0) {
+      if (add) {
+        Q.raw[i] += kap;
+        Q.kb[i] += kb;
+      } else if (kb > 0.f) {
+        prod *= 1.f - kap / kb;
+      }
+    }
+    q0 += pts;
+  }
+  return prod;
 }
 
-// chords and points of the window [ta, tb), or [ta, t1] when last; returns the chords (those
-// beyond the buffer are counted, and draw their points)
+// Chords and points of the window [ta, tb), or [ta, t1] when last; returns the chords (those
+// beyond the buffer are counted, and draw their points).  With many >= 0 sorted points
+// known: their sums instead, the buffer added to them whenever it is nearly full; returns the
+// chords left in it.
 __device__ __forceinline__ int rt_gather(const DevField& F, RtQ& Q, const Mask& M, float3 o, float3 v,
                                          float3 inv, float tmin, float tmax, float ta, float tb,
                                          bool last, uint64_t seed, uint32_t ray, uint32_t word,
-                                         const float* env, uint32_t lane, bool exact, Counters& cnt) {
+                                         const float* env, uint32_t lane, bool exact, int many, Counters& cnt) {
   const unsigned lt = (1u << lane) - 1u;
   const int cap = exact ? kRtRec / 3 : kRtRec / 2;
   int nch = 0;
@@ -141,89 +179,35 @@ __device__ __forceinline__ int rt_gather(const DevField& F, RtQ& Q, const Mask& 
       ++cnt.chords;
       if (k >= cap) {
       } else if (exact) {
-        rt_record(Q.rec + 3 * k, ch, wa, h);
+        Q.rec[3 * k] = make_float4(ch.tc, ch.tc + ch.dtin, ch.tc + ch.dtout, ch.B);
+        Q.rec[3 * k + 1] = make_float4(-0.5f * kLog2e * ch.a, -kLog2e * ch.b,
+                                       fmaf(-0.5f * kLog2e, ch.g, log2f(wa)), ch.delta);
+        Q.rec[3 * k + 2] = make_float4(h, ch.dts, sqrtf(ch.a), 0.f);
       } else {
         Q.rec[2 * k] = make_float4(ch.tc + ch.dts, ch.tc + ch.dtin, ch.tc + ch.dtout, ch.B);
         Q.rec[2 * k + 1] = make_float4(-0.5f * kLog2e * ch.a, __log2f(h),
                                        reduce_2pi(fmaf(ch.B, ch.dts, ch.delta)), sqrtf(ch.a));
       }
-      chord_points(F, ch, h, seed, ray, word, env, [&](float t, float) {
-        if (last ? t > tb : t >= tb) return false;
-        if (t >= ta) {
-          const int q = atomicAdd(&Q.npts, 1);
-          if (q >= kRtPts) return false;  // too many: the window is halved
-          Q.raw[q] = t;
-        }
-        return true;
-      });
+      if (many < 0)
+        chord_points(F, ch, h, seed, ray, word, env, [&](float t, float) {
+          if (last ? t > tb : t >= tb) return false;
+          if (t >= ta) {
+            const int q = atomicAdd(&Q.npts, 1);
+            if (q >= kRtPts) return false;  // too many: the window is halved
+            Q.raw[q] = t;
+          }
+          return true;
+        });
     }
     nch += __popc(bc);
+    if (many >= 0 && nch > cap - 32) {
+      __syncwarp();
+      (void)rt_points(Q, many, nch, true, true, env, lane, cnt);
+      nch = 0;
+    }
   });
   __syncwarp();
   return nch;
-}
-
-// The product of the factors of the window's points when its chords exceed the buffer, each
-// lane's share of it: the window is traversed again, its chords stored (exact form) and,
-// whenever the buffer is nearly full, added to the sums of the points, which the lanes hold
-// (2^sh lanes per point, up to kRtPts / 32 points per lane).
-static __device__ __noinline__ float rt_many(const DevField& F, RtQ& Q, const Mask& M, float3 o, float3 v,
-                                             float3 inv, float tmin, float tmax, float ta, float tb, int npts,
-                                             const float* env, uint32_t lane, Counters& cnt) {
-  constexpr int kGroups = kRtPts / 32;
-  const unsigned lt = (1u << lane) - 1u;
-  int sh = 0;
-  while (sh < 5 && npts << (sh + 1) <= 32) ++sh;
-  const int sub = (int)(lane & ((1u << sh) - 1u));
-  float t[kGroups], kap[kGroups], kb[kGroups];
-#pragma unroll
-  for (int g = 0; g < kGroups; ++g) {
-    const int i = 32 * g + (int)(lane >> sh);
-    t[g] = i < npts && (g == 0 || sh == 0) ? Q.pt[i] : INFINITY;
-    kap[g] = kb[g] = 0.f;
-  }
-  int n = 0;  // stored chords
-  auto add = [&]() {
-    __syncwarp();
-#pragma unroll 1
-    for (int c = sub; c < n; c += 1 << sh) {
-      const float4 a = Q.rec[3 * c];
-#pragma unroll
-      for (int g = 0; g < kGroups; ++g)
-        if (t[g] >= a.y && t[g] <= a.z) {
-          ++cnt.evals;
-          rt_terms(Q.rec + 3 * c, a, t[g], env, kap[g], kb[g]);
-        }
-    }
-    __syncwarp();
-    n = 0;
-  };
-  coop_traverse(F, Q.t, M.bits, o, inv, ta, tb, lane, cnt, [&](int j) {
-    Chord ch;
-    float w;
-    const bool ok = j >= 0 &&
-                    prim_chord(F, j, o, v, tmin, tmax,
-                               [&](uint32_t cl) { return mask_weight(M, cl); }, w, ch) &&
-                    ch.tc + ch.dtin <= tb && ch.tc + ch.dtout >= ta;
-    const unsigned bc = __ballot_sync(kFull, ok);
-    if (ok) {
-      const float wa = w * ch.absA;
-      rt_record(Q.rec + 3 * (n + __popc(bc & lt)), ch, wa, wa * expf(-0.5f * ch.qmin));
-    }
-    n += __popc(bc);
-    if (n > kRtRec / 3 - 32) add();
-  });
-  add();
-  float prod = 1.f;
-#pragma unroll
-  for (int g = 0; g < kGroups; ++g) {
-    for (int o2 = 1; o2 < 1 << sh; o2 <<= 1) {
-      kap[g] += __shfl_xor_sync(kFull, kap[g], o2);
-      kb[g] += __shfl_xor_sync(kFull, kb[g], o2);
-    }
-    if (sub == 0 && kb[g] > 0.f) prod *= 1.f - kap[g] / kb[g];
-  }
-  return prod;
 }
 
 __device__ float rt_coop(const DevField& F, RtQ& Q, const Mask& M, float3 o, float3 v, float3 inv,
@@ -231,87 +215,71 @@ __device__ float rt_coop(const DevField& F, RtQ& Q, const Mask& M, float3 o, flo
                          uint32_t word, const float* env, uint32_t lane, bool exact, Counters& cnt) {
   float prod = 1.f, ta = t0, tb = t1;
   int c8 = 0;           // points since the last multiple of kPts on the ray
+  int many = -1;        // points of a window whose chords exceed the buffer
   bool alone = false;   // to the per-thread tracker
   while (!alone) {
     const bool last = tb >= t1;
     const int nch =
         rt_gather(F, Q, M, o, v, inv, tmin, tmax, ta, tb, last, seed, ray, word, env, lane, exact,
-                  cnt);
-    int npts = Q.npts;
-    __syncwarp();
+                  many, cnt);
     const float w = tb - ta;
-    if (npts > kRtPts) {
-      if (w > 1e-6f * (1.0f + fabsf(ta))) tb = ta + 0.5f * w;
-      else alone = true;
-      exact = true;
-      continue;
-    }
-    const bool many = nch > (exact ? kRtRec / 3 : kRtRec / 2);
-    exact = exact || many;
-    // t order (so that the product does not depend on which lane drew first)
-    bool tie = false;
-    for (int i = (int)lane; i < npts; i += 32) {
-      const float t = Q.raw[i];
-      int rank = 0;
-      for (int k = 0; k < npts; ++k) {
-        const float x = Q.raw[k];
-        rank += x < t || (x == t && k < i) ? 1 : 0;
-        tie = tie || (x == t && k != i);
+    int npts = many;
+    if (many < 0) {
+      npts = Q.npts;
+      __syncwarp();
+      if (npts > kRtPts) {
+        if (w > 1e-6f * (1.0f + fabsf(ta))) tb = ta + 0.5f * w;
+        else alone = true;
+        exact = true;
+        continue;
       }
-      Q.pt[rank] = t;
-    }
-    tie = __any_sync(kFull, exact && tie);
-    __syncwarp();
-    if (tie) {  // leave out points at the end of a run (every lane writes the same)
-      int m = 0;
-      float end = -INFINITY;
-      for (int i = 0; i < npts; ++i) {
-        const float t = Q.pt[i];
+      const bool over = nch > (exact ? kRtRec / 3 : kRtRec / 2);
+      exact = exact || over;
+      // t order (so that the product does not depend on which lane drew first)
+      bool tie = false;
+      for (int i = (int)lane; i < npts; i += 32) {
+        const float t = Q.raw[i];
+        int rank = 0;
+        for (int k = 0; k < npts; ++k) {
+          const float x = Q.raw[k];
+          rank += x < t || (x == t && k < i) ? 1 : 0;
+          tie = tie || (x == t && k != i);
+        }
+        Q.pt[rank] = t;
+      }
+      tie = __any_sync(kFull, exact && tie);
+      __syncwarp();
+      if (tie) {  // leave out points at the end of a run (every lane writes the same)
+        int m = 0;
+        float end = -INFINITY;
+        for (int i = 0; i < npts; ++i) {
+          const float t = Q.pt[i];
+          __syncwarp();
+          if (t == end) continue;
+          Q.pt[m++] = t;
+          if (++c8 == kPts) {
+            c8 = 0;
+            end = t;
+          }
+        }
+        npts = m;
         __syncwarp();
-        if (t == end) continue;
-        Q.pt[m++] = t;
-        if (++c8 == kPts) {
-          c8 = 0;
-          end = t;
-        }
+      } else {
+        c8 = (c8 + npts) % kPts;
       }
-      npts = m;
-      __syncwarp();
-    } else {
-      c8 = (c8 + npts) % kPts;
+      if (lane == 0) cnt.points += (unsigned long long)npts;
+      if (over) {
+        for (int i = (int)lane; i < npts; i += 32) Q.raw[i] = Q.kb[i] = 0.f;
+        many = npts;
+        continue;  // the window again, for the sums
+      }
     }
-    if (lane == 0) cnt.points += (unsigned long long)npts;
-    if (many) prod *= rt_many(F, Q, M, o, v, inv, tmin, tmax, ta, tb, npts, env, lane, cnt);
-    for (int q0 = many ? npts : 0; q0 < npts;) {
-      const int left = npts - q0;
-      int sh = 0;  // 2^sh lanes per point
-      while (sh < 5 && left << (sh + 1) <= 32) ++sh;
-      const int pts = min(left, 32 >> sh), sub = (int)(lane & ((1u << sh) - 1u));
-      const bool act = (int)(lane >> sh) < pts;
-      const float t = act ? Q.pt[q0 + (int)(lane >> sh)] : 0.f;
-      float kap = 0.f, kb = 0.f;
-      for (int c = act ? sub : nch; c < nch; c += 1 << sh) {
-        const float4 a = Q.rec[exact ? 3 * c : 2 * c];
-        if (!(t >= a.y && t <= a.z)) continue;
-        ++cnt.evals;
-        if (exact) {
-          rt_terms(Q.rec + 3 * c, a, t, env, kap, kb);
-        } else {
-          const float4 b = Q.rec[2 * c + 1];
-          const float dt = t - a.x;
-          kap = fmaf(ex2f(fmaf(b.x, dt * dt, b.y)), cosf_fast(fmaf(a.w, dt, b.z)), kap);
-          int mm = (int)(fabsf(dt) * b.w);
-          mm = mm > 7 ? 7 : mm;
-          kb = fmaf(ex2f(b.y), env[mm], kb);  // h exp(-m^2/2)
-        }
-      }
+    prod *= rt_points(Q, npts, nch, exact, many >= 0, env, lane, cnt);
+    if (many >= 0) {
       __syncwarp();
-      for (int o2 = 1; o2 < 1 << sh; o2 <<= 1) {
-        kap += __shfl_xor_sync(kFull, kap, o2);
-        kb += __shfl_xor_sync(kFull, kb, o2);
-      }
-      if (act && sub == 0 && kb > 0.f) prod *= 1.f - kap / kb;
-      q0 += pts;
+      for (int i = (int)lane; i < npts; i += 32)
+        if (Q.kb[i] > 0.f) prod *= 1.f - Q.raw[i] / Q.kb[i];
+      many = -1;
     }
     if (last) break;
     ta = tb;
