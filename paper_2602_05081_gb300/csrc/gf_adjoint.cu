@@ -351,11 +351,11 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
   store += ((size_t)blockIdx.x * (kBackBlock / 32) + (threadIdx.x >> 5)) * kTomoChords;
   Counters cnt;
   const uint32_t nchunk = (uint32_t)((P.spp + chunk - 1) / chunk);
-  const uint32_t units = (uint32_t)(P.cam.W * P.cam.H) * nchunk;
+  const uint32_t units = (uint32_t)(P.roi_w * P.roi_h) * nchunk;
   for (;;) {
     const uint32_t u = next_tile(counter, lane);
     if (u >= units) break;
-    const int pix = (int)(u / nchunk);
+    const int pix = roi_pixel(P, u / nchunk);
     const float gI = dLdI[pix];
     if (gI == 0.f) continue;
     const int sa = P.s0 + (int)(u % nchunk) * chunk, sb = min(sa + chunk, P.s0 + P.spp);
@@ -1440,11 +1440,11 @@ __global__ void __launch_bounds__(kBackBlock, kRadBlocks)
             scratch + ((size_t)blockIdx.x * (kBackBlock / 32) + warp) * rad_warp_bytes(rad_list_cap(F.n)),
             env, lane, rad_list_cap(F.n), 0, false, Counters()};
   const uint32_t nchunk = (uint32_t)((P.spp + chunk - 1) / chunk);
-  const uint32_t units = (uint32_t)(P.cam.W * P.cam.H) * nchunk;
+  const uint32_t units = (uint32_t)(P.roi_w * P.roi_h) * nchunk;
   for (;;) {
     const uint32_t u = next_tile(counter, lane);
     if (u >= units) break;
-    const uint32_t pix = u / nchunk;
+    const uint32_t pix = (uint32_t)roi_pixel(P, u / nchunk);
     const float gI = dLdI[pix];
     if (gI == 0.f) continue;
     const float base = gI / (float)P.spp;
@@ -1565,7 +1565,8 @@ static cudaError_t launch_adjoint(const Field& F, const PathParams& P, AdjointKe
     if ((e = adjoint_stack_fits(kernel)) != cudaSuccess) return e;
     if ((e = adjoint_grid(F, kernel, smem, g)) != cudaSuccess) return e;
   }
-  const int64_t npix = (int64_t)P.cam.W * P.cam.H, warps = g * (kBackBlock / 32);
+  // (pixels whose rays all miss the scene have no part in the gradient)
+  const int64_t npix = std::max<int64_t>(1, (int64_t)P.roi_w * P.roi_h), warps = g * (kBackBlock / 32);
   int64_t nchunk = (16 * warps + npix - 1) / npix;
   nchunk = nchunk < 1 ? 1 : (nchunk > P.spp ? P.spp : nchunk);
   const int64_t chunk = (P.spp + nchunk - 1) / nchunk;

@@ -218,6 +218,49 @@ LodDev lod_dev(const gf_lod_desc& l) {
   return LodDev{l.freq_policy, l.max_band, l.cone_policy, l.beta, l.delta};
 }
 
+// The pixels whose rays can meet the scene's bounds: those around the projections of the
+// corners of the box, a little larger than it is (rounding of rays and of the box test) and
+// a pixel wider on every side.  The whole image when a corner is not in front of the camera.
+void region_of_interest(const Field& F, PathParams& P) {
+  const double W = P.cam.W, H = P.cam.H;
+  P.roi_x = P.roi_y = 0;
+  P.roi_w = P.cam.W;
+  P.roi_h = P.cam.H;
+  const double lo[3] = {F.dev.lo.x, F.dev.lo.y, F.dev.lo.z}, hi[3] = {F.dev.hi.x, F.dev.hi.y, F.dev.hi.z};
+  const double e[3] = {P.cam.eye.x, P.cam.eye.y, P.cam.eye.z};
+  const double rt[3] = {P.cam.rt.x, P.cam.rt.y, P.cam.rt.z}, up[3] = {P.cam.up.x, P.cam.up.y, P.cam.up.z},
+               fw[3] = {P.cam.fw.x, P.cam.fw.y, P.cam.fw.z};
+  double far = 0.0;
+  for (int k = 0; k < 3; ++k)
+    far += std::max(std::fabs(lo[k] - e[k]), std::fabs(hi[k] - e[k])) + std::fabs(e[k]);
+  double x0 = INFINITY, x1 = -INFINITY, y0 = INFINITY, y1 = -INFINITY;
+  for (int c = 0; c < 8; ++c) {
+    double x = 0, y = 0, z = 0;
+    for (int k = 0; k < 3; ++k) {
+      const double d = (c >> k & 1 ? hi[k] + 1e-5 * far : lo[k] - 1e-5 * far) - e[k];
+      x += d * rt[k];
+      y += d * up[k];
+      z += d * fw[k];
+    }
+    if (!(z > 1e-5 * far)) return;
+    const double px = (x / (z * P.cam.tanh * P.cam.aspect) + 1.0) * 0.5 * W;
+    const double py = (1.0 - y / (z * P.cam.tanh)) * 0.5 * H;
+    x0 = std::min(x0, px);
+    x1 = std::max(x1, px);
+    y0 = std::min(y0, py);
+    y1 = std::max(y1, py);
+  }
+  if (!(x1 >= x0 && y1 >= y0)) return;
+  // (coordinates are rounded to 1e-6 of the image in FP32)
+  const double mx = 1.0 + 1e-5 * W, my = 1.0 + 1e-5 * H;
+  const double ax = std::min(std::max(std::floor(x0 - mx), 0.0), W), bx = std::min(std::max(std::ceil(x1 + mx), 0.0), W);
+  const double ay = std::min(std::max(std::floor(y0 - my), 0.0), H), by = std::min(std::max(std::ceil(y1 + my), 0.0), H);
+  P.roi_x = (int)ax;
+  P.roi_y = (int)ay;
+  P.roi_w = (int)(bx - ax);
+  P.roi_h = (int)(by - ay);
+}
+
 gf_status camera_params(const gf_camera* c, const gf_render_opts* o, uint64_t seed,
                         const Field& F, PathParams& P) {
   if (!c || !o) return fail(GF_EINVAL, "camera/opts null");
@@ -289,6 +332,7 @@ gf_status camera_params(const gf_camera* c, const gf_render_opts* o, uint64_t se
   P.seed = seed;
   P.lod = F.lod;
   P.lod_nee = F.lod_nee;
+  region_of_interest(F, P);
   return GF_OK;
 }
 

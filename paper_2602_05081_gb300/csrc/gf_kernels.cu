@@ -14,14 +14,30 @@ namespace gf {
 constexpr int kBlock = 128;
 constexpr int kCoopBlocks = 5;  // resident blocks per SM of the one-ray-per-warp kernels
 
-// The rays of a warp: a small batch is dealt out (no counter to clear, no atomic per
-// ray), larger ones are fetched one by one (launch_transmittance).
-__device__ __forceinline__ int64_t first_ray(const TrParams& P, uint32_t lane) {
-  return P.dealt ? (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)
-                 : (int64_t)next_tile(P.counter, lane);
+struct Ray {
+  float3 o, v;
+  float tmin, tmax;
+};
+__device__ __forceinline__ Ray batch_ray(const TrParams& P, int64_t r) {
+  return Ray{make_float3(P.o[3 * r], P.o[3 * r + 1], P.o[3 * r + 2]),
+             unit_dir(make_float3(P.d[3 * r], P.d[3 * r + 1], P.d[3 * r + 2])),
+             P.trange ? P.trange[2 * r] : 0.f, P.trange ? P.trange[2 * r + 1] : INFINITY};
 }
-__device__ __forceinline__ int64_t next_ray(const TrParams& P, uint32_t lane, int64_t r) {
-  return P.dealt ? r + (int64_t)gridDim.x * (blockDim.x >> 5) : (int64_t)next_tile(P.counter, lane);
+// The next ray of a batch for the warp, after ray r (-1: the first); P.n or more at the end.
+// A small batch is dealt out (no counter to clear, no atomic per ray); of larger ones, rays
+// that miss the scene are answered by one lane.
+__device__ __forceinline__ int64_t next_ray(const DevField& F, const TrParams& P, WarpItems& S, uint32_t lane,
+                                            int spp, int64_t r) {
+  if (P.dealt)
+    return r < 0 ? (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)
+                 : r + (int64_t)gridDim.x * (blockDim.x >> 5);
+  return (int64_t)next_item(S, P.counter, (uint32_t)P.n, lane, [&](uint32_t i) {
+    const Ray y = batch_ray(P, i);
+    if (meets_scene(F, y.o, y.v, y.tmin, y.tmax)) return -1;
+    P.out_T[i] = 1.f;
+    if (P.out_tau) P.out_tau[i] = 0.f;
+    return spp;
+  });
 }
 
 // ---------------------------------------------------------------------------
@@ -35,24 +51,24 @@ __device__ __forceinline__ int64_t next_ray(const TrParams& P, uint32_t lane, in
 // ---------------------------------------------------------------------------
 template <int MODE>  // GF_TR_DETERMINISTIC or GF_TR_CLOSED_FORM
 __global__ void __launch_bounds__(kBlock, kCoopBlocks)
-    k_transmittance_coop(const __grid_constant__ DevField F, const TrParams P) {
+    k_transmittance_coop(const __grid_constant__ DevField F, const __grid_constant__ TrParams P) {
   __shared__ BlockTables sm;
   __shared__ CoopQ qs[kBlock / 32];
   init_tables(sm, F);
   const uint32_t lane = threadIdx.x & 31u;
+  __shared__ WarpItems items[kBlock / 32];
   CoopQ& Q = qs[threadIdx.x >> 5];
+  init_items(items[threadIdx.x >> 5], lane);
   Counters cnt;
   const int spp = lod_is_deterministic(P.lod) ? 1 : P.spp;
-  for (int64_t r = first_ray(P, lane); r < P.n; r = next_ray(P, lane, r)) {
-    const float3 o = make_float3(P.o[3 * r], P.o[3 * r + 1], P.o[3 * r + 2]);
-    const float3 v = unit_dir(make_float3(P.d[3 * r], P.d[3 * r + 1], P.d[3 * r + 2]));
-    const float tmin = P.trange ? P.trange[2 * r] : 0.f;
-    const float tmax = P.trange ? P.trange[2 * r + 1] : INFINITY;
+  WarpItems& S = items[threadIdx.x >> 5];
+  for (int64_t r = next_ray(F, P, S, lane, spp, -1); r < P.n; r = next_ray(F, P, S, lane, spp, r)) {
+    const Ray y = batch_ray(P, r);
     float s_acc = 0.f, c_acc = 0.f;
     for (int s = 0; s < spp; ++s) {
-      const Mask m = sample_mask(F, P.lod, v, P.seed, (uint32_t)r, (uint32_t)s, 0, TAG_MASK);
+      const Mask m = sample_mask(F, P.lod, y.v, P.seed, (uint32_t)r, (uint32_t)s, 0, TAG_MASK);
       if (lane == 0) cnt.rays += 1;
-      coop_tau<MODE>(F, Q, m, o, v, tmin, tmax, sm.glx, sm.glw, lane, s_acc, c_acc, cnt);
+      coop_tau<MODE>(F, Q, m, y.o, y.v, y.tmin, y.tmax, sm.glx, sm.glw, lane, s_acc, c_acc, cnt);
     }
     warp_sum_pair(s_acc, c_acc);
     if (lane == 0) {
@@ -61,6 +77,7 @@ __global__ void __launch_bounds__(kBlock, kCoopBlocks)
       if (P.out_tau) P.out_tau[r] = tau;
     }
   }
+  if (lane == 0) cnt.rays += S.missed;
   flush_counters(F, cnt, lane);
 }
 
@@ -297,34 +314,45 @@ __device__ float rt_coop(const DevField& F, RtQ& Q, const Mask& M, float3 o, flo
 }
 
 __global__ void __launch_bounds__(kBlock, 4)
-    k_transmittance_rt_coop(const __grid_constant__ DevField F, const TrParams P) {
+    k_transmittance_rt_coop(const __grid_constant__ DevField F, const __grid_constant__ TrParams P) {
   __shared__ BlockTables sm;
   __shared__ RtQ qs[kBlock / 32];
   init_tables(sm, F);
   const uint32_t lane = threadIdx.x & 31u;
+  __shared__ WarpItems items[kBlock / 32];
   RtQ& Q = qs[threadIdx.x >> 5];
+  init_items(items[threadIdx.x >> 5], lane);
   Counters cnt;
-  for (int64_t r = first_ray(P, lane); r < P.n; r = next_ray(P, lane, r)) {
-    const float3 o = make_float3(P.o[3 * r], P.o[3 * r + 1], P.o[3 * r + 2]);
-    const float3 v = unit_dir(make_float3(P.d[3 * r], P.d[3 * r + 1], P.d[3 * r + 2]));
-    const float tmin = P.trange ? P.trange[2 * r] : 0.f;
-    const float tmax = P.trange ? P.trange[2 * r + 1] : INFINITY;
-    const float3 inv = safe_inv(v);
+  WarpItems& S = items[threadIdx.x >> 5];
+  for (int64_t r = next_ray(F, P, S, lane, P.spp, -1); r < P.n; r = next_ray(F, P, S, lane, P.spp, r)) {
+    const Ray y = batch_ray(P, r);
+    const float3 inv = safe_inv(y.v);
     float acc = 0.f;
     for (int s = 0; s < P.spp; ++s) {
-      const Mask m = sample_mask(F, P.lod, v, P.seed, (uint32_t)r, (uint32_t)s, 0, TAG_MASK);
+      const Mask m = sample_mask(F, P.lod, y.v, P.seed, (uint32_t)r, (uint32_t)s, 0, TAG_MASK);
       if (lane == 0) cnt.rays += 1;
       float t0, t1, T = 1.f;
-      if (m.bits != 0ull && scene_span(F, o, inv, tmin, tmax, t0, t1)) {
+      if (m.bits != 0ull && scene_span(F, y.o, inv, y.tmin, y.tmax, t0, t1)) {
         if (lane == 0) cnt.windows += 1;
-        T = rt_coop(F, Q, m, o, v, inv, tmin, tmax, t0, t1, P.seed, (uint32_t)r,
+        T = rt_coop(F, Q, m, y.o, y.v, inv, y.tmin, y.tmax, t0, t1, P.seed, (uint32_t)r,
                     stream_word((uint32_t)s, 0, TAG_TRACK), sm.env, lane, P.exact, cnt);
       }
       acc += T;
     }
     if (lane == 0) P.out_T[r] = acc / (float)P.spp;
   }
+  if (lane == 0) cnt.rays += S.missed;
   flush_counters(F, cnt, lane);
+}
+
+// the pixels whose rays all miss the scene
+__global__ void k_background(const __grid_constant__ DevField F, const __grid_constant__ PathParams P, float* out,
+                             float value) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, npix = (int64_t)P.cam.W * P.cam.H;
+  if (i == 0) atomicAdd(F.stats + ST_RAYS, (unsigned long long)(npix - (int64_t)P.roi_w * P.roi_h) * P.spp);
+  if (i >= npix) return;
+  const int x = (int)(i % P.cam.W) - P.roi_x, y = (int)(i / P.cam.W) - P.roi_y;
+  if (x < 0 || x >= P.roi_w || y < 0 || y >= P.roi_h) out[i] = value;
 }
 
 // ---------------------------------------------------------------------------
@@ -340,11 +368,11 @@ __global__ void __launch_bounds__(kBlock, kCoopBlocks)
   const uint32_t lane = threadIdx.x & 31u;
   CoopQ& Q = qs[threadIdx.x >> 5];
   Counters cnt;
-  const int npix = P.cam.W * P.cam.H;
+  const int npix = P.roi_w * P.roi_h;
   for (;;) {
     const uint32_t tile = next_tile(counter, lane);
     if (tile >= (uint32_t)npix) break;
-    const int pix = (int)tile;
+    const int pix = roi_pixel(P, tile);
     float acc = 0.f;
     for (int s = P.s0; s < P.s0 + P.spp; ++s) {
       float3 o, v;
@@ -383,11 +411,11 @@ __global__ void __launch_bounds__(kBlock, kFlightBlocks)
   L.list = store + ((size_t)blockIdx.x * (kBlock / 32) + warp) * kFlightList;
   L.cap = cap;
   Counters cnt;
-  const int npix = P.cam.W * P.cam.H;
+  const int npix = P.roi_w * P.roi_h;
   for (;;) {
     const uint32_t tile = next_tile(counter, lane);
     if (tile >= (uint32_t)npix) break;
-    const uint32_t pix = tile;
+    const uint32_t pix = (uint32_t)roi_pixel(P, tile);
     float acc = 0.f;
     for (int s = P.s0; s < P.s0 + P.spp; ++s) {
       float3 o, v;
@@ -603,17 +631,22 @@ cudaError_t launch_render(const Field& F, const PathParams& P, float* out, cudaS
   if (e != cudaSuccess) return e;
   if (P.integrator == GF_INTEG_SCATTER && P.free_flight == GF_FLIGHT_DELTA)
     return launch_render_scatter(F, P, out, s);
-  const int64_t npix = (int64_t)P.cam.W * P.cam.H;
-  if (P.integrator == GF_INTEG_SCATTER) {
+  const int64_t npix = (int64_t)P.cam.W * P.cam.H, roi = (int64_t)P.roi_w * P.roi_h;
+  const bool flight = P.integrator == GF_INTEG_SCATTER;
+  if (roi < npix) {
+    k_background<<<(unsigned)((npix + 255) / 256), 256, 0, s>>>(F.dev, P, out, flight ? 0.f : 1.f);
+    if ((e = cudaGetLastError()) != cudaSuccess || roi == 0) return e;
+  }
+  if (flight) {
     auto k = P.free_flight == GF_FLIGHT_SEGMENT ? k_flight<GF_FLIGHT_SEGMENT> : k_flight<GF_FLIGHT_CDF>;
     if (!stack_fits(k)) return cudaErrorLaunchOutOfResources;
-    int64_t g = persistent_grid(F, k, npix);
+    int64_t g = persistent_grid(F, k, roi);
     const int cap = flight_lists(F, g, s);
     k<<<(unsigned)g, kBlock, 0, s>>>(F.dev, P, out, F.counter,
                                      static_cast<FlightRec*>(cap ? F.wscratch.p : nullptr), cap);
   } else {
     if (!stack_fits(k_tomo)) return cudaErrorLaunchOutOfResources;
-    k_tomo<<<persistent_grid(F, k_tomo, npix), kBlock, 0, s>>>(F.dev, P, out, F.counter);
+    k_tomo<<<persistent_grid(F, k_tomo, roi), kBlock, 0, s>>>(F.dev, P, out, F.counter);
   }
   return cudaGetLastError();
 }

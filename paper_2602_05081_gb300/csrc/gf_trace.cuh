@@ -694,6 +694,7 @@ struct PathParams {
   int fov;          // foveation: 1 = per-sample band cutoff by eccentricity
   float3 gaze;      // unit direction of the ray through the gaze point
   float fov_f0, fov_slope, fov_smooth;
+  int roi_x, roi_y, roi_w, roi_h;  // pixels outside have no ray that meets the scene's bounds
   float albedo, irradiance;
   float3 light;
   uint64_t seed;

@@ -1,12 +1,14 @@
 """Rays that miss the scene, in batches and images (GPU).
 
-A warp takes up to 32 rays (or pixels) and works only through those that meet the scene's
-bounds; the others are answered by one lane each.  Results, counters and gradients must not
-depend on how rays that hit and rays that miss lie side by side.
+A warp takes up to 32 rays of a batch and works only through those that meet the scene's
+bounds; the others are answered by one lane each.  Of an image the warps take the pixels
+around the projected bounds, and the background is filled.  Results, counters and
+gradients must not depend on how rays that hit and rays that miss lie side by side.
 """
 import numpy as np
 import pytest
 
+import oracle
 import synth
 
 torch = pytest.importorskip("torch")
@@ -96,6 +98,36 @@ def test_images_with_background(api, ctx, w, h, vfov):
         lim = 2.0 * 6 * w * h * 2.0 ** -24
         assert float((a - b).abs().max()) <= lim * float(a.abs().max()) and (float(a.abs().max()) > 0.0 or w < 100)
     f.sync()
+    f.free()
+
+
+def test_images_from_all_sides(api, ctx):
+    """Tomography images against the FP64 oracle for cameras around, beside and inside the
+    scene, near and far, wide and narrow: no pixel that a kernel reaches is taken for
+    background.  A ray's place in FP32 is off by up to 4 * 2^-24 of its distance; across a ray
+    an optical depth changes by at most 0.5 * 0.6 / 0.02 = 15 per unit and kernel, ten of
+    them: 150 * 4 * 2^-24 = 3.6e-5 times the distance."""
+    p = synth.absorption_field(30, seed=8)
+    p["weight"] = np.abs(p["weight"]).astype(np.float32)
+    p["omega"] = np.zeros_like(p["omega"])
+    p["phase"] = np.zeros_like(p["phase"])
+    f, orc = api.Field(ctx, p), oracle.Field(p)
+    rng = np.random.default_rng(4)
+    seen = 0
+    for k in range(24):
+        u = rng.standard_normal(3)
+        eye = 0.5 + (0.2, 0.9, 1.4, 4.0, 60.0)[k % 5] * u / np.linalg.norm(u)
+        at = 0.5 + (0.0, 0.4, 2.0)[k % 3] * rng.standard_normal(3)
+        vfov = float(np.clip((20.0, 70.0, 140.0)[k % 3] / (1.0 if k % 5 < 3 else 8.0), 0.5, 170.0))
+        w, h = ((31, 18), (17, 40), (64, 64))[k % 3]
+        a = [float(x) for x in eye], [float(x) for x in at], (0.0, 1.0, 0.0), vfov, w, h
+        img = f.render(api.camera(*a), api.render_opts("tomo", 2), 5)
+        f.sync()
+        ref = orc.render(oracle.camera(*a), oracle.render_opts("tomo", 2), 5)
+        err = np.abs(img.cpu().numpy() - ref)
+        assert err.max() <= 3.6e-5 * (1.0 + float(np.linalg.norm(eye - 0.5))), (k, err.max())
+        seen += int((ref < 0.999).any())
+    assert seen >= 8
     f.free()
 
 
