@@ -454,6 +454,34 @@ static __device__ __noinline__ float cdf_flight(const DevField& F, FlightQ& Q, c
 // target holds the collision e_a + u (e_b - e_a).  It is found by bisection on t that
 // stops once no chord end lies inside the bracket: every step takes tau(0, mid), the
 // chord ends inside both halves of the bracket and the nearest ends around them.
+struct SegmentEnds {
+  int n_left = 0, n_right = 0;              // chord ends in (lo, mid) and in (mid, hi)
+  float below_lo = 0.f, below_mid = 0.f;    // largest end <= lo, <= mid (or 0)
+  float above_mid = INFINITY, above_hi = INFINITY;  // smallest end >= mid, >= hi
+  __device__ __forceinline__ void add(float e, float lo, float mid, float hi) {
+    n_left += (e > lo && e < mid) ? 1 : 0;
+    n_right += (e > mid && e < hi) ? 1 : 0;
+    if (e <= lo) below_lo = fmaxf(below_lo, e);
+    if (e <= mid) below_mid = fmaxf(below_mid, e);
+    if (e >= mid) above_mid = fminf(above_mid, e);
+    if (e >= hi) above_hi = fminf(above_hi, e);
+  }
+};
+// chord r's ends into E, its part in [0, mid] into (s, c)
+__device__ __forceinline__ void segment_part(const DevField& F, const FlightRec& r, float lo, float mid, float hi,
+                                             SegmentEnds& E, float& s, float& c) {
+  const float tin = r.tc + r.dtin, tout = r.tc + r.dtout;
+  E.add(tin, lo, mid, hi);
+  E.add(tout, lo, mid, hi);
+  if (tin >= mid) return;
+  if (!(tout > mid)) {
+    neumaier_add(s, c, r.full);
+  } else {  // the chord's part in [0, mid]
+    Chord ch = flight_chord(r);
+    ch.dtout = mid - r.tc;
+    neumaier_add(s, c, r.w * chord_closed(F.wd, ch));
+  }
+}
 static __device__ __noinline__ float segment_flight(const DevField& F, FlightQ& Q, const Mask& M, float3 o,
                                              float3 v, float target, float u, uint32_t lane,
                                              const Flight& L, Counters& cnt) {
@@ -462,41 +490,20 @@ static __device__ __noinline__ float segment_flight(const DevField& F, FlightQ& 
   for (int it = 0; it < 48; ++it) {
     const float mid = 0.5f * (lo + hi);
     float s = 0.f, c = 0.f;
-    int n_left = 0, n_right = 0;              // chord ends in (lo, mid) and in (mid, hi)
-    float below_lo = 0.f, below_mid = 0.f;    // largest end <= lo, <= mid (or 0)
-    float above_mid = INFINITY, above_hi = INFINITY;  // smallest end >= mid, >= hi
-    auto end = [&](float e) {
-      n_left += (e > lo && e < mid) ? 1 : 0;
-      n_right += (e > mid && e < hi) ? 1 : 0;
-      if (e <= lo) below_lo = fmaxf(below_lo, e);
-      if (e <= mid) below_mid = fmaxf(below_mid, e);
-      if (e >= mid) above_mid = fminf(above_mid, e);
-      if (e >= hi) above_hi = fminf(above_hi, e);
-    };
-    flight_each(F, Q, M, o, v, INFINITY, lane, L, cnt, [&](const FlightRec& r) {
-      const float tin = r.tc + r.dtin, tout = r.tc + r.dtout;
-      end(tin);
-      end(tout);
-      if (tin >= mid) return;
-      if (!(tout > mid)) {
-        neumaier_add(s, c, r.full);
-      } else {  // the chord's part in [0, mid]
-        Chord ch = flight_chord(r);
-        ch.dtout = mid - r.tc;
-        neumaier_add(s, c, r.w * chord_closed(F.wd, ch));
-      }
-    });
+    SegmentEnds E;
+    flight_each(F, Q, M, o, v, INFINITY, lane, L, cnt,
+                [&](const FlightRec& r) { segment_part(F, r, lo, mid, hi, E, s, c); });
     warp_sum_pair(s, c);
     if (__fadd_rn(s, c) < target) {
       lo = mid;
-      ea = warp_max(below_mid);
-      eb = -warp_max(-above_hi);
-      if (__reduce_add_sync(kFull, n_right) == 0) break;
+      ea = warp_max(E.below_mid);
+      eb = -warp_max(-E.above_hi);
+      if (__reduce_add_sync(kFull, E.n_right) == 0) break;
     } else {
       hi = mid;
-      ea = warp_max(below_lo);
-      eb = -warp_max(-above_mid);
-      if (__reduce_add_sync(kFull, n_left) == 0) break;
+      ea = warp_max(E.below_lo);
+      eb = -warp_max(-E.above_mid);
+      if (__reduce_add_sync(kFull, E.n_left) == 0) break;
     }
     if (!(hi > lo)) break;
   }
