@@ -831,9 +831,13 @@ constexpr int64_t kLaneTau = 24, kLaneClosed = 48, kLaneTomo = 128;
 static bool lane_work(const Field& F, int64_t items, int64_t most) {
   return F.n <= std::min(most, items / 2500);
 }
+// (where the kernel's stack does not fit the limit in force, a ray per warp)
+template <class K>
+static bool lanes_fit(const Field& F, K kernel, int64_t items, int64_t most) {
+  return lane_work(F, items, most) && stack_fits(kernel);
+}
 template <class K>
 static cudaError_t launch_lanes(const Field& F, K kernel, const TrParams& P, cudaStream_t s) {
-  if (!stack_fits(kernel)) return cudaErrorLaunchOutOfResources;
   const cudaError_t e = cudaMemsetAsync(P.counter, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   kernel<<<(unsigned)persistent_grid(F, kernel, (P.n + 31) / 32), kBlock, 0, s>>>(F.dev, P);
@@ -842,17 +846,18 @@ static cudaError_t launch_lanes(const Field& F, K kernel, const TrParams& P, cud
 
 cudaError_t launch_transmittance(const Field& F, const TrParams& P, cudaStream_t s) {
   (void)cudaGetLastError();  // a stale error of an unrelated call is not ours
-  if (P.mode == GF_TR_DETERMINISTIC && lane_work(F, P.n, kLaneTau))
-    return launch_lanes(F, k_transmittance_lane<GF_TR_DETERMINISTIC>, P, s);
-  if (P.mode == GF_TR_CLOSED_FORM && lane_work(F, P.n, kLaneClosed))
-    return launch_lanes(F, k_transmittance_lane<GF_TR_CLOSED_FORM>, P, s);
+  auto det = k_transmittance_lane<GF_TR_DETERMINISTIC>;
+  auto closed = k_transmittance_lane<GF_TR_CLOSED_FORM>;
+  auto rt = k_transmittance_lane<GF_TR_RATIO_TRACKING>;
+  if (P.mode == GF_TR_DETERMINISTIC && lanes_fit(F, det, P.n, kLaneTau)) return launch_lanes(F, det, P, s);
+  if (P.mode == GF_TR_CLOSED_FORM && lanes_fit(F, closed, P.n, kLaneClosed)) return launch_lanes(F, closed, P, s);
   if (P.mode == GF_TR_DETERMINISTIC) return launch_rays(F, k_transmittance_coop<GF_TR_DETERMINISTIC>, P, s);
   if (P.mode == GF_TR_CLOSED_FORM) return launch_rays(F, k_transmittance_coop<GF_TR_CLOSED_FORM>, P, s);
   if (!stack_fits(k_transmittance_rt_coop)) return cudaErrorLaunchOutOfResources;
   TrParams Q = P;
   Q.exact = P.n * 8 > (int64_t)F.ctx.sm_count * 16 * 32;
-  if (Q.exact && lane_work(F, P.n, kLaneTau))  // (the tracker of a lane has that form)
-    return launch_lanes(F, k_transmittance_lane<GF_TR_RATIO_TRACKING>, P, s);
+  // (the tracker of a lane has that form)
+  if (Q.exact && lanes_fit(F, rt, P.n, kLaneTau)) return launch_lanes(F, rt, P, s);
   return launch_rays(F, k_transmittance_rt_coop, Q, s);
 }
 
@@ -903,7 +908,7 @@ cudaError_t launch_render(const Field& F, const PathParams& P, float* out, cudaS
     if ((e = cudaGetLastError()) != cudaSuccess || roi == 0) return e;
   }
   auto flight_lane = P.free_flight == GF_FLIGHT_SEGMENT ? k_flight_lane<GF_FLIGHT_SEGMENT> : k_flight_lane<GF_FLIGHT_CDF>;
-  if (flight && lane_work(F, roi / 3, kLaneFlight) && stack_fits(flight_lane)) {
+  if (flight && lanes_fit(F, flight_lane, roi / 3, kLaneFlight)) {
     flight_lane<<<persistent_grid(F, flight_lane, (roi + 31) / 32), kBlock, 0, s>>>(F.dev, P, out, F.counter);
   } else if (flight) {
     auto k = P.free_flight == GF_FLIGHT_SEGMENT ? k_flight<GF_FLIGHT_SEGMENT> : k_flight<GF_FLIGHT_CDF>;
@@ -912,8 +917,7 @@ cudaError_t launch_render(const Field& F, const PathParams& P, float* out, cudaS
     const int cap = flight_lists(F, g, s);
     k<<<(unsigned)g, kBlock, 0, s>>>(F.dev, P, out, F.counter,
                                      static_cast<FlightRec*>(cap ? F.wscratch.p : nullptr), cap);
-  } else if (lane_work(F, roi, kLaneTomo)) {
-    if (!stack_fits(k_tomo_lane)) return cudaErrorLaunchOutOfResources;
+  } else if (lanes_fit(F, k_tomo_lane, roi, kLaneTomo)) {
     k_tomo_lane<<<persistent_grid(F, k_tomo_lane, (roi + 31) / 32), kBlock, 0, s>>>(F.dev, P, out, F.counter);
   } else {
     if (!stack_fits(k_tomo)) return cudaErrorLaunchOutOfResources;

@@ -4,6 +4,8 @@ Up to 24 kernels (48 in closed form, 128 for images), and a 2,500th of the rays 
 ray goes to one lane instead of a warp.  At the lines, against the FP64 oracle, against small
 batches, and the time that made the difference.
 """
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -121,6 +123,31 @@ def test_flight_images_of_a_ray_per_lane(api, ctx, ff, n, w, h):
     ref = oracle.Field(p).render(cor, oracle.render_opts("scatter", 2, 3, free_flight=ff), seed=6)
     off = np.abs(img.cpu().numpy() - ref) > 1e-4 * ref.max()
     assert ref.max() > 0.0 and off.mean() <= 0.01, off.mean()
+    f.free()
+
+
+def test_a_smaller_stack_limit_takes_warps(api, ctx):
+    """Another component may lower the context's stack limit (a limit of this process).  A
+    lane's list then does not fit (1,824 bytes), and a pixel goes to a warp as in fields of
+    more kernels: same image to rounding."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    size = ctypes.c_size_t()
+    torch.zeros(1, device="cuda")
+    assert cu.cuCtxGetLimit(ctypes.byref(size), 0) == 0
+    f = api.Field(ctx, _field(3, seed=3))
+    c = synth.DEFAULT_CAMERA
+    cam = api.camera(c["eye"], c["look_at"], c["up"], 50.0, 320, 240)
+    o = api.render_opts("scatter", 1, 1, free_flight="cdf")
+    lanes = f.render(cam, o, 3).clone()
+    f.sync()
+    try:
+        assert cu.cuCtxSetLimit(0, ctypes.c_size_t(1024)) == 0
+        warps = f.render(cam, o, 3).clone()
+        f.sync()
+    finally:
+        assert cu.cuCtxSetLimit(0, size) == 0
+    off = (lanes - warps).abs() > 1e-4 * lanes.max()
+    assert float(lanes.max()) > 0.0 and float(off.float().mean()) <= 0.01
     f.free()
 
 
