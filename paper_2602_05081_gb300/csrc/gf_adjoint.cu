@@ -257,9 +257,9 @@ __device__ __forceinline__ void add_grad(const BackArgs& B, int64_t i, const flo
 // their integrals added to tau; then the warp goes through the kept chords, 32 at a
 // time, and scatters dL/dtau times their gradients.  A ray with more chords than
 // kTomoChords is traversed again with its tau known.  Bound by instruction issue.
-// Every lane used to carry its own pixel, with 15 derivatives formed at every
-// quadrature node and two traversals.  Forward and adjoint of 524,288 rays through 200k
-// kernels: 882 -> 51 ms (21 and 28.7).
+// With a pixel per lane, 15 derivatives formed at every quadrature node and two
+// traversals, forward and adjoint of 524,288 rays through 200k kernels took 882 ms, 51
+// now (20.5 and 28).
 // ---------------------------------------------------------------------------
 constexpr int kBackBlock = 128;
 constexpr int kTomoBlocks = 4;     // resident blocks per SM
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kBackBlock, kTomoBlocks)
 // The radiance adjoints run one path per warp.  Bound by instruction issue and the
 // latency of tree nodes.  With one pixel per lane 1.8 of 32 lanes ran, every window
 // visited its ray's list three times and paths were followed twice.  Through 200k
-// kernels: 305 -> 6.8 ms (128x128, 2 samples, single scattering), 697 -> 3.4 ms (96x64,
+// kernels: 305 -> 6.3 ms (128x128, 2 samples, single scattering), 697 -> 2.9 ms (96x64,
 // 1 sample, 3 bounces).
 //
 // A ray is processed over a window of t, at first all of it:

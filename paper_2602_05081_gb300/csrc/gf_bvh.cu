@@ -541,7 +541,7 @@ __device__ __forceinline__ Node4 emit_node4(int nc, const float box[4][6], const
     }
     // grid step s, never zero, and origin lo - s/64: every child keeps a margin of s/128
     // between its box and its decoded planes (254.9 s + s/64 + s/128 <= 255 s), which
-    // covers the traversal's rounding of a plane (s/512)
+    // covers the rounding of the codes' part of a plane in the traversal (s/512)
     sc[a] = __fdiv_ru(__fsub_ru(hi[a], lo[a]), 254.9f);
     const float floor_s = fmaxf(fabsf(lo[a]), fabsf(hi[a])) * 1e-7f + 1e-30f;
     sc[a] = fmaxf(sc[a], floor_s);

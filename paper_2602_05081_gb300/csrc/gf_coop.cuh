@@ -271,9 +271,8 @@ __device__ __forceinline__ void coop_tau(const DevField& F, CoopQ& Q, const Mask
 // tau(0, t) = -ln(1 - xi).
 //
 // One traversal collects the ray's chords in the warp's list with their full
-// integrals; the bisections then work on the list.  (They used to traverse the tree
-// for every one of up to 33 depths.)  A ray with more chords than the list holds
-// traverses for each depth.
+// integrals; the bisections then work on the list.  A ray with more chords than the
+// list holds traverses for each of up to 33 depths.
 // ---------------------------------------------------------------------------
 constexpr int kFlightList = 4096;  // chords per warp (global scratch)
 constexpr int kFlightActive = 512; // chords that a bisection still has to clip

@@ -29,8 +29,8 @@ enum : int {
   ERR_STACK = 1, ERR_WINDOW = 2, ERR_POINTS = 4, ERR_GUARD = 8, ERR_INPUT = 16, ERR_INDEX = 32
 };
 
-// Binary BVH node of the tree by cells (the radiance adjoints and the walks of one
-// lane, traverse_ray), holding the boxes, children and cell masks of both children
+// Binary BVH node of the tree by cells (the radiance adjoints and the walks of single
+// lanes, traverse_ray), holding the boxes, children and cell masks of both children
 // (one 80-byte fetch tests two boxes).  child >= 0: internal node; child < 0:
 // leaf of the sorted primitive ~child.
 struct __align__(16) Node {
@@ -184,7 +184,7 @@ __device__ __forceinline__ float2 faddeeva_w(const Weideman& W, float x, float y
 
 // 32 bytes of read-only memory in one load (p 32-byte aligned).  Lanes that read
 // scattered records pay per load instruction in the L1 tag stage, not per byte: a
-// 96-byte node takes 3 of these instead of 6 16-byte loads.
+// 64-byte node takes 2 of these instead of 4 16-byte loads.
 __device__ __forceinline__ void ldg32(const void* p, uint4& a, uint4& b) {
   unsigned long long r0, r1, r2, r3;
   asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(r0), "=l"(r1), "=l"(r2), "=l"(r3) : "l"(p));
@@ -518,9 +518,9 @@ __device__ __forceinline__ bool scene_span(const DevField& F, float3 o, float3 i
 __device__ __forceinline__ void set_err(const DevField& F, int code) { atomicOr(F.err, code); }
 
 // ---------------------------------------------------------------------------
-// Per-thread traversal of one ray under a cell mask, for what the traversals of a
-// whole warp leave over (windows with more chords or points than their buffers hold)
-// and for the chord lists of gf_ray_chords.  One 80-byte
+// Per-thread traversal of one ray under a cell mask, for fields of a few kernels, for what
+// the traversals of a whole warp leave over (windows with more points than their buffers
+// hold) and for the chord lists of gf_ray_chords.  One 80-byte
 // fetch gives both child boxes of a node; test(tn, tf) decides whether a child
 // whose box spans [tn, tf] along the ray can matter (the test may tighten as
 // the traversal proceeds); hit leaves go to leaf(j) at once; the nearer
@@ -745,8 +745,10 @@ __device__ __forceinline__ unsigned node4_hits(const Node4* N, float3 o, float3 
   const uint32_t qlx = __float_as_uint(v1.z), qly = __float_as_uint(v1.w);
   // slab distances straight from the codes: t = (lo + c s - o) inv.  A code byte c is
   // read as f = 1 + c 2^-15 (one byte permutation), so t = f A + B with A = 2^15 s inv
-  // and B = (lo - o) inv - A; rounding B costs up to s inv / 512, which the margin of
-  // the codes covers (emit_node4)
+  // and B = (lo - o) inv - A.  Rounding A's part of B costs up to s inv / 512, which the
+  // margin of the codes covers (emit_node4); that of (lo - o) inv is 3 2^-24 of the plane's
+  // distance, as in any slab test, and counts where a box is that small (a kernel touches
+  // its box inside a face, where the other slabs leave room)
   const float ax = v0.w * inv.x, ay = v1.x * inv.y, az = v1.y * inv.z;
   const float bx = (v0.x - o.x) * inv.x - ax, by = (v0.y - o.y) * inv.y - ay,
               bz = (v0.z - o.z) * inv.z - az;

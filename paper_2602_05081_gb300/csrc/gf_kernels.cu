@@ -1,6 +1,6 @@
 // gf_kernels.cu -- render, transmittance and test kernels of the Gabor-field
 // renderer.  Persistent warps pull work from a global counter: one ray per warp
-// (gf_coop.cuh).
+// (gf_coop.cuh), or one per lane through a few kernels.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -42,12 +42,12 @@ __device__ __forceinline__ int64_t next_ray(const DevField& F, const TrParams& P
 
 // ---------------------------------------------------------------------------
 // Optical depth of a batch of rays (Gauss-Legendre quadrature or closed-form
-// chord integrals), one ray per warp (coop_tau) at every batch size.  Bound by
-// instruction issue.  With one ray per lane the lanes part at every leaf: each
-// runs its own tree walk and its own rule of 8 to 64 nodes.  130,001 rays
-// through 100k kernels (306 chords and 4,092 nodes per ray): 65.0 ms with one
-// ray per lane, 5.6 ms with one per warp; 4,096 rays through 256 kernels: 53.6
-// us over binary nodes, 35.5 us over four-wide ones with the owner table.
+// chord integrals), one ray per warp (coop_tau) at every batch size but for fields of
+// a few kernels (lane_work).  Bound by instruction issue.  With one ray per lane the
+// lanes part at every leaf: each runs its own tree walk and its own rule of 8 to 64
+// nodes.  130,001 rays through 100k kernels (306 chords and 4,092 nodes per ray):
+// 65.0 ms with one ray per lane, 3.8 ms with one per warp; 4,096 rays through 256
+// kernels: 53.6 us over a binary tree, 29 us now.
 // ---------------------------------------------------------------------------
 template <int MODE>  // GF_TR_DETERMINISTIC or GF_TR_CLOSED_FORM
 __global__ void __launch_bounds__(kBlock, kCoopBlocks)
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kBlock, kCoopBlocks)
 // than the buffer holds is traversed once more, its chords added to the points' sums a
 // buffer at a time; one with more points is halved.  Bound by instruction issue and the
 // latency of tree nodes.  30,000 rays through 100k kernels: 38 ms with one ray per lane
-// (the per-thread tracker traverses twice per eight points, its lanes parted), 4.3 ms now;
+// (the per-thread tracker traverses twice per eight points, its lanes parted), 1.9 ms now;
 // 4,096 rays through 256 kernels: 27 us (rays dealt out).  With 445 kernels over a point
 // (14k in all), 130,000 rays: 135 ms with one ray per lane, 742 when windows were halved
 // for their chords and the rest left to one lane, 22 now.
@@ -480,7 +480,7 @@ __global__ void k_background(const __grid_constant__ DevField F, const __grid_co
 // ---------------------------------------------------------------------------
 // Tomography image: one pixel per warp, its camera rays one after the other
 // (coop_tau), T = exp(-tau) averaged in sample order.  256x256 at 8 samples
-// through 200k kernels: 222 ms with one pixel per lane, 29 ms with one per warp.
+// through 200k kernels: 222 ms with one pixel per lane, 20.5 ms with one per warp.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kBlock, kCoopBlocks)
     k_tomo(const __grid_constant__ DevField F, const PathParams P, float* out, int* counter) {
@@ -555,7 +555,7 @@ __device__ __forceinline__ float flight_path(const DevField& F, const PathParams
 // GF_FLIGHT_SEGMENT): one pixel per warp, its samples in order; every flight works on
 // the ray's collected chords, the NEE transmittance is exp(-tau) in closed form.
 // 160x120 at 2 samples through 50k kernels: 260 ms with one pixel per lane and a
-// traversal for each of up to 33 depths of a flight, 2.9 ms now.  Bound by instruction
+// traversal for each of up to 33 depths of a flight, 2.9 ms from lists.  Bound by instruction
 // issue: two traversals per collision, then the Faddeeva sums of the chord ends.
 // ---------------------------------------------------------------------------
 constexpr int kFlightBlocks = 5;  // resident blocks per SM (3.02 ms with 4, 2.85 with 5)

@@ -1,7 +1,7 @@
 // gf_trace.cuh -- per-ray work shared by the render, transmittance, adjoint and
 // server kernels: LoD mask sampling, quadrature rules and closed-form chord
-// integrals, tentative points, ratio tracking of a ray by one lane (for the windows
-// that the one-ray-per-warp kernels cannot hold), camera rays.
+// integrals, tentative points, ratio tracking of a ray by one lane (through a few
+// kernels, and for windows that the one-ray-per-warp kernel cannot hold), camera rays.
 #pragma once
 #include "../../include/gf.h"
 #include "gf_device.cuh"

@@ -39,10 +39,9 @@ constexpr int kBlocksPerSM = 4; // resident blocks per SM the kernels are built 
 constexpr int kLeafQ = 288;     // queued leaves per warp (<= 31 left + 256 new)
 constexpr int kChordQ = 64;     // queued chords per warp (<= 31 left + 32 new)
 // A window with more points or chords than its slot holds is halved and traversed
-// again: with 8 points and 256 chords that took 9 % of the windows of the 1M-kernel
-// benchmark and a third of those through 200k kernels at full detail.  13 points fill
-// the shared memory of 4 blocks per SM.  1024x1024, 8 samples, 1M kernels, stochastic
-// masks: 317 -> 303 ms; 512x512, 16 samples, 100k kernels: 196 -> 183 ms.
+// again.  13 points fill the shared memory of 4 blocks per SM.  Against 8 points and 256
+// chords: 1024x1024, 8 samples, 1M kernels, stochastic masks 214 -> 193.5 ms; 512x512, 16
+// samples, 100k kernels 93.8 -> 92.0 ms; 120x67, 1 sample, 50k kernels 310 -> 215 us.
 constexpr int kPK = 13;         // tentative points per lane and window
 constexpr int kSlotCh = 448;    // stored chords per lane and window (global scratch)
 constexpr float kFill = 0.7f;     // share of them that a ray's windows aim at (0.5 to 0.9: within 4 %)
@@ -130,9 +129,9 @@ __device__ __forceinline__ bool slot_chord(const DevField& F, const LaneRay& R, 
 }
 
 // Nodes per lane and traversal step.  Two hide each other's latency where rays visit many
-// nodes: with every cone selected, 512x512, 16 samples, 100k kernels take 98.4 ms with
-// one and 93.1 with two.  With one-cone masks (100 nodes per ray) a step seldom holds 64
-// entries and the longer code costs more: 1M kernels, 1024x1024, 8 samples 198 and 216 ms.
+// nodes: with every cone selected, 512x512, 16 samples, 100k kernels take 97.2 ms with
+// one and 92.0 with two.  With one-cone masks (100 nodes per ray) a step seldom holds 64
+// entries and the longer code costs more: 1M kernels, 1024x1024, 8 samples 193.5 and 212.5 ms.
 static int nodes_per_step(const LodDev& a, const LodDev& b) {
   return a.cone_policy == GF_CONE_ALL && b.cone_policy == GF_CONE_ALL && a.freq_policy <= GF_FREQ_CUTOFF &&
                  b.freq_policy <= GF_FREQ_CUTOFF
@@ -158,8 +157,8 @@ __device__ __forceinline__ bool walk_step(const DevField& F, WarpQ& Q, ChordItem
   const int J = (int)(c.jd & 7u);
   float dt = c.dt;
   int p = 0;  // the majorant piece holding dt: the pieces ending at or before it
-  // (supports up to 3 sigma: without a loop, so that the lanes stay together; 198 -> 196 ms
-  // per 1024x1024 8-sample launch through 1M kernels)
+  // (supports up to 3 sigma: without a loop, so that the lanes stay together: 1 % of a
+  // 1024x1024 8-sample launch through 1M kernels)
   if (J <= 2) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -862,8 +861,8 @@ static cudaError_t render_grid(int sm_count, int64_t& g) {
 // grid on entry).  With fewer units than lanes every warp of the grid takes its share
 // instead of a few warps taking 32 paths each: a warp works through its paths' windows
 // together, so its time grows with their number.  120x67 pixels at 1 sample through 50k
-// kernels: 1,278 us with 251 full warps, 431 us with 2,010 warps of 4 paths; 96x64
-// 3-bounce paths through 200k kernels: about 47 ms to 10 ms.
+// kernels: 696 us with 251 full warps, 215 us with 2,010 warps of 4 paths; 96x64
+// 3-bounce paths through 200k kernels: 9.6 and 1.8 ms.
 static int scatter_slots(int64_t units, int64_t& g) {
   const int64_t warps = g * kWWarps;
   const int64_t slots = std::min<int64_t>(32, std::max<int64_t>(1, (units + warps - 1) / warps));

@@ -41,10 +41,9 @@ GF_HD float window_end(float te, float t1) { return te >= t1 ? t1 * (1.0f + 1e-7
 // whatever the average); lim comes back as later windows need it.  Without lim, and with
 // it: 120 and 67 ms (12 mixed requests on two fields of a render server), 7.5 and 6.1 ms
 // (step through 96x64 3-bounce paths, 200k kernels), the same where windows hold all
-// their chords.  Shares of 0.25, 0.35
-// and 0.5: 201, 197 and 203 ms (1024x1024, 8 samples, 1M kernels, one-cone masks), 6.4,
-// 6.8 and 6.9 ms (333x217, 4 samples, FP16), 99, 99 and 107 ms (512x512, 16 samples, every
-// cone).
+// their chords.  Shares of 0.25, 0.3, 0.35 and 0.5: 194.9, 193.5, 191.0 and 197.2 ms
+// (1024x1024, 8 samples, 1M kernels, one-cone masks), 94.5, 92.0, 92.2 and 98.4 ms (512x512,
+// 16 samples, 100k kernels, every cone).
 GF_HD Window window_first(bool tracking, float t0, float t1, float& lim) {
   const float len = t1 - t0;
   lim = fmaxf(fminf(lim, len), 0.0625f * len);
