@@ -47,7 +47,7 @@ __device__ __forceinline__ int64_t next_ray(const DevField& F, const TrParams& P
 // lanes part at every leaf: each runs its own tree walk and its own rule of 8 to 64
 // nodes.  130,001 rays through 100k kernels (306 chords and 4,092 nodes per ray):
 // 65.0 ms with one ray per lane, 3.8 ms with one per warp; 4,096 rays through 256
-// kernels: 53.6 us over a binary tree, 29 us now.
+// kernels: 53.6 us over a binary tree, 19.4 us now.
 // ---------------------------------------------------------------------------
 template <int MODE>  // GF_TR_DETERMINISTIC or GF_TR_CLOSED_FORM
 __global__ void __launch_bounds__(kBlock, kCoopBlocks)
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(kBlock, kCoopBlocks)
 // buffer at a time; one with more points is halved.  Bound by instruction issue and the
 // latency of tree nodes.  30,000 rays through 100k kernels: 38 ms with one ray per lane
 // (the per-thread tracker traverses twice per eight points, its lanes parted), 1.9 ms now;
-// 4,096 rays through 256 kernels: 27 us (rays dealt out).  With 445 kernels over a point
+// 4,096 rays through 256 kernels: 24.7 us (rays dealt out).  With 445 kernels over a point
 // (14k in all), 130,000 rays: 135 ms with one ray per lane, 742 when windows were halved
 // for their chords and the rest left to one lane, 22 now.
 //
@@ -810,8 +810,8 @@ static int persistent_grid(const Field& F, K kernel, int64_t warps_of_work) {
 template <class K>
 static cudaError_t launch_rays(const Field& F, K kernel, TrParams P, cudaStream_t s) {
   const int64_t g = persistent_grid(F, kernel, P.n);
-  // up to four rays per warp are dealt out: 4,096 rays through 256 kernels take 32.4 us with
-  // the counter (its clearing is a launch of its own), 29.1 us without
+  // up to four rays per warp are dealt out: the counter's clearing is a launch of its own (3 us
+  // of 4,096 rays through 256 kernels)
   P.dealt = P.n <= 4 * g * (kBlock / 32);
   if (!P.dealt) {
     const cudaError_t e = cudaMemsetAsync(P.counter, 0, sizeof(int), s);

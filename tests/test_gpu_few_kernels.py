@@ -185,3 +185,24 @@ def test_few_kernels_take_little_time(api, ctx, mode, limit):
         times.append(a.elapsed_time(b))
     assert sorted(times)[2] <= limit, times
     f.free()
+
+
+def test_work_counters_add_up(api, ctx):
+    """The counters of a call, summed over its warps: a batch in two halves counts what the
+    whole does, and chord counts are those of the chord lists."""
+    f = api.Field(ctx, _field(60, seed=6))
+    o, d, tr = synth.random_rays(6_000, seed=3)
+    od, dd, trd = (torch.from_numpy(a).cuda() for a in (o, d, tr))
+    for mode in ("det", "closed"):
+        f.stats(True)
+        f.transmittance(od, dd, trd, mode=mode)
+        f.sync()
+        whole = f.stats(True)
+        for s in (slice(0, 2_500), slice(2_500, 6_000)):
+            f.transmittance(od[s].contiguous(), dd[s].contiguous(), trd[s].contiguous(), mode=mode)
+        f.sync()
+        parts = f.stats(True)
+        assert all(whole[k] == parts[k] for k in ("rays", "chords", "evals", "nodes", "windows", "leaves"))
+        counts, _, _, _ = f.chords(o, d, tr, cap=64)
+        assert whole["rays"] == 6_000 and whole["chords"] == int(counts.sum())
+    f.free()
