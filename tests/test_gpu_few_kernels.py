@@ -151,6 +151,71 @@ def test_a_smaller_stack_limit_takes_warps(api, ctx):
     f.free()
 
 
+@pytest.mark.parametrize("case", ["plain", "normalised", "clamped", "camera", "foveated"])
+def test_lanes_and_warps_agree_in_every_form(api, ctx, case):
+    """The same calls by lanes and, under a stack limit that only the warps' kernels fit, by
+    warps: ranges and none, host and device buffers, unnormalised directions, sample ranges,
+    stochastic masks, and the fields and cameras of `case`.  Optical depths within 2e-6 max(1,
+    |tau|) (the same terms in another order); flights up to 1 % of the pixels."""
+    n = 12
+    p = _field(n, seed=20)
+    kw = {}
+    if case == "normalised":
+        s3 = np.exp(np.asarray(p["log_scale"], np.float64)).prod(1)
+        p["weight"] = (p["weight"] * (2 * np.pi) ** 1.5 * s3).astype(np.float32)
+        kw["weight_mode"] = "normalized"
+    if case == "clamped":
+        kw["clamp_eps"] = 0.05
+    f = api.Field(ctx, p, **kw)
+    c = synth.DEFAULT_CAMERA
+    cam = api.camera(c["eye"], c["look_at"], c["up"], 55.0, 401, 307)
+    if case == "camera":
+        f.set_lod_camera(api.camera(c["eye"], c["look_at"], c["up"], 55.0, 40, 8))
+    fov = {"gaze": (200.0, 150.0), "f0": 60.0, "slope": 300.0, "smooth": 0.3} if case == "foveated" else None
+    o, d, tr = synth.random_rays(50_001, seed=8)
+    d = (d * np.random.default_rng(1).uniform(0.1, 30.0, (len(d), 1))).astype(np.float32)
+    od, dd, trd = (torch.from_numpy(a).cuda() for a in (o, d, tr))
+
+    def results():
+        out = {}
+        for name, lod, spp in (("all", api.lod(), 1), ("stochastic", api.lod("unif_cv", 7, "is"), 3)):
+            f.set_lod(lod)
+            for mode in ("det", "closed"):
+                _, tau = f.transmittance(od, dd, trd, mode=mode, spp=spp, seed=4)
+                out["tau", name, mode] = tau.cpu()
+                _, tau = f.transmittance(od, dd, None, mode=mode, spp=spp, seed=4)
+                out["tau", name, mode, "no range"] = tau.cpu()
+                T, tau = np.empty(len(o), np.float32), np.empty(len(o), np.float32)
+                f.transmittance(o, d, tr, mode=mode, spp=spp, seed=4, out_T=T, out_tau=tau)
+                out["tau", name, mode, "host"] = torch.from_numpy(tau)
+            out["tau", name, "image"] = f.render(cam, api.render_opts("tomo", 2, first_sample=3, foveation=fov), 5).cpu()
+            for ff in ("cdf", "segment"):
+                ro = api.render_opts("scatter", 2, 2, free_flight=ff, first_sample=1, foveation=fov)
+                out["flight", name, ff] = f.render(cam, ro, 5).cpu()
+        f.sync()
+        return out
+
+    cu = ctypes.CDLL("libcuda.so.1")
+    size = ctypes.c_size_t()
+    lanes = results()
+    assert cu.cuCtxGetLimit(ctypes.byref(size), 0) == 0
+    try:
+        assert cu.cuCtxSetLimit(0, ctypes.c_size_t(512)) == 0
+        low = ctypes.c_size_t()
+        assert cu.cuCtxGetLimit(ctypes.byref(low), 0) == 0 and low.value < 576  # the lanes' frames
+        warps = results()
+    finally:
+        assert cu.cuCtxSetLimit(0, size) == 0
+    for k, a in lanes.items():
+        d = (a - warps[k]).abs()
+        if k[0] == "tau":
+            assert bool((d <= 2e-6 * a.abs().clamp(min=1.0)).all()), (k, float(d.max()))
+            assert float(a.abs().max()) > 0.01
+        else:
+            assert float((d > 1e-4 * a.max()).float().mean()) <= 0.01, k
+    f.free()
+
+
 @pytest.mark.parametrize("ff,limit", [("cdf", 0.8), ("segment", 0.6)])
 def test_few_kernel_flights_take_little_time(api, ctx, ff, limit):
     """A 1024x1024 flight image through 8 kernels: four times what it takes (ms)."""
