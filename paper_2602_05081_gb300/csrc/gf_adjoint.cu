@@ -1550,11 +1550,7 @@ static cudaError_t launch_adjoint(const Field& F, const PathParams& P, AdjointKe
   if ((e = adjoint_grid(F, kernel, smem, g)) != cudaSuccess) return e;
   // (allocated ahead by gf_reserve, else here)
   bool scratch = true;
-  if (bare && (!F.adj || !F.rlist.p)) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    (void)cudaStreamIsCapturing(s, &cap);
-    scratch = cap == cudaStreamCaptureStatusNone;
-  }
+  if (bare && (!F.adj || !F.rlist.p)) scratch = !capturing(s);
   if (scratch && (e = grow_adjoint(F, smem ? rad_scratch(F, g) : tomo_scratch(g), g, s)) != cudaSuccess) {
     if (!bare || e != cudaErrorMemoryAllocation) return e;
     (void)cudaGetLastError();

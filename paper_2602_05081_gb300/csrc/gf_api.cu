@@ -165,23 +165,25 @@ cudaError_t grow(const Field& F, void** p, size_t& have, size_t bytes, cudaStrea
 
 cudaError_t grow_shares(const Field& F, ShareBuf& b, size_t share, int64_t& shares, cudaStream_t s) {
   const int64_t held = b.p ? (int64_t)(b.bytes / share) : 0;
+  const bool cap = capturing(s);
+  if (held > 0 && cap) b.captured = true;
   if (held >= shares) return cudaSuccess;
-  if (held > 0) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    (void)cudaStreamIsCapturing(s, &cap);
-    if (b.scarce || cap != cudaStreamCaptureStatusNone) {
-      shares = held;
-      return cudaSuccess;
-    }
+  if (held > 0 && (b.scarce || cap)) {
+    shares = held;
+    return cudaSuccess;
   }
   for (int64_t k = shares; k > held; k /= 2) {
     void* q = nullptr;
-    const cudaError_t e = F.mem.alloc(&q, share * (size_t)k, s);
+    cudaError_t e = F.mem.alloc(&q, share * (size_t)k, s);
     if (e == cudaSuccess) {
-      // (the buffer before it stays until the field is freed: work in flight and captured
-      // graphs may use it)
+      if (b.p && !b.captured) {
+        // earlier calls (on any stream) may still use the old buffer
+        if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;
+        F.mem.release(b.p, s);
+      }
       b.p = q;
       b.bytes = share * (size_t)k;
+      b.captured = false;
       shares = k;
       return e;
     }

@@ -106,7 +106,8 @@ inline __host__ __device__ int cell_fix_exp(unsigned int mb) {
 struct ShareBuf {
   void* p = nullptr;
   size_t bytes = 0;
-  bool scarce = false;  // more was refused: calls make do with what there is
+  bool scarce = false;    // more was refused: calls make do with what there is
+  bool captured = false;  // a captured graph uses it
 };
 struct Field {
   Ctx ctx;                     // copy: a field outlives the gf_ctx it came from
@@ -222,10 +223,17 @@ cudaError_t ensure_adjoint_lists(const Field& F, cudaStream_t s);
 // grow a field-owned buffer to at least `bytes` (synchronises the device before
 // returning the old one)
 cudaError_t grow(const Field& F, void** p, size_t& have, size_t bytes, cudaStream_t s);
+// whether work on the stream is being captured (nothing may be allocated or waited for)
+inline bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  (void)cudaStreamIsCapturing(s, &st);
+  return st != cudaStreamCaptureStatusNone;
+}
 // `shares` equal shares in b; when the memory is refused, half as many and so on down to one:
 // a kernel of fewer blocks, same results.  Once refused, what is held serves every later
-// call (gf_reserve asks again), and under a stream capture what is held serves anyway; a
-// buffer is never given up for one that might be refused.
+// call (gf_reserve asks again), and under a stream capture what is held serves anyway.  A
+// buffer is given back once its successor exists; one that a captured graph uses stays until
+// the field is freed.
 cudaError_t grow_shares(const Field& F, ShareBuf& b, size_t share, int64_t& shares, cudaStream_t s);
 cudaError_t launch_radiance_backward(const Field& F, const PathParams& P, const float* dLdI,
                                      float* grad, cudaStream_t s);

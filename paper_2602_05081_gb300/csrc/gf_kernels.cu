@@ -881,11 +881,7 @@ static int flight_lists(const Field& F, int64_t& g, cudaStream_t s) {
   int64_t lists = 1;
   while (lists < g) lists *= 2;
   lists = std::min(lists, flight_grid(F));
-  if (F.wscratch.bytes < kFlightShare) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    (void)cudaStreamIsCapturing(s, &cap);
-    if (cap != cudaStreamCaptureStatusNone) return 0;
-  }
+  if (F.wscratch.bytes < kFlightShare && capturing(s)) return 0;
   if (grow_shares(F, F.wscratch, kFlightShare, lists, s) != cudaSuccess) {
     (void)cudaGetLastError();
     return 0;

@@ -185,3 +185,41 @@ def test_tomography_adjoint_without_scratch(api):
             del g
             f.free()
             L.ctx.close()
+
+
+def test_outgrown_scratch_is_given_back(api):
+    """A store that a larger one replaces goes back to the allocator, but for one that a
+    captured graph uses, which stays until the field is freed."""
+    p = synth.octave_field(2000, 4, seed=4)
+    c = synth.DEFAULT_CAMERA
+    cam = api.camera(c["eye"], c["look_at"], c["up"], c["vfov_deg"], 24, 16)
+    flight, delta = api.render_opts("scatter", 1, 1, free_flight="cdf"), api.render_opts("scatter", 1, 1)
+    sizes = {}
+    for captured in (False, True):
+        L = _Limited(api, 1 << 40)
+        al = L.ctx.allocator
+        f = api.Field(L.ctx, p)
+        out = torch.empty(16, 24, device="cuda")
+        f.render(cam, flight, 3, out=out)
+        f.sync()
+        held = al.live_bytes
+        g = torch.cuda.CUDAGraph()
+        if captured:
+            s = torch.cuda.Stream()
+            s.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.graph(g, stream=s):
+                f.render(cam, flight, 3, out=out, stream=s.cuda_stream)
+        before = al.calls_free
+        f.render(cam, delta, 3)
+        f.sync()
+        assert al.calls_free - before == (0 if captured else 1)
+        sizes[captured] = al.live_bytes - held
+        if captured:
+            out.zero_()
+            g.replay()
+            torch.cuda.synchronize()
+            assert float(out.max()) > 0.0
+        del g
+        f.free()
+        L.ctx.close()
+    assert sizes[True] > sizes[False]
