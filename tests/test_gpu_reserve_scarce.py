@@ -223,3 +223,24 @@ def test_outgrown_scratch_is_given_back(api):
         f.free()
         L.ctx.close()
     assert sizes[True] > sizes[False]
+
+
+def test_tomography_adjoint_with_few_lists_takes_the_whole_grid(api):
+    """With lists for a small part of the grid's blocks the tomography adjoint goes without them
+    on every block: a ray is traversed twice."""
+    c = synth.DEFAULT_CAMERA
+    cam = api.camera(c["eye"], c["look_at"], c["up"], c["vfov_deg"], 48, 40)
+    o, dL, n = api.render_opts("tomo", 2), torch.ones(40, 48, device="cuda"), 2000
+    nodes = {}
+    for limit in (1 << 40, 1 << 20):  # 1 MiB: the arrays per kernel and ten blocks' lists
+        L = _Limited(api, 1 << 40)
+        f = api.Field(L.ctx, synth.octave_field(n, 4, seed=4))
+        f.reserve(max_pixels=48 * 40 + 16 * n)
+        L.limit = limit
+        f.stats(True)
+        f.render_backward(cam, o, 4, dL)
+        f.sync()
+        nodes[limit] = f.stats(True)["nodes"]
+        f.free()
+        L.ctx.close()
+    assert nodes[1 << 20] == 2 * nodes[1 << 40]
